@@ -75,7 +75,11 @@ enum {
                                       barriers, and every barrier wait is bounded (a
                                       block that gives up latches KG_ERR_TIMEOUT).  One
                                       thread per monomer; results equal the default
-                                      path's up to binary32 summation order            */
+                                      path's up to binary32 summation order.  A context
+                                      with one thread per monomer and at most 640
+                                      monomers per SM takes resident launches of up to
+                                      50 steps by itself; there the flag raises that to
+                                      1000                                              */
 };
 
 /* One melt (Sec. II.B): N_ch chains of N monomers in a cube of side L. */
@@ -106,7 +110,7 @@ typedef struct {
     unsigned long long seed;  /* key of every counter-based random draw                */
     int sort_interval;        /* MD steps between re-sorts of the per-monomer arrays into
                                  cell order (<= 0: 200), tested at the start of each
-                                 kg_step call and each 10-step graph; KG_FP64 results do
+                                 kg_step call and after each 10 steps; KG_FP64 results do
                                  not depend on it; in KG_MIXED a re-sort forces a Verlet
                                  build, whose timing moves positions at the binary32
                                  rounding level (~1e-7 sigma)                           */

@@ -273,8 +273,9 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
         {   // binary32 prefilter of the Verlet build on cell offsets (k_nlist):
             // the offsets (<= h), the shifted own offset (<= 2h) and the
             // difference (<= 3h) are rounded once each, and h itself once, so a
-            // component is off by at most 9 h 2^-24; the band is twice the
-            // resulting bound on r^2 near the cutoff.
+            // component is off by at most 9 h 2^-24; r^2, and r^2 - nl_hi as one
+            // chain of fused multiply-adds, round at most four times at <= rl^2
+            // 2^-24.  The band is twice the resulting bound near the cutoff.
             const double ec = 9.0 * md.h * std::ldexp(1.0, -24);
             const double er2 = 2.0 * rl * std::sqrt(3.0) * ec + 3.0 * ec * ec + 4.0 * rl * rl * std::ldexp(1.0, -24);
             md.nl_lo = (float)(rl * rl - 2.0 * er2);
@@ -334,7 +335,7 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->recb = (float4 *)A(Mp * sizeof(float4));
     // padded by a cell's worth of records: the list build reads a warp's
     // lockstep candidates past a cell's end without clamping the index
-    c->recs = (float4 *)A((Mp + kg::MAX_CELL_OCC) * sizeof(float4));
+    c->recs = (float4 *)A((Mp + kg::MAX_CELL_OCC + 4) * sizeof(float4));   // + a group of the candidate loop
     c->shtab = (float4 *)A((size_t)kg::SHIFT_SLOTS * kg::MAX_MELTS * sizeof(float4));
     if (c->precision == KG_MIXED) {
         for (int b = 0; b < 2; ++b) {
@@ -375,6 +376,7 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->scratch = (double *)A(7 * Mp * sizeof(double));
     c->flags = (unsigned *)A(16 * sizeof(unsigned));
     c->pbar = (unsigned *)A(4 * sizeof(unsigned));
+    c->resbar = (unsigned long long *)A(kg::resident_words(c->ncell_md));
     c->d_step = (long long *)A(sizeof(long long));
     c->fout = (double *)A(3 * Mp * sizeof(double));
     c->partials_cap = (int)(Mp / 128 + 2) * 5;
@@ -428,6 +430,7 @@ void kg_destroy(kg_ctx *c)
     for (void *b : bufs) dev_free(c, b);
     dev_free(c, c->d_step);
     dev_free(c, c->pbar);
+    dev_free(c, c->resbar);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     kg::graphs_reset(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -531,6 +534,25 @@ kg_status kg_set_potential_schedule(kg_ctx *c, const kg_stage *stages, int n_sta
     return upload_stage(c, c->schedule[0]);
 }
 
+// MD steps until the next re-sort test of a run of `left` steps: the tests sit
+// at the start of the run and after each whole group of steps (PERSIST_STEPS
+// with KG_FLAG_PERSISTENT, then GRAPH_STEPS, then single steps), however many
+// groups one launch covers.
+static int steps_to_sort(const kg_ctx *c, long long left, bool persistent)
+{
+    const long long most = persistent ? kg::PERSIST_MAX : kg::RESIDENT_STEPS;
+    long long n = 0;
+    while (n < left && (n == 0 || c->since_sort + n < c->sort_interval)) {
+        const long long rest = left - n;
+        const long long d = persistent && rest >= kg::PERSIST_STEPS ? kg::PERSIST_STEPS
+                            : rest >= kg::GRAPH_STEPS              ? kg::GRAPH_STEPS
+                                                                   : 1;
+        if (n + d > most) break;
+        n += d;
+    }
+    return (int)n;
+}
+
 kg_status kg_step(kg_ctx *c, long long n_steps)
 {
     if (!c || n_steps < 0) return KG_ERR_INVALID_ARG;
@@ -561,7 +583,14 @@ kg_status kg_step(kg_ctx *c, long long n_steps)
             long long n = 1;
             if (c->sort_after_load)             // after a load: one step builds the cell order to sort into
                 kg::md_step(c);
-            else if (!c->prof_on && (c->p.flags & KG_FLAG_PERSISTENT) && c->precision == KG_MIXED &&
+            else if (!c->prof_on && kg::resident_fits(c)) {
+                n = steps_to_sort(c, chunk - done, (c->p.flags & KG_FLAG_PERSISTENT) != 0);
+                if (kg::resident_launch(c, (int)n, -1, kg::RESIDENT_SPIN) != cudaSuccess) {
+                    cudaGetLastError();
+                    c->resident_failed = true;  // the launches below serve it
+                    continue;
+                }
+            } else if (!c->prof_on && (c->p.flags & KG_FLAG_PERSISTENT) && c->precision == KG_MIXED &&
                 chunk - done >= kg::PERSIST_STEPS && kg::md_persist_steps(c))
                 n = kg::PERSIST_STEPS;
             else if (!c->prof_on && c->use_graphs && chunk - done >= kg::GRAPH_STEPS && kg::md_graph_steps(c, 1))
@@ -592,7 +621,8 @@ kg_status kg_persistent_selftest(kg_ctx *c, int skip_block, unsigned spin)
         kg::set_device_step(c, c->step - 1);
         c->d_step_stale = false;
     }
-    KG_TRY(kg::persist_launch(c, c->stream, c->cur, 2, skip_block, spin));
+    if (kg::resident_fits(c)) KG_TRY(kg::resident_launch(c, 2, skip_block, spin));
+    else KG_TRY(kg::persist_launch(c, c->stream, c->cur, 2, skip_block, spin));
     c->step += 2;
     kg::md_materialize(c);
     return read_flags(c, pinned_flags());

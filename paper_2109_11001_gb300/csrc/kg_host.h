@@ -53,6 +53,9 @@ struct kg_ctx {
     cudaGraphExec_t pexec[2] = {nullptr, nullptr};   // persistent launches (KG_FLAG_PERSISTENT)
     bool persist_failed = false;
     unsigned *pbar = nullptr;    // grid-barrier words of the persistent launch
+    unsigned long long *resbar = nullptr;   // barrier words, error word and segment totals of the resident launch
+    int res_blocks = -1;         // blocks of the resident kernel the GPU holds at once (< 0: not asked yet)
+    bool resident_failed = false;
     bool use_graphs = true;
     long long graph_replays = 0;
     long long sort_interval = 200;
@@ -141,6 +144,9 @@ void dev_free(kg_ctx *c, void *p);
 
 constexpr int GRAPH_STEPS = 10;          // MD steps per captured graph (even)
 constexpr int PERSIST_STEPS = 50;        // MD steps per persistent launch (even)
+constexpr int RESIDENT_STEPS = 50;       // MD steps per resident launch (KG_FLAG_PERSISTENT: PERSIST_MAX)
+constexpr int PERSIST_MAX = 1000;
+constexpr unsigned RESIDENT_SPIN = 1u << 22;  // its barrier polls (a few hundred ns apart) before ERR_TIMEOUT
 constexpr unsigned PERSIST_SPIN = 1u << 24;   // grid-barrier polls (~64 ns apart) before ERR_TIMEOUT
 constexpr int RS = 8;                    // ints per melt in the DB commit-round array
 
@@ -163,6 +169,11 @@ void md_sort(kg_ctx *c);                     // re-sort the state into the last 
 void md_materialize(kg_ctx *c);              // mixed: x <- xb64 + dlt[cur]
 void graphs_reset(kg_ctx *c);                // drop captured step graphs (their arguments changed)
 bool md_persist_steps(kg_ctx *c);            // PERSIST_STEPS steps in one persistent launch (KG_MIXED)
+
+// kg_resident.cu
+bool resident_fits(kg_ctx *c);               // one thread per monomer, every block resident
+cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin);   // K steps in one launch
+size_t resident_words(int ncell);            // bytes of kg_ctx::resbar
 
 // kg_step.cu
 void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur);   // the mixed path's fused step kernel

@@ -346,7 +346,9 @@ __global__ void __launch_bounds__(256) k_bin_md(const SimDev *__restrict__ Sp, d
     if (!flags[1] || flags[0]) return;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= Sp->M) return;
-    bin_md_one(*Sp, s, x, xb64, recb, dcur, pgcur, pcur, xb, cellid, rank, count, slot_of, flags);
+    const unsigned err =
+        bin_md_one(*Sp, s, x, xb64, recb, dcur, pgcur, pcur, xb, cellid, rank, count, slot_of);
+    if (err) atomicOr(flags, err);
 }
 
 // DB grid: cell of each particle from its wrapped position (cells >= 1.3

@@ -29,168 +29,9 @@
 
 #include <cmath>
 
-#include "kg_host.h"
-#include "kg_rebuild.cuh"
+#include "kg_step.cuh"
 
 namespace kg {
-
-struct MeltStep {
-    int off, nc;
-    float h, L, invL, kappa;
-};
-
-struct StepArgs {
-    const float4 *recb;      // build records: offset from the Verlet-cell corner, packed cell coordinates
-    const float4 *dcur;      // displacement since the build (this step)
-    float4 *dnext;           //   ... after this step
-    const float4 *pcur;      // gather records recb + dcur
-    float4 *pnext;           //   ... after this step
-    float *u;                // [3][Mp] velocities v_{n-1/2}
-    const unsigned *nl;      // Verlet list, column-major [maxnb][Mp], entries j | q << IDX_BITS
-    const int *nn;           // list lengths
-    const int *slot_of;      // compute index -> chain-major slot (keys the noise)
-    const int4 *bp;          // compute indices of chain partners s-2, s-1, s+1, s+2 (-1 past an end)
-    unsigned *flags;         // [0] error bits, [1] rebuild request
-    const long long *stepp;  // index of the step being run
-    unsigned long long seed;
-    int M, Mp, n_melts;
-    float rc2, half_skin2;
-    float dt, gamma, amp;    // Langevin: u += dt (F - gamma u + amp g), amp = sqrt(2 gamma T / dt)
-    float c1xn, c2x6, nf;    // fr = (6 c2 r^-6 - n c1 r^-n) / r^2  (U = c1 r^-n - c2 r^-6 + 1)
-    float kf, R0sq, inv_R0sq, qmin, kf_qmin, four_R0sq;   // FENE k_n, R0^2, continuation beyond r*
-    MeltStep melt[MAX_MELTS];
-};
-
-// r^-n from r^2, 1/r^2 and 1/r^6; N4 = 4n (0: any other n, from exp2/log2)
-template <int N4>
-__device__ __forceinline__ float inv_rn(float r2, float ir2, float ir6, float nf)
-{
-    if constexpr (N4 == 0) {
-        return exp2f(-0.5f * nf * log2f(r2));
-    } else if constexpr (N4 == 23) {                 // n = 23/4: r^-6 r^(1/4)
-        return ir6 * sqrtf(sqrtf(sqrtf(r2)));
-    } else if constexpr (N4 == 26) {                 // n = 13/2: r^-6 r^(-1/2)
-        return ir6 * sqrtf(rsqrtf(r2));
-    } else {
-        static_assert(N4 % 4 == 0, "integer n");
-        constexpr int n = N4 / 4;
-        float p;
-        if constexpr (n >= 6) {
-            p = ir6;
-#pragma unroll
-            for (int k = 3; k < n / 2; ++k) p *= ir2;
-        } else {
-            p = ir2;
-#pragma unroll
-            for (int k = 1; k < n / 2; ++k) p *= ir2;
-        }
-        if constexpr (n & 1) p *= rsqrtf(r2);
-        return p;
-    }
-}
-
-// (dU_MLJ^n/dr) / r at r^2 (binary32)
-template <int N4>
-__device__ __forceinline__ float mlj_fr32(const StepArgs &P, float r2)
-{
-    const float ir2 = __fdividef(1.0f, r2);
-    const float ir6 = ir2 * ir2 * ir2;
-    const float rn = inv_rn<N4>(r2, ir2, ir6, P.nf);
-    return __fmul_rn(fmaf(P.c2x6, ir6, -__fmul_rn(P.c1xn, rn)), ir2);
-}
-
-__device__ __forceinline__ int melt_index(const StepArgs &P, int slot)
-{
-    int m = 0;
-    while (m + 1 < P.n_melts && slot >= P.melt[m + 1].off) ++m;
-    return m;
-}
-
-// Arithmetic of the step written with explicit roundings: a sum of two
-// products leaves the compiler a choice of which one to fuse, and the choice
-// can differ between the kernels that inline the step (standalone and
-// persistent), which must give the same bits.  fmaf is always fused,
-// __fmul_rn / __fadd_rn / __fsub_rn never.
-__device__ __forceinline__ float dot3(float3 a, float3 b)
-{
-    return fmaf(a.z, b.z, fmaf(a.y, b.y, __fmul_rn(a.x, b.x)));
-}
-
-__device__ __forceinline__ void axpy3(float a, float3 x, float3 &y)   // y += a x
-{
-    y.x = fmaf(a, x.x, y.x);
-    y.y = fmaf(a, x.y, y.y);
-    y.z = fmaf(a, x.z, y.z);
-}
-
-__device__ __forceinline__ float3 sub3(float3 a, float3 b)
-{
-    return make_float3(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y), __fsub_rn(a.z, b.z));
-}
-
-// a inv - c b: one term of the gradient of cos theta
-__device__ __forceinline__ float3 bend_g(float3 a, float inv, float c, float3 b)
-{
-    return make_float3(fmaf(-c, b.x, __fmul_rn(a.x, inv)), fmaf(-c, b.y, __fmul_rn(a.y, inv)),
-                       fmaf(-c, b.z, __fmul_rn(a.z, inv)));
-}
-
-// Bond (Eq. 10) and bending (Eq. 4) forces on the monomer whose gather
-// record is pi, from its chain partners bp = (s-2, s-1, s+1, s+2).
-template <int N4>
-__device__ __forceinline__ void bonded32(const StepArgs &P, const float4 *__restrict__ pcur, const MeltStep &md,
-                                         float4 pi, int4 bp, float3 &F, unsigned &err)
-{
-    const bool hm2 = bp.x >= 0, hm1 = bp.y >= 0, hp1 = bp.z >= 0, hp2 = bp.w >= 0;
-    float3 rm2 = make_float3(0.f, 0.f, 0.f), rm1 = rm2, rp1 = rm2, rp2 = rm2;
-    if (hm1) rm1 = rec_rel(pi, __ldg(pcur + bp.y), md.nc, md.h, md.L, md.invL);
-    if (hm2) rm2 = rec_rel(pi, __ldg(pcur + bp.x), md.nc, md.h, md.L, md.invL);
-    if (hp1) rp1 = rec_rel(pi, __ldg(pcur + bp.z), md.nc, md.h, md.L, md.invL);
-    if (hp2) rp2 = rec_rel(pi, __ldg(pcur + bp.w), md.nc, md.h, md.L, md.invL);
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-        if (side == 0 ? hm1 : hp1) {
-            const float3 d = side == 0 ? rm1 : rp1;
-            const float r2 = dot3(d, d);
-            float q = 1.0f - r2 * P.inv_R0sq, fr;
-            if (P.qmin > 0.0f && q < P.qmin) {          // continuation beyond r* (kg_params.fene_qmin)
-                fr = P.kf_qmin;
-                if (!(r2 < P.four_R0sq)) err |= ERR_OVERSTRETCH;
-            } else {
-                if (!(r2 < P.R0sq)) err |= ERR_OVERSTRETCH;
-                q = fmaxf(q, 1e-6f);                    // finite even when flagged
-                fr = P.kf * __fdividef(1.0f, q);
-            }
-            const float fl = mlj_fr32<N4>(P, r2);
-            fr += r2 < P.rc2 ? fl : 0.0f;
-            axpy3(fr, d, F);
-        }
-    }
-    const float kap = md.kappa;
-    if (kap != 0.0f) {
-        const float3 Bm2 = sub3(rm1, rm2);
-        const float3 Bm1 = make_float3(-rm1.x, -rm1.y, -rm1.z), B0 = rp1;
-        const float3 Bp1 = sub3(rp2, rp1);
-        if (hm1 && hp1) {                     // vertex s: force kappa (g1 - g2)
-            const float l1 = dot3(Bm1, Bm1), l2 = dot3(B0, B0);
-            const float inv = rsqrtf(__fmul_rn(l1, l2)), cs = __fmul_rn(dot3(Bm1, B0), inv);
-            const float c1 = __fmul_rn(cs, __fdividef(1.0f, l1)), c2 = __fmul_rn(cs, __fdividef(1.0f, l2));
-            axpy3(kap, sub3(bend_g(B0, inv, c1, Bm1), bend_g(Bm1, inv, c2, B0)), F);
-        }
-        if (hp2) {                            // vertex s+1, s its first end: -kappa g1
-            const float l1 = dot3(B0, B0), l2 = dot3(Bp1, Bp1);
-            const float inv = rsqrtf(__fmul_rn(l1, l2)), cs = __fmul_rn(dot3(B0, Bp1), inv);
-            const float c1 = __fmul_rn(cs, __fdividef(1.0f, l1));
-            axpy3(-kap, bend_g(Bp1, inv, c1, B0), F);
-        }
-        if (hm2) {                            // vertex s-1, s its last end: +kappa g2
-            const float l1 = dot3(Bm2, Bm2), l2 = dot3(Bm1, Bm1);
-            const float inv = rsqrtf(__fmul_rn(l1, l2)), cs = __fmul_rn(dot3(Bm2, Bm1), inv);
-            const float c2 = __fmul_rn(cs, __fdividef(1.0f, l2));
-            axpy3(kap, bend_g(Bm2, inv, c2, Bm1), F);
-        }
-    }
-}
 
 constexpr int STEP_ILP = 4;      // Verlet-list entries in flight per lane
 // One tile of blockDim threads (all threads of the block call it together):
@@ -254,7 +95,7 @@ __device__ __forceinline__ void step_tile(const StepArgs &P, int t0, const float
     }
     float4 rb = make_float4(0.f, 0.f, 0.f, 0.f), dc = rb;
     if (live) {
-        if (sub == 0) bonded32<N4>(P, pcur, md, pi, __ldg(P.bp + s), F, err);
+        if (sub == 0) bonded32<N4>(P, [&](int, int j) { return __ldg(pcur + j); }, md, pi, __ldg(P.bp + s), F, err);
         if (sub == TPM - 1)
             gn = gauss3_f(draw(P.seed, m, 0, (unsigned long long)step, (uint32_t)(slot - md.off)));
         rb = __ldg(P.recb + s);
@@ -289,18 +130,6 @@ __device__ __forceinline__ void step_tile(const StepArgs &P, int t0, const float
     // leaves without waiting for the block's longest)
     if (__any_sync(0xffffffffu, rebuild) && lane == 0) atomicOr(P.flags + 1, 1u);
     if (err) atomicOr(P.flags, err);
-}
-
-// per-block setup of the step body: the stencil offsets of the 27 codes,
-// one table per axis
-__device__ __forceinline__ void step_block_setup(float *dk)
-{
-    if (threadIdx.x < 27) {
-        const int q = threadIdx.x;
-        dk[q] = (float)(q % 3 - 1);
-        dk[32 + q] = (float)((q / 3) % 3 - 1);
-        dk[64 + q] = (float)(q / 9 - 1);
-    }
 }
 
 // One MD step of every monomer.  (256, 8): at most 32 registers, full
@@ -467,8 +296,11 @@ __global__ void __launch_bounds__(PERSIST_BLOCK, 5) k_persist(const __grid_const
         const int cur = A.cur0 ^ (it & 1);
         if (snap_s.y) {                                       // Verlet rebuild
             for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < P.M; s += nthreads)
-                bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.pg[cur], nullptr, nullptr, A.cellid, A.rank,
-                           A.ccount, P.slot_of, P.flags);
+            {
+                const unsigned err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.pg[cur], nullptr, nullptr,
+                                                A.cellid, A.rank, A.ccount, P.slot_of);
+                if (err) atomicOr(P.flags, err);
+            }
             if (!grid_sync(A, &ok_s, &snap_s)) return;
             for (int g = blockIdx.x; g < nseg; g += gridDim.x) scan_seg(A, g, wsum);
             if (!grid_sync(A, &ok_s, &snap_s)) return;
@@ -500,7 +332,7 @@ __global__ void __launch_bounds__(PERSIST_BLOCK, 5) k_persist(const __grid_const
 }
 
 // 4n of a stage exponent with its own kernel instantiation, 0 otherwise
-static int n4_of(double n)
+int n4_of(double n)
 {
     const double q = 4.0 * n;
     const int k = (int)std::lround(q);
@@ -520,7 +352,7 @@ static void launch_n4(const StepArgs &a, int tpm, int block, long long M, cudaSt
     else k_step32<N4, 1><<<nb, block, 0, st>>>(a);
 }
 
-static StepArgs step_args(const kg_ctx *c, int cur)
+StepArgs step_args(const kg_ctx *c, int cur)
 {
     const StageDev &sg = c->stage;
     StepArgs a{};
@@ -582,8 +414,6 @@ void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur)
         default: launch_n4<0>(a, tpm, blk, M, st); break;
     }
 }
-
-NlArgs nl_args(const kg_ctx *c);                 // kg_md.cu
 
 template <int N4>
 static cudaError_t launch_persist(const PersistArgs &a, cudaStream_t st)

@@ -3,6 +3,9 @@
 // repeated calls give identical results.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "kg_host.h"
 
 namespace kg {
@@ -191,120 +194,254 @@ void msd_permute(kg_ctx *c, const int *order)
 
 // ---------------------------------------------------------------------------
 // static structure factor (App. A): S(q) = |sum_j exp(i q . r_j)|^2 / M for
-// q = 2 pi (h, k, l) / L.  The phase is reduced to [0, 1) turns in binary64
-// (so unwrapped positions of any size keep their precision) and evaluated by
-// sincospif in binary32; sums are binary64, block trees then block order.
+// q = 2 pi (h, k, l) / L.  The turns of q . r_j are formed exactly: every
+// coordinate once as a 64-bit fraction of the box, u = frac(x / L) 2^64, then
+// h u_x + k u_y + l u_z in integers modulo 2^64, whose upper word is the
+// phase (so unwrapped positions of any size and any (h, k, l) keep their
+// precision).  sincospif evaluates it in binary32; the cosines and sines are
+// summed as integers of 2^-30 (2^-31 rounding, below the binary32 value's own),
+// exactly and in any order.  With the phases, the floor and the sums in
+// binary64 the kernel sat on the binary64 pipe (ten of its operations per pair
+// of a wave vector and a monomer, two lanes a clock): 256 vectors x 80,000
+// monomers took 559 us.
+// A thread takes SQ_Q wave vectors, so a monomer's 24 bytes serve that many.
 // ---------------------------------------------------------------------------
-constexpr int SQ_CHUNKS = 64;
+constexpr int SQ_Q = 4;
 
-__global__ void __launch_bounds__(256) k_sq(const double *__restrict__ x, int Mp, int off, int M, double invL,
-                                           const int *__restrict__ hkl, double *__restrict__ part)
+__global__ void __launch_bounds__(256) k_sq_turns(const double *__restrict__ x, int Mp, int off, int M, double invL,
+                                                 unsigned long long *__restrict__ u, long long *__restrict__ bad)
 {
-    __shared__ double sre[256], sim[256];
-    const int q = blockIdx.x;
-    const double h = hkl[3 * q], k = hkl[3 * q + 1], l = hkl[3 * q + 2];
-    double re = 0.0, im = 0.0;
-    for (int r = blockIdx.y * blockDim.x + threadIdx.x; r < M; r += gridDim.y * blockDim.x) {
-        const int j = off + r;
-        const double t = (h * x[j] + k * x[(size_t)Mp + j] + l * x[2 * (size_t)Mp + j]) * invL;
-        float sn, cs;
-        sincospif(2.0f * (float)(t - floor(t)), &sn, &cs);
-        re += cs;
-        im += sn;
-    }
-    sre[threadIdx.x] = re;
-    sim[threadIdx.x] = im;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            sre[threadIdx.x] += sre[threadIdx.x + w];
-            sim[threadIdx.x] += sim[threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        part[2 * ((size_t)q * gridDim.y + blockIdx.y)] = sre[0];
-        part[2 * ((size_t)q * gridDim.y + blockIdx.y) + 1] = sim[0];
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= M) return;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const double t = x[(size_t)d * Mp + off + r] * invL;
+        if (!isfinite(t)) *bad = 1;                        // S is then not a number
+        u[(size_t)d * M + r] = __double2ull_rz((t - floor(t)) * 18446744073709551616.0);
     }
 }
 
-__global__ void __launch_bounds__(256) k_sq_sum(const double *__restrict__ part, int nq, int G, int M,
+__global__ void __launch_bounds__(256) k_sq(const unsigned long long *__restrict__ u, int M,
+                                           const int *__restrict__ hkl, int nq, long long *__restrict__ part)
+{
+    const int q0 = blockIdx.x * SQ_Q;
+    long long h[SQ_Q], k[SQ_Q], l[SQ_Q], re[SQ_Q], im[SQ_Q];
+#pragma unroll
+    for (int i = 0; i < SQ_Q; ++i) {
+        const int q = min(q0 + i, nq - 1);
+        h[i] = hkl[3 * q];
+        k[i] = hkl[3 * q + 1];
+        l[i] = hkl[3 * q + 2];
+        re[i] = im[i] = 0;
+    }
+    for (int r = blockIdx.y * blockDim.x + threadIdx.x; r < M; r += gridDim.y * blockDim.x) {
+        const unsigned long long ux = u[r], uy = u[(size_t)M + r], uz = u[2 * (size_t)M + r];
+#pragma unroll
+        for (int i = 0; i < SQ_Q; ++i) {
+            const unsigned long long t = (unsigned long long)h[i] * ux + (unsigned long long)k[i] * uy +
+                                         (unsigned long long)l[i] * uz;
+            float sn, cs;
+            sincospif((float)(int)(t >> 32) * 4.656612873077392578125e-10f, &sn, &cs);   // half turns: 2^-31
+            re[i] += __float2int_rn(cs * 1073741824.0f);
+            im[i] += __float2int_rn(sn * 1073741824.0f);
+        }
+    }
+    __shared__ long long sum[2 * SQ_Q];
+    if (threadIdx.x < 2 * SQ_Q) sum[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SQ_Q; ++i) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            re[i] += __shfl_down_sync(0xffffffffu, re[i], o);
+            im[i] += __shfl_down_sync(0xffffffffu, im[i], o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd((unsigned long long *)sum + 2 * i, (unsigned long long)re[i]);
+            atomicAdd((unsigned long long *)sum + 2 * i + 1, (unsigned long long)im[i]);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * SQ_Q && q0 + (int)threadIdx.x / 2 < nq)
+        atomicAdd((unsigned long long *)part + 2 * q0 + threadIdx.x, (unsigned long long)sum[threadIdx.x]);
+}
+
+// part[2 nq]: a position was not finite
+__global__ void __launch_bounds__(256) k_sq_sum(const long long *__restrict__ part, int nq, int M,
                                                double *__restrict__ S)
 {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= nq) return;
-    double re = 0.0, im = 0.0;
-    for (int g = 0; g < G; ++g) {
-        re += part[2 * ((size_t)q * G + g)];
-        im += part[2 * ((size_t)q * G + g) + 1];
-    }
-    S[q] = (re * re + im * im) / (double)M;
+    const double re = (double)part[2 * q] * 9.31322574615478515625e-10, im = (double)part[2 * q + 1] * 9.31322574615478515625e-10;
+    S[q] = part[2 * nq] ? nan("") : (re * re + im * im) / (double)M;
 }
 
-void sq_eval(kg_ctx *c, int melt, const int *hkl_dev, int nq, double *part_dev, double *S_dev)
+// part_dev: 2 nq + 1 zeroed integers
+void sq_eval(kg_ctx *c, int melt, const int *hkl_dev, int nq, long long *part_dev, double *S_dev)
 {
     const MeltDev &md = c->sim.melt[melt];
-    c->launches += 2;
-    k_sq<<<dim3(nq, SQ_CHUNKS), 256, 0, c->stream>>>(c->x, c->Mp, md.off, md.M, md.invL, hkl_dev, part_dev);
-    k_sq_sum<<<(nq + 255) / 256, 256, 0, c->stream>>>(part_dev, nq, SQ_CHUNKS, md.M, S_dev);
+    c->launches += 3;
+    unsigned long long *u = (unsigned long long *)c->scratch;
+    k_sq_turns<<<nb256(md.M), 256, 0, c->stream>>>(c->x, c->Mp, md.off, md.M, md.invL, u, part_dev + 2 * nq);
+    const int nqb = (nq + SQ_Q - 1) / SQ_Q;                // about eight blocks per SM in all
+    const int chunks = std::max(1, std::min(nb256(md.M), 152 * 8 / nqb));
+    k_sq<<<dim3(nqb, chunks), 256, 0, c->stream>>>(u, md.M, hkl_dev, nq, part_dev);
+    k_sq_sum<<<nb256(nq), 256, 0, c->stream>>>(part_dev, nq, md.M, S_dev);
 }
 
 // ---------------------------------------------------------------------------
-// pair distribution (App. A): ordered pairs i != j with minimum-image
-// distance r < r_max, counted in bins of width dr, on the double-bridging cell
-// grid (cells >= 1.3 sigma, stencil of +-R cells, each cell once).  The
-// distance is the binary64 expression ((dx*dx + dy*dy) + dz*dz), dx = d - L
-// rint(d/L), its IEEE square root and bin floor(r / dr): integer counts, so
-// the histogram does not depend on the order of the additions.
+// pair distribution (App. A): pairs with minimum-image distance r < r_max,
+// counted in bins of width dr, on the double-bridging cell grid (cells >= 1.3
+// sigma, stencil of +-R cells).  A pair's bin is by definition that of the
+// binary64 expression ((dx*dx + dy*dy) + dz*dz), dx = d - L rint(d/L), its IEEE
+// square root and floor(r / dr).  The binary32 records on that grid (offset
+// from the cell corner and cell coordinates) settle it for every pair whose
+// r / dr is further than tol from an integer, tol bounding their rounding;
+// only the others (~6e-4 of them at dr = 0.01) take the binary64 expression,
+// whose divides and square root cost ~100 operations at two lanes a clock:
+// with every candidate in binary64 80,000 monomers at r_max = 3 took 11.4 ms.
+// Counts are integers, so neither the order nor the two kinds of decision
+// show.  Both calls of App. A there (this and 256 wave vectors): 12.1 -> 0.28 ms.
+// One thread per monomer in cell order and group of stencil rows: the grid is
+// numbered x first, so a row of 2R + 1 cells is one run of records (two where
+// it wraps), read in order.  Each pair is counted once, from the half stencil
+// (in small boxes, whose rows hold every cell, from the lower position).
 // ---------------------------------------------------------------------------
 constexpr int GR_MAX_BINS = 2048;
 
-__global__ void __launch_bounds__(256) k_gr(const SimDev *__restrict__ Sp, int melt, const double *__restrict__ x,
-                                           const int *__restrict__ cell, const int *__restrict__ start,
-                                           const int *__restrict__ list, int R, double r_max, double dr,
-                                           int nbins, unsigned long long *__restrict__ hist)
+struct GrArgs {
+    const float4 *rec;           // records in cell order
+    const int *start, *list;     // cell starts; compute index of each position
+    const double *x;
+    int off, M, Mp, n, cell0, R, nrow, nbins;
+    bool all;                    // 2R + 1 >= n: every row holds every cell
+    float h, L, invL, inv_dr, tol, cut2;
+    double Ld, r_max, dr;
+    unsigned long long *hist;
+};
+
+__global__ void __launch_bounds__(256) k_gr_sort(const float4 *__restrict__ rec, const int *__restrict__ list, int n,
+                                                float4 *__restrict__ out)
 {
-    __shared__ unsigned int sh[GR_MAX_BINS];
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) sh[b] = 0u;
-    __syncthreads();
-    const SimDev &S = *Sp;
-    const MeltDev &md = S.melt[melt];
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < md.M) {
-        const int i = md.off + r, n = md.ndb;
-        const int c0 = cell[i] - md.dbcell_off;
-        const int cx = c0 % n, cy = (c0 / n) % n, cz = c0 / (n * n);
-        const int w = 2 * R + 1 < n ? 2 * R + 1 : n;         // each cell of the stencil once
-        const int o = 2 * R + 1 < n ? -R : 0;
-        for (int a = 0; a < w; ++a)
-            for (int b = 0; b < w; ++b)
-                for (int e = 0; e < w; ++e) {
-                    const int zz = 2 * R + 1 < n ? ((cz + o + a) % n + n) % n : a;
-                    const int yy = 2 * R + 1 < n ? ((cy + o + b) % n + n) % n : b;
-                    const int xx = 2 * R + 1 < n ? ((cx + o + e) % n + n) % n : e;
-                    const int cc = md.dbcell_off + (zz * n + yy) * n + xx;
-                    for (int k = start[cc]; k < start[cc + 1]; ++k) {
-                        const int j = list[k];
-                        if (j == i) continue;
-                        const double rr = sqrt(dist2_exact(x, S.Mp, md.L, i, j));
-                        if (!(rr < r_max)) continue;
-                        const int bin = (int)__ddiv_rn(rr, dr);
-                        if (bin < nbins) atomicAdd(&sh[bin], 1u);
-                    }
-                }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x)
-        if (sh[b]) atomicAdd(hist + b, (unsigned long long)sh[b]);
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < n) out[p] = rec[list[p]];
 }
 
+// bin of a pair by the binary64 definition (-1: none)
+__device__ __noinline__ int gr_exact(const GrArgs &A, int p, int k)
+{
+    const double r = sqrt(dist2_exact(A.x, A.Mp, A.Ld, A.list[p], A.list[k]));
+    return r < A.r_max ? (int)__ddiv_rn(r, A.dr) : -1;
+}
+
+__global__ void __launch_bounds__(256) k_gr(const __grid_constant__ GrArgs A)
+{
+    __shared__ unsigned int sh[GR_MAX_BINS];
+    for (int b = threadIdx.x; b < A.nbins; b += blockDim.x) sh[b] = 0u;
+    __syncthreads();
+    const int p = A.off + blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < A.off + A.M) {
+        const float4 ri = A.rec[p];
+        const unsigned code = __float_as_uint(ri.w);
+        const int cx = (int)(code & CODE_MASK), cy = (int)((code >> CODE_BITS) & CODE_MASK);
+        const int cz = (int)(code >> (2 * CODE_BITS)), n = A.n, R = A.R, w = 2 * R + 1;
+        float oy = 0.f, oz = 0.f;
+        // records [k0, k1), seen at cell x - cxs from the own one
+        auto run = [&](int k0, int k1, int cxs) {
+            for (int k = k0; k < k1; ++k) {
+                const float4 r = __ldg(A.rec + k);
+                const int dc = (int)(__float_as_uint(r.w) & CODE_MASK) - cxs;
+                float ex = fmaf((float)dc, A.h, r.x - ri.x), ey = r.y - oy, ez = r.z - oz;
+                if (A.all) {
+                    ex -= A.L * rintf(ex * A.invL);
+                    ey -= A.L * rintf(ey * A.invL);
+                    ez -= A.L * rintf(ez * A.invL);
+                }
+                const float r2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
+                if (r2 < A.cut2) {
+                    const float t = sqrtf(r2) * A.inv_dr;
+                    int b = (int)t;
+                    const float f = t - (float)b;
+                    if (f < A.tol || f > 1.0f - A.tol) b = gr_exact(A, p, k);
+                    if ((unsigned)b < (unsigned)A.nbins) atomicAdd(&sh[b], 1u);
+                }
+            }
+        };
+        for (int row = blockIdx.y; row < A.nrow; row += gridDim.y) {
+            int dy, dz, yy, zz;
+            if (A.all) {
+                zz = row / n;
+                yy = row - zz * n;
+                dz = wrap_dk(zz - cz, n);
+                dy = wrap_dk(yy - cy, n);
+            } else {                                 // dz = 0: dy = 0..R; dz = 1..R: dy = -R..R
+                dz = row <= R ? 0 : 1 + (row - R - 1) / w;
+                dy = row <= R ? row : (row - R - 1) % w - R;
+                zz = cz + dz >= n ? cz + dz - n : cz + dz;
+                yy = cy + dy;
+                yy = yy < 0 ? yy + n : (yy >= n ? yy - n : yy);
+            }
+            oy = fmaf((float)-dy, A.h, ri.y);
+            oz = fmaf((float)-dz, A.h, ri.z);
+            const int *start = A.start + A.cell0 + (zz * n + yy) * n;
+            if (A.all) {
+                run(max(start[0], p + 1), start[n], cx);
+            } else {
+                const bool own = row == 0;           // the own row: behind p in its cell, then the cells after it
+                const int xa = own ? cx : cx - R, xb = cx + R;
+                const int k0 = start[max(xa, 0)], k1 = start[min(xb, n - 1) + 1];
+                run(own ? max(k0, p + 1) : k0, k1, cx);
+                if (xa < 0) run(start[n + xa], start[n], cx + n);
+                if (xb >= n) run(start[0], start[xb - n + 1], cx - n);
+            }
+        }
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < A.nbins; b += blockDim.x)
+        if (sh[b]) atomicAdd(A.hist + b, (unsigned long long)sh[b]);
+}
+
+// hist_dev: nbins zeroed counts; receives the unordered pairs of each bin
 void gr_eval(kg_ctx *c, int melt, int R, double r_max, double dr, int nbins, unsigned long long *hist_dev)
 {
     const MeltDev &md = c->sim.melt[melt];
-    ++c->launches;
-    cudaMemsetAsync(hist_dev, 0, sizeof(unsigned long long) * nbins, c->stream);
-    k_gr<<<nb256(md.M), 256, 0, c->stream>>>(c->d_sim, melt, c->x, c->dbcell, c->dbstart, c->dblist, R, r_max,
-                                             dr, nbins, hist_dev);
+    c->launches += 2;
+    k_gr_sort<<<nb256(c->M), 256, 0, c->stream>>>(c->dbrec, c->dblist, c->M, c->recs);   // recs: free between builds
+    GrArgs a{};
+    a.rec = c->recs;
+    a.start = c->dbstart;
+    a.list = c->dblist;
+    a.x = c->x;
+    a.off = md.off;
+    a.M = md.M;
+    a.Mp = c->Mp;
+    a.n = md.ndb;
+    a.cell0 = md.dbcell_off;
+    a.all = 2 * R + 1 >= md.ndb;
+    a.R = R;
+    a.nrow = a.all ? md.ndb * md.ndb : (R + 1) + R * (2 * R + 1);
+    a.nbins = nbins;
+    a.h = md.hdbf;
+    a.L = md.Lf;
+    a.invL = md.invLf;
+    a.Ld = md.L;
+    a.r_max = r_max;
+    a.dr = dr;
+    a.hist = hist_dev;
+    // A component adds two offsets (rounded at <= h 2^-24 each), up to Rm + 1
+    // cell sides (h itself rounded) and two roundings of a value below (Rm + 2)
+    // h, in small boxes an image of L as well; the square root and r / dr add a
+    // few roundings of r.  Twice that bound decides.
+    const double Rm = a.all ? md.ndb : R, ulp = std::ldexp(1.0, -24);
+    const double ec = (3.0 * Rm + 7.0) * md.hdb * ulp + (a.all ? 3.0 * md.L * ulp : 0.0);
+    const double er = 2.0 * (std::sqrt(3.0) * ec + 4.0 * r_max * ulp);
+    a.inv_dr = (float)(1.0 / dr);
+    a.tol = (float)std::min(1.0, er / dr + 4.0 * nbins * ulp);
+    a.cut2 = (float)((r_max + er) * (r_max + er) * 1.000001);
+    const int nb = nb256(md.M);
+    // rows over blocks until about eight blocks per SM are in flight
+    const int split = std::max(1, std::min(a.nrow, 152 * 8 / nb));
+    k_gr<<<dim3(nb, split), 256, 0, c->stream>>>(a);
 }
 
 // <R^2(n)> without any allocation (kg_r2n_noalloc)

@@ -10,95 +10,305 @@
 
 namespace kg {
 
-// One block per chain: the chain's unwrapped positions in shared memory;
-// thread t accumulates sum_i |x_{i+n} - x_i|^2 for n = t+1, t+1+blockDim, ...
+// <R^2(n)> of one chain and a share of its lags (block (c, y) of gridDim.y):
+// sum_i |x_{i+n} - x_i|^2 for every lag n.  In binary64 the three differences
+// and three fused multiply-adds of a pair are 96 clocks of an SM's binary64
+// pipe per warp (two lanes a clock), and nothing else counts: 500 chains of
+// 800 took 2584 us, and take 518 us here (the wide integer multiplies bound it).  Here a chain's positions become 53-bit integers t = (x -
+// x_0) 2^(52-e), 2^e above the chain's extent, split as t = 2^30 hi + lo, and a
+// pair's t^2 = 2^60 dhi^2 + 2^31 dhi dlo + dlo^2 is three products a component,
+// accumulated as 64-bit integers: dhi^2 exactly, dhi dlo exactly (moved to
+// binary64 every R2N_CHUNK terms, before it can overflow), dlo^2 from the upper
+// 22 of its 30 bits (2^-21 of a unit of dhi^2).  The quantum, 2^(e-52), is of
+// the order of one binary64 ulp at the chain's extent.
+// A thread takes R2N_W consecutive lags at once: monomer i + n0 + k serves lag
+// k of step i and lag k - 1 of step i + 1, so one shared-memory read of a
+// position (six words, each array padded by one word in 32 against bank
+// conflicts between lanes four monomers apart) serves R2N_W pairs.  The window
+// at the short end of the lags and its mirror image at the long end go to
+// the same thread, so threads have equal work.
+// A chain with a position that is not finite takes binary64, which says so.
 // The row stride Mp is 64-bit: a caller's rows may sit 2^30 or more doubles
 // apart, and every index into x is formed in 64-bit arithmetic.
-__global__ void __launch_bounds__(256) k_r2n_chain(const double *__restrict__ x, long long Mp, int off, int N,
-                                                  double *__restrict__ out /* [n_ch][N] */,
-                                                  const int *__restrict__ comp_of /* NULL: slot order */)
+constexpr int R2N_W = 4, R2N_CHUNK = 256, R2N_THREADS = 128;
+
+// words of one of the six arrays of a chain of N monomers; sh: padding shift (31: none, the longest chains)
+__host__ __device__ __forceinline__ int r2n_words(int N, int sh) { return N + (N >> sh); }
+
+__global__ void __launch_bounds__(R2N_THREADS) k_r2n_chain(const double *__restrict__ x, long long Mp, int off, int N,
+                                                          double *__restrict__ out /* [n_ch][N] */,
+                                                          const int *__restrict__ comp_of /* NULL: slot order */,
+                                                          int sh)
 {
-    extern __shared__ double pos[];          // 3N
-    const int c = blockIdx.x;
+    extern __shared__ __align__(16) int words[];   // hi x, y, z, lo x, y, z (first the warps' extents)
+    static_assert(2 * 24 >= 8 * (R2N_THREADS / 32), "the extents fit the shortest chain's words");
+    double *ext_s = reinterpret_cast<double *>(words);
+    const int c = blockIdx.x, P = r2n_words(N, sh);
     const long long base = (long long)off + (long long)c * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    const long long j0 = comp_of ? (long long)comp_of[base] : base;
+    const double o[3] = {x[j0], x[Mp + j0], x[2 * Mp + j0]};
+    double ext = 0.0;
+    bool bad = false;
+    for (int i = threadIdx.x; i < N; i += R2N_THREADS) {
         const long long j = comp_of ? (long long)comp_of[base + i] : base + i;
-        pos[i] = x[j];
-        pos[N + i] = x[Mp + j];
-        pos[2 * N + i] = x[2 * Mp + j];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double t = fabs(x[d * Mp + j] - o[d]);
+            bad |= !isfinite(t);
+            ext = fmax(ext, t);
+        }
     }
-    __syncthreads();
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-        double s = 0.0;
-        if (n > 0)
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) ext = fmax(ext, __shfl_xor_sync(0xffffffffu, ext, w));
+    if ((threadIdx.x & 31) == 0) ext_s[threadIdx.x >> 5] = ext;
+    bad = __syncthreads_or(bad);
+#pragma unroll
+    for (int w = 0; w < R2N_THREADS / 32; ++w) ext = fmax(ext, ext_s[w]);
+    __syncthreads();                                // before the words replace them
+    if (blockIdx.y == 0 && threadIdx.x == 0) out[(size_t)c * N] = 0.0;
+    if (bad || ext < 1e-200 || ext > 1e200) {       // not finite, a point, or past the scaling's range
+        for (int n = 1 + blockIdx.y * R2N_THREADS + threadIdx.x; n < N; n += gridDim.y * R2N_THREADS) {
+            double s = 0.0;
             for (int i = 0; i + n < N; ++i) {
-                const double dx = pos[i + n] - pos[i], dy = pos[N + i + n] - pos[N + i],
-                             dz = pos[2 * N + i + n] - pos[2 * N + i];
+                const long long p = comp_of ? (long long)comp_of[base + i] : base + i;
+                const long long q = comp_of ? (long long)comp_of[base + i + n] : base + i + n;
+                const double dx = x[q] - x[p], dy = x[Mp + q] - x[Mp + p], dz = x[2 * Mp + q] - x[2 * Mp + p];
                 s += dx * dx + dy * dy + dz * dz;
             }
-        out[(size_t)c * N + n] = s;
+            out[(size_t)c * N + n] = s;
+        }
+        return;
     }
+    const int e = ilogb(ext) + 1;
+    const double scale = scalbn(1.0, 52 - e);
+    for (int i = threadIdx.x; i < N; i += R2N_THREADS) {
+        const long long j = comp_of ? (long long)comp_of[base + i] : base + i;
+        const int w = i + (i >> sh);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const long long t = __double2ll_rn((x[d * Mp + j] - o[d]) * scale);
+            words[d * P + w] = (int)(t >> 30);
+            words[(3 + d) * P + w] = (int)(t & ((1 << 30) - 1));
+        }
+    }
+    __syncthreads();
+    const double unit = scalbn(1.0, 2 * (e - 52) + 30);
+    const int nwin = (N - 1 + R2N_W - 1) / R2N_W;   // windows of lags 1 + R2N_W w ...
+    auto get = [&](int i, int *p) {
+        const int w = i + (i >> sh);
+#pragma unroll
+        for (int d = 0; d < 6; ++d) p[d] = words[d * P + w];
+    };
+    for (int u = blockIdx.y * R2N_THREADS + threadIdx.x; 2 * u < nwin; u += gridDim.y * R2N_THREADS)
+        for (int half = 0; half < 2; ++half) {
+            const int w = half ? nwin - 1 - u : u;
+            if (half && w == u) break;
+            const int n0 = 1 + R2N_W * w;
+            long long hh[R2N_W], hl[R2N_W], ll[R2N_W];
+            double mid[R2N_W];
+            int ring[R2N_W][6];                      // monomers i + n0 ... i + n0 + 3, at (i + k) % 4
+#pragma unroll
+            for (int k = 0; k < R2N_W; ++k) {
+                hh[k] = hl[k] = ll[k] = 0;
+                mid[k] = 0.0;
+                if (k) get(min(n0 + k - 1, N - 1), ring[k - 1]);
+            }
+            auto pair = [&](int k, const int *a, const int *b) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const int dh = b[d] - a[d], dl = b[3 + d] - a[3 + d], dq = dl >> 8;
+                    hh[k] += (long long)dh * dh;
+                    hl[k] += (long long)dh * dl;
+                    ll[k] += (long long)dq * dq;
+                }
+            };
+            const int full = max(0, N - n0 - (R2N_W - 1));      // steps whose R2N_W lags all end in the chain
+            int i = 0;
+            for (; i + R2N_W <= full; i += R2N_W) {
+#pragma unroll
+                for (int r = 0; r < R2N_W; ++r) {
+                    int a[6];
+                    get(i + r, a);
+                    get(i + r + n0 + R2N_W - 1, ring[(r + R2N_W - 1) % R2N_W]);
+#pragma unroll
+                    for (int k = 0; k < R2N_W; ++k) pair(k, a, ring[(r + k) % R2N_W]);
+                }
+                if ((i & (R2N_CHUNK - 1)) == R2N_CHUNK - R2N_W) {
+#pragma unroll
+                    for (int k = 0; k < R2N_W; ++k) {
+                        mid[k] += (double)hl[k];
+                        hl[k] = 0;
+                    }
+                }
+            }
+            for (; i + n0 < N; ++i) {                // the ends, lag by lag (at most 2 R2N_W - 2 steps)
+                int a[6], p[6];
+                get(i, a);
+#pragma unroll
+                for (int k = 0; k < R2N_W; ++k)
+                    if (i + n0 + k < N) {
+                        get(i + n0 + k, p);
+                        pair(k, a, p);
+                    }
+            }
+#pragma unroll
+            for (int k = 0; k < R2N_W; ++k)
+                if (n0 + k < N)
+                    out[(size_t)c * N + n0 + k] =
+                        ((double)hh[k] * 1073741824.0 + (2.0 * (mid[k] + (double)hl[k]) + (double)ll[k] * 6.103515625e-05)) *
+                        unit;                                // 2^30, 2^-14
+        }
 }
 
-// column sums over chains, in chain order, divided by the number of pairs
-__global__ void __launch_bounds__(256) k_r2n_reduce(const double *__restrict__ in, int n_ch, int N,
-                                                   double *__restrict__ out)
+// column sums over chains divided by the number of pairs: R2N_ROWS partial
+// sums of every R2N_ROWS-th chain in order, then a fixed tree (500 x 800: 43 ->
+// 8 us against one thread per column)
+constexpr int R2N_ROWS = 16;
+
+__global__ void __launch_bounds__(32 * R2N_ROWS) k_r2n_reduce(const double *__restrict__ in, int n_ch, int N,
+                                                             double *__restrict__ out)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+    __shared__ double sh[R2N_ROWS][33];
+    const int n = blockIdx.x * 32 + threadIdx.x;
     double s = 0.0;
-    for (int c = 0; c < n_ch; ++c) s += in[(size_t)c * N + n];
-    out[n] = n == 0 ? 0.0 : s / ((double)n_ch * (double)(N - n));
+    if (n < N)
+        for (int c = threadIdx.y; c < n_ch; c += R2N_ROWS) s += in[(size_t)c * N + n];
+    sh[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    for (int w = R2N_ROWS / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.y < w) sh[threadIdx.y][threadIdx.x] += sh[threadIdx.y + w][threadIdx.x];
+        __syncthreads();
+    }
+    if (threadIdx.y == 0 && n < N)
+        out[n] = n == 0 ? 0.0 : sh[0][threadIdx.x] / ((double)n_ch * (double)(N - n));
+}
+
+// bond-length and cos(theta) counts.  A value's bin is by definition that of
+// the binary64 expressions below (min_image_exact and IEEE square roots and
+// divides: about 170 binary64 operations a monomer, 180 us for 400,000
+// monomers).  The bond vector itself is the plain difference whenever no
+// component is near half a box, so three subtractions stay; length and cosine
+// in binary32 settle the bin unless they are within their rounding of an
+// edge.  Counts go to shared memory first (bins up to HIST_SHARED).  18 us.
+constexpr int HIST_SHARED = 4096;
+
+struct Bond64 {
+    double v[3];
+};
+
+__device__ __noinline__ int hist_bond_exact(Bond64 b, double R0, int nbins)
+{
+    const double len = sqrt(b.v[0] * b.v[0] + b.v[1] * b.v[1] + b.v[2] * b.v[2]);
+    const int k = (int)floor(len / R0 * nbins);
+    return k >= 0 && k < nbins ? k : -1;
+}
+
+__device__ __noinline__ int hist_cos_exact(Bond64 a, Bond64 b, int nbins)
+{
+    const double cs = (a.v[0] * b.v[0] + a.v[1] * b.v[1] + a.v[2] * b.v[2])
+                      / (sqrt(a.v[0] * a.v[0] + a.v[1] * a.v[1] + a.v[2] * a.v[2])
+                         * sqrt(b.v[0] * b.v[0] + b.v[1] * b.v[1] + b.v[2] * b.v[2]));
+    const int k = (int)floor((cs + 1.0) * 0.5 * nbins);
+    return k < 0 ? 0 : (k >= nbins ? nbins - 1 : k);
 }
 
 __global__ void __launch_bounds__(256) k_hist(const double *__restrict__ x, int Mp, int off, int M, int N,
                                              double L, double R0, int nbins, int *__restrict__ bond_h,
                                              int *__restrict__ cos_h, const int *__restrict__ comp_of)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= M) return;
-    const int s = off + r, i = r % N;
-    const int j0 = comp_of[s], jm = i >= 1 ? comp_of[s - 1] : j0, jp = i + 1 < N ? comp_of[s + 1] : j0;
-    double b1[3], b2[3];
-    if (i + 1 < N) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) b2[k] = min_image_exact(x[k * Mp + jp] - x[k * Mp + j0], L);
-        const double len = sqrt(b2[0] * b2[0] + b2[1] * b2[1] + b2[2] * b2[2]);
-        const int b = (int)floor(len / R0 * nbins);
-        if (b >= 0 && b < nbins) atomicAdd(bond_h + b, 1);
+    __shared__ int sh[2 * HIST_SHARED];
+    const bool local = nbins <= HIST_SHARED;
+    int *hb = local ? sh : bond_h, *hc = local ? sh + nbins : cos_h;
+    if (local) {
+        for (int b = threadIdx.x; b < 2 * nbins; b += blockDim.x) sh[b] = 0;
+        __syncthreads();
     }
-    if (i >= 1 && i + 1 < N) {
+    const float half = (float)(0.49 * L), binsf = (float)nbins, per = (float)((double)nbins / R0);
+    // rounding of the binary32 length (relative 3 2^-24, and the bin's) and cosine (absolute 12 2^-24), in bins, doubled
+    const float ulp = 5.9604644775390625e-8f, tol = 32.0f * binsf * ulp;
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < M; r += gridDim.x * blockDim.x) {
+        const int s = off + r, i = r % N;
+        const int j0 = comp_of[s], jm = i >= 1 ? comp_of[s - 1] : j0, jp = i + 1 < N ? comp_of[s + 1] : j0;
+        auto bond = [&](int from, int to, Bond64 &b, float3 &f) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) b1[k] = min_image_exact(x[k * Mp + j0] - x[k * Mp + jm], L);
-        const double cs = (b1[0] * b2[0] + b1[1] * b2[1] + b1[2] * b2[2])
-                          / (sqrt(b1[0] * b1[0] + b1[1] * b1[1] + b1[2] * b1[2])
-                             * sqrt(b2[0] * b2[0] + b2[1] * b2[1] + b2[2] * b2[2]));
-        int b = (int)floor((cs + 1.0) * 0.5 * nbins);
-        b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
-        atomicAdd(cos_h + b, 1);
+            for (int k = 0; k < 3; ++k) b.v[k] = x[(size_t)k * Mp + to] - x[(size_t)k * Mp + from];
+            f = make_float3((float)b.v[0], (float)b.v[1], (float)b.v[2]);
+            if (!(fmaxf(fmaxf(fabsf(f.x), fabsf(f.y)), fabsf(f.z)) < half)) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) b.v[k] = min_image_exact(b.v[k], L);
+                f = make_float3((float)b.v[0], (float)b.v[1], (float)b.v[2]);
+            }
+        };
+        if (i + 1 >= N) continue;
+        Bond64 b2;
+        float3 f2;
+        bond(j0, jp, b2, f2);
+        const float l2 = fmaf(f2.z, f2.z, fmaf(f2.y, f2.y, f2.x * f2.x));
+        {
+            const float t = sqrtf(l2) * per;
+            int b = t < 2.0f * binsf ? (int)t : nbins;
+            const float q = t - (float)b;
+            // every value below two histogram widths that sits near an edge, and anything not comparable
+            if (!(t >= 2.0f * binsf) && !(q > tol && q < 1.0f - tol)) b = hist_bond_exact(b2, R0, nbins);
+            if (b >= 0 && b < nbins) atomicAdd(hb + b, 1);
+        }
+        if (i >= 1) {
+            Bond64 b1;
+            float3 f1;
+            bond(jm, j0, b1, f1);
+            const float l1 = fmaf(f1.z, f1.z, fmaf(f1.y, f1.y, f1.x * f1.x));
+            const float cs = fmaf(f1.z, f2.z, fmaf(f1.y, f2.y, f1.x * f2.x)) * rsqrtf(l1) * rsqrtf(l2);
+            const float t = (cs + 1.0f) * 0.5f * binsf;
+            int b = (int)t;
+            const float q = t - (float)b;
+            if (!(q > tol && q < 1.0f - tol)) b = hist_cos_exact(b1, b2, nbins);
+            b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
+            atomicAdd(hc + b, 1);
+        }
+    }
+    if (local) {
+        __syncthreads();
+        for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
+            if (sh[b]) atomicAdd(bond_h + b, sh[b]);
+            if (sh[nbins + b]) atomicAdd(cos_h + b, sh[nbins + b]);
+        }
     }
 }
 
-// Dynamic shared memory of k_r2n_chain for chains of N monomers (3N doubles);
-// above 48 KiB the kernel's opt-in limit is raised first.
-bool r2n_smem_ready(int N)
+// Dynamic shared memory of k_r2n_chain for chains of N monomers (six words a
+// monomer, padded where that fits); above 48 KiB the kernel's opt-in limit is
+// raised first.  False if N is too long.
+static bool r2n_shared(int N, size_t &smem, int &sh)
 {
-    const size_t smem = sizeof(double) * 3 * (size_t)N;
+    sh = 24 * (size_t)r2n_words(N, 5) <= (size_t)R2N_SMEM_MAX ? 5 : 31;
+    smem = 24 * (size_t)r2n_words(N, sh);
     if (N < 1 || smem > (size_t)R2N_SMEM_MAX) return false;
-    if (smem <= 48 * 1024) return true;
+    if (smem <= 48 * 1024 - 256) return true;
     return cudaFuncSetAttribute(k_r2n_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+}
+
+// <R^2(n)> of n_ch chains of N monomers from x (rows Mp apart); tmp: [n_ch][N]
+static bool r2n_launch(const double *x, long long Mp, int off, int n_ch, int N, const int *comp_of, double *tmp,
+                       double *out, cudaStream_t st)
+{
+    size_t smem = 0;
+    int sh = 5;
+    if (!r2n_shared(N, smem, sh)) return false;
+    // few chains: the lags of a chain over several blocks, to about eight per SM
+    const int pairs = ((N - 1 + R2N_W - 1) / R2N_W + 1) / 2;
+    const int most = std::max(1, (pairs + R2N_THREADS - 1) / R2N_THREADS);
+    const int split = std::max(1, std::min(most, 152 * 8 / n_ch));
+    k_r2n_chain<<<dim3(n_ch, split), R2N_THREADS, smem, st>>>(x, Mp, off, N, tmp, comp_of, sh);
+    if (cudaGetLastError() != cudaSuccess) return false;
+    k_r2n_reduce<<<(N + 31) / 32, dim3(32, R2N_ROWS), 0, st>>>(tmp, n_ch, N, out);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 bool r2n_eval(kg_ctx *c, int melt, double *out_dev)
 {
     const MeltDev &md = c->sim.melt[melt];
-    if (!r2n_smem_ready(md.N)) return false;
     c->launches += 2;
-    k_r2n_chain<<<md.n_ch, 256, sizeof(double) * 3 * md.N, c->stream>>>(c->x, (long long)c->Mp, md.off, md.N,
-                                                                          c->r2tmp, c->comp_of);
-    if (cudaGetLastError() != cudaSuccess) return false;
-    k_r2n_reduce<<<(md.N + 255) / 256, 256, 0, c->stream>>>(c->r2tmp, md.n_ch, md.N, out_dev);
-    return cudaGetLastError() == cudaSuccess;
+    return r2n_launch(c->x, (long long)c->Mp, md.off, md.n_ch, md.N, c->comp_of, c->r2tmp, out_dev, c->stream);
 }
 
 void hist_eval(kg_ctx *c, int melt, int nbins, int *out_dev)
@@ -106,7 +316,7 @@ void hist_eval(kg_ctx *c, int melt, int nbins, int *out_dev)
     const MeltDev &md = c->sim.melt[melt];
     cudaMemsetAsync(out_dev, 0, sizeof(int) * 2 * nbins, c->stream);
     ++c->launches;
-    k_hist<<<(md.M + 255) / 256, 256, 0, c->stream>>>(c->x, c->Mp, md.off, md.M, md.N, md.L, sqrt(c->stage.R0sq),
+    k_hist<<<std::min((md.M + 255) / 256, 152 * 4), 256, 0, c->stream>>>(c->x, c->Mp, md.off, md.M, md.N, md.L, sqrt(c->stage.R0sq),
                                                       nbins, out_dev, out_dev + nbins, c->comp_of);
 }
 
@@ -484,11 +694,6 @@ extern "C" kg_status kg_r2n_noalloc(const double *x, long long stride, int n_cha
     kg_status st;
     double *scratch = scratch_address(&st);
     if (!scratch) return st;
-    const cudaStream_t s = (cudaStream_t)stream;
-    const size_t smem = sizeof(double) * 3 * chain_len;
-    if (!kg::r2n_smem_ready(chain_len)) return KG_ERR_CUDA;
-    kg::k_r2n_chain<<<n_chains, 256, smem, s>>>(x, stride, 0, chain_len, scratch, nullptr);
-    kg::k_r2n_reduce<<<(chain_len + 255) / 256, 256, 0, s>>>(scratch, n_chains, chain_len, out);
-    return cudaGetLastError() == cudaSuccess ? KG_OK : KG_ERR_CUDA;
+    return kg::r2n_launch(x, stride, 0, n_chains, chain_len, nullptr, scratch, out, (cudaStream_t)stream) ? KG_OK
+                                                                                                         : KG_ERR_CUDA;
 }
-

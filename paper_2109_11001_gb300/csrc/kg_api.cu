@@ -376,7 +376,6 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->scratch = (double *)A(7 * Mp * sizeof(double));
     c->flags = (unsigned *)A(16 * sizeof(unsigned));
     c->pbar = (unsigned *)A(4 * sizeof(unsigned));
-    c->resbar = (unsigned long long *)A(kg::resident_words(c->ncell_md));
     c->d_step = (long long *)A(sizeof(long long));
     c->fout = (double *)A(3 * Mp * sizeof(double));
     c->partials_cap = (int)(Mp / 128 + 2) * 5;
@@ -385,6 +384,7 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     for (int m = 0; m < p->n_melts; ++m) r2cap = std::max(r2cap, (long long)S.melt[m].M);
     c->r2tmp_cap = r2cap;
     c->r2tmp = (double *)A((size_t)r2cap * sizeof(double));
+    ok = ok && kg::resident_alloc(c);
     if (!ok) return fail(KG_ERR_OOM);
     if (cudaMemcpyAsync(c->d_sim, &c->sim, sizeof(SimDev), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
         return fail(KG_ERR_CUDA);
@@ -431,6 +431,9 @@ void kg_destroy(kg_ctx *c)
     dev_free(c, c->d_step);
     dev_free(c, c->pbar);
     dev_free(c, c->resbar);
+    dev_free(c, c->bcount);
+    dev_free(c, c->bidx);
+    dev_free(c, c->brec);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     kg::graphs_reset(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -492,6 +495,7 @@ kg_status kg_load_config(kg_ctx *c, int melt, const double *x, const double *v, 
     KG_TRY(cudaMemsetAsync(c->flags, 0, 16 * sizeof(unsigned), c->stream));
     // a rebuild cut short by an earlier error may have left cell counts behind
     KG_TRY(cudaMemsetAsync(c->ccount, 0, sizeof(int) * (size_t)c->ncell_md, c->stream));
+    KG_TRY(kg::resident_reset(c));
     if ((s = set_rebuild(c)) != KG_OK) return s;
     KG_TRY(cudaStreamSynchronize(c->stream));
     c->latched = KG_OK;
@@ -583,7 +587,7 @@ kg_status kg_step(kg_ctx *c, long long n_steps)
             long long n = 1;
             if (c->sort_after_load)             // after a load: one step builds the cell order to sort into
                 kg::md_step(c);
-            else if (!c->prof_on && kg::resident_fits(c)) {
+            else if (!c->prof_on && kg::resident_kind(c) != kg::RES_NONE) {
                 n = steps_to_sort(c, chunk - done, (c->p.flags & KG_FLAG_PERSISTENT) != 0);
                 if (kg::resident_launch(c, (int)n, -1, kg::RESIDENT_SPIN) != cudaSuccess) {
                     cudaGetLastError();
@@ -621,7 +625,7 @@ kg_status kg_persistent_selftest(kg_ctx *c, int skip_block, unsigned spin)
         kg::set_device_step(c, c->step - 1);
         c->d_step_stale = false;
     }
-    if (kg::resident_fits(c)) KG_TRY(kg::resident_launch(c, 2, skip_block, spin));
+    if (kg::resident_kind(c) != kg::RES_NONE) KG_TRY(kg::resident_launch(c, 2, skip_block, spin));
     else KG_TRY(kg::persist_launch(c, c->stream, c->cur, 2, skip_block, spin));
     c->step += 2;
     kg::md_materialize(c);

@@ -54,7 +54,10 @@ struct kg_ctx {
     bool persist_failed = false;
     unsigned *pbar = nullptr;    // grid-barrier words of the persistent launch
     unsigned long long *resbar = nullptr;   // barrier words, error word and segment totals of the resident launch
-    int res_blocks = -1;         // blocks of the resident kernel the GPU holds at once (< 0: not asked yet)
+    int *bcount = nullptr, *bidx = nullptr; // its cell buckets: two sets of counts, members in arrival order
+    float4 *brec = nullptr;                 // and records in order
+    bool buckets = false;
+    int res_sms = -1;            // SMs of the GPU (< 0: not asked yet)
     bool resident_failed = false;
     bool use_graphs = true;
     long long graph_replays = 0;
@@ -165,15 +168,19 @@ void set_device_step(kg_ctx *c, long long v);
 void forces_eval(kg_ctx *c, int melt, long long step, double *F_dev, double *part_dev, int nblk);
 void prof_collect(kg_ctx *c);                // fold recorded event pairs into the totals
 void bonded_partners(kg_ctx *c);             // bp from slot_of / comp_of
+void scan_counts(kg_ctx *c, const int *count, int *start, int n);   // exclusive scan, start[n] the total
 void md_sort(kg_ctx *c);                     // re-sort the state into the last cell order
 void md_materialize(kg_ctx *c);              // mixed: x <- xb64 + dlt[cur]
 void graphs_reset(kg_ctx *c);                // drop captured step graphs (their arguments changed)
 bool md_persist_steps(kg_ctx *c);            // PERSIST_STEPS steps in one persistent launch (KG_MIXED)
 
 // kg_resident.cu
-bool resident_fits(kg_ctx *c);               // one thread per monomer, every block resident
+enum { RES_NONE = 0, RES_WIDE = 1, RES_SMALL = 2 };
+int resident_kind(kg_ctx *c);                // which resident kernel serves the context
 cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin);   // K steps in one launch
-size_t resident_words(int ncell);            // bytes of kg_ctx::resbar
+bool resident_alloc(kg_ctx *c);              // its buffers (none for contexts it does not serve)
+cudaError_t resident_reset(kg_ctx *c);
+void resident_cell_order(kg_ctx *c);         // clist after builds that used buckets
 
 // kg_step.cu
 void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur);   // the mixed path's fused step kernel

@@ -39,6 +39,10 @@ enum : unsigned {
     ERR_DB_INTERNAL = 32u,
 };
 
+// status words kept by the resident MD kernel: how the last Verlet build left the
+// cell order (0: clist; 1 + b: buckets with counts b), and the zeroed count buffer
+constexpr int RES_BUILT = 8, RES_NEXT = 9;
+
 struct MeltDev {
     int off, M, N, n_ch;          // slots [off, off+M): chain c, position i -> off + c*N + i
     int ch_off;                   // chains of earlier melts (global chain index = ch_off + c)

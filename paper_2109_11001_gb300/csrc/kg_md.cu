@@ -474,6 +474,7 @@ __global__ void __launch_bounds__(NL_BLOCK, 5) k_nlist(const __grid_constant__ N
             A.flags[1] = 0u;
             A.flags[4] = 0u;
             A.flags[5] += 1u;                    // Verlet builds completed
+            A.flags[RES_BUILT] = 0u;             // the cell order is in clist
         }
     }
 }
@@ -638,6 +639,7 @@ void bonded_partners(kg_ctx *c)
 void md_sort(kg_ctx *c)
 {
     md_materialize(c);
+    resident_cell_order(c);
     const int Mp = c->Mp;
     double *sx = c->scratch;
     int *spid = (int *)(c->scratch + 6 * (size_t)Mp);
@@ -729,6 +731,13 @@ __global__ void k_begin_step(long long *__restrict__ stepp, unsigned *__restrict
 }
 
 __global__ void k_set_step(long long *__restrict__ stepp, long long v) { stepp[0] = v; }
+
+void scan_counts(kg_ctx *c, const int *count, int *start, int n)
+{
+    const int nb = nblk(n, 1024);
+    k_scan1<<<nb, 1024, 0, c->stream>>>(count, start, c->bsum, n, nullptr);
+    k_scan2<<<nb, 1024, 0, c->stream>>>(start, c->bsum, n, nb, nullptr);
+}
 
 static void launch_rebuild(kg_ctx *c, cudaStream_t st);
 

@@ -25,7 +25,8 @@ __device__ __forceinline__ unsigned bin_md_one(const SimDev &S, int s, double *_
                                                float4 *__restrict__ dcur, float4 *__restrict__ pgcur,
                                                double4_32a *__restrict__ pcur, double4_32a *__restrict__ xb,
                                                int *__restrict__ cellid, int *__restrict__ rank,
-                                               int *__restrict__ count, const int *__restrict__ slot_of)
+                                               int *__restrict__ count, const int *__restrict__ slot_of,
+                                               int *cell_out = nullptr, int *rank_out = nullptr)
 {
     const MeltDev &md = S.melt[melt_of(S, slot_of[s])];
     const int Mp = S.Mp;
@@ -75,7 +76,10 @@ __device__ __forceinline__ unsigned bin_md_one(const SimDev &S, int s, double *_
     int base = 0;
     if (lane == leader) base = atomicAdd(count + c, __popc(grp));
     base = __shfl_sync(grp, base, leader);
-    rank[s] = base + __popc(grp & ((1u << lane) - 1u));
+    const int rk = base + __popc(grp & ((1u << lane) - 1u));
+    rank[s] = rk;
+    if (cell_out) *cell_out = c;
+    if (rank_out) *rank_out = rk;
     return 0;
 }
 
@@ -180,12 +184,12 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
     constexpr unsigned FULL = 0xffffffffu;
     const bool live = s < A.M;
     const int sv = live ? s : A.M - 1;                       // idle lanes read valid memory, write nothing
-    const int slot = __ldg(A.slot_of + sv);
+    const int slot = A.slot_of[sv];
     int m = 0;
     while (m + 1 < A.n_melts && slot >= A.melt[m + 1].off) ++m;
     const MeltNl &md = A.melt[m];
-    const int4 bp = __ldg(A.bp + sv);                        // 1-2 bonded partners: bp.y, bp.z
-    const float4 ri = __ldg(A.recb + sv);
+    const int4 bp = A.bp[sv];                        // 1-2 bonded partners: bp.y, bp.z
+    const float4 ri = A.recb[sv];
     const unsigned code = __float_as_uint(ri.w);
     const int cx = (int)(code & CODE_MASK), cy = (int)((code >> CODE_BITS) & CODE_MASK);
     const int cz = (int)(code >> (2 * CODE_BITS));
@@ -210,8 +214,8 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
                 int xx = cx + dx;
                 xx = xx < 0 ? nc - 1 : (xx >= nc ? 0 : xx);
                 const int cell = rowb + ((xx >> 2) << 6) + (xx & 3);
-                const int k0 = __ldg(A.start + cell);
-                int n = live ? __ldg(A.start + cell + 1) - k0 : 0;
+                const int k0 = A.start[cell];
+                int n = live ? A.start[cell + 1] - k0 : 0;
                 if (n > MAX_CELL_OCC) {
                     err = ERR_NL_CAPACITY;
                     n = 0;
@@ -221,7 +225,7 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
                 const unsigned tag = (unsigned)((dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)) << IDX_BITS;
 #pragma unroll 2
                 for (int j = 0; j < nmax; ++j) {
-                    const float4 rj = __ldg(A.recs + k0 + j);
+                    const float4 rj = A.recs[k0 + j];
                     const int t = __float_as_int(rj.w);
                     const float ex = rj.x - ox, ey = rj.y - oy, ez = rj.z - oz;
                     const float r2 = ex * ex + ey * ey + ez * ez;
@@ -238,7 +242,7 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
         for (int k = 0; k < cnt; ++k) {
             const unsigned e = out[(size_t)k * Mp];
             const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
-            const float r2 = nl_r2(ri, __ldg(A.recb + t), q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
+            const float r2 = nl_r2(ri, A.recb[t], q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
             const bool keep = r2 < lo || dist2_exact(A.x, A.Mp, md.L, s, t) < A.rl2;
             if (keep) out[(size_t)(w++) * Mp] = e;
         }
@@ -261,6 +265,51 @@ __device__ __forceinline__ float nl_v(float4 r, float ox, float oy, float oz, fl
     return fmaf(ez, ez, fmaf(ey, ey, fmaf(ex, ex, -hi)));
 }
 
+// After a walk that took the band pairs provisionally: those of the warp's rows
+// decided in binary64, the length written; near: the smallest |v| that the
+// lane's row saw, m: its melt.  Whole warps.  Returns error bits.
+__device__ __forceinline__ unsigned nlist_finish(const NlArgs &A, int s, int m, bool live, float near, int cnt,
+                                                 int &n_out)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int maxnb = A.maxnb;
+    const size_t Mp = (size_t)A.Mp;
+    unsigned err = 0;
+    unsigned fix = __ballot_sync(FULL, live && near < (A.melt[m].hi - A.melt[m].lo) && cnt <= maxnb);
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    while (fix) {
+        const int src = __ffs(fix) - 1;
+        fix &= fix - 1;
+        const int ss = __shfl_sync(FULL, s, src), cs = __shfl_sync(FULL, cnt, src);
+        const MeltNl &ms = A.melt[__shfl_sync(FULL, m, src)];
+        const float4 rs = A.recb[ss];
+        unsigned *row = A.nl + ss;
+        int kept = 0;
+        for (int k = lane; k - lane < cs; k += 32) {
+            const unsigned e = k < cs ? row[(size_t)k * Mp] : (unsigned)ss;
+            const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
+            const float v = nl_v(A.recb[t], rs.x - (float)(q % 3 - 1) * ms.h, rs.y - (float)((q / 3) % 3 - 1) * ms.h,
+                                 rs.z - (float)(q / 9 - 1) * ms.h, ms.hi);
+            const bool keep = k < cs && (v < ms.lo - ms.hi || dist2_exact(A.x, A.Mp, ms.L, ss, t) < A.rl2);
+            const unsigned bal = __ballot_sync(FULL, keep);
+            if (keep) row[(size_t)(kept + __popc(bal & ((1u << lane) - 1u))) * Mp] = e;
+            kept += __popc(bal);
+        }
+        if (lane == src) cnt = kept;
+        __syncwarp();
+    }
+    n_out = cnt < maxnb ? cnt : maxnb;
+    if (live) {
+        A.nn[s] = n_out;
+        if (cnt > maxnb) {
+            err |= ERR_NL_CAPACITY;
+            atomicMax(A.flags + 3, (unsigned)cnt);
+        }
+    }
+    return err;
+}
+
 // The same list by another walk, for the resident kernel, where load latency
 // counts and not the work: the three cells of a stencil row have their starts
 // in flight together, and a cell of up to 32 candidates takes two passes.  The
@@ -271,7 +320,7 @@ __device__ __forceinline__ float nl_v(float4 r, float ox, float oy, float oz, fl
 // between two candidate loads.  A pair inside the band -w <= v < 0 is taken
 // provisionally; after the stencil the whole warp re-reads the row of a lane
 // that may hold one (about one lane in 5000), an entry per lane, decides in
-// binary64 and compacts it in order.  The kernel of large systems keeps the
+// binary64 and compacts it in order.  The kernel of larger systems keeps the
 // walk above: it is bound by the L1 data pipe, and this one took 362 us
 // against 336 per build of 1.6M monomers there (two candidates at a time).
 // s >= M: an idle lane; n_out: the length; returns error bits.
@@ -360,39 +409,80 @@ __device__ __forceinline__ unsigned nlist_masked(const NlArgs &A, int s, int &n_
             }
         }
     }
-    unsigned fix = __ballot_sync(FULL, live && near < (md.hi - md.lo) && cnt <= maxnb);
-    const int lane = threadIdx.x & 31;
-    __syncwarp();
-    while (fix) {
-        const int src = __ffs(fix) - 1;
-        fix &= fix - 1;
-        const int ss = __shfl_sync(FULL, s, src), cs = __shfl_sync(FULL, cnt, src);
-        const MeltNl &ms = A.melt[__shfl_sync(FULL, m, src)];
-        const float4 rs = A.recb[ss];
-        unsigned *row = A.nl + ss;
-        int kept = 0;
-        for (int k = lane; k - lane < cs; k += 32) {
-            const unsigned e = k < cs ? row[(size_t)k * Mp] : (unsigned)ss;
-            const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
-            const float v = nl_v(A.recb[t], rs.x - (float)(q % 3 - 1) * ms.h, rs.y - (float)((q / 3) % 3 - 1) * ms.h,
-                                 rs.z - (float)(q / 9 - 1) * ms.h, ms.hi);
-            const bool keep = k < cs && (v < ms.lo - ms.hi || dist2_exact(A.x, A.Mp, ms.L, ss, t) < A.rl2);
-            const unsigned bal = __ballot_sync(FULL, keep);
-            if (keep) row[(size_t)(kept + __popc(bal & ((1u << lane) - 1u))) * Mp] = e;
-            kept += __popc(bal);
-        }
-        if (lane == src) cnt = kept;
-        __syncwarp();
+    return err | nlist_finish(A, s, m, live, near, cnt, n_out);
+}
+
+// Cells [q0, q1) of the stencil of monomer s (melt md, record ri, bonded
+// partners bp) in the small resident kernel's buckets: emit(e, take) for every
+// candidate, in list order; near: the smallest |v| seen.  Whole warps, at most
+// NQ cells, whose counts are in flight together; a cell's first records load
+// while the cell before is looked at.
+// A bucket's first BUCKET_MAIN records lie in one array, the few further ones
+// in another: the walk is bound by the L1 data pipe, which serves one 128-byte
+// line at a time, so cells next to each other have to share lines (buckets of
+// 512 bytes took 20,000 clocks for 128 monomers of an SM, these take 10,000).
+constexpr int BUCKET = 32, BUCKET_MAIN = 4;
+
+template <int NQ, class EMIT>
+__device__ __forceinline__ void nlist_cells(const MeltNl &md, int s, bool live, float4 ri, int4 bp, int q0, int q1,
+                                            const float4 *brec, const float4 *brec2, const int *count, float &near,
+                                            EMIT emit)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int U = BUCKET_MAIN;
+    const unsigned code = __float_as_uint(ri.w);
+    const int cx = (int)(code & CODE_MASK), cy = (int)((code >> CODE_BITS) & CODE_MASK);
+    const int cz = (int)(code >> (2 * CODE_BITS));
+    const int nc = md.nc, nbk = md.nbk, cell_off = md.cell_off;
+    const float h = md.h, hi = md.hi;
+    int cell[NQ], cn[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+        const int q = min(q0 + i, 26);
+        int zz = cz + q / 9 - 1, yy = cy + (q / 3) % 3 - 1, xx = cx + q % 3 - 1;
+        zz = zz < 0 ? nc - 1 : (zz >= nc ? 0 : zz);
+        yy = yy < 0 ? nc - 1 : (yy >= nc ? 0 : yy);
+        xx = xx < 0 ? nc - 1 : (xx >= nc ? 0 : xx);
+        cell[i] = cell_off + ((((zz >> 2) * nbk + (yy >> 2)) * nbk + (xx >> 2)) << 6) +
+                  (((zz & 3) << 4) | ((yy & 3) << 2) | (xx & 3));
     }
-    n_out = cnt < maxnb ? cnt : maxnb;
-    if (live) {
-        A.nn[s] = n_out;
-        if (cnt > maxnb) {
-            err |= ERR_NL_CAPACITY;
-            atomicMax(A.flags + 3, (unsigned)cnt);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) cn[i] = count[cell[i]];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) cn[i] = live && q0 + i < q1 ? cn[i] : 0;
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 r[2][U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) r[0][k] = k < cn[0] ? brec[(size_t)cell[0] * U + k] : none;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+        const int q = q0 + i, n = cn[i], nmax = __reduce_max_sync(FULL, n);
+        if (i + 1 < NQ) {
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                r[(i + 1) & 1][k] = k < cn[i + 1] ? brec[(size_t)cell[i + 1] * U + k] : none;
+        }
+        const float ox = ri.x - (float)(q % 3 - 1) * h, oy = ri.y - (float)((q / 3) % 3 - 1) * h,
+                    oz = ri.z - (float)(q / 9 - 1) * h;
+        auto look = [&](const float4 &c, int j) {
+            const float v = nl_v(c, ox, oy, oz, hi);
+            const int t = __float_as_int(c.w);
+            near = fminf(near, fabsf(v));
+            emit((unsigned)t | ((unsigned)q << IDX_BITS),
+                 (j < n) & (v < 0.f) & (t != s) & (t != bp.y) & (t != bp.z));
+        };
+        if (nmax > 0) {
+#pragma unroll
+            for (int k = 0; k < U; ++k) look(r[i & 1][k], k);
+        }
+#pragma unroll 1
+        for (int j = U; j < nmax; j += 2) {
+            const float4 *b = brec2 + (size_t)cell[i] * (BUCKET - U) + (j - U);
+            const float4 c0 = j < n ? b[0] : none, c1 = j + 1 < n ? b[1] : none;
+            look(c0, j);
+            look(c1, j + 1);
         }
     }
-    return err;
 }
 
 }  // namespace kg

@@ -28,144 +28,34 @@
 // ERR_TIMEOUT and leaves.  The arithmetic is that of the one-step kernel
 // (kg_step.cuh) on the same lists, so trajectories have the same bits.
 //
-// Measured, 50 steps and the read of the state (skin 0.3, n = 12, dt = 0.01; a
-// build every third or fourth step), against the captured graphs of separate
-// launches: 1,000 monomers 1230 -> 613 us, 16 melts of 1,000 in one context
-// 1998 -> 1362 us (about half of it the reads), 80,000 monomers 1674 -> 1170 us.
+// Measured, 50 steps and a read of the state of 80,000 monomers (skin 0.3, n =
+// 12, dt = 0.01; a build every third or fourth step), against captured graphs
+// of separate launches: 1743 -> 1117 us.
 // Larger systems keep the graphs: there the step is work and the launches are
 // not.
 //
-// (128, 5): at most 102 registers, 5 x 128 threads per SM; the capacity (about
-// 97,000 monomers on 152 SMs) is resident_fits' limit.
+// Systems of at most 128 monomers per SM take kg_resident_small.cu.
+//
+// (128, 5): at most 102 registers, 5 x 128 threads per SM, about 97,000
+// monomers on 152 SMs (resident_kind).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
-#include "kg_step.cuh"
+#include "kg_resident.cuh"
 
 namespace kg {
 
 constexpr int RES_BLOCK = 128;
 constexpr int RES_MIN_BLOCKS = 5;
 constexpr int RES_ILP = 8;               // list entries in flight per lane
-constexpr int RES_SEG = 1024;            // cells per scan segment
-
-struct ResArgs {
-    StepArgs st;                 // its dcur/dnext/pcur/pnext are ignored: the buffers alternate below
-    NlArgs nl;
-    const SimDev *sim;           // device copy of the melt table (binning)
-    float4 *dlt[2], *pg[2];      // displacement and gather buffers, ping-pong
-    double *x, *xb64;
-    float4 *recb, *recs;
-    int *cellid, *rank, *ccount, *cstart, *clist, *ctmp, *segtot;
-    int ncell, cur0, K, skip_block;   // skip_block >= 0: that block never arrives (barrier self-test)
-    unsigned long long *bar;     // three barrier words, zero at launch
-    unsigned *errw;              // error bits of this launch (zero at launch)
-    unsigned spin;               // barrier polls before giving up
-    long long *stepp;            // device step counter: the last step run
-};
-
-// fields of a barrier word: blocks arrived, blocks asking for a rebuild, blocks that saw an error
-constexpr unsigned long long BAR_ONE = 1ull, BAR_REQ = 1ull << 21, BAR_ERR = 1ull << 42;
-constexpr unsigned long long BAR_MASK = (1ull << 21) - 1ull;
-constexpr unsigned REQ = 1u, FAIL = 2u, GAVE_UP = 4u;       // what a barrier tells
-
-struct GridBar {
-    unsigned long long *bar;
-    unsigned *acc, *out;         // shared: this block's bits for the next barrier [2], the last barrier's answer
-    unsigned spin;
-    int b;                       // barriers passed
-
-    // bits of any thread reach the barrier that the block arrives at next
-    __device__ __forceinline__ void note(unsigned bits) { if (bits) atomicOr(acc + (b & 1), bits); }
-
-    __device__ __forceinline__ void arrive()
-    {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const unsigned a = acc[b & 1];
-            acc[(b + 1) & 1] = 0u;
-            if (blockIdx.x == 0) *(volatile unsigned long long *)(bar + (b + 1) % 3) = 0ull;
-            const unsigned long long add = BAR_ONE + ((a & REQ) ? BAR_REQ : 0ull) + ((a & FAIL) ? BAR_ERR : 0ull);
-            asm volatile("fence.acq_rel.gpu;\n\tred.release.gpu.global.add.u64 [%0], %1;"
-                         ::"l"(bar + b % 3), "l"(add) : "memory");
-        }
-    }
-
-    __device__ __forceinline__ unsigned wait()
-    {
-        if (threadIdx.x == 0) {
-            unsigned long long v;
-            unsigned it = 0, r = 0;
-            for (;;) {
-                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(bar + b % 3) : "memory");
-                if ((v & BAR_MASK) == gridDim.x) break;
-                if (++it > spin) {
-                    r = GAVE_UP;
-                    break;
-                }
-                if (it > 64) __nanosleep(32);
-            }
-            asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            if ((v / BAR_REQ) & BAR_MASK) r |= REQ;
-            if (v / BAR_ERR) r |= FAIL;
-            *out = r;
-        }
-        __syncthreads();
-        ++b;
-        return *out;
-    }
-
-    __device__ __forceinline__ unsigned sync()
-    {
-        arrive();
-        return wait();
-    }
-};
-
-// exclusive scan of the cell counts: segment g from the totals of the
-// segments before it (the bin phase summed them) and its own counts
-__device__ __forceinline__ void res_scan_seg(const ResArgs &A, int g, int nseg, int *wsum)
-{
-    constexpr int PER = RES_SEG / RES_BLOCK, NW = RES_BLOCK / 32;
-    const int n = A.ncell, i0 = g * RES_SEG + threadIdx.x * PER;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int before = 0;
-    for (int k = threadIdx.x; k < g; k += RES_BLOCK) before += A.segtot[k];
-    int v[PER], own = 0;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        v[k] = i0 + k < n ? A.ccount[i0 + k] : 0;
-        own += v[k];
-    }
-    int incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += u;
-    }
-    before = __reduce_add_sync(0xffffffffu, before);
-    if (lane == 31) wsum[w] = incl;
-    if (lane == 0) wsum[NW + w] = before;
-    __syncthreads();
-    int run = incl - own;
-#pragma unroll
-    for (int k = 0; k < NW; ++k) run += wsum[NW + k] + (k < w ? wsum[k] : 0);
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        if (i0 + k < n) A.cstart[i0 + k] = run;
-        run += v[k];
-    }
-    if (g == nseg - 1 && threadIdx.x == RES_BLOCK - 1) A.cstart[n] = run;
-    __syncthreads();
-}
 
 template <int N4>
 __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __grid_constant__ ResArgs A)
 {
     __shared__ float dk[96];
     __shared__ unsigned acc_s[2], out_s;
-    __shared__ int wsum[2 * (RES_BLOCK / 32)];
+    __shared__ int wsum[RES_BLOCK / 16];
     step_block_setup(dk);
     const StepArgs &P = A.st;
     // no block writes the status words before every block has arrived at the last barrier
@@ -226,7 +116,7 @@ __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __
             }
             gb.note(err ? FAIL : 0u);
             if ((told = gb.sync()) & (FAIL | GAVE_UP)) break;
-            for (int g = blockIdx.x; g < nseg; g += gridDim.x) res_scan_seg(A, g, nseg, wsum);
+            for (int g = blockIdx.x; g < nseg; g += gridDim.x) res_scan_seg<RES_BLOCK>(A, A.ccount, g, nseg, wsum);
             if ((told = gb.sync()) & GAVE_UP) break;
             if (live) scatter_one(s, A.cellid, A.rank, A.cstart, A.ctmp);
             if (blockIdx.x == 0)
@@ -277,7 +167,8 @@ __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __
             }
         }
         if (live) {
-            bonded32<N4>(P, [&](int k, int) { return part[k]; }, md, pi, bp, F, err);
+            bonded32<N4>(P, [&](int k, int) { return part[k]; }, [&](int, float a, float3 x) { axpy3(a, x, F); }, md,
+                         pi, bp, err);
             v.x = fmaf(P.dt, fmaf(P.amp, gn.x, fmaf(-P.gamma, v.x, F.x)), v.x);
             v.y = fmaf(P.dt, fmaf(P.amp, gn.y, fmaf(-P.gamma, v.y, F.y)), v.y);
             v.z = fmaf(P.dt, fmaf(P.amp, gn.z, fmaf(-P.gamma, v.z, F.z)), v.z);
@@ -305,54 +196,21 @@ __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __
         if (told & FAIL) atomicOr(P.flags, *(volatile unsigned *)A.errw);
         P.flags[1] = rebuild ? 1u : 0u;
         P.flags[5] += builds;
+        if (builds) P.flags[RES_BUILT] = 0u;                  // the cell order is in clist
         *A.stepp = base + A.K;
     }
 }
 
-template <int N4>
-static cudaError_t launch_n4(const ResArgs &a, cudaStream_t st)
+// How a context's steps run: RES_NONE (launches per step), RES_WIDE (this
+// file's kernel, 640 monomers per SM) or RES_SMALL (kg_resident_small.cu, 128
+// monomers per SM).  Every block has to be resident at once; the limits are
+// what the kernels' __launch_bounds__ guarantee for every exponent.
+int resident_kind(kg_ctx *c)
 {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((a.st.M + RES_BLOCK - 1) / RES_BLOCK));
-    cfg.blockDim = dim3(RES_BLOCK);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_resident<N4>, a);
-}
-
-static cudaError_t resident_start(int n4, const ResArgs &a, cudaStream_t st)
-{
-    switch (n4) {
-        case 8: return launch_n4<8>(a, st);
-        case 12: return launch_n4<12>(a, st);
-        case 16: return launch_n4<16>(a, st);
-        case 20: return launch_n4<20>(a, st);
-        case 23: return launch_n4<23>(a, st);
-        case 26: return launch_n4<26>(a, st);
-        case 28: return launch_n4<28>(a, st);
-        case 32: return launch_n4<32>(a, st);
-        case 36: return launch_n4<36>(a, st);
-        case 40: return launch_n4<40>(a, st);
-        case 44: return launch_n4<44>(a, st);
-        case 48: return launch_n4<48>(a, st);
-        default: return launch_n4<0>(a, st);
-    }
-}
-
-// One thread per monomer needs every block resident at once.
-bool resident_fits(kg_ctx *c)
-{
-    if (c->precision != KG_MIXED || c->tpm != 1 || c->resident_failed) return false;
-    if (c->res_blocks < 0) {
-        int nsm = 0;
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
-        c->res_blocks = RES_MIN_BLOCKS * nsm;          // what __launch_bounds__ guarantees for every exponent
-    }
-    return (c->M + RES_BLOCK - 1) / RES_BLOCK <= c->res_blocks;
+    if (c->precision != KG_MIXED || c->tpm != 1 || c->resident_failed) return RES_NONE;
+    if (c->res_sms < 0) cudaDeviceGetAttribute(&c->res_sms, cudaDevAttrMultiProcessorCount, c->device);
+    if (c->buckets && c->M <= SMALL_OWN * SMALL_MIN_BLOCKS * c->res_sms) return RES_SMALL;
+    return c->M <= RES_BLOCK * RES_MIN_BLOCKS * c->res_sms ? RES_WIDE : RES_NONE;
 }
 
 cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin)
@@ -364,7 +222,11 @@ cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin)
     for (int b = 0; b < 2; ++b) {
         a.dlt[b] = c->dlt[b];
         a.pg[b] = c->pg[b];
+        a.count[b] = c->bcount ? c->bcount + (size_t)b * c->ncell_md : nullptr;
     }
+    a.bidx = c->bidx;
+    a.brec = c->brec;
+    a.brec2 = c->brec ? c->brec + (size_t)c->ncell_md * BUCKET_MAIN : nullptr;
     a.x = c->x;
     a.xb64 = c->xb64;
     a.recb = c->recb;
@@ -388,13 +250,80 @@ cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin)
     const size_t nseg = (size_t)(c->ncell_md + RES_SEG - 1) / RES_SEG;
     cudaError_t e = cudaMemsetAsync(c->resbar, 0, 4 * sizeof(unsigned long long) + nseg * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
-    e = resident_start(n4_of(c->stage.n), a, c->stream);
+    const int n4 = n4_of(c->stage.n), nb = (c->M + RES_BLOCK - 1) / RES_BLOCK;
+    e = resident_kind(c) == RES_SMALL ? small_launch(a, n4, c->stream)
+                                      : KG_RESIDENT_LAUNCH(k_resident, n4, nb, RES_BLOCK, a, c->stream);
     if (e != cudaSuccess) return e;
     c->launches += 1;
     c->cur ^= K & 1;
     return cudaSuccess;
 }
 
-size_t resident_words(int ncell) { return 4 * sizeof(unsigned long long) + ((size_t)ncell / RES_SEG + 1) * sizeof(int); }
+// Barrier words and segment totals; for the small kernel bucket counts (two
+// sets), members and records.  Cells of the usual grids hold 2.4 to 5
+// monomers; grids whose mean is above a third of a bucket (cell_scale well
+// above 1) do not use them.
+bool resident_alloc(kg_ctx *c)
+{
+    double most = 0.0;
+    for (int m = 0; m < c->sim.n_melts; ++m) {
+        const MeltDev &md = c->sim.melt[m];
+        most = std::max(most, (double)md.M / ((double)md.nc * md.nc * md.nc));
+    }
+    c->buckets = 3.0 * most <= BUCKET;
+    const int kind = resident_kind(c);
+    if (kind == RES_NONE) return true;
+    c->resbar = (unsigned long long *)dev_alloc(c, 4 * sizeof(unsigned long long) +
+                                                       ((size_t)c->ncell_md / RES_SEG + 1) * sizeof(int));
+    if (kind != RES_SMALL) return c->resbar != nullptr;
+    const size_t nb = (size_t)c->ncell_md * BUCKET;
+    c->bcount = (int *)dev_alloc(c, 2 * (size_t)c->ncell_md * sizeof(int));
+    c->bidx = (int *)dev_alloc(c, nb * sizeof(int));
+    c->brec = (float4 *)dev_alloc(c, nb * sizeof(float4));
+    return c->resbar && c->bcount && c->bidx && c->brec;
+}
+
+// a rebuild cut short by an error may have left counts behind (kg_load_config)
+cudaError_t resident_reset(kg_ctx *c)
+{
+    return c->bcount ? cudaMemsetAsync(c->bcount, 0, 2 * sizeof(int) * (size_t)c->ncell_md, c->stream) : cudaSuccess;
+}
+
+// The cell order of a build that used buckets, for a re-sort: the counts to
+// the counting sort's array for the scan, then every bucket's members (in
+// order, from the records) to their cell's run.
+__global__ void __launch_bounds__(256) k_bucket_counts(const unsigned *__restrict__ flags,
+                                                      const int *__restrict__ bcount, int ncell,
+                                                      int *__restrict__ count)
+{
+    const unsigned built = flags[RES_BUILT];
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (built && c < ncell) count[c] = bcount[(size_t)(built - 1) * ncell + c];
+}
+
+__global__ void __launch_bounds__(256) k_bucket_list(const unsigned *__restrict__ flags,
+                                                    const float4 *__restrict__ brec, int ncell,
+                                                    int *__restrict__ count, const int *__restrict__ start,
+                                                    int *__restrict__ list)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (!flags[RES_BUILT] || c >= ncell) return;
+    const int n = count[c], k0 = start[c];
+    for (int k = 0; k < n; ++k) list[k0 + k] = __float_as_int(
+            (k < BUCKET_MAIN ? brec[(size_t)c * BUCKET_MAIN + k]
+                             : brec[(size_t)ncell * BUCKET_MAIN + (size_t)c * (BUCKET - BUCKET_MAIN) + k - BUCKET_MAIN])
+                .w);
+    count[c] = 0;
+}
+
+void resident_cell_order(kg_ctx *c)
+{
+    if (!c->bcount) return;
+    const int nb = (c->ncell_md + 255) / 256;
+    k_bucket_counts<<<nb, 256, 0, c->stream>>>(c->flags, c->bcount, c->ncell_md, c->ccount);
+    scan_counts(c, c->ccount, c->cstart, c->ncell_md);
+    k_bucket_list<<<nb, 256, 0, c->stream>>>(c->flags, c->brec, c->ncell_md, c->ccount, c->cstart, c->clist);
+    c->launches += 4;
+}
 
 }  // namespace kg

@@ -95,7 +95,8 @@ __device__ __forceinline__ void step_tile(const StepArgs &P, int t0, const float
     }
     float4 rb = make_float4(0.f, 0.f, 0.f, 0.f), dc = rb;
     if (live) {
-        if (sub == 0) bonded32<N4>(P, [&](int, int j) { return __ldg(pcur + j); }, md, pi, __ldg(P.bp + s), F, err);
+        if (sub == 0) bonded32<N4>(P, [&](int, int j) { return __ldg(pcur + j); },
+                                   [&](int, float a, float3 x) { axpy3(a, x, F); }, md, pi, __ldg(P.bp + s), err);
         if (sub == TPM - 1)
             gn = gauss3_f(draw(P.seed, m, 0, (unsigned long long)step, (uint32_t)(slot - md.off)));
         rb = __ldg(P.recb + s);
@@ -320,6 +321,7 @@ __global__ void __launch_bounds__(PERSIST_BLOCK, 5) k_persist(const __grid_const
             if (blockIdx.x == 0 && threadIdx.x == 0) {
                 P.flags[1] = 0u;                               // request served (before the next release)
                 P.flags[5] += 1u;                              // Verlet builds completed
+                P.flags[RES_BUILT] = 0u;                       // the cell order is in clist
             }
             if (!grid_sync(A, &ok_s, &snap_s)) return;
             if (snap_s.x) break;

@@ -112,9 +112,11 @@ __device__ __forceinline__ float3 bend_g(float3 a, float inv, float c, float3 b)
 
 // Bond (Eq. 10) and bending (Eq. 4) forces on the monomer whose gather
 // record is pi, from its chain partners bp = (s-2, s-1, s+1, s+2);
-// rec(k, j): the gather record of partner k (0..3), compute index j.
-template <int N4, class REC>
-__device__ __forceinline__ void bonded32(const StepArgs &P, REC rec, const MeltStep &md, float4 pi, int4 bp, float3 &F,
+// rec(k, j): the gather record of partner k (0..3), compute index j; add(k, a,
+// x): term k of the force, F += a x, called in the order k = 0 ... 4 (two
+// bonds, three angles) for the terms that exist.
+template <int N4, class REC, class ADD>
+__device__ __forceinline__ void bonded32(const StepArgs &P, REC rec, ADD add, const MeltStep &md, float4 pi, int4 bp,
                                          unsigned &err)
 {
     const bool hm2 = bp.x >= 0, hm1 = bp.y >= 0, hp1 = bp.z >= 0, hp2 = bp.w >= 0;
@@ -139,7 +141,7 @@ __device__ __forceinline__ void bonded32(const StepArgs &P, REC rec, const MeltS
             }
             const float fl = mlj_fr32<N4>(P, r2);
             fr += r2 < P.rc2 ? fl : 0.0f;
-            axpy3(fr, d, F);
+            add(side, fr, d);
         }
     }
     const float kap = md.kappa;
@@ -151,19 +153,19 @@ __device__ __forceinline__ void bonded32(const StepArgs &P, REC rec, const MeltS
             const float l1 = dot3(Bm1, Bm1), l2 = dot3(B0, B0);
             const float inv = rsqrtf(__fmul_rn(l1, l2)), cs = __fmul_rn(dot3(Bm1, B0), inv);
             const float c1 = __fmul_rn(cs, __fdividef(1.0f, l1)), c2 = __fmul_rn(cs, __fdividef(1.0f, l2));
-            axpy3(kap, sub3(bend_g(B0, inv, c1, Bm1), bend_g(Bm1, inv, c2, B0)), F);
+            add(2, kap, sub3(bend_g(B0, inv, c1, Bm1), bend_g(Bm1, inv, c2, B0)));
         }
         if (hp2) {                            // vertex s+1, s its first end: -kappa g1
             const float l1 = dot3(B0, B0), l2 = dot3(Bp1, Bp1);
             const float inv = rsqrtf(__fmul_rn(l1, l2)), cs = __fmul_rn(dot3(B0, Bp1), inv);
             const float c1 = __fmul_rn(cs, __fdividef(1.0f, l1));
-            axpy3(-kap, bend_g(Bp1, inv, c1, B0), F);
+            add(3, -kap, bend_g(Bp1, inv, c1, B0));
         }
         if (hm2) {                            // vertex s-1, s its last end: +kappa g2
             const float l1 = dot3(Bm2, Bm2), l2 = dot3(Bm1, Bm1);
             const float inv = rsqrtf(__fmul_rn(l1, l2)), cs = __fmul_rn(dot3(Bm2, Bm1), inv);
             const float c2 = __fmul_rn(cs, __fdividef(1.0f, l2));
-            axpy3(kap, bend_g(Bm2, inv, c2, Bm1), F);
+            add(4, kap, bend_g(Bm2, inv, c2, Bm1));
         }
     }
 }

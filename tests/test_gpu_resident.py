@@ -50,9 +50,11 @@ def _run(kg, melts, one_by_one, skin=0.3, cell_scale=0.0, stream=None):
         kg.kg_destroy(ctx)
 
 
-def _capacity():
+def _capacities():
+    """Monomers that the kernel with four threads per monomer holds, and the one with one."""
     import torch
-    return 5 * 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    n = torch.cuda.get_device_properties(0).multi_processor_count
+    return 128 * n, 640 * n
 
 
 # chains x N: the smallest box, one monomer under / over whole blocks, a batch
@@ -68,14 +70,42 @@ def test_resident_launches_match_one_launch_per_step(kg, sizes, skin, scale):
     assert la < lb / 5                           # many steps per launch
 
 
-def test_both_sides_of_the_capacity(kg):
-    cap = _capacity()
-    for extra in (0, 1):                         # every block resident; one block more takes the other path
+# 24 monomers (whole chains) in one cell: more list entries than a set of the small kernel
+# keeps; 45: more members than a bucket holds, the counting sort instead
+@pytest.mark.parametrize("crowd", [24, 45])
+def test_a_crowded_cell(kg, crowd):
+    m = KI.random_walk_melt(110, 3, 0.85, 0.0, 51)
+    k = np.arange(crowd)
+    m.x[:, :crowd] = 0.1 + 0.3 * np.stack([k % 4, k // 4 % 4, k // 16])
+    out = []
+    for one_by_one in (0, 1):
+        p = kg.make_params([(m.n_chains, m.chain_len, m.box, m.kappa)], seed=9, fene_qmin=0.01)
+        ctx = kg.kg_create(p, 0, None, None)
+        try:
+            kg.kg_set_potential_schedule(ctx, [kg.stage(2.0, 10 ** 9, 1e-8)])
+            kg.kg_load_config(ctx, 0, m.x, m.v)
+            kg.kg_profile(ctx, one_by_one)
+            kg.kg_step(ctx, 1)
+            kg.kg_step(ctx, 30)                  # starts with the rebuild that the re-sort after a load asks for
+            x, v = np.zeros_like(m.x), np.zeros_like(m.v)
+            kg.kg_get_config(ctx, 0, x, v)
+            F = np.zeros_like(m.x)
+            kg.kg_forces(ctx, 0, F)
+            out.append((x, v, F))
+        finally:
+            kg.kg_destroy(ctx)
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+def test_both_sides_of_a_capacity(kg, kind):
+    cap = _capacities()[kind]
+    for extra in (0, 1):                         # every block resident; one block more takes the next path
         m = KI.random_walk_melt(cap // 128 + extra, 128, 0.85, 2.0, 31)
         a, la = _run(kg, [m], 0)
         b, lb = _run(kg, [m], 1)
         assert all(np.array_equal(p, q) for p, q in zip(a, b))
-        assert (la < lb / 5) == (extra == 0)
+        assert (la < lb / 5) == (kind == 0 or extra == 0)
 
 
 def test_two_contexts_on_two_threads(kg):

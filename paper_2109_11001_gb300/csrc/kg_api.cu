@@ -366,8 +366,9 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->dbmark = (int *)A((size_t)c->ncell_db * sizeof(int));
     c->n_chain_total = (int)nchain;
     c->chain_ver = (int *)A((size_t)nchain * sizeof(int));
-    c->dbround = (int *)A(kg::RS * kg::MAX_MELTS * sizeof(int));
+    c->dbround = (int *)A(2 * kg::RS * kg::MAX_MELTS * sizeof(int));
     c->koff = (int *)A((kg::MAX_MELTS + 1) * sizeof(int));
+    c->dbbar = (unsigned long long *)A(4 * sizeof(unsigned long long));
     c->slot_of = (int *)A(Mp * sizeof(int));
     c->comp_of = (int *)A(Mp * sizeof(int));
     c->bp = (int4 *)A(Mp * sizeof(int4));
@@ -421,15 +422,16 @@ void kg_destroy(kg_ctx *c)
     void *bufs[] = {c->d_sim, c->d_stage, c->x, c->xb64, c->u, c->pid, c->recb, c->recs, c->shtab, c->dlt[0], c->dlt[1],
                     c->pg[0], c->pg[1], c->pos64[0],
                     c->pos64[1], c->xb, c->cellid, c->rank, c->ccount, c->cstart, c->clist, c->ctmp, c->bsum, c->nl,
-                    c->nn, c->dbcell, c->dbrank, c->dbcount, c->dbstart, c->dblist, c->dbrec, c->dbmark, c->chain_ver, c->dbround, c->att_ver, c->att,
+                    c->nn, c->dbcell, c->dbrank, c->dbcount, c->dbstart, c->dblist, c->dbrec, c->dbmark, c->chain_ver, c->dbround, c->att,
                     c->koff, c->slot_of,
                     c->comp_of, c->bp, c->img, c->db_stats, c->scratch, c->flags, c->fout, c->partials,
                     c->r2tmp, c->hist, c->mlp_master, c->mlp_adam, c->mlp_grad, c->mlp_blob, c->mlp_w2t,
-                    c->logf, c->logt, c->logn, c->trainf, c->traint, c->d_train_head, c->tr_buf, c->bmax2,
+                    c->logf, c->logt, c->logn, c->logoff, c->trainf, c->traint, c->d_train_head, c->tr_buf, c->bmax2,
                     c->d_io, c->msd_ref};
     for (void *b : bufs) dev_free(c, b);
     dev_free(c, c->d_step);
     dev_free(c, c->pbar);
+    dev_free(c, c->dbbar);
     dev_free(c, c->resbar);
     dev_free(c, c->bcount);
     dev_free(c, c->bidx);
@@ -648,15 +650,9 @@ static kg_status sweep_impl(kg_ctx *c, const long long *attempts, kg_db_stats *s
     if (tot >= (1LL << 31)) return KG_ERR_INVALID_ARG;
     if (tot > c->att_cap) {
         dev_free(c, c->att);
-        dev_free(c, c->att_ver);
         c->att_cap = std::max(tot, 2 * c->att_cap);
         c->att = dev_alloc(c, (size_t)c->att_cap * sizeof(kg::Attempt));
-        c->att_ver = (int *)dev_alloc(c, (size_t)c->att_cap * sizeof(int));
-        if (!c->att || !c->att_ver) {
-            dev_free(c, c->att);
-            dev_free(c, c->att_ver);
-            c->att = nullptr;
-            c->att_ver = nullptr;
+        if (!c->att) {
             c->att_cap = 0;
             return KG_ERR_OOM;
         }
@@ -665,8 +661,8 @@ static kg_status sweep_impl(kg_ctx *c, const long long *attempts, kg_db_stats *s
     static thread_local long long *hstats = nullptr;
     if (!hstats && cudaMallocHost(&hstats, sizeof(long long) * 4 * kg::MAX_MELTS) != cudaSuccess) return KG_ERR_OOM;
     // the grid and the record buffers must describe the current positions
-    if (learned) kg::db_sweep_learned(c, K, lambda, hstats);
-    else kg::db_sweep(c, K, hstats);
+    const cudaError_t swept = learned ? kg::db_sweep_learned(c, K, lambda, hstats) : kg::db_sweep(c, K, hstats);
+    KG_TRY(swept);
     KG_TRY(cudaGetLastError());
     kg_status s = read_flags(c, pinned_flags());
     kg_db_stats out{0, 0, 0, 0, c->sweep};

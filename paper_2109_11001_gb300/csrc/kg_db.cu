@@ -15,20 +15,18 @@
 //      during a sweep: swaps only relabel slots) and write its binary32 record
 //      there; the 1.3 sigma criterion is decided on the records outside a
 //      rounding band and in binary64 inside it, so decisions are exact;
-//   2. k_db_eval: every attempt evaluated in parallel against the pre-sweep
-//      topology, one warp each (the 27 cells of a partner scan on its lanes).
-//      A "monomer" here is its compute index; the topology is the pair of
-//      maps slot -> monomer (comp_of) and monomer -> slot (slot_of);
-//   3. commit rounds (kg_db.cuh): an attempt's record is stale when an
-//      earlier accepted swap in the sweep touched one of its two chains, or
-//      put a junction monomer (whose bonds changed) within one cell of a
-//      monomer whose neighbourhood it scanned.  Nothing else an evaluation
-//      reads can change: swaps preserve positions, the bonds inside moved
-//      segments, and the lengths of the two pieces on either side of every
-//      bond.  Each round, k_db_restale re-evaluates the stale records across
-//      the GPU, then k_db_commit_next (one block per melt) commits the first
-//      accepted attempt: the two maps are rewritten for the slots of its two
-//      chains and box shifts are added to a per-monomer counter;
+//   2. k_db_eval: every attempt drawn in parallel against the pre-sweep
+//      topology, one warp each (the 27 cells of a partner scan on its lanes):
+//      its partner set and its partner.  A "monomer" here is its compute index;
+//      the topology is the pair of maps slot -> monomer (comp_of) and monomer ->
+//      slot (slot_of);
+//   3. k_db_rounds (kg_db.cuh): drawn swaps are decided, and committed in order
+//      in rounds: an attempt's record is stale when an earlier accepted swap in
+//      the sweep touched one of its two chains, or put a junction monomer (whose
+//      bonds changed) within one cell of a monomer whose neighbourhood it
+//      scanned.  Nothing else an evaluation reads can change: swaps preserve
+//      positions, the bonds inside moved segments, and the lengths of the two
+//      pieces on either side of every bond;
 //   4. k_db_finish: the box shifts are added to the positions in place; no
 //      monomer data moves (the maps are the topology).
 #include <cuda_runtime.h>
@@ -39,63 +37,80 @@
 
 namespace kg {
 
-// One attempt, one warp (the partner scans are warp-wide; lane 0 forms dE
-// and the decision in binary64 and broadcasts the record).
+// Attempt k: the drawn bond, its partner set and the partner drawn from it
+// (one warp).  flags 0 (empty set, or a capacity error, which is flagged), or
+// 1 | 4: to be decided from the parts below.
 template <class V>
-__device__ Attempt evaluate(const DBC &C, const V &v, WarpCand &wc, unsigned long long seed, long long sweep, int k,
-                            int paper, unsigned &err)
+__device__ void draw_attempt(const DBC &C, const V &v, WarpCand &wc, unsigned long long seed, long long sweep, int k,
+                             Attempt &a, unsigned &err)
 {
-    const int lane = threadIdx.x & 31;
     const MeltDev &md = C.md;
     const int N = md.N, off = md.off;
-    Attempt a;
     a.flags = 0;
     a.d = -1;
-    a.kind = a.A = a.B = a.pA = a.pB = 0;
-    a.jp[2] = a.jp[3] = -1;
+    a.kind = a.A = a.B = a.pA = a.pB = a.q = 0;
+    a.ver = 0;
+    a.cell[2] = a.cell[3] = -1;
+    a.p = a.dE = 0.0;
     const uint4 r = draw(seed, C.melt, 1, (unsigned long long)sweep, (uint32_t)k);
     const uint4 r2 = draw(seed, C.melt, 2, (unsigned long long)sweep, (uint32_t)k);
     const long long nbonds = (long long)md.n_ch * (N - 1);
     const long long bond = mul_hi64(((unsigned long long)r.y << 32) | r.x, (unsigned long long)nbonds);
-    const double uacc = ((double)(r.z >> 5) * 67108864.0 + (double)(r.w >> 6)) * (1.0 / 9007199254740992.0);
     const int c = (int)(bond / (N - 1)), b = (int)(bond % (N - 1));
     a.c = c;
-    a.jp[0] = v.occ(off + c * N + b);
-    a.jp[1] = v.occ(off + c * N + b + 1);
-    const int n1 = warp_partners<true>(C, v, c, b, wc, err);
-    if (n1 <= 0) return a;                              // empty, or a capacity error (flagged)
-    const Cand m = wc.cand[mul_hi64(((unsigned long long)r2.y << 32) | r2.x, (unsigned long long)n1)];
-    a.flags = 1;
+    a.cell[0] = C.cell[v.occ(off + c * N + b)];
+    a.cell[1] = C.cell[v.occ(off + c * N + b + 1)];
+    a.n = warp_partners<true>(C, v, c, b, wc, err);
+    if (a.n <= 0) return;
+    const Cand m = wc.cand[mul_hi64(((unsigned long long)r2.y << 32) | r2.x, (unsigned long long)a.n)];
+    a.flags = 1 | 4;
     a.d = m.d;
-    a.jp[2] = v.occ(off + m.d * N + m.q);
-    a.jp[3] = v.occ(off + m.d * N + m.q + 1);
-    const int n2 = warp_partners<false>(C, v, m.d, m.q, wc, err);
-    if (n2 <= 0) { err |= n2 < 0 ? ERR_DB_CAPACITY : ERR_DB_INTERNAL; return a; }
-    const int A = c < m.d ? c : m.d, B = c < m.d ? m.d : c;
-    const int pA = A == c ? b : m.q, pB = A == c ? m.q : b;
-    a.kind = m.kind; a.A = A; a.B = B; a.pA = pA; a.pB = pB;
-    const ViewMove<V> w{v, m.kind, A, B, pA, pB, N, off};
-    const int r1 = warp_partners<false>(C, w, A, pA, wc, err);
-    const int rr2 = warp_partners<false>(C, w, B, pB, wc, err);
-    if (r1 <= 0 || rr2 <= 0) { err |= (r1 < 0 || rr2 < 0) ? ERR_DB_CAPACITY : ERR_DB_INTERNAL; return a; }
-    int acc_bit = 0;
-    if (lane == 0) {
-        double dE = bond_fene(C, w, A, pA) + bond_fene(C, w, B, pB) - bond_fene(C, v, A, pA) - bond_fene(C, v, B, pB);
-        dE += bend(C, w, A, pA) + bend(C, w, A, pA + 1) + bend(C, w, B, pB) + bend(C, w, B, pB + 1);
-        dE -= bend(C, v, A, pA) + bend(C, v, A, pA + 1) + bend(C, v, B, pB) + bend(C, v, B, pB + 1);
-        const double ratio = (1.0 / r1 + 1.0 / rr2) / (1.0 / n1 + 1.0 / n2);
-        double acc = exp(-dE / C.T);
-        if (!paper) acc *= ratio;
-        acc_bit = uacc < acc;
+    a.q = m.q;
+    a.cell[2] = C.cell[v.occ(off + m.d * N + m.q)];
+    a.cell[3] = C.cell[v.occ(off + m.d * N + m.q + 1)];
+    a.kind = m.kind;
+    a.A = c < m.d ? c : m.d;
+    a.B = c < m.d ? m.d : c;
+    a.pA = a.A == c ? b : m.q;
+    a.pB = a.A == c ? m.q : b;
+}
+
+// Part t of deciding a drawn swap (one warp): the sizes of the partner sets of
+// the partner bond and, in the topology after the swap, of both new bonds, and
+// the energy change.
+constexpr int UNIFORM_TASKS = 4;
+
+template <class V>
+__device__ double swap_part(const DBC &C, const V &v, WarpCand &wc, const Attempt &a, int t, unsigned &err)
+{
+    const int lane = threadIdx.x & 31;
+    const ViewMove<V> w{v, a.kind, a.A, a.B, a.pA, a.pB, C.md.N, C.md.off};
+    if (t < 3) {
+        const int n = t == 0 ? warp_partners<false>(C, v, a.d, a.q, wc, err)
+                             : warp_partners<false>(C, w, t == 1 ? a.A : a.B, t == 1 ? a.pA : a.pB, wc, err);
+        if (n <= 0) err |= n < 0 ? ERR_DB_CAPACITY : ERR_DB_INTERNAL;
+        return (double)n;
     }
-    if (__shfl_sync(FULL_MASK, acc_bit, 0)) a.flags |= 2;
-    return a;
+    // dE: a lane per term (a binary64 square root, divide or logarithm is a long
+    // dependent chain), the sum in the order new bonds, old bonds, new angles, old angles
+    double term = 0.0;
+    if (lane < 4) {
+        term = bond_fene(C, ViewEither<V>{w, lane < 2}, lane & 1 ? a.B : a.A, lane & 1 ? a.pB : a.pA);
+    } else if (lane < 12) {
+        const int i = lane & 3;
+        term = bend(C, ViewEither<V>{w, lane < 8}, i < 2 ? a.A : a.B, (i < 2 ? a.pA : a.pB) + (i & 1));
+    }
+    auto at = [&](int k) { return __shfl_sync(FULL_MASK, term, k); };
+    double dE = at(0) + at(1) - at(2) - at(3);
+    dE += at(4) + at(5) + at(6) + at(7);
+    dE -= at(8) + at(9) + at(10) + at(11);
+    return dE;
 }
 
 constexpr int EVAL_WARPS_U = 4;                 // attempts (warps) per block of k_db_eval
 
 // (128, 12): at most 40 registers; the partner scans are latency-bound, and
-// more resident warps beat the spills (244 against 499 us for 160,000 attempts)
+// more resident warps beat the spills (160,000 attempts: 168 us)
 __global__ void __launch_bounds__(32 * EVAL_WARPS_U, 12) k_db_eval(const SimDev *__restrict__ Sp,
                                                               const StageDev *__restrict__ stp,
                                                               const double *__restrict__ x,
@@ -120,8 +135,8 @@ __global__ void __launch_bounds__(32 * EVAL_WARPS_U, 12) k_db_eval(const SimDev 
     while (g >= koff[m + 1]) ++m;
     const DBC C = make_dbc(S, *stp, m, x, pid, cell, start, list, rec, stp->T);
     unsigned err = 0;
-    const Attempt a = evaluate(C, ViewMap{comp_of, slot_of}, wcs[warp], S.seed, sweep, g - koff[m],
-                               S.paper_metropolis, err);
+    Attempt a;
+    draw_attempt(C, ViewMap{comp_of, slot_of}, wcs[warp], S.seed, sweep, g - koff[m], a, err);
     if (lane == 0) {
         att[g] = a;
         if (err) atomicOr(flags, err);
@@ -139,53 +154,48 @@ struct UniformEval {
     const int *comp_of, *slot_of;
     long long sweep;
     unsigned *flags;
-    WarpCand *wc;
-    __device__ void eval(int m, int k, int, Attempt &out)
+    WarpCand *wc;                // set by the kernel
+    static constexpr int TASKS = UNIFORM_TASKS;
+    __device__ DBC dbc(int m) const { return make_dbc(*S, *st, m, x, pid, cell, start, list, rec, st->T); }
+    __device__ void say(unsigned err) const
     {
-        const DBC C = make_dbc(*S, *st, m, x, pid, cell, start, list, rec, st->T);
+        if (err && (threadIdx.x & 31) == 0) atomicOr(flags, err);
+    }
+    __device__ void scan(int m, int k, int, Attempt &a)
+    {
         unsigned err = 0;
-        const Attempt a = evaluate(C, ViewMap{comp_of, slot_of}, *wc, S->seed, sweep, k, S->paper_metropolis, err);
-        if ((threadIdx.x & 31) == 0) {
-            out = a;
-            if (err) atomicOr(flags, err);
-        }
+        draw_attempt(dbc(m), ViewMap{comp_of, slot_of}, *wc, S->seed, sweep, k, a, err);
+        say(err);
+    }
+    __device__ double task(int m, const Attempt &a, int t)
+    {
+        unsigned err = 0;
+        const double v = swap_part(dbc(m), ViewMap{comp_of, slot_of}, *wc, a, t, err);
+        say(err);
+        return v;
+    }
+    __device__ bool accepts(int m, int k, const Attempt &a, const double *p) const
+    {
+        if (!(p[0] > 0.0 && p[1] > 0.0 && p[2] > 0.0)) return false;     // an error, flagged
+        double acc = exp(-p[3] / st->T);
+        if (!S->paper_metropolis) acc *= (1.0 / p[1] + 1.0 / p[2]) / (1.0 / a.n + 1.0 / p[0]);
+        return accept_u(S->seed, m, sweep, k) < acc;
     }
 };
 
 struct UniformRadius {
-    __device__ void init() {}
     __device__ int radius(const MeltDev &) const { return 1; }
 };
 
-constexpr int RESTALE_WARPS = 8;
+constexpr int ROUND_WARPS = 8;
 
-__global__ void __launch_bounds__(32 * RESTALE_WARPS) k_db_restale(
-    const SimDev *__restrict__ Sp, const StageDev *__restrict__ stp, const double *__restrict__ x,
-    const int *__restrict__ pid, const int *__restrict__ cell, const int *__restrict__ start,
-    const int *__restrict__ list, const float4 *__restrict__ rec, const int *__restrict__ koff,
-    const int *__restrict__ comp_of, const int *__restrict__ slot_of, Attempt *__restrict__ att, int *__restrict__ ver,
-    const int *__restrict__ chain_ver, const int *__restrict__ cell_ver, int *__restrict__ round, long long sweep,
-    unsigned *flags)
+// (256, 3): three records' checks and evaluations per scheduler in flight hide more than the registers cost
+__global__ void __launch_bounds__(32 * ROUND_WARPS, 3) k_db_rounds(RoundArgs R, UniformEval ev)
 {
-    __shared__ WarpCand wcs[RESTALE_WARPS];
-    if (flags[0]) return;                          // a latched error stops the sweep
-    UniformEval ev{Sp, stp, x, pid, cell, start, list, rec, comp_of, slot_of, sweep, flags,
-                   wcs + (threadIdx.x >> 5)};
-    restale_body(ev, *Sp, koff, att, ver, chain_ver, cell, cell_ver, round);
-}
-
-constexpr int COMMIT_THREADS = 512;
-
-__global__ void __launch_bounds__(COMMIT_THREADS) k_db_commit_next(
-    const SimDev *__restrict__ Sp, const double *__restrict__ x, const int *__restrict__ cell,
-    const int *__restrict__ koff, const Attempt *__restrict__ att, int *__restrict__ occ, int *__restrict__ curmap,
-    int *__restrict__ img, int *__restrict__ chain_ver, int *__restrict__ cell_ver, int *__restrict__ round,
-    long long *__restrict__ stats, unsigned *flags)
-{
-    extern __shared__ int old_occ[];              // 2N ints
+    __shared__ WarpCand wcs[ROUND_WARPS];
+    ev.wc = wcs + (threadIdx.x >> 5);
     UniformRadius pol;
-    commit_next_body(pol, *Sp, x, cell, koff, att, occ, curmap, img, chain_ver, cell_ver, round, stats, flags,
-                     old_occ);
+    rounds_body<32 * ROUND_WARPS>(ev, pol, R);
 }
 
 // end of a sweep: box shifts into the positions (x + L*img, as one rounding of
@@ -253,25 +263,37 @@ void db_finish(kg_ctx *c, long long *host_stats)
     cudaMemcpyAsync(host_stats, c->db_stats, sizeof(long long) * 4 * c->sim.n_melts, cudaMemcpyDeviceToHost, st);
 }
 
-void db_rounds_reset(kg_ctx *c, long long tot)
+void db_rounds_reset(kg_ctx *c)
 {
     cudaStream_t st = c->stream;
     cudaMemsetAsync(c->chain_ver, 0xFF, sizeof(int) * (size_t)c->n_chain_total, st);    // -1: untouched
     cudaMemsetAsync(c->dbmark, 0xFF, sizeof(int) * (size_t)c->ncell_db, st);
-    std::vector<int> r0((size_t)RS * MAX_MELTS, 0);
-    for (int m = 0; m < MAX_MELTS; ++m) r0[(size_t)RS * m + 4] = INT_MAX;   // no accepted attempt known
+    std::vector<int> r0((size_t)2 * RS * MAX_MELTS, 0);
+    for (int m = 0; m < 2 * MAX_MELTS; ++m) r0[(size_t)RS * m + 4] = INT_MAX;   // no accepted attempt known
     cudaMemcpyAsync(c->dbround, r0.data(), sizeof(int) * r0.size(), cudaMemcpyHostToDevice, st);
-    if (tot > 0) cudaMemsetAsync(c->att_ver, 0, sizeof(int) * (size_t)tot, st);
 }
 
-int db_max_chain_len(const kg_ctx *c)
+RoundArgs round_args(kg_ctx *c)
 {
-    int maxN = 0;
-    for (int m = 0; m < c->sim.n_melts; ++m) maxN = maxN > c->sim.melt[m].N ? maxN : c->sim.melt[m].N;
-    return maxN;
+    RoundArgs r{};
+    r.sim = c->d_sim;
+    r.x = c->x;
+    r.cell = c->dbcell;
+    r.koff = c->koff;
+    r.att = (Attempt *)c->att;
+    r.occ = c->comp_of;
+    r.curmap = c->slot_of;
+    r.img = c->img;
+    r.chain_ver = c->chain_ver;
+    r.cell_ver = c->dbmark;
+    r.round = c->dbround;
+    r.old = (int *)c->scratch;
+    r.stats = c->db_stats;
+    r.flags = c->flags;
+    return r;
 }
 
-void db_sweep(kg_ctx *c, const std::vector<long long> &K, long long *host_stats)
+cudaError_t db_sweep(kg_ctx *c, const std::vector<long long> &K, long long *host_stats)
 {
     cudaStream_t st = c->stream;
     const int nm = c->sim.n_melts;
@@ -285,25 +307,14 @@ void db_sweep(kg_ctx *c, const std::vector<long long> &K, long long *host_stats)
             c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist, c->dbrec, c->koff, c->comp_of,
             c->slot_of, att, c->sweep, c->flags);
     // ordered commit in rounds (kg_db.cuh)
-    db_rounds_reset(c, tot);
-    const int maxN = db_max_chain_len(c);
-    const size_t sm = sizeof(int) * 2 * (size_t)maxN;
-    cudaFuncSetAttribute(k_db_commit_next, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    const int rgrid = std::max(1, std::min(nblk(tot, 32 * RESTALE_WARPS), 152 * 8));
-    db_rounds(c, tot,
-              [&] {
-                  k_db_restale<<<rgrid, 32 * RESTALE_WARPS, 0, st>>>(
-                      c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist, c->dbrec, c->koff,
-                      c->comp_of, c->slot_of, att, c->att_ver, c->chain_ver, c->dbmark, c->dbround, c->sweep,
-                      c->flags);
-              },
-              [&] {
-                  k_db_commit_next<<<nm, COMMIT_THREADS, sm, st>>>(c->d_sim, c->x, c->dbcell, c->koff, att,
-                                                                   c->comp_of, c->slot_of, c->img, c->chain_ver,
-                                                                   c->dbmark, c->dbround, c->db_stats, c->flags);
-              });
+    db_rounds_reset(c);
+    const UniformEval ev{c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist, c->dbrec,
+                         c->comp_of, c->slot_of, c->sweep, c->flags, nullptr};
+    const cudaError_t e = rounds_launch(c, k_db_rounds, 32 * ROUND_WARPS, 0, tot, nm, round_args(c), ev);
+    if (e != cudaSuccess) return e;
     c->launches += 1;
     db_finish(c, host_stats);
+    return cudaSuccess;
 }
 
 }  // namespace kg

@@ -4,8 +4,10 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 
+#include "kg_gridbar.cuh"
 #include "kg_host.h"
 
 namespace kg {
@@ -75,6 +77,13 @@ __device__ __forceinline__ bool within(const DBC &C, int a, int b)
     return d2(C, a, b) <= C.lim2;
 }
 
+// the acceptance uniform of attempt k
+__device__ __forceinline__ double accept_u(unsigned long long seed, int melt, long long sweep, int k)
+{
+    const uint4 r = draw(seed, melt, 1, (unsigned long long)sweep, (uint32_t)k);
+    return ((double)(r.z >> 5) * 67108864.0 + (double)(r.w >> 6)) * (1.0 / 9007199254740992.0);
+}
+
 // per-warp candidate scratch of one partner enumeration
 struct __align__(16) WarpCand {
     Cand tmp[CAND_CAP];
@@ -102,17 +111,30 @@ __device__ int warp_partners(const DBC &C, const V &v, int c, int b, WarpCand &w
     __syncwarp();
     bool bad = false;
     if (lane < 27) {
-        const int n = md.ndb, c0 = C.cell[pu] - md.dbcell_off;
-        const int cx = c0 % n, cy = (c0 / n) % n, cz = c0 / (n * n);
+        // the record names the cell; list entries, and then their slots, are
+        // loaded four at a time: an evaluation is a chain of L2 round trips
+        const int n = md.ndb;
+        const unsigned code = __float_as_uint(__ldg(C.rec + pu).w);
+        const int cx = (int)(code & CODE_MASK), cy = (int)((code >> CODE_BITS) & CODE_MASK);
+        const int cz = (int)(code >> (2 * CODE_BITS));
         const int dz = lane / 9 - 1, dy = (lane / 3) % 3 - 1, dx = lane % 3 - 1;
         const int cell = md.dbcell_off + (((cz + dz + n) % n) * n + (cy + dy + n) % n) * n + (cx + dx + n) % n;
         const int b0 = C.start[cell], e = C.start[cell + 1];
         if (e - b0 > MAX_CELL_OCC) {
             bad = true;
         } else {
+            int tt[4], sl[4];
             for (int k = b0; k < e; ++k) {
-                const int t = C.list[k];
-                const int ts = v.cur(t), r = ts - md.off, d = r / N, i = r - d * N;
+                if (((k - b0) & 3) == 0) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) tt[u] = C.list[min(k + u, e - 1)];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) sl[u] = v.cur(tt[u]);
+                }
+                const int u = (k - b0) & 3;
+                const int t = u == 0 ? tt[0] : u == 1 ? tt[1] : u == 2 ? tt[2] : tt[3];
+                const int ts = u == 0 ? sl[0] : u == 1 ? sl[1] : u == 2 ? sl[2] : sl[3];
+                const int r = ts - md.off, d = r / N, i = r - d * N;
                 if (d == c) continue;
                 if (i != b + 1 && i != N - 2 - b) continue;   // neither kind can use t
                 if (!within(C, pu, t)) continue;
@@ -197,6 +219,17 @@ __device__ double bend(const DBC &C, const V &v, int chain, int i)
     return C.md.kappa * (1.0 - vcos(C, v, chain, i));
 }
 
+// v or the topology after a swap, chosen per lane
+template <class V>
+struct ViewEither {
+    ViewMove<V> m;
+    bool moved;
+    __device__ __forceinline__ int occ(int s) const
+    {
+        return m.b.occ(moved ? swap_slot(s, m.kind, m.A, m.B, m.pA, m.pB, m.N, m.off) : s);
+    }
+};
+
 __device__ __forceinline__ DBC make_dbc(const SimDev &S, const StageDev &st, int m, const double *x,
                                         const int *pid, const int *cell, const int *start, const int *list,
                                         const float4 *rec, double T)
@@ -210,219 +243,318 @@ __device__ __forceinline__ DBC make_dbc(const SimDev &S, const StageDev &st, int
 
 // ---------------------------------------------------------------------------
 // Ordered commit in rounds.  Every attempt record carries the number of swaps
-// committed (in its melt) when it was evaluated, ver[k]; chains and cells of
-// the 1.3 sigma grid carry the number of the last commit that touched them
-// (chain_ver, cell_ver; -1 for none).  A record is stale when a commit at or
-// after its version touched one of its two chains, or stamped a cell within
-// P::radius cells of one of its junction monomers: only then can its
-// evaluation differ, since swaps preserve positions, the bonds inside moved
-// segments and the lengths of the pieces on either side of every bond.
+// committed (in its melt) when it was evaluated; chains and cells of the 1.3
+// sigma grid carry the number of the last commit that touched them (chain_ver,
+// cell_ver; -1 for none).  A record is stale when a commit at or after its
+// version touched one of its two chains, or stamped a cell within P::radius
+// cells of one of its junction monomers: only then can its evaluation differ,
+// since swaps preserve positions, the bonds inside moved segments and the
+// lengths of the pieces on either side of every bond.
 // One round: (A) every stale record at or after the melt's position is
-// re-evaluated against the current topology, across the whole GPU, one warp
-// per attempt; (B) one block per melt finds the first accepted attempt from
-// its position (every record there is now current), commits it (slot maps,
-// box shifts, chain and cell stamps) and moves the position past it, or, if
-// there is none, finishes the melt (statistics).  Rounds repeat until every
-// melt is finished: as many rounds as accepted swaps plus one, and the result
-// is that of the strictly sequential loop over attempts.
-// round[RS m + 0..4] = position, commits, finished, re-evaluations, and the
-// first accepted attempt at or after the position (INT_MAX: none), which pass
-// (A) records while it reads every current record, so (B) needs no search.
+// re-evaluated against the current topology, across the whole GPU; (B) the
+// first accepted attempt of each melt from its position (every record there is
+// now current) is committed: one block rewrites the slot maps and adds the
+// box shifts, all blocks stamp cells; or, if there is none, the melt is
+// finished (statistics).  Rounds repeat until every melt is finished: as many
+// rounds as accepted swaps plus one, and the result is that of the strictly
+// sequential loop over attempts.
+// All rounds run in one cooperative launch, two grid barriers a round, the
+// second of which also says whether a melt is left.  An evaluation is a long
+// chain of dependent loads and binary64 operations, and a round waits for its
+// slowest one, so it is cut in two: the draw and the partner scan of the drawn
+// bond, one warp per record (most sets are empty, and done); then, for a
+// non-empty set, E::TASKS independent parts on as many warps.  160,000
+// attempts of a 1.6M-monomer melt (21 swaps): 536 us, against about 1,450 as two
+// launches a round with the host reading the finished flags now and then, an
+// attempt evaluated by one warp and the dE of a swap by one lane.
+// round[RS m + 0..5] of one of two buffers (by round parity: commits write the
+// next round's while every block reads this one's) = position, commits,
+// finished, re-evaluations, the first accepted attempt at or after the position
+// (INT_MAX: none), empty records.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool stale_rec(const Attempt &a, int v, const int *__restrict__ chain_ver, int choff,
-                                          const int *__restrict__ cell, const int *__restrict__ cell_ver)
+__device__ __forceinline__ bool stale_rec(int4 head, int4 cells, const int *chain_ver, int choff, const int *cell_ver)
 {
-    if (chain_ver[choff + a.c] >= v) return true;
-    if ((a.flags & 1) && chain_ver[choff + a.d] >= v) return true;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        if (a.jp[q] >= 0 && cell_ver[cell[a.jp[q]]] >= v) return true;
-    return false;
+    const int v = head.w;
+    int newest = chain_ver[choff + head.y];                    // loads of one latency, then one comparison
+    if (head.x & 1) newest = max(newest, chain_ver[choff + head.z]);
+    if (cells.x >= 0) newest = max(newest, cell_ver[cells.x]);
+    if (cells.y >= 0) newest = max(newest, cell_ver[cells.y]);
+    if (cells.z >= 0) newest = max(newest, cell_ver[cells.z]);
+    if (cells.w >= 0) newest = max(newest, cell_ver[cells.w]);
+    return newest >= v;
 }
 
-// (A) E provides eval(m, k_in_melt, k_global, Attempt &out) for one whole warp
-// (lane 0 leaves the record in out).
-template <class E>
-__device__ void restale_body(E &ev, const SimDev &S, const int *__restrict__ koff, Attempt *__restrict__ att,
-                             int *__restrict__ ver, const int *__restrict__ chain_ver, const int *__restrict__ cell,
-                             const int *__restrict__ cell_ver, int *__restrict__ round)
+struct RoundArgs {
+    const SimDev *sim;
+    const double *x;
+    const int *cell, *koff;
+    Attempt *att;
+    int *occ, *curmap, *img, *chain_ver, *cell_ver;
+    int *round;                  // [2][MAX_MELTS][RS]
+    int *old;                    // [2 M]: slot maps of the two chains of a commit, per melt
+    long long *stats;
+    unsigned *flags;
+    unsigned long long *bar;     // three barrier words, zero at launch
+    unsigned spin;
+    long long most;              // rounds (attempts + 1)
+};
+
+// (A) by blocks of THREADS records.  E provides, each for one whole warp,
+//   scan(m, k, g, Attempt &a): draw attempt k (global index g) of melt m and its partner; flags 0, or 1 | 4
+//   task(m, a, t): part t < TASKS of deciding a, as a binary64 value
+// and for one thread accepts(m, k, a, const double *parts).
+template <int THREADS, class E>
+__device__ void restale_pass(E &ev, const RoundArgs &R, int *round, bool first)
 {
-    const int lane = threadIdx.x & 31;
-    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarp = (int)((gridDim.x * blockDim.x) >> 5);
-    const int Ktot = koff[S.n_melts];
-    for (int base = gw * 32; base < Ktot; base += nwarp * 32) {
-        const int k = base + lane;
-        bool st = false, live = false;
+    __shared__ int todo[THREADS], und[THREADS], n_todo, n_und;
+    __shared__ double part[THREADS][E::TASKS];
+    const SimDev &S = *R.sim;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = THREADS / 32;
+    const int Ktot = R.koff[S.n_melts];
+    auto melt = [&](int k) {
         int m = 0;
+        while (k >= R.koff[m + 1]) ++m;
+        return m;
+    };
+    for (int base = blockIdx.x * THREADS; base < Ktot; base += gridDim.x * THREADS) {
+        const int k = base + threadIdx.x;
+        bool st = false, un = false, acc = false, empty = false;
+        int m = 0;
+        if (threadIdx.x == 0) n_todo = n_und = 0;
         if (k < Ktot) {
-            while (k >= koff[m + 1]) ++m;
-            const int *R = round + RS * m;
-            if (!R[2] && k - koff[m] >= R[0]) {
-                st = stale_rec(att[k], ver[k], chain_ver, S.melt[m].ch_off, cell, cell_ver);
-                live = true;
+            m = melt(k);
+            const int *rd = round + RS * m;
+            if (!rd[2] && k - R.koff[m] >= rd[0]) {
+                const int4 *rec = reinterpret_cast<const int4 *>(R.att + k);
+                const int4 head = rec[0], cells = rec[1];
+                st = stale_rec(head, cells, R.chain_ver, S.melt[m].ch_off, R.cell_ver);
+                un = !st && (head.x & 4);
+                acc = !st && (head.x & 2);
+                empty = !(head.x & 1);
             }
         }
-        // fresh records are current: note the first accepted one of each melt
+        // fresh records are current: note the first accepted one of each melt (and, once, count the empty ones)
         const int m0 = __shfl_sync(FULL_MASK, m, 0);
-        const bool acc = live && !st && (att[k].flags & 2);
-        if (__all_sync(FULL_MASK, !live || m == m0)) {  // one melt in the warp: one atomic
-            const int first = __reduce_min_sync(FULL_MASK, acc ? k - koff[m] : INT_MAX);
-            if (lane == 0 && first != INT_MAX) atomicMin(round + RS * m0 + 4, first);
-        } else if (acc) {
-            atomicMin(round + RS * m + 4, k - koff[m]);
+        if (__all_sync(FULL_MASK, k >= Ktot || m == m0)) {       // one melt in the warp: one atomic
+            const int f = __reduce_min_sync(FULL_MASK, acc ? k - R.koff[m] : INT_MAX);
+            const int ne = __popc(__ballot_sync(FULL_MASK, empty));
+            if (lane == 0 && f != INT_MAX) atomicMin(round + RS * m0 + 4, f);
+            if (lane == 0 && first && ne) atomicAdd(round + RS * m0 + 5, ne);
+        } else {
+            if (acc) atomicMin(round + RS * m + 4, k - R.koff[m]);
+            if (first && empty) atomicAdd(round + RS * m + 5, 1);
         }
-        unsigned bal = __ballot_sync(FULL_MASK, st);
-        while (bal) {
-            const int src = __ffs(bal) - 1;
-            bal &= bal - 1;
-            const int kk = __shfl_sync(FULL_MASK, k, src), mm = __shfl_sync(FULL_MASK, m, src);
+        if (!__syncthreads_or(st || un)) continue;
+        if (st) todo[atomicAdd(&n_todo, 1)] = k;
+        if (un) und[atomicAdd(&n_und, 1)] = k;
+        __syncthreads();
+        for (int i = warp; i < n_todo; i += NW) {
+            const int kk = todo[i], mm = melt(kk);
             Attempt a;
-            ev.eval(mm, kk - koff[mm], kk, a);
+            ev.scan(mm, kk - R.koff[mm], kk, a);
             if (lane == 0) {
-                att[kk] = a;
-                ver[kk] = round[RS * mm + 1];
+                const int was = R.att[kk].flags & 1, is = a.flags & 1;
+                a.ver = round[RS * mm + 1];
+                R.att[kk] = a;
                 atomicAdd(round + RS * mm + 3, 1);
-                if (a.flags & 2) atomicMin(round + RS * mm + 4, kk - koff[mm]);
+                if (was != is) atomicAdd(round + RS * mm + 5, was - is);
+                if (is) und[atomicAdd(&n_und, 1)] = kk;
             }
             __syncwarp();
         }
+        __syncthreads();
+        const int nu = n_und;
+        for (int i = warp; i < nu * E::TASKS; i += NW) {
+            const int kk = und[i / E::TASKS], t = i % E::TASKS;
+            const double v = ev.task(melt(kk), R.att[kk], t);
+            if (lane == 0) part[i / E::TASKS][t] = v;
+            __syncwarp();
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < nu) {
+            const int kk = und[threadIdx.x], mm = melt(kk);
+            const bool yes = ev.accepts(mm, kk - R.koff[mm], R.att[kk], part[threadIdx.x]);
+            R.att[kk].flags = yes ? 3 : 1;
+            if (yes) atomicMin(round + RS * mm + 4, kk - R.koff[mm]);
+        }
+        __syncthreads();
     }
 }
 
-// (B) one block per melt; P provides init (block-wide) and radius.
+// (B) every block; block m % gridDim.x rewrites melt m's maps.  P provides
+// radius.  nx: the next round's state.  True while the melt is unfinished.
 template <class P>
-__device__ void commit_next_body(P &pol, const SimDev &S, const double *__restrict__ x, const int *__restrict__ cell,
-                                 const int *__restrict__ koff, const Attempt *__restrict__ att,
-                                 int *__restrict__ occ, int *__restrict__ curmap, int *__restrict__ img,
-                                 int *__restrict__ chain_ver, int *__restrict__ cell_ver, int *__restrict__ round,
-                                 long long *__restrict__ stats, unsigned *flags, int *old_occ)
+__device__ bool commit_pass(P &pol, const RoundArgs &A, int m, const int *round, int *next)
 {
-    __shared__ int found_s, sh[6], done_s;
-    __shared__ unsigned long long n_empty;
-    const int m = blockIdx.x, tid = threadIdx.x;
-    int *R = round + RS * m;
-    if (tid == 0) done_s = R[2] || flags[0] != 0;
-    __syncthreads();
-    if (done_s) return;
+    __shared__ int sh[6];
+    const SimDev &S = *A.sim;
+    const int tid = threadIdx.x;
+    const int *R = round + RS * m;
+    int *X = next + RS * m;
     const MeltDev &md = S.melt[m];
     const int N = md.N, off = md.off, Mp = S.Mp;
-    const int k0 = koff[m], K = koff[m + 1] - k0;
-    // the first accepted attempt at or after the position, as pass (A) found it
-    if (tid == 0) found_s = R[4] < K ? R[4] : K;
-    __syncthreads();
-    const int found = found_s;
-    if (found == K) {                              // the melt is finished
-        if (tid == 0) n_empty = 0;
-        __syncthreads();
-        unsigned long long e = 0;
-        for (int k = tid; k < K; k += blockDim.x) e += !(att[k0 + k].flags & 1);
-        atomicAdd(&n_empty, e);
-        __syncthreads();
-        if (tid == 0) {
-            stats[4 * m + 0] = K;
-            stats[4 * m + 1] = (long long)n_empty;
-            stats[4 * m + 2] = R[1];
-            stats[4 * m + 3] = R[3];
-            if (R[1]) atomicOr(flags + 1, 1u);
-            R[2] = 1;
+    const int k0 = A.koff[m], K = A.koff[m + 1] - k0;
+    const bool mine = m % (int)gridDim.x == (int)blockIdx.x;
+    const int found = min(R[4], K);                // the first accepted attempt at or after the position
+    const int nc = R[1];
+    if (R[2] || found == K) {                      // the melt is finished
+        if (mine && tid == 0) {
+            if (!R[2]) {
+                A.stats[4 * m + 0] = K;
+                A.stats[4 * m + 1] = R[5];
+                A.stats[4 * m + 2] = nc;
+                A.stats[4 * m + 3] = R[3];
+                if (nc) atomicOr(A.flags + 1, 1u);
+            }
+            X[2] = 1;
         }
-        return;
+        return false;
     }
-    pol.init();
+    const Attempt &a = A.att[k0 + found];
     const int Rr = pol.radius(md);
-    const Attempt a = att[k0 + found];
-    const int kind = a.kind, A = a.A, Bc = a.B, pA = a.pA, pB = a.pB, nc = R[1];
-    const int baseA = off + A * N, baseB = off + Bc * N;
-    for (int j = tid; j < N; j += blockDim.x) {
-        old_occ[j] = occ[baseA + j];
-        old_occ[N + j] = occ[baseB + j];
-    }
-    __syncthreads();
-    for (int j = tid; j < 2 * N; j += blockDim.x) {
-        const int s = j < N ? baseA + j : baseB + (j - N);
-        const int src = swap_slot(s, kind, A, Bc, pA, pB, N, off);
-        const int val = src - baseA < N && src >= baseA ? old_occ[src - baseA] : old_occ[N + src - baseB];
-        occ[s] = val;
-        curmap[val] = s;
-    }
-    __syncthreads();
-    if (tid < 2) {
-        // segment 0: A' slots pA+1..N-1 anchored at A' slot pA;
-        // segment 1: kind 0 -> B' slots pA+1..N-1 at pA; kind 1 -> B' slots 0..pB at pB+1
-        int f, an;
-        if (tid == 0) { f = occ[baseA + pA + 1]; an = occ[baseA + pA]; }
-        else if (kind == 0) { f = occ[baseB + pA + 1]; an = occ[baseB + pA]; }
-        else { f = occ[baseB + pB]; an = occ[baseB + pB + 1]; }
-#pragma unroll
-        for (int d = 0; d < 3; ++d)
-            sh[3 * tid + d] = -((int)rint(__ddiv_rn(__dsub_rn(x[d * Mp + f], x[d * Mp + an]), md.L))
-                                + img[d * Mp + f] - img[d * Mp + an]);
-    }
-    __syncthreads();
-    for (int j = tid; j < 2 * N; j += blockDim.x) {
-        int seg = -1, s;
-        if (j < N) {
-            s = baseA + j;
-            if (j > pA) seg = 0;
-        } else {
-            const int jj = j - N;
-            s = baseB + jj;
-            if ((kind == 0 && jj > pA) || (kind == 1 && jj <= pB)) seg = 1;
-        }
-        if (seg >= 0) {
-            const int p = occ[s];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) img[d * Mp + p] += sh[3 * seg + d];
-        }
-    }
-    // stamp the two chains and the cells within Rr of the four junction monomers
+    // stamp the cells within Rr of the four junction monomers, over the grid
     const int n = md.ndb, W = 2 * Rr + 1;
-    for (int q = 0; q < 4; ++q) {
-        const int p = a.jp[q];
-        if (p < 0) continue;
-        const int c0 = cell[p] - md.dbcell_off;
+    for (int t = blockIdx.x * blockDim.x + tid; t < 4 * W * W * W; t += gridDim.x * blockDim.x) {
+        const int q = t / (W * W * W), r = t - q * W * W * W;
+        const int cq = a.cell[q];
+        if (cq < 0) continue;
+        const int c0 = cq - md.dbcell_off;
         const int cx = c0 % n, cy = (c0 / n) % n, cz = c0 / (n * n);
-        for (int t = tid; t < W * W * W; t += blockDim.x) {
-            const int dx = t % W - Rr, dy = (t / W) % W - Rr, dz = t / (W * W) - Rr;
-            const int xx = ((cx + dx) % n + n) % n, yy = ((cy + dy) % n + n) % n;
-            const int zz = ((cz + dz) % n + n) % n;
-            cell_ver[md.dbcell_off + (zz * n + yy) * n + xx] = nc;
+        const int dx = r % W - Rr, dy = (r / W) % W - Rr, dz = r / (W * W) - Rr;
+        const int xx = ((cx + dx) % n + n) % n, yy = ((cy + dy) % n + n) % n;
+        const int zz = ((cz + dz) % n + n) % n;
+        A.cell_ver[md.dbcell_off + (zz * n + yy) * n + xx] = nc;
+    }
+    if (!mine) return true;
+    const int kind = a.kind, cA = a.A, cB = a.B, pA = a.pA, pB = a.pB;
+    const int baseA = off + cA * N, baseB = off + cB * N;
+    // box shifts of the moved segments; segment 0: A' slots pA+1..N-1 anchored at A' slot pA; segment 1: kind 0 ->
+    // B' slots pA+1..N-1 at pA, kind 1 -> B' slots 0..pB at pB+1 (maps still before the swap)
+    if (tid < 6) {
+        const int seg = tid / 3, d = tid % 3;
+        const int fs = seg == 0 ? baseA + pA + 1 : (kind == 0 ? baseB + pA + 1 : baseB + pB);
+        const int as = seg == 0 ? baseA + pA : (kind == 0 ? baseB + pA : baseB + pB + 1);
+        const int f = A.occ[swap_slot(fs, kind, cA, cB, pA, pB, N, off)];
+        const int an = A.occ[swap_slot(as, kind, cA, cB, pA, pB, N, off)];
+        sh[tid] = -((int)rint(__ddiv_rn(__dsub_rn(A.x[d * Mp + f], A.x[d * Mp + an]), md.L))
+                    + A.img[d * Mp + f] - A.img[d * Mp + an]);
+    }
+    // new slot maps: read whole before they are written, PER entries of a
+    // thread in registers (all loads in flight together); longer chains go
+    // through a copy of the two chains' maps
+    constexpr int PER = 16;
+    const bool copy = 2 * N > PER * (int)blockDim.x;
+    int *old_occ = A.old + 2 * off;
+    int val[PER];
+    if (copy) {
+        for (int j = tid; j < 2 * N; j += blockDim.x) old_occ[j] = A.occ[j < N ? baseA + j : baseB + (j - N)];
+    } else {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int j = tid + q * blockDim.x;
+            if (j < 2 * N)
+                val[q] = A.occ[swap_slot(j < N ? baseA + j : baseB + (j - N), kind, cA, cB, pA, pB, N, off)];
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        chain_ver[md.ch_off + A] = nc;
-        chain_ver[md.ch_off + Bc] = nc;
-        R[1] = nc + 1;
-        R[0] = found + 1;
-        R[4] = INT_MAX;                            // to be found again by the next pass (A)
+    auto moved = [&](int j, int p) {                 // entry j of the two chains is now monomer p
+        const int s = j < N ? baseA + j : baseB + (j - N);
+        A.occ[s] = p;
+        A.curmap[p] = s;
+        const int jj = j - N;
+        const int seg = j < N ? (j > pA ? 0 : -1) : (((kind == 0 && jj > pA) || (kind == 1 && jj <= pB)) ? 1 : -1);
+        if (seg >= 0) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                if (sh[3 * seg + d]) A.img[d * Mp + p] += sh[3 * seg + d];
+        }
+    };
+    if (copy) {
+        for (int j = tid; j < 2 * N; j += blockDim.x) {
+            const int src = swap_slot(j < N ? baseA + j : baseB + (j - N), kind, cA, cB, pA, pB, N, off);
+            moved(j, src - baseA < N && src >= baseA ? old_occ[src - baseA] : old_occ[N + src - baseB]);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int j = tid + q * blockDim.x;
+            if (j < 2 * N) moved(j, val[q]);
+        }
     }
+    if (tid == 0) {
+        A.chain_ver[md.ch_off + cA] = nc;
+        A.chain_ver[md.ch_off + cB] = nc;
+        X[0] = found + 1;
+        X[1] = nc + 1;
+        X[2] = 0;
+        X[3] = R[3];
+        X[4] = INT_MAX;                            // to be found again by the next pass (A)
+        X[5] = R[5];
+    }
+    __syncthreads();                               // sh is used again for the next melt
+    return true;
 }
 
-// Commit rounds until every melt is finished (host).  restale() and
-// commit_next() enqueue one pass each; the host reads the per-melt finished
-// flags after rounds 1, 2, 4, 8 and then every 8 (the passes of a finished melt
-// return at once), and stops on a latched device error.
-template <class FA, class FB>
-void db_rounds(kg_ctx *c, long long tot, FA restale, FB commit_next)
+// all rounds of a sweep; every block of a cooperative launch (ev, pol as above)
+template <int THREADS, class E, class P>
+__device__ void rounds_body(E &ev, P &pol, const RoundArgs &R)
 {
-    static thread_local int *hround = nullptr;
-    if (!hround && cudaMallocHost(&hround, sizeof(int) * (RS * MAX_MELTS + 1)) != cudaSuccess) return;
-    const int nm = c->sim.n_melts;
-    long long r = 0, next_check = 1;
-    while (r <= tot) {                              // at most one round per accepted swap, plus one
-        restale();
-        commit_next();
-        c->launches += 2;
-        if (++r < next_check) continue;
-        cudaMemcpyAsync(hround, c->dbround, sizeof(int) * RS * nm, cudaMemcpyDeviceToHost, c->stream);
-        cudaMemcpyAsync(hround + RS * MAX_MELTS, c->flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-        if (cudaStreamSynchronize(c->stream) != cudaSuccess) return;
-        bool all = true;
-        for (int m = 0; m < nm; ++m) all = all && hround[RS * m + 2] != 0;
-        if (all || hround[RS * MAX_MELTS] != 0) return;
-        next_check = r < 8 ? 2 * r : r + 8;
+    __shared__ unsigned acc_s[2], out_s;
+    const bool stop = *(volatile unsigned *)R.flags != 0u;     // a latched error stops the sweep; written only after
+    if (threadIdx.x < 2) acc_s[threadIdx.x] = 0u;              //   every block has arrived at the first barrier
+    __syncthreads();
+    if (stop) return;
+    GridBar gb{R.bar, acc_s, &out_s, R.spin, 0};
+    unsigned told = 0;
+    for (long long r = 0; r <= R.most; ++r) {
+        int *round = R.round + (r & 1) * RS * MAX_MELTS, *next = R.round + ((r + 1) & 1) * RS * MAX_MELTS;
+        restale_pass<THREADS>(ev, R, round, r == 0);
+        if (threadIdx.x == 0 && r > 0 && *(volatile unsigned *)R.flags) gb.note(FAIL);
+        if ((told = gb.sync()) & (FAIL | GAVE_UP)) break;
+        bool left = false;
+        for (int m = 0; m < R.sim->n_melts; ++m) left |= commit_pass(pol, R, m, round, next);
+        if (threadIdx.x == 0 && left) gb.note(REQ);
+        told = gb.sync();
+        if (!(told & REQ) || (told & (FAIL | GAVE_UP))) break;
     }
+    if (threadIdx.x == 0 && (told & GAVE_UP)) atomicOr(R.flags, ERR_TIMEOUT);
+}
+
+RoundArgs round_args(kg_ctx *c);                // kg_db.cu
+
+constexpr unsigned ROUNDS_SPIN = 1u << 24;         // barrier polls (tens of ns at least) before giving up
+
+// Launches kernel K (blocks of `threads`, smem bytes, RoundArgs in r, then the
+// evaluator's arguments) on as many blocks as the attempts need and the GPU holds.
+template <class KERNEL, class... ARGS>
+cudaError_t rounds_launch(kg_ctx *c, KERNEL K, int threads, size_t smem, long long tot, int nm, RoundArgs r, ARGS... args)
+{
+    int dev = 0, nsm = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, K, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (per < 1) return cudaErrorCooperativeLaunchTooLarge;
+    const long long want = (tot + threads - 1) / threads;      // a thread looks at one record
+    const long long nb = std::min((long long)per * nsm, std::max((long long)nm, std::max(want, 1LL)));
+    e = cudaMemsetAsync(c->dbbar, 0, 3 * sizeof(unsigned long long), c->stream);
+    if (e != cudaSuccess) return e;
+    r.bar = c->dbbar;
+    r.spin = ROUNDS_SPIN;
+    r.most = tot;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)nb);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    c->launches += 1;
+    return cudaLaunchKernelEx(&cfg, K, r, args...);
 }
 
 }  // namespace kg

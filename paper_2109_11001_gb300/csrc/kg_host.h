@@ -90,10 +90,10 @@ struct kg_ctx {
     int *chain_ver = nullptr;    // per chain: number of the last commit of the sweep that touched it
     int n_chain_total = 0;
     int *dbround = nullptr;      // per melt: position, commits, finished, re-evaluations
-    int *att_ver = nullptr;      // per attempt: commits seen by its record
     void *att = nullptr;         // kg::Attempt[att_cap]
     long long att_cap = 0;
     int *koff = nullptr;         // [n_melts+1] attempt offsets
+    unsigned long long *dbbar = nullptr;   // grid-barrier words of the commit rounds
     int *img = nullptr;
     long long *db_stats = nullptr;   // [n_melts][4]
 
@@ -106,7 +106,7 @@ struct kg_ctx {
     long long adam_t = 0;                // Adam steps taken
     long long train_iter = 0;            // minibatches drawn
     double *logf = nullptr, *logt = nullptr;   // per-attempt staging of the sweep log
-    int *logn = nullptr;
+    int *logn = nullptr, *logoff = nullptr;    // rows of each attempt, their offsets (and the scan's block sums)
     long long log_att_cap = 0;
     double *trainf = nullptr, *traint = nullptr;  // training ring [train_cap][24], [train_cap]
     long long train_cap = 0;
@@ -153,11 +153,18 @@ constexpr unsigned RESIDENT_SPIN = 1u << 22;  // its barrier polls (a few hundre
 constexpr unsigned PERSIST_SPIN = 1u << 24;   // grid-barrier polls (~64 ns apart) before ERR_TIMEOUT
 constexpr int RS = 8;                    // ints per melt in the DB commit-round array
 
-struct Attempt {
-    int flags;                   // 1: non-empty partner set, 2: accepted
+// A sweep's record of one attempt.  The staleness check of every round reads
+// the first 32 bytes only.
+struct __align__(16) Attempt {
+    int flags;                   // 1: non-empty partner set, 2: accepted, 4: partner drawn, not yet decided
     int c, d;                    // chain of the drawn bond, chain of the chosen partner
+    int ver;                     // commits of the melt that the evaluation had seen
+    int cell[4];                 // 1.3 sigma cells of the junction monomers (-1: unused)
     int kind, A, B, pA, pB;      // canonical move
-    int jp[4];                   // junction particles (-1: unused)
+    int q;                       // partner bond of chain d
+    int n;                       // partners of the drawn bond
+    int pad;
+    double p, dE;                // learned proposal: probability of the pick, energy change
 };
 
 // kg_md.cu
@@ -168,7 +175,7 @@ void set_device_step(kg_ctx *c, long long v);
 void forces_eval(kg_ctx *c, int melt, long long step, double *F_dev, double *part_dev, int nblk);
 void prof_collect(kg_ctx *c);                // fold recorded event pairs into the totals
 void bonded_partners(kg_ctx *c);             // bp from slot_of / comp_of
-void scan_counts(kg_ctx *c, const int *count, int *start, int n);   // exclusive scan, start[n] the total
+void scan_counts(kg_ctx *c, const int *count, int *start, int n, int *bsum);   // exclusive scan, start[n] the total
 void md_sort(kg_ctx *c);                     // re-sort the state into the last cell order
 void md_materialize(kg_ctx *c);              // mixed: x <- xb64 + dlt[cur]
 void graphs_reset(kg_ctx *c);                // drop captured step graphs (their arguments changed)
@@ -193,16 +200,15 @@ void pid_to_slots(kg_ctx *c, int melt, int *out_dev);
 int forces_blocks(const kg_ctx *c, int melt);
 
 // kg_db.cu
-void db_sweep(kg_ctx *c, const std::vector<long long> &K, long long *host_stats /*[n_melts][4]*/);
+cudaError_t db_sweep(kg_ctx *c, const std::vector<long long> &K, long long *host_stats /*[n_melts][4]*/);
 void db_bin(kg_ctx *c, const std::vector<long long> &K);     // attempt offsets + the >= 1.3 sigma grid
 void db_finish(kg_ctx *c, long long *host_stats);             // box shifts, chain partners, stats to host
-int db_max_chain_len(const kg_ctx *c);
 // reset the commit bookkeeping of a sweep (versions, stamps, rounds)
-void db_rounds_reset(kg_ctx *c, long long tot);
+void db_rounds_reset(kg_ctx *c);
 
 
 // kg_learned.cu
-void db_sweep_learned(kg_ctx *c, const std::vector<long long> &K, double lambda, long long *host_stats);
+cudaError_t db_sweep_learned(kg_ctx *c, const std::vector<long long> &K, double lambda, long long *host_stats);
 bool db_proposal(kg_ctx *c, int melt, int chain, int bond, double lambda, int *h_n, int *h_ints /*[3][48]*/,
                  double *h_f /*[48][24]*/, double *h_s /*[48]*/, double *h_pi /*[48]*/);
 

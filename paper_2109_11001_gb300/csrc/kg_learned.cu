@@ -26,8 +26,8 @@
 // in 16-row tiles, and lane 0 forms pi in FP64 in list order.  The forward
 // probability of the partner bond and the two reverse probabilities repeat
 // this for three more bonds (the reverse ones in the swapped topology view).
-// Attempts are evaluated speculatively in parallel and committed in order by
-// the shared commit walk (kg_db.cuh); a learned evaluation reads monomers up
+// Attempts are drawn speculatively in parallel, then decided and committed in
+// order by the shared commit rounds (kg_db.cuh); a learned evaluation reads monomers up
 // to 2 b_lim + 3 b_max from its junction monomers (b_lim = 1.3 the swap bond
 // limit, b_max the longest bond at sweep start), so an accepted swap with a
 // junction monomer within that many cells forces a re-evaluation.
@@ -55,6 +55,7 @@ struct __align__(16) WarpProp : WarpCand {
     double pi[CAND_CAP];
     double dE[CAND_CAP];
     float s[CAND_CAP];
+    double f[24];                       // features of the candidate in work
     __nv_bfloat16 F[CAND_CAP * S1];     // features of the candidates, bf16 rows
 };
 
@@ -73,10 +74,13 @@ __device__ __forceinline__ void sort4(double *v)
     }
 }
 
-// Features of swap m of bond (c, b) in view v (one lane).
+// Features of swap m of bond (c, b) in view v into f (shared), whole warp: a
+// lane per bond length and per cosine (each a dependent chain of binary64
+// square roots and divides), then lane 0 sorts and sums them.
 template <class V>
 __device__ void move_features(const DBC &C, const V &v, int c, int b, const Cand &m, double *f)
 {
+    const int lane = threadIdx.x & 31;
     const MeltDev &md = C.md;
     const int N = md.N, off = md.off;
     const int u = v.occ(off + c * N + b), w = v.occ(off + c * N + b + 1);
@@ -88,47 +92,65 @@ __device__ void move_features(const DBC &C, const V &v, int c, int b, const Cand
         X = v.occ(off + m.d * N + m.q);
         Y = v.occ(off + m.d * N + m.q + 1);
     }
-    const double o1 = sqrt(d2(C, u, w)), o2 = sqrt(d2(C, X, Y));
-    const double n1 = sqrt(d2(C, u, X)), n2 = sqrt(d2(C, Y, w));
-    f[0] = o1 < o2 ? o1 : o2;
-    f[1] = o1 < o2 ? o2 : o1;
-    f[2] = n1 < n2 ? n1 : n2;
-    f[3] = n1 < n2 ? n2 : n1;
-    f[4] = fene_of_r(C, n1) + fene_of_r(C, n2) - fene_of_r(C, o1) - fene_of_r(C, o2);
     const int A = c < m.d ? c : m.d, B = c < m.d ? m.d : c;
     const int pA = A == c ? b : m.q, pB = A == c ? m.q : b;
-    double before[4] = {vcos(C, v, A, pA), vcos(C, v, A, pA + 1), vcos(C, v, B, pB), vcos(C, v, B, pB + 1)};
-    double outer[4] = {vcos(C, v, A, pA - 1), vcos(C, v, A, pA + 2), vcos(C, v, B, pB - 1),
-                       vcos(C, v, B, pB + 2)};
-    const ViewMove<V> mv{v, m.kind, A, B, pA, pB, N, off};
-    double after[4] = {vcos(C, mv, A, pA), vcos(C, mv, A, pA + 1), vcos(C, mv, B, pB), vcos(C, mv, B, pB + 1)};
-    double db = 0.0;
+    // lanes 0-3: lengths of u-w, X-Y, u-X, Y-w and their FENE terms; 4-7, 8-11,
+    // 12-15: cosines at the four junction vertices before and after, and one
+    // vertex further out; 16: cosine between u->w and X->Y
+    double val = 0.0, fene = 0.0;
+    if (lane < 4) {
+        val = sqrt(d2(C, lane & 1 ? (lane == 1 ? X : Y) : u, lane == 0 || lane == 3 ? w : (lane == 1 ? Y : X)));
+        fene = fene_of_r(C, val);
+    } else if (lane < 16) {
+        const int t = lane & 3, far = lane >= 12 ? ((t & 1) ? 1 : -1) : 0;
+        const ViewEither<V> e{ViewMove<V>{v, m.kind, A, B, pA, pB, N, off}, lane >= 8 && lane < 12};
+        val = vcos(C, e, t < 2 ? A : B, (t < 2 ? pA : pB) + (t & 1) + far);
+    } else if (lane == 16) {
+        double e1[3], e2[3];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) db += md.kappa * ((1.0 - after[i]) - (1.0 - before[i]));
-    f[5] = db;
-    sort4(before);
-    sort4(after);
-    sort4(outer);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        f[6 + i] = before[i];
-        f[10 + i] = after[i];
-        f[14 + i] = outer[i];
+        for (int k = 0; k < 3; ++k) {
+            e1[k] = min_image_exact(C.x[k * C.Mp + w] - C.x[k * C.Mp + u], md.L);
+            e2[k] = min_image_exact(C.x[k * C.Mp + Y] - C.x[k * C.Mp + X], md.L);
+        }
+        val = (e1[0] * e2[0] + e1[1] * e2[1] + e1[2] * e2[2])
+              / (sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]) *
+                 sqrt(e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]));
     }
-    double e1[3], e2[3];
+    auto at = [&](int k) { return __shfl_sync(FULL, val, k); };
+    const double o1 = at(0), o2 = at(1), n1 = at(2), n2 = at(3);
+    double before[4] = {at(4), at(5), at(6), at(7)}, after[4] = {at(8), at(9), at(10), at(11)};
+    double outer[4] = {at(12), at(13), at(14), at(15)};
+    const double cross = at(16);
+    const double fo1 = __shfl_sync(FULL, fene, 0), fo2 = __shfl_sync(FULL, fene, 1);
+    const double fn1 = __shfl_sync(FULL, fene, 2), fn2 = __shfl_sync(FULL, fene, 3);
+    if (lane == 0) {
+        f[0] = o1 < o2 ? o1 : o2;
+        f[1] = o1 < o2 ? o2 : o1;
+        f[2] = n1 < n2 ? n1 : n2;
+        f[3] = n1 < n2 ? n2 : n1;
+        f[4] = fn1 + fn2 - fo1 - fo2;
+        double db = 0.0;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        e1[k] = min_image_exact(C.x[k * C.Mp + w] - C.x[k * C.Mp + u], md.L);
-        e2[k] = min_image_exact(C.x[k * C.Mp + Y] - C.x[k * C.Mp + X], md.L);
+        for (int i = 0; i < 4; ++i) db += md.kappa * ((1.0 - after[i]) - (1.0 - before[i]));
+        f[5] = db;
+        sort4(before);
+        sort4(after);
+        sort4(outer);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            f[6 + i] = before[i];
+            f[10 + i] = after[i];
+            f[14 + i] = outer[i];
+        }
+        f[18] = cross;
+        f[19] = md.kappa / 4.0;
+        f[20] = C.nexp / 12.0;
+        const int lo = b + 1 < N - 1 - b ? b + 1 : N - 1 - b;
+        f[21] = (double)lo / N;
+        f[22] = f[4] + f[5];
+        f[23] = 1.0;
     }
-    f[18] = (e1[0] * e2[0] + e1[1] * e2[1] + e1[2] * e2[2])
-            / (sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]) * sqrt(e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]));
-    f[19] = md.kappa / 4.0;
-    f[20] = C.nexp / 12.0;
-    const int lo = b + 1 < N - 1 - b ? b + 1 : N - 1 - b;
-    f[21] = (double)lo / N;
-    f[22] = f[4] + f[5];
-    f[23] = 1.0;
+    __syncwarp();
 }
 
 // Proposal weights of bond (c, b) in view v: wp.cand[0..n), wp.pi, and (when
@@ -150,28 +172,21 @@ __device__ int proposal(const DBC &C, const V &v, const MlpSmem &W, WarpProp &wp
     const bool net = la.lambda < 1.0 && (n > 1 || logits);
     if (net || features) {
         const int nr = (n + 15) & ~15;
-        for (int j = lane; j < nr; j += 32) {
+        for (int j = 0; j < n; ++j) {                  // most lists have one entry
+            move_features(C, v, c, b, wp.cand[j], wp.f);
             __nv_bfloat16 *row = wp.F + j * S1;
-            if (j < n) {
-                double f[24];
-                move_features(C, v, c, b, wp.cand[j], f);
-                wp.dE[j] = f[22];
-#pragma unroll
-                for (int i = 0; i < 24; ++i) row[i] = __double2bfloat16(f[i]);
+            row[lane] = lane < 24 ? __double2bfloat16(wp.f[lane]) : __float2bfloat16(0.f);
+            if (log_att >= 0 && lane < 24) la.logf[(log_att * CAND_CAP + j) * 24 + lane] = wp.f[lane];
+            if (lane == 0) {
+                wp.dE[j] = wp.f[22];
                 if (log_att >= 0) {
-                    double *o = la.logf + (log_att * CAND_CAP + j) * 24;
-#pragma unroll
-                    for (int i = 0; i < 24; ++i) o[i] = f[i];
-                    const double de = f[22] / C.T;
+                    const double de = wp.f[22] / C.T;
                     la.logt[log_att * CAND_CAP + j] = de > 0.0 ? exp(-de) : 1.0;
                 }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 24; ++i) row[i] = __float2bfloat16(0.f);
             }
-#pragma unroll
-            for (int i = 24; i < 32; ++i) row[i] = __float2bfloat16(0.f);
+            __syncwarp();
         }
+        for (int j = n; j < nr; ++j) wp.F[j * S1 + lane] = __float2bfloat16(0.f);
         if (log_att >= 0 && lane == 0) la.logn[log_att] = n;
         __syncwarp();
     }
@@ -225,59 +240,54 @@ __device__ double match_prob(const DBC &C, const V &v, const MlpSmem &W, WarpPro
     return p;
 }
 
-// One attempt (k of this melt's sweep; g its global index), whole warp.
+// Attempt k of this melt's sweep (g its global index): the drawn bond, its
+// proposal and the partner picked from it (one warp).  flags 0 (empty set, or a
+// capacity error, which is flagged), or 1 | 4: to be decided from the parts.
 template <class V>
-__device__ Attempt learned_eval(const DBC &C, const V &v, const MlpSmem &W, WarpProp &wp, const LearnedArgs &la,
-                                unsigned long long seed, long long sweep, int k, int g, unsigned &err)
+__device__ void learned_draw(const DBC &C, const V &v, const MlpSmem &W, WarpProp &wp, const LearnedArgs &la,
+                             unsigned long long seed, long long sweep, int k, int g, Attempt &a, unsigned &err)
 {
     const int lane = threadIdx.x & 31;
     const MeltDev &md = C.md;
     const int N = md.N, off = md.off;
-    Attempt a;
     a.flags = 0;
     a.d = -1;
-    a.kind = a.A = a.B = a.pA = a.pB = 0;
-    a.jp[2] = a.jp[3] = -1;
+    a.kind = a.A = a.B = a.pA = a.pB = a.q = 0;
+    a.ver = 0;
+    a.cell[2] = a.cell[3] = -1;
+    a.p = a.dE = 0.0;
     const uint4 r = draw(seed, C.melt, 1, (unsigned long long)sweep, (uint32_t)k);
     const uint4 r2 = draw(seed, C.melt, 2, (unsigned long long)sweep, (uint32_t)k);
     const long long nbonds = (long long)md.n_ch * (N - 1);
     const long long bond = mul_hi64(((unsigned long long)r.y << 32) | r.x, (unsigned long long)nbonds);
-    const double uacc = ((double)(r.z >> 5) * 67108864.0 + (double)(r.w >> 6)) * (1.0 / 9007199254740992.0);
     const double upick = (double)((((unsigned long long)r2.y << 32) | r2.x) >> 11) * (1.0 / 9007199254740992.0);
     const int c = (int)(bond / (N - 1)), b = (int)(bond % (N - 1));
     a.c = c;
-    a.jp[0] = v.occ(off + c * N + b);
-    a.jp[1] = v.occ(off + c * N + b + 1);
+    a.cell[0] = C.cell[v.occ(off + c * N + b)];
+    a.cell[1] = C.cell[v.occ(off + c * N + b + 1)];
     if (la.logn && lane == 0) la.logn[g] = 0;
-    const int n1 = proposal(C, v, W, wp, la, c, b, true, la.logf ? (long long)g : -1LL, err);
-    if (n1 <= 0) return a;                         // empty, or a capacity error (bit set)
+    a.n = proposal(C, v, W, wp, la, c, b, true, la.logf ? (long long)g : -1LL, err);
+    if (a.n <= 0) return;
     int j = 0;
     if (lane == 0) {
         double cum = wp.pi[0];
-        while (j + 1 < n1 && upick >= cum) cum += wp.pi[++j];
+        while (j + 1 < a.n && upick >= cum) cum += wp.pi[++j];
     }
     j = __shfl_sync(FULL, j, 0);
     const Cand m = wp.cand[j];
-    const double pij = wp.pi[j], dE = wp.dE[j];
+    a.p = wp.pi[j];
+    a.dE = wp.dE[j];
     __syncwarp();
-    a.flags = 1;
+    a.flags = 1 | 4;
     a.d = m.d;
-    a.jp[2] = v.occ(off + m.d * N + m.q);
-    a.jp[3] = v.occ(off + m.d * N + m.q + 1);
-    const int A = c < m.d ? c : m.d, B = c < m.d ? m.d : c;
-    const int pA = A == c ? b : m.q, pB = A == c ? m.q : b;
-    a.kind = m.kind; a.A = A; a.B = B; a.pA = pA; a.pB = pB;
-    const double q_fwd = pij + match_prob(C, v, W, wp, la, m.d, m.q, m.kind, A, B, pA, pB, err);
-    const ViewMove<V> w{v, m.kind, A, B, pA, pB, N, off};
-    const double q_rev = match_prob(C, w, W, wp, la, A, pA, m.kind, A, B, pA, pB, err)
-                         + match_prob(C, w, W, wp, la, B, pB, m.kind, A, B, pA, pB, err);
-    if (!(q_rev > 0.0) || !(q_fwd > 0.0)) {
-        err |= ERR_DB_INTERNAL;
-        return a;
-    }
-    const double acc = exp(-dE / C.T) * q_rev / q_fwd;
-    if (uacc < acc) a.flags |= 2;
-    return a;
+    a.q = m.q;
+    a.cell[2] = C.cell[v.occ(off + m.d * N + m.q)];
+    a.cell[3] = C.cell[v.occ(off + m.d * N + m.q + 1)];
+    a.kind = m.kind;
+    a.A = c < m.d ? c : m.d;
+    a.B = c < m.d ? m.d : c;
+    a.pA = a.A == c ? b : m.q;
+    a.pB = a.A == c ? m.q : b;
 }
 
 constexpr int EVAL_WARPS = 4;
@@ -311,7 +321,8 @@ __global__ void __launch_bounds__(32 * EVAL_WARPS) k_dbl_eval(const SimDev *__re
     while (g >= koff[m + 1]) ++m;
     const DBC C = make_dbc(S, *stp, m, x, pid, cell, start, list, la.rec, stp->T);
     unsigned err = 0;
-    const Attempt a = learned_eval(C, ViewMap{comp_of, slot_of}, W, wps[warp], la, S.seed, sweep, g - koff[m], g, err);
+    Attempt a;
+    learned_draw(C, ViewMap{comp_of, slot_of}, W, wps[warp], la, S.seed, sweep, g - koff[m], g, a, err);
     if (lane == 0) {
         att[g] = a;
         if (err) atomicOr(flags, err);
@@ -329,24 +340,48 @@ struct LearnedEval {
     long long sweep;
     unsigned *flags;
     LearnedArgs la;
-    const MlpSmem *W;
+    const MlpSmem *W;            // set by the kernel
     WarpProp *wp;
-    __device__ void eval(int m, int k, int g, Attempt &out)
+    static constexpr int TASKS = 3;
+    __device__ DBC dbc(int m) const { return make_dbc(*S, *st, m, x, pid, cell, start, list, la.rec, st->T); }
+    __device__ void say(unsigned err) const
     {
-        const DBC C = make_dbc(*S, *st, m, x, pid, cell, start, list, la.rec, st->T);
+        if (err && (threadIdx.x & 31) == 0) atomicOr(flags, err);
+    }
+    __device__ void scan(int m, int k, int g, Attempt &a)
+    {
         unsigned err = 0;
-        const Attempt a = learned_eval(C, ViewMap{comp_of, slot_of}, *W, *wp, la, S->seed, sweep, k, g, err);
-        if ((threadIdx.x & 31) == 0) {
-            out = a;
-            if (err) atomicOr(flags, err);
+        learned_draw(dbc(m), ViewMap{comp_of, slot_of}, *W, *wp, la, S->seed, sweep, k, g, a, err);
+        say(err);
+    }
+    // probability that the partner bond proposes the swap, and that either new bond proposes the one back
+    __device__ double task(int m, const Attempt &a, int t)
+    {
+        const DBC C = dbc(m);
+        const ViewMap v{comp_of, slot_of};
+        const ViewMove<ViewMap> w{v, a.kind, a.A, a.B, a.pA, a.pB, C.md.N, C.md.off};
+        unsigned err = 0;
+        const double p =
+            t == 0 ? match_prob(C, v, *W, *wp, la, a.d, a.q, a.kind, a.A, a.B, a.pA, a.pB, err)
+                   : match_prob(C, w, *W, *wp, la, t == 1 ? a.A : a.B, t == 1 ? a.pA : a.pB, a.kind, a.A, a.B, a.pA, a.pB,
+                                err);
+        say(err);
+        return p;
+    }
+    __device__ bool accepts(int m, int k, const Attempt &a, const double *p) const
+    {
+        const double q_fwd = a.p + p[0], q_rev = p[1] + p[2];
+        if (!(q_rev > 0.0) || !(q_fwd > 0.0)) {
+            atomicOr(flags, ERR_DB_INTERNAL);
+            return false;
         }
+        return accept_u(S->seed, m, sweep, k) < exp(-a.dE / st->T) * q_rev / q_fwd;
     }
 };
 
 struct LearnedRadius {
     const unsigned long long *bmax2;
     double lim;                                    // swap bond limit (1.3)
-    __device__ void init() {}
     // cells within 2 lim + 3 max(b_max, lim) of a junction monomer, one extra
     // cell against rounding at cell faces
     __device__ int radius(const MeltDev &md) const
@@ -357,39 +392,17 @@ struct LearnedRadius {
     }
 };
 
-__host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
-
-__host__ __device__ constexpr size_t restale_smem() { return sizeof(MlpSmem) + EVAL_WARPS * sizeof(WarpProp); }
-
-__global__ void __launch_bounds__(32 * EVAL_WARPS) k_dbl_restale(
-    const SimDev *__restrict__ Sp, const StageDev *__restrict__ stp, const double *__restrict__ x,
-    const int *__restrict__ pid, const int *__restrict__ cell, const int *__restrict__ start,
-    const int *__restrict__ list, const int *__restrict__ koff, const int *__restrict__ comp_of,
-    const int *__restrict__ slot_of, Attempt *__restrict__ att, int *__restrict__ ver,
-    const int *__restrict__ chain_ver, const int *__restrict__ cell_ver, int *__restrict__ round, long long sweep,
-    unsigned *flags, LearnedArgs la)
+__global__ void __launch_bounds__(32 * EVAL_WARPS) k_dbl_rounds(RoundArgs R, LearnedEval ev)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     MlpSmem &W = *reinterpret_cast<MlpSmem *>(smem);
     WarpProp *wps = reinterpret_cast<WarpProp *>(smem + sizeof(MlpSmem));
-    mlp_load(W, la.w);
+    mlp_load(W, ev.la.w);
     __syncthreads();
-    if (flags[0]) return;                          // a latched error stops the sweep (no block barrier follows)
-    LearnedEval ev{Sp, stp, x, pid, cell, start, list, comp_of, slot_of, sweep, flags, la, &W,
-                   wps + (threadIdx.x >> 5)};
-    restale_body(ev, *Sp, koff, att, ver, chain_ver, cell, cell_ver, round);
-}
-
-__global__ void __launch_bounds__(256) k_dbl_commit_next(
-    const SimDev *__restrict__ Sp, const double *__restrict__ x, const int *__restrict__ cell,
-    const int *__restrict__ koff, const Attempt *__restrict__ att, int *__restrict__ occ, int *__restrict__ curmap,
-    int *__restrict__ img, int *__restrict__ chain_ver, int *__restrict__ cell_ver, int *__restrict__ round,
-    long long *__restrict__ stats, unsigned *flags, const unsigned long long *bmax2)
-{
-    extern __shared__ int old_occ[];              // 2N ints
-    LearnedRadius pol{bmax2, sqrt(Sp->db_lim2)};
-    commit_next_body(pol, *Sp, x, cell, koff, att, occ, curmap, img, chain_ver, cell_ver, round, stats, flags,
-                     old_occ);
+    ev.W = &W;
+    ev.wp = wps + (threadIdx.x >> 5);
+    LearnedRadius pol{ev.la.bmax2, sqrt(R.sim->db_lim2)};
+    rounds_body<32 * EVAL_WARPS>(ev, pol, R);
 }
 
 // longest bond of all melts, squared, as ordered binary64 bits
@@ -408,53 +421,40 @@ __global__ void __launch_bounds__(256) k_bond_max(const SimDev *__restrict__ Sp,
     if ((threadIdx.x & 31) == 0 && r2 > 0.0) atomicMax(bmax2, (unsigned long long)__double_as_longlong(r2));
 }
 
-// Append the sweep's log rows (attempt order, list order within an attempt)
-// to the training ring; one block.
-__global__ void __launch_bounds__(1024) k_log_append(const int *__restrict__ logn, int Ktot,
-                                                    const double *__restrict__ sf, const double *__restrict__ st,
-                                                    double *__restrict__ rf, double *__restrict__ rt, long long cap,
-                                                    long long *head, const unsigned *flags)
+// Append the sweep's log rows (attempt order, list order within an attempt) to
+// the training ring: rows of attempt k go to head + off[k] (off the scan of
+// the row counts), a warp copies the rows of its 32 attempts one attempt after
+// the other (almost all have none).  One block walking the attempts with a
+// scan of its own per 1,024 took 236 us for 80,000 attempts.
+__global__ void __launch_bounds__(256) k_log_append(const int *__restrict__ logn, const int *__restrict__ off, int Ktot,
+                                                   const double *__restrict__ sf, const double *__restrict__ st,
+                                                   double *__restrict__ rf, double *__restrict__ rt, long long cap,
+                                                   const long long *__restrict__ head, const unsigned *flags)
 {
-    __shared__ int scan[1024];
-    __shared__ long long base, total;
     if (flags[0]) return;
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        base = *head;
-        total = 0;
-    }
-    __syncthreads();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int n = k < Ktot ? logn[k] : 0, o = k < Ktot ? off[k] : 0;
     // rows that an append of more than `cap` rows overwrites within itself are
     // skipped, so no two writes of one pass land on the same ring slot
-    long long mine = 0;
-    for (int k = tid; k < Ktot; k += 1024) mine += logn[k];
-    atomicAdd(reinterpret_cast<unsigned long long *>(&total), (unsigned long long)mine);
-    __syncthreads();
-    const long long keep_from = base + total - cap;
-    for (int k0 = 0; k0 < Ktot; k0 += 1024) {
-        const int k = k0 + tid;
-        const int n = k < Ktot ? logn[k] : 0;
-        scan[tid] = n;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            const int add = tid >= o ? scan[tid - o] : 0;
-            __syncthreads();
-            scan[tid] += add;
-            __syncthreads();
+    const long long base = *head, keep_from = base + off[Ktot] - cap;
+    unsigned bal = __ballot_sync(FULL, n > 0);
+    while (bal) {
+        const int src = __ffs(bal) - 1;
+        bal &= bal - 1;
+        const int nn = __shfl_sync(FULL, n, src), kk = __shfl_sync(FULL, k, src);
+        const long long d0 = base + __shfl_sync(FULL, o, src);
+        for (int j = 0; j < nn; ++j) {
+            if (d0 + j < keep_from) continue;
+            const long long dst = (d0 + j) % cap;
+            if (lane < 24) rf[dst * 24 + lane] = sf[((long long)kk * CAND_CAP + j) * 24 + lane];
+            if (lane == 24) rt[dst] = st[(long long)kk * CAND_CAP + j];
         }
-        const long long dst0 = base + scan[tid] - n;
-        for (int j = 0; j < n; ++j) {
-            if (dst0 + j < keep_from) continue;
-            const long long dst = (dst0 + j) % cap;
-            const double *src = sf + ((long long)k * CAND_CAP + j) * 24;
-            for (int i = 0; i < 24; ++i) rf[dst * 24 + i] = src[i];
-            rt[dst] = st[(long long)k * CAND_CAP + j];
-        }
-        __syncthreads();
-        if (tid == 0) base += scan[1023];
-        __syncthreads();
     }
-    if (tid == 0) *head = base;
+}
+
+__global__ void k_log_head(const int *__restrict__ off, int Ktot, long long *head, const unsigned *flags)
+{
+    if (!flags[0]) *head += off[Ktot];
 }
 
 // One bond's learned proposal in the current topology (introspection).
@@ -498,11 +498,14 @@ static bool ensure_log_staging(kg_ctx *c, long long tot)
     dev_free(c, c->logf);
     dev_free(c, c->logt);
     dev_free(c, c->logn);
+    dev_free(c, c->logoff);
     const long long cap = tot > 2 * c->log_att_cap ? tot : 2 * c->log_att_cap;
     c->logf = (double *)dev_alloc(c, sizeof(double) * 24 * CAND_CAP * (size_t)cap);
     c->logt = (double *)dev_alloc(c, sizeof(double) * CAND_CAP * (size_t)cap);
     c->logn = (int *)dev_alloc(c, sizeof(int) * (size_t)cap);
-    c->log_att_cap = (c->logf && c->logt && c->logn) ? cap : 0;
+    // offsets of the attempts' rows, and the block sums of their scan
+    c->logoff = (int *)dev_alloc(c, sizeof(int) * ((size_t)cap + 1 + (size_t)cap / 1024 + 2));
+    c->log_att_cap = (c->logf && c->logt && c->logn && c->logoff) ? cap : 0;
     return c->log_att_cap > 0;
 }
 
@@ -519,7 +522,7 @@ static LearnedArgs make_args(kg_ctx *c, double lambda, bool log)
     return la;
 }
 
-void db_sweep_learned(kg_ctx *c, const std::vector<long long> &K, double lambda, long long *host_stats)
+cudaError_t db_sweep_learned(kg_ctx *c, const std::vector<long long> &K, double lambda, long long *host_stats)
 {
     cudaStream_t st = c->stream;
     const int nm = c->sim.n_melts;
@@ -538,30 +541,23 @@ void db_sweep_learned(kg_ctx *c, const std::vector<long long> &K, double lambda,
             att, c->sweep, c->flags, la);
     }
     // ordered commit in rounds (kg_db.cuh)
-    db_rounds_reset(c, tot);
-    const int maxN = db_max_chain_len(c);
-    const size_t sm = sizeof(int) * 2 * (size_t)maxN;
-    cudaFuncSetAttribute(k_dbl_commit_next, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_dbl_restale, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)restale_smem());
-    const int rgrid = std::max(1, std::min(nblk(tot, 32 * EVAL_WARPS), 152 * 4));
-    db_rounds(c, tot,
-              [&] {
-                  k_dbl_restale<<<rgrid, 32 * EVAL_WARPS, restale_smem(), st>>>(
-                      c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist, c->koff, c->comp_of,
-                      c->slot_of, att, c->att_ver, c->chain_ver, c->dbmark, c->dbround, c->sweep, c->flags, la);
-              },
-              [&] {
-                  k_dbl_commit_next<<<nm, 256, sm, st>>>(c->d_sim, c->x, c->dbcell, c->koff, att, c->comp_of,
-                                                         c->slot_of, c->img, c->chain_ver, c->dbmark, c->dbround,
-                                                         c->db_stats, c->flags, c->bmax2);
-              });
+    db_rounds_reset(c);
+    cudaFuncSetAttribute(k_dbl_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eval_smem());
+    const LearnedEval ev{c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist,
+                         c->comp_of, c->slot_of, c->sweep, c->flags, la, nullptr, nullptr};
+    const cudaError_t e = rounds_launch(c, k_dbl_rounds, 32 * EVAL_WARPS, eval_smem(), tot, nm, round_args(c), ev);
+    if (e != cudaSuccess) return e;
     c->launches += 2;
     if (log && tot > 0) {
-        k_log_append<<<1, 1024, 0, st>>>(c->logn, (int)tot, c->logf, c->logt, c->trainf, c->traint, c->train_cap,
-                                         c->d_train_head, c->flags);
+        scan_counts(c, c->logn, c->logoff, (int)tot, c->logoff + tot + 1);
+        k_log_append<<<nblk(tot, 256), 256, 0, st>>>(c->logn, c->logoff, (int)tot, c->logf, c->logt, c->trainf,
+                                                     c->traint, c->train_cap, c->d_train_head, c->flags);
+        k_log_head<<<1, 1, 0, st>>>(c->logoff, (int)tot, c->d_train_head, c->flags);
+        c->launches += 3;
         ++c->launches;
     }
     db_finish(c, host_stats);
+    return cudaSuccess;
 }
 
 bool db_proposal(kg_ctx *c, int melt, int chain, int bond, double lambda, int *h_n, int *h_ints, double *h_f,

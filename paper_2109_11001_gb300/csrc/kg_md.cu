@@ -732,11 +732,11 @@ __global__ void k_begin_step(long long *__restrict__ stepp, unsigned *__restrict
 
 __global__ void k_set_step(long long *__restrict__ stepp, long long v) { stepp[0] = v; }
 
-void scan_counts(kg_ctx *c, const int *count, int *start, int n)
+void scan_counts(kg_ctx *c, const int *count, int *start, int n, int *bsum)
 {
     const int nb = nblk(n, 1024);
-    k_scan1<<<nb, 1024, 0, c->stream>>>(count, start, c->bsum, n, nullptr);
-    k_scan2<<<nb, 1024, 0, c->stream>>>(start, c->bsum, n, nb, nullptr);
+    k_scan1<<<nb, 1024, 0, c->stream>>>(count, start, bsum, n, nullptr);
+    k_scan2<<<nb, 1024, 0, c->stream>>>(start, bsum, n, nb, nullptr);
 }
 
 static void launch_rebuild(kg_ctx *c, cudaStream_t st);

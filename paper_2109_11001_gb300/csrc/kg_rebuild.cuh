@@ -184,12 +184,12 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
     constexpr unsigned FULL = 0xffffffffu;
     const bool live = s < A.M;
     const int sv = live ? s : A.M - 1;                       // idle lanes read valid memory, write nothing
-    const int slot = A.slot_of[sv];
+    const int slot = __ldg(A.slot_of + sv);
     int m = 0;
     while (m + 1 < A.n_melts && slot >= A.melt[m + 1].off) ++m;
     const MeltNl &md = A.melt[m];
-    const int4 bp = A.bp[sv];                        // 1-2 bonded partners: bp.y, bp.z
-    const float4 ri = A.recb[sv];
+    const int4 bp = __ldg(A.bp + sv);                        // 1-2 bonded partners: bp.y, bp.z
+    const float4 ri = __ldg(A.recb + sv);
     const unsigned code = __float_as_uint(ri.w);
     const int cx = (int)(code & CODE_MASK), cy = (int)((code >> CODE_BITS) & CODE_MASK);
     const int cz = (int)(code >> (2 * CODE_BITS));
@@ -214,8 +214,8 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
                 int xx = cx + dx;
                 xx = xx < 0 ? nc - 1 : (xx >= nc ? 0 : xx);
                 const int cell = rowb + ((xx >> 2) << 6) + (xx & 3);
-                const int k0 = A.start[cell];
-                int n = live ? A.start[cell + 1] - k0 : 0;
+                const int k0 = __ldg(A.start + cell);
+                int n = live ? __ldg(A.start + cell + 1) - k0 : 0;
                 if (n > MAX_CELL_OCC) {
                     err = ERR_NL_CAPACITY;
                     n = 0;
@@ -225,7 +225,7 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
                 const unsigned tag = (unsigned)((dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)) << IDX_BITS;
 #pragma unroll 2
                 for (int j = 0; j < nmax; ++j) {
-                    const float4 rj = A.recs[k0 + j];
+                    const float4 rj = __ldg(A.recs + k0 + j);
                     const int t = __float_as_int(rj.w);
                     const float ex = rj.x - ox, ey = rj.y - oy, ez = rj.z - oz;
                     const float r2 = ex * ex + ey * ey + ez * ez;
@@ -242,7 +242,7 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
         for (int k = 0; k < cnt; ++k) {
             const unsigned e = out[(size_t)k * Mp];
             const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
-            const float r2 = nl_r2(ri, A.recb[t], q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
+            const float r2 = nl_r2(ri, __ldg(A.recb + t), q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
             const bool keep = r2 < lo || dist2_exact(A.x, A.Mp, md.L, s, t) < A.rl2;
             if (keep) out[(size_t)(w++) * Mp] = e;
         }

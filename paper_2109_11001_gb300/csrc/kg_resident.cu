@@ -321,7 +321,7 @@ void resident_cell_order(kg_ctx *c)
     if (!c->bcount) return;
     const int nb = (c->ncell_md + 255) / 256;
     k_bucket_counts<<<nb, 256, 0, c->stream>>>(c->flags, c->bcount, c->ncell_md, c->ccount);
-    scan_counts(c, c->ccount, c->cstart, c->ncell_md);
+    scan_counts(c, c->ccount, c->cstart, c->ncell_md, c->bsum);
     k_bucket_list<<<nb, 256, 0, c->stream>>>(c->flags, c->brec, c->ncell_md, c->ccount, c->cstart, c->clist);
     c->launches += 4;
 }

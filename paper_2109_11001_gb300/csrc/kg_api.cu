@@ -504,25 +504,41 @@ kg_status kg_load_config(kg_ctx *c, int melt, const double *x, const double *v, 
     return KG_OK;
 }
 
+// whether a kernel of the context can write n elements of `size` bytes at p: device memory of its GPU, aligned
+static bool writable(const kg_ctx *c, const void *p, size_t size)
+{
+    cudaPointerAttributes a;
+    if ((size_t)p % size != 0 || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
+
 kg_status kg_get_config(kg_ctx *c, int melt, double *x, double *v, int *pid)
 {
     kg_status s = check_melt(c, melt);
     if (s != KG_OK) return s;
     const MeltDev &md = c->sim.melt[melt];
     const size_t Mm = md.M;
-    if (x) {
-        kg::to_slots(c, melt, c->x, c->scratch, 3);
-        KG_TRY(cudaMemcpyAsync(x, c->scratch, 3 * Mm * sizeof(double), cudaMemcpyDefault, c->stream));
-    }
-    if (v) {
-        kg::u_to_slots(c, melt, c->scratch + 3 * Mm);
-        KG_TRY(cudaMemcpyAsync(v, c->scratch + 3 * Mm, 3 * Mm * sizeof(double), cudaMemcpyDefault, c->stream));
-    }
-    if (pid) {
-        int *tmp = (int *)(c->scratch + 6 * Mm);
-        kg::pid_to_slots(c, melt, tmp);
-        KG_TRY(cudaMemcpyAsync(pid, tmp, Mm * sizeof(int), cudaMemcpyDefault, c->stream));
-    }
+    // one kernel for everything asked for, into the caller's memory where it
+    // is this GPU's, else into scratch and copied from there
+    const char *lo[3] = {(const char *)x, (const char *)v, (const char *)pid};
+    const size_t bytes[3] = {3 * Mm * sizeof(double), 3 * Mm * sizeof(double), Mm * sizeof(int)};
+    bool direct = true;                                    // no two outputs share memory
+    for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b)
+            if (a != b && lo[a] && lo[b] && lo[a] < lo[b] + bytes[b] && lo[b] < lo[a] + bytes[a]) direct = false;
+    double *xd = c->scratch, *vd = c->scratch + 3 * Mm;
+    int *pd = (int *)(c->scratch + 6 * Mm);
+    const bool dx = x && direct && writable(c, x, sizeof(double)), dv = v && direct && writable(c, v, sizeof(double));
+    const bool dp = pid && direct && writable(c, pid, sizeof(int));
+    if (x || v || pid)
+        kg::state_to_slots(c, melt, x ? (dx ? x : xd) : nullptr, v ? (dv ? v : vd) : nullptr,
+                           pid ? (dp ? pid : pd) : nullptr);
+    if (x && !dx) KG_TRY(cudaMemcpyAsync(x, xd, bytes[0], cudaMemcpyDefault, c->stream));
+    if (v && !dv) KG_TRY(cudaMemcpyAsync(v, vd, bytes[1], cudaMemcpyDefault, c->stream));
+    if (pid && !dp) KG_TRY(cudaMemcpyAsync(pid, pd, bytes[2], cudaMemcpyDefault, c->stream));
     KG_TRY(cudaStreamSynchronize(c->stream));
     return KG_OK;
 }

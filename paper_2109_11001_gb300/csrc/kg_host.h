@@ -195,8 +195,7 @@ void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur);   // the mixed path
 // block skip the barriers (self-test of the bounded waits)
 cudaError_t persist_launch(kg_ctx *c, cudaStream_t st, int cur, int K, int skip_block, unsigned spin);
 void to_slots(kg_ctx *c, int melt, const double *in_comp, double *out_dev, int dims);
-void u_to_slots(kg_ctx *c, int melt, double *out_dev);
-void pid_to_slots(kg_ctx *c, int melt, int *out_dev);
+void state_to_slots(kg_ctx *c, int melt, double *x_dev, double *u_dev, int *pid_dev);   // null: not wanted
 int forces_blocks(const kg_ctx *c, int melt);
 
 // kg_db.cu

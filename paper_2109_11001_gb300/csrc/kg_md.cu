@@ -606,21 +606,24 @@ __global__ void __launch_bounds__(256) k_to_slots(const double *__restrict__ in,
     for (int d = 0; d < dims; ++d) out[(size_t)d * out_stride + r] = in[(size_t)d * in_stride + j];
 }
 
-__global__ void __launch_bounds__(256) k_to_slots_f(const float *__restrict__ in, int in_stride,
-                                                   const int *__restrict__ comp_of, int off, int n,
-                                                   double *__restrict__ out, int out_stride)
+// State of a melt in slot order, in one pass: positions, velocities (binary32
+// state widened) and ids, each where asked for (null: not).
+template <typename U>
+__global__ void __launch_bounds__(256) k_state_to_slots(const double *__restrict__ x, const U *__restrict__ u,
+                                                       const int *__restrict__ pid, int Mp,
+                                                       const int *__restrict__ comp_of, int off, int n,
+                                                       double *__restrict__ xo, double *__restrict__ uo,
+                                                       int *__restrict__ po)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int j = comp_of[off + r];
-    for (int d = 0; d < 3; ++d) out[(size_t)d * out_stride + r] = (double)in[(size_t)d * in_stride + j];
-}
-
-__global__ void __launch_bounds__(256) k_to_slots_i(const int *__restrict__ in, const int *__restrict__ comp_of,
-                                                   int off, int n, int *__restrict__ out)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < n) out[r] = in[comp_of[off + r]];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (xo) xo[(size_t)d * n + r] = x[(size_t)d * Mp + j];
+        if (uo) uo[(size_t)d * n + r] = (double)u[(size_t)d * Mp + j];
+    }
+    if (po) po[r] = pid[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -697,23 +700,17 @@ void to_slots(kg_ctx *c, int melt, const double *in_comp, double *out_dev, int d
                                                        dims);
 }
 
-void u_to_slots(kg_ctx *c, int melt, double *out_dev)
+void state_to_slots(kg_ctx *c, int melt, double *x_dev, double *u_dev, int *pid_dev)
 {
     const MeltDev &md = c->sim.melt[melt];
     ++c->launches;
+    const int nb = nblk(md.M, 256);
     if (c->precision == KG_MIXED)
-        k_to_slots_f<<<nblk(md.M, 256), 256, 0, c->stream>>>((const float *)c->u, c->Mp, c->comp_of, md.off, md.M,
-                                                             out_dev, md.M);
+        k_state_to_slots<float><<<nb, 256, 0, c->stream>>>(c->x, (const float *)c->u, c->pid, c->Mp, c->comp_of, md.off,
+                                                           md.M, x_dev, u_dev, pid_dev);
     else
-        k_to_slots<<<nblk(md.M, 256), 256, 0, c->stream>>>((const double *)c->u, c->Mp, c->comp_of, md.off, md.M,
-                                                           out_dev, md.M, 3);
-}
-
-void pid_to_slots(kg_ctx *c, int melt, int *out_dev)
-{
-    const MeltDev &md = c->sim.melt[melt];
-    ++c->launches;
-    k_to_slots_i<<<nblk(md.M, 256), 256, 0, c->stream>>>(c->pid, c->comp_of, md.off, md.M, out_dev);
+        k_state_to_slots<double><<<nb, 256, 0, c->stream>>>(c->x, (const double *)c->u, c->pid, c->Mp, c->comp_of,
+                                                            md.off, md.M, x_dev, u_dev, pid_dev);
 }
 
 // First kernel of every MD step: advance the device step counter (the index

@@ -337,11 +337,9 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     // lockstep candidates past a cell's end without clamping the index
     c->recs = (float4 *)A((Mp + kg::MAX_CELL_OCC + 4) * sizeof(float4));   // + a group of the candidate loop
     c->shtab = (float4 *)A((size_t)kg::SHIFT_SLOTS * kg::MAX_MELTS * sizeof(float4));
+    for (int b = 0; b < 2; ++b) c->pg[b] = (float4 *)A(Mp * sizeof(float4));
     if (c->precision == KG_MIXED) {
-        for (int b = 0; b < 2; ++b) {
-            c->dlt[b] = (float4 *)A(Mp * sizeof(float4));
-            c->pg[b] = (float4 *)A(Mp * sizeof(float4));
-        }
+        for (int b = 0; b < 2; ++b) c->dlt[b] = (float4 *)A(Mp * sizeof(float4));
     } else {
         c->pos64[0] = (double4_32a *)A(Mp * sizeof(double4_32a));
         c->pos64[1] = (double4_32a *)A(Mp * sizeof(double4_32a));

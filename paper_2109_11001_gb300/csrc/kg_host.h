@@ -67,7 +67,7 @@ struct kg_ctx {
     float4 *recb = nullptr;      // build records: offset from the Verlet-cell corner, cell coordinates
     float4 *recs = nullptr;      // the same in cell order (Verlet-list build)
     float4 *dlt[2] = {nullptr, nullptr};   // (mixed) displacement since the build
-    float4 *pg[2] = {nullptr, nullptr};    // (mixed) gather records recb + dlt
+    float4 *pg[2] = {nullptr, nullptr};    // gather records recb + displacement (binary64: for the near-pair test)
     float4 *shtab = nullptr;     // image shift of each stencil code, SHIFT_SLOTS per melt
     double4_32a *pos64[2] = {nullptr, nullptr};
     double4_32a *xb = nullptr;

@@ -57,10 +57,8 @@ __device__ __forceinline__ unsigned bin_md_one(const SimDev &S, int s, double *_
     for (int d = 0; d < 3; ++d) cell[d] = cell_of(xs[d], md.h, md.invh, md.nc, off[d]);
     const float4 rb = make_float4(off[0], off[1], off[2], __uint_as_float(pack_code(cell[0], cell[1], cell[2])));
     recb[s] = rb;
-    if (dcur) {
-        dcur[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-        pgcur[s] = make_float4(rb.x + 0.f, rb.y + 0.f, rb.z + 0.f, rb.w);
-    }
+    if (dcur) dcur[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+    pgcur[s] = make_float4(rb.x + 0.f, rb.y + 0.f, rb.z + 0.f, rb.w);
     if (pcur) {
         const double4_32a p = make_double4_32a(xs[0], xs[1], xs[2], 0.0);
         pcur[s] = p;

@@ -69,17 +69,15 @@ enum {
     KG_FLAG_PAPER_METROPOLIS = 1, /* accept DB swaps with exp(-dE/T) alone (Fig. 1),
                                       without the proposal ratio                      */
     KG_FLAG_PERSISTENT = 2        /* KG_MIXED (ignored with KG_FP64): kg_step advances
-                                      every melt in persistent cooperative launches of
-                                      50 steps, each held in a captured CUDA graph; the
-                                      Verlet rebuild runs inside the launch between grid
-                                      barriers, and every barrier wait is bounded (a
-                                      block that gives up latches KG_ERR_TIMEOUT).  One
-                                      thread per monomer; results equal the default
-                                      path's up to binary32 summation order.  A context
-                                      with one thread per monomer and at most 640
-                                      monomers per SM takes resident launches of up to
-                                      50 steps by itself; there the flag raises that to
-                                      1000                                              */
+                                      every melt in cooperative launches of up to 1000
+                                      steps; the Verlet rebuild runs inside the launch
+                                      between grid barriers, and every barrier wait is
+                                      bounded (a block that gives up latches
+                                      KG_ERR_TIMEOUT).  One thread per monomer; results
+                                      equal the default path's up to binary32 summation
+                                      order.  Contexts with threads_per_monomer 1 and at
+                                      most 1280 monomers per SM take such launches, of
+                                      up to 50 steps, without the flag               */
 };
 
 /* One melt (Sec. II.B): N_ch chains of N monomers in a cube of side L. */

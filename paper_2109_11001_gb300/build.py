@@ -14,13 +14,14 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libkg.so")
-SOURCES = ["kg_api.cu", "kg_md.cu", "kg_step.cu", "kg_resident.cu", "kg_resident_small.cu", "kg_db.cu", "kg_obs.cu", "kg_learned.cu", "kg_mlp.cu", "kg_ppa.cu"]
+SOURCES = ["kg_api.cu", "kg_md.cu", "kg_step.cu", "kg_resident.cu", "kg_resident_small.cu", "kg_resident_tiled.cu", "kg_db.cu", "kg_obs.cu", "kg_learned.cu", "kg_mlp.cu", "kg_ppa.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # the mixed path's step kernels: binary32 denormals flushed to zero and the
 # approximate divide and square root (its arithmetic never meets a denormal;
 # the rounding changes stay far inside the parity bars)
 STEP_FLAGS = ["-ftz=true", "-prec-div=false", "-prec-sqrt=false"]
-PER_FILE = {"kg_step.cu": STEP_FLAGS, "kg_resident.cu": STEP_FLAGS, "kg_resident_small.cu": STEP_FLAGS}
+PER_FILE = {"kg_step.cu": STEP_FLAGS, "kg_resident.cu": STEP_FLAGS, "kg_resident_small.cu": STEP_FLAGS,
+            "kg_resident_tiled.cu": STEP_FLAGS}
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 

@@ -374,7 +374,6 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->db_stats = (long long *)A(4 * kg::MAX_MELTS * sizeof(long long));
     c->scratch = (double *)A(7 * Mp * sizeof(double));
     c->flags = (unsigned *)A(16 * sizeof(unsigned));
-    c->pbar = (unsigned *)A(4 * sizeof(unsigned));
     c->d_step = (long long *)A(sizeof(long long));
     c->fout = (double *)A(3 * Mp * sizeof(double));
     c->partials_cap = (int)(Mp / 128 + 2) * 5;
@@ -428,7 +427,6 @@ void kg_destroy(kg_ctx *c)
                     c->d_io, c->msd_ref};
     for (void *b : bufs) dev_free(c, b);
     dev_free(c, c->d_step);
-    dev_free(c, c->pbar);
     dev_free(c, c->dbbar);
     dev_free(c, c->resbar);
     dev_free(c, c->bcount);
@@ -610,10 +608,7 @@ kg_status kg_step(kg_ctx *c, long long n_steps)
                     c->resident_failed = true;  // the launches below serve it
                     continue;
                 }
-            } else if (!c->prof_on && (c->p.flags & KG_FLAG_PERSISTENT) && c->precision == KG_MIXED &&
-                chunk - done >= kg::PERSIST_STEPS && kg::md_persist_steps(c))
-                n = kg::PERSIST_STEPS;
-            else if (!c->prof_on && c->use_graphs && chunk - done >= kg::GRAPH_STEPS && kg::md_graph_steps(c, 1))
+            } else if (!c->prof_on && c->use_graphs && chunk - done >= kg::GRAPH_STEPS && kg::md_graph_steps(c, 1))
                 n = kg::GRAPH_STEPS;
             else
                 kg::md_step(c);
@@ -641,8 +636,7 @@ kg_status kg_persistent_selftest(kg_ctx *c, int skip_block, unsigned spin)
         kg::set_device_step(c, c->step - 1);
         c->d_step_stale = false;
     }
-    if (kg::resident_kind(c) != kg::RES_NONE) KG_TRY(kg::resident_launch(c, 2, skip_block, spin));
-    else KG_TRY(kg::persist_launch(c, c->stream, c->cur, 2, skip_block, spin));
+    KG_TRY(kg::resident_launch(c, 2, skip_block, spin));
     c->step += 2;
     kg::md_materialize(c);
     return read_flags(c, pinned_flags());

@@ -50,9 +50,6 @@ struct kg_ctx {
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     bool graph_failed = false;
-    cudaGraphExec_t pexec[2] = {nullptr, nullptr};   // persistent launches (KG_FLAG_PERSISTENT)
-    bool persist_failed = false;
-    unsigned *pbar = nullptr;    // grid-barrier words of the persistent launch
     unsigned long long *resbar = nullptr;   // barrier words, error word and segment totals of the resident launch
     int *bcount = nullptr, *bidx = nullptr; // its cell buckets: two sets of counts, members in arrival order
     float4 *brec = nullptr;                 // and records in order
@@ -146,11 +143,10 @@ void *dev_alloc(kg_ctx *c, size_t bytes);
 void dev_free(kg_ctx *c, void *p);
 
 constexpr int GRAPH_STEPS = 10;          // MD steps per captured graph (even)
-constexpr int PERSIST_STEPS = 50;        // MD steps per persistent launch (even)
+constexpr int PERSIST_STEPS = 50;        // MD steps between re-sort tests with KG_FLAG_PERSISTENT
 constexpr int RESIDENT_STEPS = 50;       // MD steps per resident launch (KG_FLAG_PERSISTENT: PERSIST_MAX)
 constexpr int PERSIST_MAX = 1000;
 constexpr unsigned RESIDENT_SPIN = 1u << 22;  // its barrier polls (a few hundred ns apart) before ERR_TIMEOUT
-constexpr unsigned PERSIST_SPIN = 1u << 24;   // grid-barrier polls (~64 ns apart) before ERR_TIMEOUT
 constexpr int RS = 8;                    // ints per melt in the DB commit-round array
 
 // A sweep's record of one attempt.  The staleness check of every round reads
@@ -179,10 +175,9 @@ void scan_counts(kg_ctx *c, const int *count, int *start, int n, int *bsum);   /
 void md_sort(kg_ctx *c);                     // re-sort the state into the last cell order
 void md_materialize(kg_ctx *c);              // mixed: x <- xb64 + dlt[cur]
 void graphs_reset(kg_ctx *c);                // drop captured step graphs (their arguments changed)
-bool md_persist_steps(kg_ctx *c);            // PERSIST_STEPS steps in one persistent launch (KG_MIXED)
 
 // kg_resident.cu
-enum { RES_NONE = 0, RES_WIDE = 1, RES_SMALL = 2 };
+enum { RES_NONE = 0, RES_WIDE = 1, RES_SMALL = 2, RES_TILED = 3 };
 int resident_kind(kg_ctx *c);                // which resident kernel serves the context
 cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin);   // K steps in one launch
 bool resident_alloc(kg_ctx *c);              // its buffers (none for contexts it does not serve)
@@ -191,9 +186,6 @@ void resident_cell_order(kg_ctx *c);         // clist after builds that used buc
 
 // kg_step.cu
 void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur);   // the mixed path's fused step kernel
-// K steps of every melt in one cooperative launch; skip_block >= 0 makes that
-// block skip the barriers (self-test of the bounded waits)
-cudaError_t persist_launch(kg_ctx *c, cudaStream_t st, int cur, int K, int skip_block, unsigned spin);
 void to_slots(kg_ctx *c, int melt, const double *in_comp, double *out_dev, int dims);
 void state_to_slots(kg_ctx *c, int melt, double *x_dev, double *u_dev, int *pid_dev);   // null: not wanted
 int forces_blocks(const kg_ctx *c, int melt);

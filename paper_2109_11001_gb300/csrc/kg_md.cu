@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(NL_BLOCK, 5) k_nlist(const __grid_constant__ N
     __syncthreads();
     if (!go) return;                                         // block-uniform
     const int s = blockIdx.x * NL_BLOCK + threadIdx.x;
-    const unsigned err = nlist_one(A, s);
+    const unsigned err = nlist_one<true>(A, s);
     if (err) atomicOr(A.flags, err);
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -938,45 +938,7 @@ void graphs_reset(kg_ctx *c)
             cudaGraphExecDestroy(c->gexec[k]);
             c->gexec[k] = nullptr;
         }
-        if (c->pexec[k]) {
-            cudaGraphExecDestroy(c->pexec[k]);
-            c->pexec[k] = nullptr;
-        }
     }
-}
-
-// PERSIST_STEPS MD steps as one captured graph holding the persistent
-// cooperative launch (the barrier words reset first); one graph per starting
-// buffer parity.  False if capture or launch is not possible.
-bool md_persist_steps(kg_ctx *c)
-{
-    const int parity = c->cur;
-    if (!c->pexec[parity]) {
-        if (c->persist_failed) return false;
-        if (!c->cap_stream) {
-            if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
-                cudaStreamCreateWithFlags(&c->cap_stream2, cudaStreamNonBlocking) != cudaSuccess) {
-                c->persist_failed = true;
-                return false;
-            }
-        }
-        cudaGraph_t g = nullptr;
-        bool ok = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) ok = persist_launch(c, c->cap_stream, parity, PERSIST_STEPS, -1, PERSIST_SPIN) == cudaSuccess;
-        const bool ended = cudaStreamEndCapture(c->cap_stream, &g) == cudaSuccess;
-        ok = ok && ended && cudaGraphInstantiate(&c->pexec[parity], g, 0) == cudaSuccess;
-        if (g) cudaGraphDestroy(g);
-        if (!ok) {
-            cudaGetLastError();
-            c->pexec[parity] = nullptr;
-            c->persist_failed = true;
-            return false;
-        }
-    }
-    if (cudaGraphLaunch(c->pexec[parity], c->stream) != cudaSuccess) return false;
-    c->launches += 2;                          // barrier reset + the persistent kernel
-    c->cur ^= PERSIST_STEPS & 1;
-    return true;
 }
 
 void set_device_step(kg_ctx *c, long long v)

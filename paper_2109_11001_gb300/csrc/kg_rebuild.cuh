@@ -1,6 +1,6 @@
 // kg_rebuild.cuh -- per-item work of the Verlet-list rebuild chain (binning,
 // scatter into cell order, in-cell rank, list build), shared by the
-// standalone rebuild kernels and the persistent step kernel, so both run the
+// standalone rebuild kernels and the resident kernels, so both run the
 // same arithmetic.
 #pragma once
 #include <cuda_runtime.h>
@@ -166,6 +166,16 @@ __device__ __forceinline__ void st_pred(unsigned *addr, unsigned v, bool p)
                  ::"l"(addr), "r"(v), "r"((unsigned)p) : "memory");
 }
 
+// the same, for memory that the code around it does not read before nl_fence():
+// loads may move across it
+__device__ __forceinline__ void st_pred_free(unsigned *addr, unsigned v, bool p)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.u32 [%0], %1;\n\t}"
+                 ::"l"(addr), "r"(v), "r"((unsigned)p));
+}
+
+__device__ __forceinline__ void nl_fence() { asm volatile("" ::: "memory"); }
+
 // binary32 squared distance of the build records of s (ri) and t (rj) for a
 // pair in stencil cell (dx, dy, dz) of s: the same expression as the build's
 __device__ __forceinline__ float nl_r2(float4 ri, float4 rj, int dx, int dy, int dz, float h)
@@ -176,18 +186,27 @@ __device__ __forceinline__ float nl_r2(float4 ri, float4 rj, int dx, int dy, int
 }
 
 // The list of monomer s (s >= M: an idle lane that takes part in the warp's
-// lockstep and writes nothing); returns error bits.
+// lockstep and writes nothing); returns error bits.  READ_ONLY: what it loads is not written
+// in the same launch (non-coherent loads).
+template <bool READ_ONLY, typename T>
+__device__ __forceinline__ T nl_ld(const T *p)
+{
+    if constexpr (READ_ONLY) return __ldg(p);
+    else return *p;
+}
+
+template <bool READ_ONLY>
 __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const bool live = s < A.M;
     const int sv = live ? s : A.M - 1;                       // idle lanes read valid memory, write nothing
-    const int slot = __ldg(A.slot_of + sv);
+    const int slot = nl_ld<READ_ONLY>(A.slot_of + sv);
     int m = 0;
     while (m + 1 < A.n_melts && slot >= A.melt[m + 1].off) ++m;
     const MeltNl &md = A.melt[m];
-    const int4 bp = __ldg(A.bp + sv);                        // 1-2 bonded partners: bp.y, bp.z
-    const float4 ri = __ldg(A.recb + sv);
+    const int4 bp = nl_ld<READ_ONLY>(A.bp + sv);                        // 1-2 bonded partners: bp.y, bp.z
+    const float4 ri = nl_ld<READ_ONLY>(A.recb + sv);
     const unsigned code = __float_as_uint(ri.w);
     const int cx = (int)(code & CODE_MASK), cy = (int)((code >> CODE_BITS) & CODE_MASK);
     const int cz = (int)(code >> (2 * CODE_BITS));
@@ -212,8 +231,8 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
                 int xx = cx + dx;
                 xx = xx < 0 ? nc - 1 : (xx >= nc ? 0 : xx);
                 const int cell = rowb + ((xx >> 2) << 6) + (xx & 3);
-                const int k0 = __ldg(A.start + cell);
-                int n = live ? __ldg(A.start + cell + 1) - k0 : 0;
+                const int k0 = nl_ld<READ_ONLY>(A.start + cell);
+                int n = live ? nl_ld<READ_ONLY>(A.start + cell + 1) - k0 : 0;
                 if (n > MAX_CELL_OCC) {
                     err = ERR_NL_CAPACITY;
                     n = 0;
@@ -223,24 +242,25 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
                 const unsigned tag = (unsigned)((dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)) << IDX_BITS;
 #pragma unroll 2
                 for (int j = 0; j < nmax; ++j) {
-                    const float4 rj = __ldg(A.recs + k0 + j);
+                    const float4 rj = nl_ld<READ_ONLY>(A.recs + k0 + j);
                     const int t = __float_as_int(rj.w);
                     const float ex = rj.x - ox, ey = rj.y - oy, ez = rj.z - oz;
                     const float r2 = ex * ex + ey * ey + ez * ez;
                     const bool take = (j < n) & (r2 < hi) & (t != s) & (t != bp.y) & (t != bp.z);
                     nband += (take & (r2 >= lo)) ? 1 : 0;
-                    st_pred(out + (size_t)cnt * Mp, (unsigned)t | tag, take & (cnt < maxnb));
+                    st_pred_free(out + (size_t)cnt * Mp, (unsigned)t | tag, take & (cnt < maxnb));
                     cnt += take ? 1 : 0;
                 }
             }
         }
     }
+    nl_fence();
     if (nband > 0 && cnt <= maxnb) {                         // rare: decide the band entries in binary64
         int w = 0;
         for (int k = 0; k < cnt; ++k) {
             const unsigned e = out[(size_t)k * Mp];
             const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
-            const float r2 = nl_r2(ri, __ldg(A.recb + t), q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
+            const float r2 = nl_r2(ri, nl_ld<READ_ONLY>(A.recb + t), q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
             const bool keep = r2 < lo || dist2_exact(A.x, A.Mp, md.L, s, t) < A.rl2;
             if (keep) out[(size_t)(w++) * Mp] = e;
         }

@@ -202,15 +202,21 @@ __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __
 }
 
 // How a context's steps run: RES_NONE (launches per step), RES_WIDE (this
-// file's kernel, 640 monomers per SM) or RES_SMALL (kg_resident_small.cu, 128
-// monomers per SM).  Every block has to be resident at once; the limits are
-// what the kernels' __launch_bounds__ guarantee for every exponent.
+// file's kernel, 640 monomers per SM), RES_SMALL (kg_resident_small.cu, 128
+// monomers per SM) or RES_TILED (kg_resident_tiled.cu, any number; by default
+// while a block has one tile of 256).  Every block has to be resident at once;
+// the limits are what the kernels' __launch_bounds__ guarantee for every
+// exponent.
+constexpr int TILED_MOST = 5 * 256;
+
 int resident_kind(kg_ctx *c)
 {
-    if (c->precision != KG_MIXED || c->tpm != 1 || c->resident_failed) return RES_NONE;
+    if (c->precision != KG_MIXED || c->resident_failed) return RES_NONE;
+    if (c->tpm != 1 && !(c->p.flags & KG_FLAG_PERSISTENT)) return RES_NONE;
     if (c->res_sms < 0) cudaDeviceGetAttribute(&c->res_sms, cudaDevAttrMultiProcessorCount, c->device);
     if (c->buckets && c->M <= SMALL_OWN * SMALL_MIN_BLOCKS * c->res_sms) return RES_SMALL;
-    return c->M <= RES_BLOCK * RES_MIN_BLOCKS * c->res_sms ? RES_WIDE : RES_NONE;
+    if (c->M <= RES_BLOCK * RES_MIN_BLOCKS * c->res_sms) return RES_WIDE;
+    return c->M <= TILED_MOST * c->res_sms || (c->p.flags & KG_FLAG_PERSISTENT) ? RES_TILED : RES_NONE;
 }
 
 cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin)
@@ -251,8 +257,10 @@ cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin)
     cudaError_t e = cudaMemsetAsync(c->resbar, 0, 4 * sizeof(unsigned long long) + nseg * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
     const int n4 = n4_of(c->stage.n), nb = (c->M + RES_BLOCK - 1) / RES_BLOCK;
-    e = resident_kind(c) == RES_SMALL ? small_launch(a, n4, c->stream)
-                                      : KG_RESIDENT_LAUNCH(k_resident, n4, nb, RES_BLOCK, a, c->stream);
+    const int kind = resident_kind(c);
+    e = kind == RES_SMALL  ? small_launch(a, n4, c->stream)
+        : kind == RES_WIDE ? KG_RESIDENT_LAUNCH(k_resident, n4, nb, RES_BLOCK, a, c->stream)
+                           : tiled_launch(a, n4, c->res_sms, c->stream);
     if (e != cudaSuccess) return e;
     c->launches += 1;
     c->cur ^= K & 1;
@@ -272,7 +280,7 @@ bool resident_alloc(kg_ctx *c)
     }
     c->buckets = 3.0 * most <= BUCKET;
     const int kind = resident_kind(c);
-    if (kind == RES_NONE) return true;
+    if (c->precision != KG_MIXED) return true;
     c->resbar = (unsigned long long *)dev_alloc(c, 4 * sizeof(unsigned long long) +
                                                        ((size_t)c->ncell_md / RES_SEG + 1) * sizeof(int));
     if (kind != RES_SMALL) return c->resbar != nullptr;

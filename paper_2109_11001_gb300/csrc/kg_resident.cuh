@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kg_gridbar.cuh"
 #include "kg_step.cuh"
 
@@ -113,5 +115,7 @@ __device__ __forceinline__ void res_scan_seg(const ResArgs &A, const int *count,
 // kg_resident_small.cu
 constexpr int SMALL_OWN = 64, SMALL_MIN_BLOCKS = 2;   // monomers of a block of the small kernel, blocks per SM
 cudaError_t small_launch(const ResArgs &a, int n4, cudaStream_t st);
+// kg_resident_tiled.cu
+cudaError_t tiled_launch(const ResArgs &a, int n4, int sms, cudaStream_t st);
 
 }  // namespace kg

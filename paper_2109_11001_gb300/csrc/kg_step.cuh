@@ -1,6 +1,6 @@
 // kg_step.cuh -- arithmetic of the mixed path's MD step, shared by the one-step
-// kernel, the persistent kernel (kg_step.cu) and the resident kernel
-// (kg_resident.cu): all three give the same bits.
+// kernel (kg_step.cu) and the resident kernels (kg_resident*.cu): all give the
+// same bits.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -179,6 +179,114 @@ __device__ __forceinline__ void step_block_setup(float *dk)
         dk[32 + q] = (float)((q / 3) % 3 - 1);
         dk[64 + q] = (float)(q / 9 - 1);
     }
+}
+
+constexpr int STEP_ILP = 4;      // Verlet-list entries in flight per lane
+// One tile of blockDim threads (all threads of the block call it together):
+// the step of the monomers of threads t0 + threadIdx.x.  TPM threads per
+// monomer (1 or 2, adjacent lanes): the lanes split the list (entries k =
+// sub, sub + TPM, ...); with two, lane 0 adds the bonded terms and lane 1
+// draws the noise, the forces are combined with a shuffle, and lane 0 writes
+// the state.  The pair loop comes first and holds only its own state (the
+// own gather record, the force, the entries in flight), so the kernel fits
+// 32 registers at full occupancy; the bonded terms, the noise and the build
+// record and displacement for the update follow.  The pair loop runs to the
+// warp's longest list in groups of STEP_ILP entries with per-lane
+// predicates: an entry past the lane's own list becomes the lane's own record
+// with the zero shift (code 13), a valid gather whose term is masked.
+// READ_ONLY: nothing it loads is written in the same launch (non-coherent
+// loads).  vote(rebuild, err), by every lane of the warp: its monomer left its
+// skin, and its error bits.
+template <bool READ_ONLY, typename T>
+__device__ __forceinline__ T step_ld(const T *p)
+{
+    if constexpr (READ_ONLY) return __ldg(p);
+    else return *p;
+}
+
+template <int N4, int TPM, bool READ_ONLY, class VOTE>
+__device__ __forceinline__ void step_tile(const StepArgs &P, int t0, const float4 *dcur, float4 *dnext,
+                                          const float4 *pcur, float4 *pnext, long long step, const float *dk,
+                                          VOTE vote)
+{
+    constexpr bool RO = READ_ONLY;
+    const int lane = threadIdx.x & 31;
+    const int t = t0 + threadIdx.x;
+    const int s = t / TPM, sub = t % TPM;
+    const bool live = s < P.M;
+    const int cnt = live ? step_ld<RO>(P.nn + s) : 0;
+    const int kmax = __reduce_max_sync(0xffffffffu, cnt);
+    unsigned err = 0;
+    float3 F = make_float3(0.f, 0.f, 0.f), gn = F;
+    int slot = 0, m = 0;
+    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) {
+        slot = __ldg(P.slot_of + s);
+        m = melt_index(P, slot);
+        pi = step_ld<RO>(pcur + s);
+    }
+    const MeltStep &md = P.melt[m];
+    const float h = md.h, rc2 = P.rc2;
+    const unsigned self = (unsigned)(live ? s : 0) | (13u << IDX_BITS);
+    const size_t Mp = (size_t)P.Mp;
+    const unsigned *col = P.nl + (live ? s : 0);
+    for (int k0 = sub; k0 < kmax; k0 += STEP_ILP * TPM) {
+        unsigned e[STEP_ILP];
+        float4 pj[STEP_ILP];
+#pragma unroll
+        for (int i = 0; i < STEP_ILP; ++i) {
+            const int k = k0 + i * TPM;
+            e[i] = k < cnt ? step_ld<RO>(col + (size_t)k * Mp) : self;
+        }
+#pragma unroll
+        for (int i = 0; i < STEP_ILP; ++i) pj[i] = step_ld<RO>(pcur + (e[i] & IDX_MASK));
+#pragma unroll
+        for (int i = 0; i < STEP_ILP; ++i) {
+            const unsigned q = e[i] >> IDX_BITS;
+            const float dx = fmaf(dk[q], h, pj[i].x - pi.x);
+            const float dy = fmaf(dk[32 + q], h, pj[i].y - pi.y);
+            const float dz = fmaf(dk[64 + q], h, pj[i].z - pi.z);
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
+            float fr = mlj_fr32<N4>(P, r2);
+            fr = (k0 + i * TPM < cnt && r2 < rc2) ? fr : 0.0f;
+            F.x = fmaf(fr, dx, F.x); F.y = fmaf(fr, dy, F.y); F.z = fmaf(fr, dz, F.z);
+        }
+    }
+    float4 rb = make_float4(0.f, 0.f, 0.f, 0.f), dc = rb;
+    if (live) {
+        if (sub == 0) bonded32<N4>(P, [&](int, int j) { return step_ld<RO>(pcur + j); },
+                                   [&](int, float a, float3 x) { axpy3(a, x, F); }, md, pi, __ldg(P.bp + s), err);
+        if (sub == TPM - 1)
+            gn = gauss3_f(draw(P.seed, m, 0, (unsigned long long)step, (uint32_t)(slot - md.off)));
+        rb = step_ld<RO>(P.recb + s);
+        dc = step_ld<RO>(dcur + s);
+    }
+    if (TPM == 2) {                        // every lane takes part: s is shared by lanes 2i, 2i+1
+        F.x += __shfl_xor_sync(0xffffffffu, F.x, 1);
+        F.y += __shfl_xor_sync(0xffffffffu, F.y, 1);
+        F.z += __shfl_xor_sync(0xffffffffu, F.z, 1);
+        const int src = lane | 1;
+        gn.x = __shfl_sync(0xffffffffu, gn.x, src);
+        gn.y = __shfl_sync(0xffffffffu, gn.y, src);
+        gn.z = __shfl_sync(0xffffffffu, gn.z, src);
+    }
+    bool rebuild = false;
+    if (live && sub == 0) {
+        const int Mpi = P.Mp;
+        float *u = P.u;
+        float3 v = make_float3(u[s], u[Mpi + s], u[2 * Mpi + s]);
+        v.x = fmaf(P.dt, fmaf(P.amp, gn.x, fmaf(-P.gamma, v.x, F.x)), v.x);
+        v.y = fmaf(P.dt, fmaf(P.amp, gn.y, fmaf(-P.gamma, v.y, F.y)), v.y);
+        v.z = fmaf(P.dt, fmaf(P.amp, gn.z, fmaf(-P.gamma, v.z, F.z)), v.z);
+        u[s] = v.x; u[Mpi + s] = v.y; u[2 * Mpi + s] = v.z;
+        float4 d = dc;
+        d.x = fmaf(P.dt, v.x, d.x); d.y = fmaf(P.dt, v.y, d.y); d.z = fmaf(P.dt, v.z, d.z);
+        dnext[s] = d;
+        pnext[s] = make_float4(rb.x + d.x, rb.y + d.y, rb.z + d.z, rb.w);
+        rebuild = fmaf(d.z, d.z, fmaf(d.y, d.y, __fmul_rn(d.x, d.x))) > P.half_skin2;
+        if (!isfinite(v.x + v.y + v.z)) err |= ERR_NONFINITE;
+    }
+    vote(rebuild, err);
 }
 
 // 4n of a stage exponent with its own kernel instantiation, 0 otherwise

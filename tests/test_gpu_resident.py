@@ -26,9 +26,9 @@ def kg():
     return kg
 
 
-def _run(kg, melts, one_by_one, skin=0.3, cell_scale=0.0, stream=None):
+def _run(kg, melts, one_by_one, skin=0.3, cell_scale=0.0, stream=None, flags=0):
     p = kg.make_params([(m.n_chains, m.chain_len, m.box, m.kappa) for m in melts], seed=9, fene_qmin=0.01, skin=skin,
-                       sort_interval=40, cell_scale=cell_scale)
+                       sort_interval=40 if not flags else 10 ** 9, cell_scale=cell_scale, flags=flags)
     ctx = kg.kg_create(p, 0, stream, None)
     try:
         # n = 2, then 5 (another instantiation), a stage change inside a call
@@ -100,12 +100,25 @@ def test_a_crowded_cell(kg, crowd):
 @pytest.mark.parametrize("kind", [0, 1])
 def test_both_sides_of_a_capacity(kg, kind):
     cap = _capacities()[kind]
-    for extra in (0, 1):                         # every block resident; one block more takes the next path
+    for extra in (0, 1):                         # every block resident; one block more takes the next kernel
         m = KI.random_walk_melt(cap // 128 + extra, 128, 0.85, 2.0, 31)
         a, la = _run(kg, [m], 0)
         b, lb = _run(kg, [m], 1)
         assert all(np.array_equal(p, q) for p, q in zip(a, b))
-        assert (la < lb / 5) == (kind == 0 or extra == 0)
+        assert la < lb / 5
+
+
+# one tile of 256 monomers for every block; a few blocks with a second, which
+# only the flag asks for
+@pytest.mark.parametrize("extra,flags", [(0, 0), (3, 2)])
+def test_tiles(kg, extra, flags):
+    import torch
+    n = torch.cuda.get_device_properties(0).multi_processor_count
+    m = KI.random_walk_melt(10 * n + extra, 128, 0.85, 2.0, 33)
+    a, la = _run(kg, [m], 0, flags=flags)
+    b, lb = _run(kg, [m], 1, flags=flags)
+    assert all(np.array_equal(p, q) for p, q in zip(a, b))
+    assert la < lb / 5
 
 
 def test_two_contexts_on_two_threads(kg):

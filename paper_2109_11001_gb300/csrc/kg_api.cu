@@ -128,11 +128,11 @@ __global__ void k_iota(int *__restrict__ a, int n, int base)
 }
 
 // Read the device status word; translate latched error bits.
-kg_status read_flags(kg_ctx *c, unsigned *host4)
+kg_status read_flags(kg_ctx *c, unsigned *host8)
 {
-    KG_TRY(cudaMemcpyAsync(host4, c->flags, sizeof(unsigned) * 4, cudaMemcpyDeviceToHost, c->stream));
+    KG_TRY(cudaMemcpyAsync(host8, c->flags, sizeof(unsigned) * 8, cudaMemcpyDeviceToHost, c->stream));
     KG_TRY(cudaStreamSynchronize(c->stream));
-    const unsigned e = host4[0];
+    const unsigned e = host8[0];
     kg_status s = KG_OK;
     if (e & kg::ERR_OVERSTRETCH) s = KG_ERR_BOND_OVERSTRETCH;
     else if (e & kg::ERR_NONFINITE) s = KG_ERR_NONFINITE;
@@ -375,6 +375,7 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->scratch = (double *)A(7 * Mp * sizeof(double));
     c->flags = (unsigned *)A(16 * sizeof(unsigned));
     c->d_step = (long long *)A(sizeof(long long));
+    c->loop = (kg::LoopDev *)A(sizeof(kg::LoopDev));
     c->fout = (double *)A(3 * Mp * sizeof(double));
     c->partials_cap = (int)(Mp / 128 + 2) * 5;
     c->partials = (double *)A((size_t)c->partials_cap * sizeof(double));
@@ -428,6 +429,7 @@ void kg_destroy(kg_ctx *c)
     for (void *b : bufs) dev_free(c, b);
     dev_free(c, c->d_step);
     dev_free(c, c->dbbar);
+    dev_free(c, c->loop);
     dev_free(c, c->resbar);
     dev_free(c, c->bcount);
     dev_free(c, c->bidx);
@@ -435,7 +437,6 @@ void kg_destroy(kg_ctx *c)
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     kg::graphs_reset(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
-    if (c->cap_stream2) cudaStreamDestroy(c->cap_stream2);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -555,10 +556,9 @@ kg_status kg_set_potential_schedule(kg_ctx *c, const kg_stage *stages, int n_sta
 // MD steps until the next re-sort test of a run of `left` steps: the tests sit
 // at the start of the run and after each whole group of steps (PERSIST_STEPS
 // with KG_FLAG_PERSISTENT, then GRAPH_STEPS, then single steps), however many
-// groups one launch covers.
-static int steps_to_sort(const kg_ctx *c, long long left, bool persistent)
+// groups one launch covers, `most` steps in all.
+static int steps_to_sort(const kg_ctx *c, long long left, bool persistent, long long most)
 {
-    const long long most = persistent ? kg::PERSIST_MAX : kg::RESIDENT_STEPS;
     long long n = 0;
     while (n < left && (n == 0 || c->since_sort + n < c->sort_interval)) {
         const long long rest = left - n;
@@ -576,6 +576,7 @@ kg_status kg_step(kg_ctx *c, long long n_steps)
     if (!c || n_steps < 0) return KG_ERR_INVALID_ARG;
     if (c->latched != KG_OK) return KG_ERR_STATE;
     if (cudaSetDevice(c->device) != cudaSuccess) return KG_ERR_CUDA;
+    const long long asked = n_steps;
     while (n_steps > 0) {
         // advance past exhausted stages
         while (c->stage_left == 0 && c->stage_idx + 1 < c->schedule.size()) {
@@ -602,16 +603,19 @@ kg_status kg_step(kg_ctx *c, long long n_steps)
             if (c->sort_after_load)             // after a load: one step builds the cell order to sort into
                 kg::md_step(c);
             else if (!c->prof_on && kg::resident_kind(c) != kg::RES_NONE) {
-                n = steps_to_sort(c, chunk - done, (c->p.flags & KG_FLAG_PERSISTENT) != 0);
+                const bool longer = (c->p.flags & KG_FLAG_PERSISTENT) != 0;
+                n = steps_to_sort(c, chunk - done, longer, longer ? kg::PERSIST_MAX : kg::RESIDENT_STEPS);
                 if (kg::resident_launch(c, (int)n, -1, kg::RESIDENT_SPIN) != cudaSuccess) {
                     cudaGetLastError();
                     c->resident_failed = true;  // the launches below serve it
                     continue;
                 }
-            } else if (!c->prof_on && c->use_graphs && chunk - done >= kg::GRAPH_STEPS && kg::md_graph_steps(c, 1))
-                n = kg::GRAPH_STEPS;
-            else
+            } else if (!c->prof_on && chunk - done >= kg::GRAPH_STEPS && !c->graph_failed) {
+                n = steps_to_sort(c, chunk - done, false, kg::PERSIST_MAX);
+                if (!kg::md_loop_steps(c, (int)n)) continue;   // graph_failed: the launches below serve it
+            } else {
                 kg::md_step(c);
+            }
             c->clist_valid = true;              // a Verlet build has run since the last load / sort
             c->step += n;
             c->since_sort += n;
@@ -624,7 +628,11 @@ kg_status kg_step(kg_ctx *c, long long n_steps)
     kg::md_materialize(c);                      // current binary64 positions for every other call
     KG_TRY(cudaGetLastError());
     unsigned *h = pinned_flags();
-    return read_flags(c, h);
+    const kg_status s = read_flags(c, h);
+    const unsigned builds = h[5] - c->builds_seen;
+    if (asked >= kg::LOOP_MAX) c->build_every = builds ? (double)asked / builds : (double)kg::LOOP_MAX;
+    c->builds_seen = h[5];
+    return s;
 }
 
 kg_status kg_persistent_selftest(kg_ctx *c, int skip_block, unsigned spin)
@@ -1221,11 +1229,11 @@ kg_status kg_profile_read(kg_ctx *c, double *ms, long long *n, long long *launch
     if (ms) *ms = c->prof_ms;
     if (n) *n = c->prof_n;
     if (launches) {
-        // inside graphs the six rebuild kernels run only when requested; the
-        // device counts those runs in flags[6]
+        // the device counts a captured loop's passes in flags[6]: chain, end
+        // kernel and the steps that returned at once
         unsigned f[8];
         if (cudaMemcpy(f, c->flags, sizeof(f), cudaMemcpyDeviceToHost) != cudaSuccess) return KG_ERR_CUDA;
-        *launches = c->launches + 6LL * (long long)f[6];
+        *launches = c->launches + (long long)f[6];
     }
     return KG_OK;
 }

@@ -48,16 +48,17 @@ struct kg_ctx {
     long long *d_step = nullptr;   // device step counter (index of the step being run)
     bool d_step_stale = true;      // host must write it before the next step
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+    cudaGraphExec_t gexec[kg::LOOP_MAX / 4] = {};   // captured step loops with bodies of 4, 8, 12 and 16 steps
     bool graph_failed = false;
+    kg::LoopDev *loop = nullptr;   // their state on the device
+    double build_every = 8.0;      // MD steps between Verlet builds in the last call long enough to tell
+    unsigned builds_seen = 0;      // builds counted on the device up to the end of the last call
     unsigned long long *resbar = nullptr;   // barrier words, error word and segment totals of the resident launch
     int *bcount = nullptr, *bidx = nullptr; // its cell buckets: two sets of counts, members in arrival order
     float4 *brec = nullptr;                 // and records in order
     bool buckets = false;
     int res_sms = -1;            // SMs of the GPU (< 0: not asked yet)
     bool resident_failed = false;
-    bool use_graphs = true;
-    long long graph_replays = 0;
     long long sort_interval = 200;
     int block = 128;             // threads per block of the fused step kernel
     int tpm = 1;                 // threads per monomer of the mixed step kernel (1 or 2)
@@ -142,9 +143,9 @@ namespace kg {
 void *dev_alloc(kg_ctx *c, size_t bytes);
 void dev_free(kg_ctx *c, void *p);
 
-constexpr int GRAPH_STEPS = 10;          // MD steps per captured graph (even)
+constexpr int GRAPH_STEPS = 10;          // MD steps between re-sort tests
 constexpr int PERSIST_STEPS = 50;        // MD steps between re-sort tests with KG_FLAG_PERSISTENT
-constexpr int RESIDENT_STEPS = 50;       // MD steps per resident launch (KG_FLAG_PERSISTENT: PERSIST_MAX)
+constexpr int RESIDENT_STEPS = 50;       // MD steps per resident launch (KG_FLAG_PERSISTENT, step loop: PERSIST_MAX)
 constexpr int PERSIST_MAX = 1000;
 constexpr unsigned RESIDENT_SPIN = 1u << 22;  // its barrier polls (a few hundred ns apart) before ERR_TIMEOUT
 constexpr int RS = 8;                    // ints per melt in the DB commit-round array
@@ -166,7 +167,7 @@ struct __align__(16) Attempt {
 // kg_md.cu
 void rebuild_md(kg_ctx *c);                  // conditional on flags[1]
 void md_step(kg_ctx *c);                     // one fused force + integrate step (direct launches)
-bool md_graph_steps(kg_ctx *c, long long nrep);  // nrep replays of a GRAPH_STEPS-step graph
+bool md_loop_steps(kg_ctx *c, int n);        // n steps in one launch of the captured step loop
 void set_device_step(kg_ctx *c, long long v);
 void forces_eval(kg_ctx *c, int melt, long long step, double *F_dev, double *part_dev, int nblk);
 void prof_collect(kg_ctx *c);                // fold recorded event pairs into the totals
@@ -185,7 +186,8 @@ cudaError_t resident_reset(kg_ctx *c);
 void resident_cell_order(kg_ctx *c);         // clist after builds that used buckets
 
 // kg_step.cu
-void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur);   // the mixed path's fused step kernel
+// the mixed path's fused step kernel; loop, k: its place in a captured step loop
+void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur, LoopDev *loop, int k);
 void to_slots(kg_ctx *c, int melt, const double *in_comp, double *out_dev, int dims);
 void state_to_slots(kg_ctx *c, int melt, double *x_dev, double *u_dev, int *pid_dev);   // null: not wanted
 int forces_blocks(const kg_ctx *c, int melt);

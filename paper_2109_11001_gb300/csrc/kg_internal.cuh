@@ -39,6 +39,17 @@ enum : unsigned {
     ERR_DB_INTERNAL = 32u,
 };
 
+constexpr int LOOP_MAX = 16;             // steps in the body of a captured step loop, at most (multiple of 4)
+
+// State of a captured step loop (kg_md.cu) on the device.
+struct LoopDev {
+    int rem;                 // MD steps still to run
+    int n;                   // of them in the present pass of the loop body
+    int src;                 // buffer that holds the state when the pass begins (1 only before a list build)
+    int par;                 // buffer that holds it after the last pass
+    unsigned req;            // bit k: step k of the pass asked for a list rebuild (later ones of the pass are skipped)
+};
+
 // status words kept by the resident MD kernel: how the last Verlet build left the
 // cell order (0: clist; 1 + b: buckets with counts b), and the zeroed count buffer
 constexpr int RES_BUILT = 8, RES_NEXT = 9;

@@ -13,6 +13,10 @@
 // the random draws so results do not depend on the order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cstddef>
+#include <cstdlib>
+
 #include "kg_host.h"
 #include "kg_rebuild.cuh"
 
@@ -393,12 +397,22 @@ __global__ void __launch_bounds__(256) k_step_f64(const SimDev *__restrict__ Sp,
                                                  const unsigned *__restrict__ nl,
                                                  const int *__restrict__ nn, const int *__restrict__ slot_of,
                                                  const int4 *__restrict__ bp, unsigned *__restrict__ flags,
-                                                 const long long *__restrict__ stepp)
+                                                 const long long *__restrict__ stepp, LoopDev *loop, int kstep)
 {
-    if (flags[0]) return;                  // a latched error stops the run
+    __shared__ unsigned stop;
+    if (threadIdx.x == 0) {                // a latched error, the end of the loop or an earlier step's rebuild request
+        unsigned f = *(volatile unsigned *)flags;
+        if (loop) {
+            const volatile LoopDev *lp = loop;
+            if (kstep >= lp->n || (lp->req & ((1u << kstep) - 1u))) f = 1u;
+        }
+        stop = f;
+    }
+    __syncthreads();
+    if (stop) return;
     const SimDev &S = *Sp;
     const StageDev &st = *stp;
-    const long long step = *stepp;
+    const long long step = *stepp + (loop ? 1 + kstep : 0);
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     bool rebuild = false;
     unsigned err = 0;
@@ -460,7 +474,10 @@ __global__ void __launch_bounds__(256) k_step_f64(const SimDev *__restrict__ Sp,
         rebuild = !(fmaf(dz, dz, fmaf(dy, dy, dx * dx)) <= S.half_skin2f * (1.0f - 1e-6f));
         if (!isfinite(v.x + v.y + v.z)) err |= ERR_NONFINITE;
     }
-    if (__syncthreads_or(rebuild) && threadIdx.x == 0) atomicOr(flags + 1, 1u);
+    if (__syncthreads_or(rebuild) && threadIdx.x == 0) {
+        if (loop) atomicOr(&loop->req, 1u << kstep);
+        else atomicOr(flags + 1, 1u);
+    }
     if (err) atomicOr(flags, err);
 }
 
@@ -472,17 +489,19 @@ __global__ void __launch_bounds__(256) k_step_f64(const SimDev *__restrict__ Sp,
 // gather buffers reset, Verlet-grid cell + rank within it
 __global__ void __launch_bounds__(256) k_bin_md(const SimDev *__restrict__ Sp, double *__restrict__ x,
                                                double *__restrict__ xb64,
-                                               float4 *__restrict__ recb, float4 *__restrict__ dcur,
+                                               float4 *__restrict__ recb, float4 *dcur,
                                                float4 *__restrict__ pgcur, double4_32a *__restrict__ pcur,
                                                double4_32a *__restrict__ xb, int *__restrict__ cellid,
                                                int *__restrict__ rank, int *__restrict__ count,
-                                               const int *__restrict__ slot_of, unsigned *__restrict__ flags)
+                                               const int *__restrict__ slot_of, unsigned *__restrict__ flags,
+                                               const float4 *dother, const LoopDev *__restrict__ loop)
 {
     if (!flags[1] || flags[0]) return;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= Sp->M) return;
     const unsigned err =
-        bin_md_one(*Sp, s, x, xb64, recb, dcur, pgcur, pcur, xb, cellid, rank, count, slot_of);
+        bin_md_one(*Sp, s, x, xb64, recb, loop && loop->src ? dother : dcur, dcur, pgcur, pcur, xb, cellid, rank, count,
+                   slot_of);                       // a loop's pass starts in buffer 0 wherever the last one ended
     if (err) atomicOr(flags, err);
 }
 
@@ -848,19 +867,9 @@ void state_to_slots(kg_ctx *c, int melt, double *x_dev, double *u_dev, int *pid_
                                                             md.off, md.M, x_dev, u_dev, pid_dev);
 }
 
-// First kernel of every MD step: advance the device step counter (the index
-// of the step about to run) and, inside a captured graph, arm the conditional
-// rebuild node with the rebuild request.
-__global__ void k_begin_step(long long *__restrict__ stepp, unsigned *__restrict__ flags,
-                             cudaGraphConditionalHandle h, int armed)
-{
-    stepp[0] += 1;
-    if (armed) {
-        const unsigned go = (flags[1] && !flags[0]) ? 1u : 0u;
-        cudaGraphSetConditional(h, go);
-        flags[6] += go;                        // rebuild bodies run inside graphs
-    }
-}
+// First kernel of a directly launched MD step: advance the device step counter
+// (the index of the step about to run).
+__global__ void k_begin_step(long long *__restrict__ stepp) { stepp[0] += 1; }
 
 __global__ void k_set_step(long long *__restrict__ stepp, long long v) { stepp[0] = v; }
 
@@ -871,12 +880,12 @@ void scan_counts(kg_ctx *c, const int *count, int *start, int n, int *bsum)
     k_scan2<<<nb, 1024, 0, c->stream>>>(start, bsum, n, nb, nullptr);
 }
 
-static void launch_rebuild(kg_ctx *c, cudaStream_t st);
+static void launch_rebuild(kg_ctx *c, cudaStream_t st, int cur, LoopDev *loop);
 
 void rebuild_md(kg_ctx *c)
 {
     c->launches += 6;
-    launch_rebuild(c, c->stream);
+    launch_rebuild(c, c->stream, c->cur, nullptr);
 }
 
 NlArgs nl_args(const kg_ctx *c)
@@ -903,12 +912,13 @@ NlArgs nl_args(const kg_ctx *c)
     return a;
 }
 
-static void launch_rebuild(kg_ctx *c, cudaStream_t st)
+static void launch_rebuild(kg_ctx *c, cudaStream_t st, int cur, LoopDev *loop)
 {
     const bool mixed = c->precision == KG_MIXED;
     k_bin_md<<<nblk(c->M, 256), 256, 0, st>>>(c->d_sim, c->x, mixed ? c->xb64 : nullptr, c->recb,
-                                              mixed ? c->dlt[c->cur] : nullptr, c->pg[c->cur], mixed ? nullptr : c->pos64[c->cur],
-                                              c->xb, c->cellid, c->rank, c->ccount, c->slot_of, c->flags);
+                                              mixed ? c->dlt[cur] : nullptr, c->pg[cur], mixed ? nullptr : c->pos64[cur],
+                                              c->xb, c->cellid, c->rank, c->ccount, c->slot_of, c->flags,
+                                              mixed ? c->dlt[cur ^ 1] : nullptr, loop);
     const int nb = nblk(c->ncell_md, 1024);
     k_scan1<<<nb, 1024, 0, st>>>(c->ccount, c->cstart, c->bsum, c->ncell_md, c->flags);
     k_scan2<<<nb, 1024, 0, st>>>(c->cstart, c->bsum, c->ncell_md, nb, c->flags);
@@ -918,26 +928,24 @@ static void launch_rebuild(kg_ctx *c, cudaStream_t st)
     k_nlist<<<nblk(c->M, NL_BLOCK), NL_BLOCK, 0, st>>>(nl_args(c));
 }
 
-static void launch_step_kernel(kg_ctx *c, cudaStream_t st, int cur)
+static void launch_step_kernel(kg_ctx *c, cudaStream_t st, int cur, LoopDev *loop, int k)
 {
     if (c->precision == KG_MIXED) {
-        step_mixed_launch(c, st, cur);
+        step_mixed_launch(c, st, cur, loop, k);
         return;
     }
     const int nb = nblk(c->M, c->block);
     k_step_f64<<<nb, c->block, 0, st>>>(c->d_sim, c->d_stage, c->x, (double *)c->u, c->pos64[cur], c->pos64[cur ^ 1],
-                                        c->xb, c->recb, c->pg[cur], c->pg[cur ^ 1], c->nl, c->nn, c->slot_of, c->bp, c->flags, c->d_step);
+                                        c->xb, c->recb, c->pg[cur], c->pg[cur ^ 1], c->nl, c->nn, c->slot_of, c->bp, c->flags, c->d_step, loop, k);
 }
 
 // Captured graphs hold the step kernel's by-value arguments (stage
 // parameters among them): drop them when those change.
 void graphs_reset(kg_ctx *c)
 {
-    for (int k = 0; k < 2; ++k) {
-        if (c->gexec[k]) {
-            cudaGraphExecDestroy(c->gexec[k]);
-            c->gexec[k] = nullptr;
-        }
+    for (cudaGraphExec_t &e : c->gexec) {
+        if (e) cudaGraphExecDestroy(e);
+        e = nullptr;
     }
 }
 
@@ -964,7 +972,7 @@ void prof_collect(kg_ctx *c)
 
 void md_step(kg_ctx *c)
 {
-    k_begin_step<<<1, 1, 0, c->stream>>>(c->d_step, c->flags, cudaGraphConditionalHandle{}, 0);
+    k_begin_step<<<1, 1, 0, c->stream>>>(c->d_step);
     ++c->launches;
     rebuild_md(c);
     cudaEvent_t e1 = nullptr;
@@ -979,90 +987,128 @@ void md_step(kg_ctx *c)
         ++c->ev_used;
     }
     ++c->launches;
-    launch_step_kernel(c, c->stream, c->cur);
+    launch_step_kernel(c, c->stream, c->cur, nullptr, 0);
     if (e1) cudaEventRecord(e1, c->stream);
     c->cur ^= 1;
 }
 
-// A CUDA graph of GRAPH_STEPS MD steps: per step, the begin kernel, a
-// conditional node holding the rebuild chain (run only when a rebuild was
-// requested), and the fused step kernel.  GRAPH_STEPS is even, so a replay
-// leaves the ping-pong buffers as it found them; one graph per starting buffer.
-static bool capture_graph(kg_ctx *c, int parity)
+// ---------------------------------------------------------------------------
+// captured step loop: a graph with one while node, whose body is the rebuild
+// chain (its kernels return at once without a request), up to LOOP_MAX step
+// kernels and a one-thread kernel that ends the pass.  A step that asks for a
+// rebuild sets its bit; the later steps of the pass see it and return at once,
+// and the next pass starts with the chain.  So the graph's control (a while
+// node's turn, ~10 us) is paid once per list build, where a conditional node
+// in front of every step cost about 13 us a step (the step kernel of 200,000
+// monomers takes 14, that of 1.6M 91).  The body is as long as the measured
+// number of steps between builds, so few step kernels are launched in vain.
+// Passes start in buffer 0 (a build writes it, and the body's length is even);
+// k_loop_settle moves the result there when the last pass ended in buffer 1.
+// ---------------------------------------------------------------------------
+__global__ void k_loop_begin(LoopDev *lp, int steps, int len)
+{
+    lp->rem = steps;
+    lp->n = steps < len ? steps : len;
+    lp->src = lp->par = 0;
+    lp->req = 0u;
+}
+
+__global__ void k_loop_end(LoopDev *lp, int len, long long *__restrict__ stepp, unsigned *__restrict__ flags,
+                           cudaGraphConditionalHandle h)
+{
+    const int done = lp->req ? min(lp->n, __ffs((int)lp->req)) : lp->n;
+    stepp[0] += done;
+    const int rem = lp->rem - done;
+    lp->rem = rem;
+    lp->n = rem < len ? rem : len;
+    const bool more = rem > 0 && !flags[0];
+    lp->src = done & 1;                        // every pass starts in buffer 0, or with a build that writes it
+    lp->par = more ? 0 : done & 1;
+    if (lp->req) flags[1] = 1u;
+    lp->req = 0u;
+    flags[6] += 7 + len - done;                // kernels launched in loops, less the steps done (the host counts those)
+    cudaGraphSetConditional(h, more ? 1u : 0u);
+}
+
+__global__ void __launch_bounds__(256) k_loop_settle(const LoopDev *__restrict__ lp, bool always,
+                                                    float4 *__restrict__ a0, const float4 *__restrict__ a1, int na,
+                                                    float4 *__restrict__ b0, const float4 *__restrict__ b1, int nb)
+{
+    if (!always && !lp->par) return;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < na; i += gridDim.x * blockDim.x) a0[i] = a1[i];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) b0[i] = b1[i];
+}
+
+static bool capture_loop(kg_ctx *c, int len, cudaGraphExec_t *exec)
 {
     cudaGraph_t g = nullptr;
     if (cudaGraphCreate(&g, 0) != cudaSuccess) return false;
-    bool ok = cudaStreamBeginCaptureToGraph(c->cap_stream, g, nullptr, nullptr, 0,
-                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    int cur = parity;
-    for (int i = 0; ok && i < GRAPH_STEPS; ++i) {
-        cudaGraphConditionalHandle h;
-        ok = cudaGraphConditionalHandleCreate(&h, g, 0, 0) == cudaSuccess;
-        if (!ok) break;
-        k_begin_step<<<1, 1, 0, c->cap_stream>>>(c->d_step, c->flags, h, 1);
-        cudaStreamCaptureStatus cs;
-        cudaGraph_t cg = nullptr;
-        const cudaGraphNode_t *deps = nullptr;
-        size_t nd = 0;
-        ok = cudaStreamGetCaptureInfo(c->cap_stream, &cs, nullptr, &cg, &deps, nullptr, &nd) == cudaSuccess;
-        if (!ok) break;
-        cudaGraphNodeParams cp{};
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeIf;
-        cp.conditional.size = 1;
-        cudaGraphNode_t cn;
-        ok = cudaGraphAddNode(&cn, cg, deps, nullptr, nd, &cp) == cudaSuccess &&
-             cudaStreamUpdateCaptureDependencies(c->cap_stream, &cn, nullptr, 1,
-                                                 cudaStreamSetCaptureDependencies) == cudaSuccess;
-        if (!ok) break;
+    cudaGraphConditionalHandle h;
+    bool ok = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = h;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t cn;
+    ok = ok && cudaGraphAddNode(&cn, g, nullptr, nullptr, 0, &cp) == cudaSuccess;
+    if (ok) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
-        ok = cudaStreamBeginCaptureToGraph(c->cap_stream2, body, nullptr, nullptr, 0,
+        ok = cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0,
                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (!ok) break;
-        const int save = c->cur;
-        c->cur = cur;
-        launch_rebuild(c, c->cap_stream2);
-        c->cur = save;
-        ok = cudaStreamEndCapture(c->cap_stream2, &body) == cudaSuccess;
-        if (!ok) break;
-        launch_step_kernel(c, c->cap_stream, cur);
-        cur ^= 1;
+        if (ok) {
+            launch_rebuild(c, c->cap_stream, 0, c->loop);
+            for (int k = 0; k < len; ++k) launch_step_kernel(c, c->cap_stream, k & 1, c->loop, k);
+            k_loop_end<<<1, 1, 0, c->cap_stream>>>(c->loop, len, c->d_step, c->flags, h);
+            ok = cudaStreamEndCapture(c->cap_stream, &body) == cudaSuccess && cudaGetLastError() == cudaSuccess;
+        }
     }
-    cudaGraph_t out = nullptr;
-    const bool ended = cudaStreamEndCapture(c->cap_stream, &out) == cudaSuccess;
-    ok = ok && ended && cudaGetLastError() == cudaSuccess &&
-         cudaGraphInstantiate(&c->gexec[parity], g, 0) == cudaSuccess;
+    ok = ok && cudaGraphInstantiate(exec, g, 0) == cudaSuccess;
     cudaGraphDestroy(g);
     if (!ok) {
         cudaGetLastError();
-        c->gexec[parity] = nullptr;
+        *exec = nullptr;
     }
     return ok;
 }
 
-bool md_graph_steps(kg_ctx *c, long long nrep)
+// buffer 1 of the state that alternates between steps to buffer 0
+static void loop_settle(kg_ctx *c, bool always)
 {
-    const int parity = c->cur;
-    if (!c->gexec[parity]) {
-        if (c->graph_failed) return false;
-        if (!c->cap_stream) {
-            if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
-                cudaStreamCreateWithFlags(&c->cap_stream2, cudaStreamNonBlocking) != cudaSuccess) {
-                c->graph_failed = true;
-                return false;
-            }
+    const bool mixed = c->precision == KG_MIXED;
+    ++c->launches;
+    k_loop_settle<<<std::min(nblk(c->M, 256), 152 * 8), 256, 0, c->stream>>>(
+        c->loop, always, mixed ? c->dlt[0] : (float4 *)c->pos64[0], mixed ? c->dlt[1] : (const float4 *)c->pos64[1],
+        mixed ? c->M : 2 * c->M, c->pg[0], c->pg[1], c->M);
+}
+
+bool md_loop_steps(kg_ctx *c, int n)
+{
+    if (c->graph_failed) return false;
+    // the multiple of four at or above the measured number of steps between builds
+    int q = 0;
+    while (4 * (q + 1) < LOOP_MAX && c->build_every > 4.0 * (q + 1)) ++q;
+    const int len = 4 * (q + 1);
+    if (!c->gexec[q]) {
+        if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+            c->graph_failed = true;
+            return false;
         }
-        if (!capture_graph(c, parity)) {
+        if (!capture_loop(c, len, &c->gexec[q])) {
             c->graph_failed = true;
             return false;
         }
     }
-    for (long long r = 0; r < nrep; ++r) {
-        if (cudaGraphLaunch(c->gexec[parity], c->stream) != cudaSuccess) return false;
-        c->launches += 2 * GRAPH_STEPS;        // begin + step kernels; executed rebuilds counted on the device
-        ++c->graph_replays;
+    k_loop_begin<<<1, 1, 0, c->stream>>>(c->loop, n, len);
+    if (c->cur) loop_settle(c, true);          // after an odd number of direct steps: start from buffer 0
+    c->cur = 0;
+    if (cudaGraphLaunch(c->gexec[q], c->stream) != cudaSuccess) {
+        cudaGetLastError();
+        c->graph_failed = true;
+        return false;
     }
+    loop_settle(c, false);
+    c->launches += 1 + n;                      // begin and steps; the passes' chains are counted on the device
     return true;
 }
 

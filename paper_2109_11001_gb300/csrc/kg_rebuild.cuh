@@ -15,14 +15,14 @@ __device__ __forceinline__ bool finite64(double v)
     return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
 }
 
-// Monomer s: its position (mixed: build position + displacement since the
+// Monomer s: its position (mixed: build position + displacement dread since the
 // build, folded into the binary64 arrays), its Verlet-grid cell and offset
 // from the cell corner (the build record), the gather records reset to the
 // record, and its rank within its cell (atomic count, aggregated per warp).
 // Returns error bits.
 __device__ __forceinline__ unsigned bin_md_one(const SimDev &S, int s, double *__restrict__ x,
                                                double *__restrict__ xb64, float4 *__restrict__ recb,
-                                               float4 *__restrict__ dcur, float4 *__restrict__ pgcur,
+                                               const float4 *dread, float4 *dcur, float4 *__restrict__ pgcur,
                                                double4_32a *__restrict__ pcur, double4_32a *__restrict__ xb,
                                                int *__restrict__ cellid, int *__restrict__ rank,
                                                int *__restrict__ count, const int *__restrict__ slot_of,
@@ -32,7 +32,7 @@ __device__ __forceinline__ unsigned bin_md_one(const SimDev &S, int s, double *_
     const int Mp = S.Mp;
     double xs[3];
     if (xb64) {                        // mixed: the build position plus the displacement since
-        const float4 e = dcur[s];
+        const float4 e = dread[s];
         xs[0] = __dadd_rn(xb64[s], (double)e.x);
         xs[1] = __dadd_rn(xb64[Mp + s], (double)e.y);
         xs[2] = __dadd_rn(xb64[2 * Mp + s], (double)e.z);

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __
             unsigned err = 0;
             if (live) {
                 A.dlt[cur][s] = make_float4(d.x, d.y, d.z, 0.f);
-                err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.pg[cur], nullptr, nullptr, A.cellid,
+                err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.dlt[cur], A.pg[cur], nullptr, nullptr, A.cellid,
                                  A.rank, A.ccount, P.slot_of);
                 if (err) atomicOr(A.errw, err);
                 else {                                        // one atomic per segment and warp

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, SMALL_MIN_BLOCKS) k_resident_sm
             int *count = A.count[next], cell = 0, rk = 0;
             if (set == 0 && live) {
                 A.dlt[cur][s] = make_float4(d.x, d.y, d.z, 0.f);
-                err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.pg[cur], nullptr, nullptr, A.cellid,
+                err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.dlt[cur], A.pg[cur], nullptr, nullptr, A.cellid,
                                  A.rank, count, P.slot_of, &cell, &rk);
                 if (err) {
                     atomicOr(A.errw, err);

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(TILE, 5) k_resident_tiled(const __grid_constan
         if (rebuild) {                                        // Verlet rebuild; grid-uniform
             for (int s = first + threadIdx.x; s < P.M; s += nthreads) {
                 int cell = 0;
-                const unsigned err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.pg[cur], nullptr, nullptr,
+                const unsigned err = bin_md_one(*A.sim, s, A.x, A.xb64, A.recb, A.dlt[cur], A.dlt[cur], A.pg[cur], nullptr, nullptr,
                                                 A.cellid, A.rank, A.ccount, P.slot_of, &cell);
                 if (err) {
                     atomicOr(A.errw, err);

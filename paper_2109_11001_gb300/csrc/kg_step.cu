@@ -44,15 +44,25 @@ __global__ void __launch_bounds__(256, 8) k_step32(const __grid_constant__ StepA
     __shared__ float dk[96];
     __shared__ unsigned stop;
     step_block_setup(dk);
-    if (threadIdx.x == 0) stop = *(volatile unsigned *)P.flags;    // a latched error stops the run
+    if (threadIdx.x == 0) {
+        unsigned st = *(volatile unsigned *)P.flags;               // a latched error stops the run
+        if (P.loop) {                                              // so do the end of the loop and a rebuild request of
+            const volatile LoopDev *lp = P.loop;                   //   an earlier step of the pass (this one's own bit
+            if (P.k >= lp->n || (lp->req & ((1u << P.k) - 1u))) st = 1u;   //   may already be set by another block)
+        }
+        stop = st;
+    }
     __syncthreads();
     if (stop) return;                                              // block-uniform
-    step_tile<N4, TPM, true>(P, blockIdx.x * blockDim.x, P.dcur, P.dnext, P.pcur, P.pnext, *P.stepp, dk,
+    const long long step = *P.stepp + (P.loop ? 1 + P.k : 0);
+    step_tile<N4, TPM, true>(P, blockIdx.x * blockDim.x, P.dcur, P.dnext, P.pcur, P.pnext, step, dk,
                              // the rebuild vote per warp (no block barrier: a warp with short
                              // lists leaves without waiting for the block's longest)
                              [&](bool rebuild, unsigned err) {
-                                 if (__any_sync(0xffffffffu, rebuild) && (threadIdx.x & 31) == 0)
-                                     atomicOr(P.flags + 1, 1u);
+                                 if (__any_sync(0xffffffffu, rebuild) && (threadIdx.x & 31) == 0) {
+                                     if (P.loop) atomicOr(&P.loop->req, 1u << P.k);
+                                     else atomicOr(P.flags + 1, 1u);
+                                 }
                                  if (err) atomicOr(P.flags, err);
                              });
 }
@@ -119,9 +129,11 @@ StepArgs step_args(const kg_ctx *c, int cur)
     return a;
 }
 
-void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur)
+void step_mixed_launch(kg_ctx *c, cudaStream_t st, int cur, LoopDev *loop, int k)
 {
-    const StepArgs a = step_args(c, cur);
+    StepArgs a = step_args(c, cur);
+    a.loop = loop;
+    a.k = k;
     const int tpm = c->tpm, blk = c->block;
     const long long M = c->M;
     switch (n4_of(c->stage.n)) {

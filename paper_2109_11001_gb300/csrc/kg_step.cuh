@@ -26,7 +26,9 @@ struct StepArgs {
     const int *slot_of;      // compute index -> chain-major slot (keys the noise)
     const int4 *bp;          // compute indices of chain partners s-2, s-1, s+1, s+2 (-1 past an end)
     unsigned *flags;         // [0] error bits, [1] rebuild request
-    const long long *stepp;  // index of the step being run
+    const long long *stepp;  // index of the step being run (in a loop: of the last one before the pass)
+    LoopDev *loop;           // captured step loop (null: none), and the step's place in its body
+    int k;
     unsigned long long seed;
     int M, Mp, n_melts;
     float rc2, half_skin2;

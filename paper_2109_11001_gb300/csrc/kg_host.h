@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <functional>
 #include <vector>
 
 #include "kg.h"
@@ -167,6 +168,9 @@ struct __align__(16) Attempt {
 // kg_md.cu
 void rebuild_md(kg_ctx *c);                  // conditional on flags[1]
 void md_step(kg_ctx *c);                     // one fused force + integrate step (direct launches)
+// captured step loop: its start, and the graph of a while node whose body `pass` enqueues on s
+void loop_begin(cudaStream_t st, LoopDev *lp, long long steps, int len);
+bool capture_loop(cudaStream_t s, cudaGraphExec_t *exec, const std::function<void(cudaGraphConditionalHandle)> &pass);
 bool md_loop_steps(kg_ctx *c, int n);        // n steps in one launch of the captured step loop
 void set_device_step(kg_ctx *c, long long v);
 void forces_eval(kg_ctx *c, int melt, long long step, double *F_dev, double *part_dev, int nblk);

@@ -43,12 +43,32 @@ constexpr int LOOP_MAX = 16;             // steps in the body of a captured step
 
 // State of a captured step loop (kg_md.cu) on the device.
 struct LoopDev {
-    int rem;                 // MD steps still to run
+    long long rem;           // steps still to run
     int n;                   // of them in the present pass of the loop body
     int src;                 // buffer that holds the state when the pass begins (1 only before a list build)
     int par;                 // buffer that holds it after the last pass
     unsigned req;            // bit k: step k of the pass asked for a list rebuild (later ones of the pass are skipped)
 };
+
+// Ends a pass of `len` steps: counts the steps done (those up to the first
+// that asked for a build), passes the request on (flags[1]) and returns true if
+// another pass has to run.  flags[6] counts the pass's kernels other than these
+// steps: six of the build chain, the end kernel, steps that returned at once.
+__device__ __forceinline__ bool loop_finish(LoopDev *lp, int len, long long *stepp, unsigned *flags)
+{
+    const int done = lp->req ? min(lp->n, __ffs((int)lp->req)) : lp->n;
+    stepp[0] += done;
+    const long long rem = lp->rem - done;
+    const bool more = rem > 0 && !flags[0];
+    lp->rem = rem;
+    lp->n = (int)(rem < len ? rem : len);
+    lp->src = done & 1;                        // every pass starts in buffer 0, or with a build that writes it
+    lp->par = more ? 0 : done & 1;
+    flags[1] = lp->req ? 1u : 0u;
+    lp->req = 0u;
+    flags[6] += 7 + len - done;
+    return more;
+}
 
 // status words kept by the resident MD kernel: how the last Verlet build left the
 // cell order (0: clist; 1 + b: buckets with counts b), and the zeroed count buffer

@@ -1005,10 +1005,10 @@ void md_step(kg_ctx *c)
 // Passes start in buffer 0 (a build writes it, and the body's length is even);
 // k_loop_settle moves the result there when the last pass ended in buffer 1.
 // ---------------------------------------------------------------------------
-__global__ void k_loop_begin(LoopDev *lp, int steps, int len)
+__global__ void k_loop_begin(LoopDev *lp, long long steps, int len)
 {
     lp->rem = steps;
-    lp->n = steps < len ? steps : len;
+    lp->n = (int)(steps < len ? steps : len);
     lp->src = lp->par = 0;
     lp->req = 0u;
 }
@@ -1016,19 +1016,11 @@ __global__ void k_loop_begin(LoopDev *lp, int steps, int len)
 __global__ void k_loop_end(LoopDev *lp, int len, long long *__restrict__ stepp, unsigned *__restrict__ flags,
                            cudaGraphConditionalHandle h)
 {
-    const int done = lp->req ? min(lp->n, __ffs((int)lp->req)) : lp->n;
-    stepp[0] += done;
-    const int rem = lp->rem - done;
-    lp->rem = rem;
-    lp->n = rem < len ? rem : len;
-    const bool more = rem > 0 && !flags[0];
-    lp->src = done & 1;                        // every pass starts in buffer 0, or with a build that writes it
-    lp->par = more ? 0 : done & 1;
-    if (lp->req) flags[1] = 1u;
-    lp->req = 0u;
-    flags[6] += 7 + len - done;                // kernels launched in loops, less the steps done (the host counts those)
+    const bool more = loop_finish(lp, len, stepp, flags);
     cudaGraphSetConditional(h, more ? 1u : 0u);
 }
+
+void loop_begin(cudaStream_t st, LoopDev *lp, long long steps, int len) { k_loop_begin<<<1, 1, 0, st>>>(lp, steps, len); }
 
 __global__ void __launch_bounds__(256) k_loop_settle(const LoopDev *__restrict__ lp, bool always,
                                                     float4 *__restrict__ a0, const float4 *__restrict__ a1, int na,
@@ -1039,9 +1031,10 @@ __global__ void __launch_bounds__(256) k_loop_settle(const LoopDev *__restrict__
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) b0[i] = b1[i];
 }
 
-static bool capture_loop(kg_ctx *c, int len, cudaGraphExec_t *exec)
+bool capture_loop(cudaStream_t s, cudaGraphExec_t *exec, const std::function<void(cudaGraphConditionalHandle)> &pass)
 {
     cudaGraph_t g = nullptr;
+    *exec = nullptr;
     if (cudaGraphCreate(&g, 0) != cudaSuccess) return false;
     cudaGraphConditionalHandle h;
     bool ok = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
@@ -1054,13 +1047,11 @@ static bool capture_loop(kg_ctx *c, int len, cudaGraphExec_t *exec)
     ok = ok && cudaGraphAddNode(&cn, g, nullptr, nullptr, 0, &cp) == cudaSuccess;
     if (ok) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
-        ok = cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0,
-                                           cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        ok = cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
+             cudaSuccess;
         if (ok) {
-            launch_rebuild(c, c->cap_stream, 0, c->loop);
-            for (int k = 0; k < len; ++k) launch_step_kernel(c, c->cap_stream, k & 1, c->loop, k);
-            k_loop_end<<<1, 1, 0, c->cap_stream>>>(c->loop, len, c->d_step, c->flags, h);
-            ok = cudaStreamEndCapture(c->cap_stream, &body) == cudaSuccess && cudaGetLastError() == cudaSuccess;
+            pass(h);
+            ok = cudaStreamEndCapture(s, &body) == cudaSuccess && cudaGetLastError() == cudaSuccess;
         }
     }
     ok = ok && cudaGraphInstantiate(exec, g, 0) == cudaSuccess;
@@ -1094,12 +1085,17 @@ bool md_loop_steps(kg_ctx *c, int n)
             c->graph_failed = true;
             return false;
         }
-        if (!capture_loop(c, len, &c->gexec[q])) {
+        const cudaStream_t s = c->cap_stream;
+        if (!capture_loop(s, &c->gexec[q], [&](cudaGraphConditionalHandle h) {
+                launch_rebuild(c, s, 0, c->loop);
+                for (int k = 0; k < len; ++k) launch_step_kernel(c, s, k & 1, c->loop, k);
+                k_loop_end<<<1, 1, 0, s>>>(c->loop, len, c->d_step, c->flags, h);
+            })) {
             c->graph_failed = true;
             return false;
         }
     }
-    k_loop_begin<<<1, 1, 0, c->stream>>>(c->loop, n, len);
+    loop_begin(c->stream, c->loop, n, len);
     if (c->cur) loop_settle(c, true);          // after an odd number of direct steps: start from buffer 0
     c->cur = 0;
     if (cudaGraphLaunch(c->gexec[q], c->stream) != cudaSuccess) {

@@ -30,12 +30,16 @@
 // moved more than skin / 2 since the last build (flag word 1).  Candidates are
 // tested in binary32 on the monomers' offsets from their cells' corners, with
 // a margin that keeps every pair within r_c + skin: the list only has to
-// contain the pairs, so its edge need not be exact.  Steps run as a captured
-// CUDA graph of 25 steps, each step drift, a one-thread kernel that arms a
-// conditional graph node with the build request, the node holding the build
-// kernels, and the force kernel, the scheme of the MD graphs; steps outside
-// whole graphs launch the build kernels directly, which return at once without
-// a request.
+// contain the pairs, so its edge need not be exact.
+//
+// A step is the force at the present positions, the kick that ends the
+// previous velocity Verlet step and the drift that begins the next (no kick in
+// the first, no drift in the last of the n_iter + 1).  They run as the captured
+// step loop of the MD path (kg_md.cu): passes of the list build, which returns
+// at once without a request, and PPA_PASS steps, those after a request left to
+// the next pass.  A contraction rebuilds its list every few steps: 200 steps
+// of 200,000 monomers with 51 builds took 11.5 ms with drift and force apart
+// and a conditional node per step.
 //
 // Two force kernels.  Binary64 (KG_FP64): minimum-image distances and forces
 // in binary64, the same update order as the definition.  Mixed (KG_MIXED), the
@@ -47,7 +51,9 @@
 // position plus d, and every step runs in binary32 (a bond vector is its
 // build value, a binary64 difference rounded to binary32, plus the
 // difference of the two displacements); the build folds d into the binary64
-// position.
+// position.  Force, kick and drift are one kernel there: records and
+// displacements alternate between two buffers from step to step, since
+// neighbours read them while their owner moves on.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -69,8 +75,11 @@ namespace {
 constexpr double PPA_RC = 1.122462048309373;   // 2^(1/6)
 constexpr int PPA_MAXNB = 128;                  // list entries per monomer (overflow: capacity error)
 constexpr int PPA_CELL_CAP = 1024;              // monomers per cell the build accepts
-constexpr int PPA_GRAPH_ITERS = 25;             // steps per captured graph
+constexpr int PPA_PASS = 6;                     // steps per pass of the captured loop (even)
+constexpr int PPA_DIRECT_PASS = 2;              // the same without a graph
+constexpr long long PPA_GRAPH_MIN = 16;         // steps that are worth a capture (~0.2 ms)
 constexpr int PPA_BLOCK = 128;
+constexpr int PPA_ILP = 4;                      // list entries in flight per thread (mixed force)
 constexpr unsigned FIXED_BIT = 0x80000000u;     // record word w: chain index | FIXED_BIT at a chain end
 
 struct PpaArgs {
@@ -80,14 +89,18 @@ struct PpaArgs {
     double half_skin2;           // (skin / 2)^2
     double dt, gamma, k, R0sq;
     float dtf, gammaf, kf, invR0sqf, half_skin2f;
-    // double-buffered per-monomer state (storage order), buffer flags[3] in use
+    long long n_iter;
+    // per-monomer state in storage order, moved from buffer to buffer by a build; buffer flags[3] in use
     double *x0, *x1;             // (3, M) positions (mixed: positions at the last build)
-    double *v0, *v1, *F0, *F1;   // (3, M) velocities and forces, binary64 mode
-    float *u0, *u1, *G0, *G1;    // (3, M) velocities and forces, mixed mode
+    double *v0, *v1;             // (3, M) velocities, binary64 mode
+    float *u0, *u1;              // (3, M) velocities, mixed mode
     int *slot0, *slot1;          // storage index -> slot
     // single-buffered, rewritten at each build (storage order of the new buffer)
     double *xb;                  // positions at the build (binary64 mode)
-    float4 *rec, *pg, *dl;       // build offset + (chain | FIXED_BIT); offset + d; d
+    double *F;                   // (3, M) forces of the step, binary64 mode
+    float *G;                    // (3, M) forces of the last step, mixed mode
+    float4 *rec;                 // build offset + (chain | FIXED_BIT)
+    float4 *pg[2], *dl[2];       // mixed: offset + d; d (buffers alternate between steps)
     float4 *off;                 // bin output in the old order: offset + cell index
     float4 *bvec;                // mixed: bond vector to the next monomer at the build
     int2 *bp;                    // storage indices of the bonded partners (-1 past an end)
@@ -95,10 +108,14 @@ struct PpaArgs {
     int *cellof;                 // packed cell coordinates of each storage index
     int *rank, *count, *start, *list, *nn;
     unsigned *nl;                // entries j | q << IDX_BITS, column-major
-    unsigned *flags;             // [0] error bits, [1] rebuild request, [2] builds, [3] buffer in use
+    unsigned *flags;             // [0] error bits, [1] rebuild request, [2] builds, [3] buffer in use, [6] launches
+    LoopDev *loop;
+    long long *steps;            // steps completed before the present pass
 };
 
 __device__ __forceinline__ int cur_buf(const PpaArgs &a) { return (int)(a.flags[3] & 1u); }
+// the buffer of the steps of a pass: a build requested before it has moved the arrays to the other one
+__device__ __forceinline__ int step_buf(const PpaArgs &a) { return (int)((a.flags[3] ^ a.flags[1]) & 1u); }
 __device__ __forceinline__ bool build_requested(const PpaArgs &a) { return a.flags[1] && !a.flags[0]; }
 
 __device__ __forceinline__ double min_image(double d, const PpaArgs &a)
@@ -106,32 +123,39 @@ __device__ __forceinline__ double min_image(double d, const PpaArgs &a)
     return __dsub_rn(d, __dmul_rn(a.L, rint(__dmul_rn(d, a.invL))));
 }
 
-// image shift q h of stencil code q = (dz + 1) 9 + (dy + 1) 3 + (dx + 1)
-__device__ __forceinline__ float3 stencil_shift(unsigned q, float h)
+// the stop test of a step kernel, one thread's answer for the block: a latched
+// error, the end of the loop, or an earlier step of the pass that asked for a
+// build (this step's own bit may already be set)
+__device__ __forceinline__ bool step_off(const PpaArgs &a, int k)
 {
-    const int dx = (int)(q % 3u) - 1, dy = (int)((q / 3u) % 3u) - 1, dz = (int)(q / 9u) - 1;
-    return make_float3((float)dx * h, (float)dy * h, (float)dz * h);
+    __shared__ unsigned off;
+    if (threadIdx.x == 0) {
+        const volatile LoopDev *lp = a.loop;
+        off = *(volatile unsigned *)a.flags | (unsigned)(k >= lp->n) | (lp->req & ((1u << k) - 1u));
+    }
+    __syncthreads();
+    return off != 0u;
 }
 
 __device__ __forceinline__ bool is_fixed(const float4 &r) { return (__float_as_uint(r.w) & FIXED_BIT) != 0u; }
 
-// ---- one step: drift, (conditional) build, force ----
+// ---- one step: force and kick, drift ----
 
-// first half kick and drift of the mobile monomers:
+// binary64: first half kick and drift of the mobile monomers:
 // v <- v + (dt/2) F; x <- x + dt v; request a rebuild past skin / 2
-__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_drift_f64(PpaArgs a)
+__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_drift_f64(PpaArgs a, int k)
 {
+    if (step_off(a, k) || *a.steps + k == a.n_iter) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.M || is_fixed(a.rec[p])) return;
-    const int cb = cur_buf(a);
+    const int cb = step_buf(a);
     double *x = cb ? a.x1 : a.x0, *v = cb ? a.v1 : a.v0;
-    const double *F = cb ? a.F1 : a.F0;
     const double hdt = 0.5 * a.dt;
     double dr2 = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const size_t o = (size_t)d * a.M + p;
-        const double vh = __dadd_rn(v[o], __dmul_rn(hdt, F[o]));
+        const double vh = __dadd_rn(v[o], __dmul_rn(hdt, a.F[o]));
         const double xn = __dadd_rn(x[o], __dmul_rn(a.dt, vh));
         v[o] = vh;
         x[o] = xn;
@@ -140,37 +164,7 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_drift_f64(PpaArgs a)
     }
     if (!(dr2 <= a.half_skin2)) {
         if (!isfinite(dr2)) atomicOr(a.flags, ERR_NONFINITE);
-        atomicOr(a.flags + 1, 1u);
-    }
-}
-
-// mixed: the same step with binary32 v and F; the drift goes into the
-// binary32 displacement d since the build, and the gather record becomes o + d
-__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_drift_mixed(PpaArgs a)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.M) return;
-    const float4 r = a.rec[p];
-    if (is_fixed(r)) return;
-    const int cb = cur_buf(a);
-    float *u = cb ? a.u1 : a.u0;
-    const float *G = cb ? a.G1 : a.G0;
-    const float hdt = 0.5f * a.dtf;
-    const float4 d0 = a.dl[p];
-    float dd[3] = {d0.x, d0.y, d0.z};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const size_t o = (size_t)d * a.M + p;
-        const float vh = u[o] + hdt * G[o];
-        u[o] = vh;
-        dd[d] += a.dtf * vh;
-    }
-    a.dl[p] = make_float4(dd[0], dd[1], dd[2], 0.f);
-    a.pg[p] = make_float4(r.x + dd[0], r.y + dd[1], r.z + dd[2], r.w);
-    const float dr2 = dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2];
-    if (!(dr2 <= a.half_skin2f)) {
-        if (!isfinite(dr2)) atomicOr(a.flags, ERR_NONFINITE);
-        atomicOr(a.flags + 1, 1u);
+        atomicOr(&a.loop->req, 1u << k);
     }
 }
 
@@ -184,7 +178,7 @@ __global__ void __launch_bounds__(256) k_ppa_bin(PpaArgs a)
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.M) return;
     double *x = cur_buf(a) ? a.x1 : a.x0;
-    const float4 dp = a.u0 ? a.dl[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 dp = a.u0 ? a.dl[a.loop->src][p] : make_float4(0.f, 0.f, 0.f, 0.f);
     const float dd[3] = {dp.x, dp.y, dp.z};
     int cc[3];
     float o[3];
@@ -199,52 +193,46 @@ __global__ void __launch_bounds__(256) k_ppa_bin(PpaArgs a)
     }
     const int c = (cc[2] * a.nc + cc[1]) * a.nc + cc[0];
     a.off[p] = make_float4(o[0], o[1], o[2], __int_as_float(c));
-    a.rank[p] = atomicAdd(a.count + c, 1);
+    // one atomic per cell and warp: neighbours in storage order share cells
+    const unsigned act = __activemask(), grp = __match_any_sync(act, c);
+    const int lane = threadIdx.x & 31, leader = __ffs(grp) - 1;
+    int base = 0;
+    if (lane == leader) base = atomicAdd(a.count + c, __popc(grp));
+    base = __shfl_sync(grp, base, leader);
+    a.rank[p] = base + __popc(grp & ((1u << lane) - 1u));
 }
 
-// build 2: the current storage indices in cell order
+// build 2: the current storage indices by cell, in no fixed order within one;
+// clear the counts for the next build
 __global__ void __launch_bounds__(256) k_ppa_scatter(PpaArgs a)
 {
     if (!build_requested(a)) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int c = p; c < a.ncell; c += gridDim.x * blockDim.x) {
+        if (a.count[c] > PPA_CELL_CAP) atomicOr(a.flags, ERR_NL_CAPACITY);
+        a.count[c] = 0;
+    }
     if (p >= a.M) return;
     a.list[a.start[__float_as_int(a.off[p].w)] + a.rank[p]] = p;
 }
 
-// build 3: each cell's run ordered by current storage index (deterministic);
-// clear the counts for the next build
-__global__ void __launch_bounds__(256) k_ppa_cellsort(PpaArgs a)
-{
-    if (!build_requested(a)) return;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= a.ncell) return;
-    const int b0 = a.start[c], b1 = a.start[c + 1];
-    a.count[c] = 0;
-    if (b1 - b0 > PPA_CELL_CAP) {
-        atomicOr(a.flags, ERR_NL_CAPACITY);
-        return;
-    }
-    for (int k = b0 + 1; k < b1; ++k) {
-        const int v = a.list[k];
-        int j = k - 1;
-        while (j >= b0 && a.list[j] > v) {
-            a.list[j + 1] = a.list[j];
-            --j;
-        }
-        a.list[j + 1] = v;
-    }
-}
-
-// build 4: move every per-monomer array into cell order (the other buffer);
-// the records, displacement, build positions and slot -> storage map
+// build 3: move every per-monomer array into cell order (the other buffer),
+// a cell's run ordered by present storage index (deterministic): the new index
+// is the cell's start plus the number of its members with a lower one; the
+// records, displacement, build positions and slot -> storage map
 __global__ void __launch_bounds__(256) k_ppa_permute(PpaArgs a)
 {
     if (!build_requested(a)) return;
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= a.M) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= a.M) return;
     const int cb = cur_buf(a);
-    const int p = a.list[q];
+    const int p = a.list[t];
     const size_t M = a.M;
+    const float4 o = a.off[p];
+    const int c = __float_as_int(o.w);
+    const int b0 = a.start[c], b1 = a.start[c + 1];
+    int q = b0;
+    for (int k = b0; k < b1; ++k) q += a.list[k] < p;
     const double *xs = cb ? a.x1 : a.x0;
     double *xd = cb ? a.x0 : a.x1;
 #pragma unroll
@@ -254,50 +242,35 @@ __global__ void __launch_bounds__(256) k_ppa_permute(PpaArgs a)
         if (a.xb) a.xb[d * M + q] = xv;
     }
     if (a.u0) {
-        const float *us = cb ? a.u1 : a.u0, *Gs = cb ? a.G1 : a.G0;
-        float *ud = cb ? a.u0 : a.u1, *Gd = cb ? a.G0 : a.G1;
+        const float *us = cb ? a.u1 : a.u0;
+        float *ud = cb ? a.u0 : a.u1;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            ud[d * M + q] = us[d * M + p];
-            Gd[d * M + q] = Gs[d * M + p];
-        }
+        for (int d = 0; d < 3; ++d) ud[d * M + q] = us[d * M + p];
     } else {
-        const double *vs = cb ? a.v1 : a.v0, *Fs = cb ? a.F1 : a.F0;
-        double *vd = cb ? a.v0 : a.v1, *Fd = cb ? a.F0 : a.F1;
+        const double *vs = cb ? a.v1 : a.v0;
+        double *vd = cb ? a.v0 : a.v1;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            vd[d * M + q] = vs[d * M + p];
-            Fd[d * M + q] = Fs[d * M + p];
-        }
+        for (int d = 0; d < 3; ++d) vd[d * M + q] = vs[d * M + p];
     }
     const int s = (cb ? a.slot1 : a.slot0)[p];
     (cb ? a.slot0 : a.slot1)[q] = s;
     a.pos_of[s] = q;
     const int i = s % a.N;
     const unsigned w = (unsigned)(s / a.N) | ((i == 0 || i == a.N - 1) ? FIXED_BIT : 0u);
-    const float4 o = a.off[p];
     const float4 r = make_float4(o.x, o.y, o.z, __uint_as_float(w));
     a.rec[q] = r;
-    a.pg[q] = r;
-    a.dl[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int c = __float_as_int(o.w);
+    if (a.u0) {
+        a.pg[0][q] = r;
+        a.dl[0][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     a.cellof[q] = (int)pack_code(c % a.nc, (c / a.nc) % a.nc, c / (a.nc * a.nc));
 }
 
-// build 5 (one thread): the new buffer becomes the one in use
-__global__ void k_ppa_flip(PpaArgs a)
+// storage indices of monomer p's bonded partners; mixed: the bond vector to
+// the next monomer (binary64 difference rounded to binary32); cb: the buffer
+// that the permutation wrote
+__device__ __forceinline__ void partners_one(const PpaArgs &a, int p, int cb)
 {
-    if (build_requested(a)) a.flags[3] ^= 1u;
-}
-
-// build 6: storage indices of each monomer's bonded partners; mixed: the
-// bond vector to the next monomer (binary64 difference rounded to binary32)
-__global__ void __launch_bounds__(256) k_ppa_partners(PpaArgs a)
-{
-    if (!build_requested(a)) return;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.M) return;
-    const int cb = cur_buf(a);
     const int s = (cb ? a.slot1 : a.slot0)[p];
     const int i = s % a.N;
     const int2 b = make_int2(i > 0 ? a.pos_of[s - 1] : -1, i < a.N - 1 ? a.pos_of[s + 1] : -1);
@@ -310,15 +283,20 @@ __global__ void __launch_bounds__(256) k_ppa_partners(PpaArgs a)
     }
 }
 
-// build 7: interchain Verlet list of monomer p from the binary32 build
-// offsets: every t of another chain in the 27 cells around p whose vector
-// o_t - o_p + q h is shorter than r_c + skin (plus a margin above the offsets'
-// rounding)
+// build 4: bonded partners and the interchain Verlet list of monomer p from
+// the binary32 build offsets: every t of another chain in the 27 cells around
+// p whose vector o_t - o_p + q h is shorter than r_c + skin (plus a margin
+// above the offsets' rounding).  The three cells of a row in x are walked as
+// one run, four candidates in flight: the lanes of a warp diverge at the ends
+// of 9 runs of ~12 instead of 27 of ~4.  The thread of monomer 0 counts the
+// build; the loop's end kernel makes the new buffer the one in use.
 __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_nlist(PpaArgs a)
 {
     if (!build_requested(a)) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.M) return;
+    if (p == 0) a.flags[2] += 1u;
+    partners_one(a, p, cur_buf(a) ^ 1);
     const float4 rp = a.rec[p];
     const unsigned chain = __float_as_uint(rp.w) & ~FIXED_BIT;
     const unsigned code = (unsigned)a.cellof[p];
@@ -326,24 +304,36 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_nlist(PpaArgs a)
               cz = (int)(code >> (2 * CODE_BITS));
     const int nc = a.nc;
     auto wrap = [nc](int v) { return v < 0 ? v + nc : (v >= nc ? v - nc : v); };
+    const int xl = wrap(cx - 1), xr = wrap(cx + 1);
     int n = 0;
-    unsigned q = 0;
-    for (int dz = -1; dz <= 1; ++dz) {
-        const int z = wrap(cz + dz);
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int zy = (z * nc + wrap(cy + dy)) * nc;
-            for (int dx = -1; dx <= 1; ++dx, ++q) {
-                const int cn = zy + wrap(cx + dx);
-                const float sx = (float)dx * a.hf - rp.x, sy = (float)dy * a.hf - rp.y, sz = (float)dz * a.hf - rp.z;
-                const int j1 = __ldg(a.start + cn + 1);
-                for (int j = __ldg(a.start + cn); j < j1; ++j) {
-                    const float4 rj = __ldg(a.rec + j);
-                    if ((__float_as_uint(rj.w) & ~FIXED_BIT) == chain) continue;
-                    const float ex = rj.x + sx, ey = rj.y + sy, ez = rj.z + sz;
-                    if (ex * ex + ey * ey + ez * ez < a.rl2f) {
-                        if (n < PPA_MAXNB) a.nl[(size_t)n * a.M + p] = (unsigned)j | (q << IDX_BITS);
-                        ++n;
-                    }
+    for (int r = 0; r < 9; ++r) {
+        const int dz = r / 3 - 1, dy = r % 3 - 1;
+        const int zy = (wrap(cz + dz) * nc + wrap(cy + dy)) * nc;
+        const float sy = (float)dy * a.hf - rp.y, sz = (float)dz * a.hf - rp.z;
+        // the row's cells left, centre, right as one run of candidates
+        const int b0 = __ldg(a.start + zy + xl), b1 = __ldg(a.start + zy + cx), b2 = __ldg(a.start + zy + xr);
+        const int n0 = __ldg(a.start + zy + xl + 1) - b0;
+        const int n1 = n0 + __ldg(a.start + zy + cx + 1) - b1;
+        const int n2 = n1 + __ldg(a.start + zy + xr + 1) - b2;
+        for (int k = 0; k < n2; k += 4) {
+            float4 rj[4];
+            int j[4];
+            int dx[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int t = min(k + i, n2 - 1);
+                j[i] = t < n0 ? b0 + t : t < n1 ? b1 + (t - n0) : b2 + (t - n1);
+                dx[i] = t < n0 ? -1 : t < n1 ? 0 : 1;
+                rj[i] = __ldg(a.rec + j[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float sx = (float)dx[i] * a.hf - rp.x;
+                const float ex = rj[i].x + sx, ey = rj[i].y + sy, ez = rj[i].z + sz;
+                if (k + i < n2 && (__float_as_uint(rj[i].w) & ~FIXED_BIT) != chain &&
+                    ex * ex + ey * ey + ez * ez < a.rl2f) {
+                    if (n < PPA_MAXNB) a.nl[(size_t)n * a.M + p] = (unsigned)j[i] | ((unsigned)(3 * r + 1 + dx[i]) << IDX_BITS);
+                    ++n;
                 }
             }
         }
@@ -355,33 +345,23 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_nlist(PpaArgs a)
     a.nn[p] = n;
 }
 
-// the thread of monomer 0 retires the build request of this step (every build
-// kernel has run) and counts the build
-__device__ __forceinline__ void retire_build(const PpaArgs &a, int p)
-{
-    if (p == 0 && a.flags[1]) {
-        if (!a.flags[0]) a.flags[2] += 1u;
-        a.flags[1] = 0u;
-    }
-}
-
 // binary64 force: minimum-image pair vectors, LJ 12-6 between chains, FENE
 // bonds; F <- F_c(x) - gamma v; v <- v + half dt F (half = 0 for the first force)
-__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_f64(PpaArgs a, double half)
+__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_f64(PpaArgs a, int k)
 {
+    if (step_off(a, k)) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    retire_build(a, p);
     if (p >= a.M || is_fixed(a.rec[p])) return;
-    const int cb = cur_buf(a);
+    const int cb = step_buf(a);
     const double *x = cb ? a.x1 : a.x0;
-    double *v = cb ? a.v1 : a.v0, *F = cb ? a.F1 : a.F0;
+    double *v = cb ? a.v1 : a.v0, *F = a.F;
     const size_t M = a.M;
     const double xs = x[p], ys = x[M + p], zs = x[2 * M + p];
     double fx = 0.0, fy = 0.0, fz = 0.0;
     const int n = a.nn[p];
     const double rc2 = PPA_RC * PPA_RC;
-    for (int k = 0; k < n; ++k) {
-        const int j = (int)(a.nl[(size_t)k * M + p] & IDX_MASK);
+    for (int i = 0; i < n; ++i) {
+        const int j = (int)(a.nl[(size_t)i * M + p] & IDX_MASK);
         const double ex = min_image(__dsub_rn(x[j], xs), a);
         const double ey = min_image(__dsub_rn(x[M + j], ys), a);
         const double ez = min_image(__dsub_rn(x[2 * M + j], zs), a);
@@ -410,7 +390,7 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_f64(PpaArgs a, double h
         fy += gb * by;
         fz += gb * bz;
     }
-    const double hdt = half * a.dt;
+    const double hdt = (*a.steps + k ? 0.5 : 0.0) * a.dt;
     const double f[3] = {fx, fy, fz};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -422,42 +402,64 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_f64(PpaArgs a, double h
     }
 }
 
-// mixed force, all binary32: pair vectors from the gather records, LJ 12-6;
-// bond vectors from the build's bond vectors and the displacements; FENE,
-// friction and kick
-__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_mixed(PpaArgs a, float half)
+// One step of the mixed path, all binary32.  Pair vectors from the gather
+// records, LJ 12-6; bond vectors from the build's bond vectors and the
+// displacements; FENE, friction, the kick, and the next step's half kick and
+// drift into the displacement since the build; a build request past skin / 2.
+// Bound by the latency of the list and record gathers: PPA_ILP entries are in
+// flight per thread, and the image shifts come from a word table in shared
+// memory (27 words in 27 banks).
+__global__ void __launch_bounds__(PPA_BLOCK) k_ppa_step_mixed(PpaArgs a, int k)
 {
+    __shared__ float sh[96];
+    for (int q = threadIdx.x; q < 96; q += PPA_BLOCK) {
+        const int i = q & 31, c = i < 27 ? (q < 32 ? i % 3 : q < 64 ? (i / 3) % 3 : i / 9) - 1 : 0;
+        sh[q] = (float)c * a.hf;
+    }
+    if (step_off(a, k)) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    retire_build(a, p);
     if (p >= a.M) return;
-    const float4 ps = a.pg[p];
-    if (is_fixed(ps)) return;
-    const int cb = cur_buf(a);
-    float *u = cb ? a.u1 : a.u0, *G = cb ? a.G1 : a.G0;
+    const float4 *__restrict__ pg = a.pg[k & 1], *__restrict__ dl = a.dl[k & 1];
+    const long long step = *a.steps + k;
+    const float4 ps = pg[p];
+    if (is_fixed(ps)) {
+        a.pg[~k & 1][p] = ps;
+        a.dl[~k & 1][p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
+    float *u = step_buf(a) ? a.u1 : a.u0;
     const size_t M = a.M;
     float fx = 0.f, fy = 0.f, fz = 0.f;
     const int n = a.nn[p];
-    for (int k = 0; k < n; ++k) {
-        const unsigned e = __ldg(a.nl + (size_t)k * M + p);
-        const float4 pj = __ldg(a.pg + (e & IDX_MASK));
-        const float3 sh = stencil_shift(e >> IDX_BITS, a.hf);
-        const float ex = (pj.x - ps.x) + sh.x, ey = (pj.y - ps.y) + sh.y, ez = (pj.z - ps.z) + sh.z;
-        const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < a.rc2f) {
-            const float ir2 = __frcp_rn(r2);
-            const float ir6 = ir2 * ir2 * ir2;
-            const float g = (48.f * ir6 * ir6 - 24.f * ir6) * ir2;   // -U'(r)/r, U = 4(r^-12 - r^-6) + 1
-            fx -= g * ex;
-            fy -= g * ey;
-            fz -= g * ez;
+    for (int i0 = 0; i0 < n; i0 += PPA_ILP) {
+        unsigned e[PPA_ILP];
+        float4 pj[PPA_ILP];
+#pragma unroll
+        for (int i = 0; i < PPA_ILP; ++i) e[i] = i0 + i < n ? __ldg(a.nl + (size_t)(i0 + i) * M + p) : (unsigned)p;
+#pragma unroll
+        for (int i = 0; i < PPA_ILP; ++i) pj[i] = __ldg(pg + (e[i] & IDX_MASK));
+#pragma unroll
+        for (int i = 0; i < PPA_ILP; ++i) {
+            const unsigned q = e[i] >> IDX_BITS;
+            const float ex = (pj[i].x - ps.x) + sh[q], ey = (pj[i].y - ps.y) + sh[32 + q],
+                        ez = (pj[i].z - ps.z) + sh[64 + q];
+            const float r2 = ex * ex + ey * ey + ez * ez;
+            if (r2 < a.rc2f && i0 + i < n) {
+                const float ir2 = __frcp_rn(r2);
+                const float ir6 = ir2 * ir2 * ir2;
+                const float g = (48.f * ir6 * ir6 - 24.f * ir6) * ir2;   // -U'(r)/r, U = 4(r^-12 - r^-6) + 1
+                fx -= g * ex;
+                fy -= g * ey;
+                fz -= g * ez;
+            }
         }
     }
     const int2 b = a.bp[p];
-    const float4 dp = a.dl[p];
+    const float4 dp = dl[p];
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
         const int t = side ? b.y : b.x;
-        const float4 dt_ = __ldg(a.dl + t);
+        const float4 dt_ = __ldg(dl + t);
         const float4 bv = __ldg(a.bvec + (side ? p : t));
         const float sg = side ? 1.f : -1.f;             // the previous bond is -(its bond to p)
         const float bx = sg * bv.x + (dt_.x - dp.x), by = sg * bv.y + (dt_.y - dp.y),
@@ -472,15 +474,32 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_mixed(PpaArgs a, float 
         fy += gb * by;
         fz += gb * bz;
     }
-    const float hdt = half * a.dtf;
+    const float hdt = (step ? 0.5f : 0.f) * a.dtf, hdt2 = 0.5f * a.dtf;
     const float f[3] = {fx, fy, fz};
+    const bool last = step == a.n_iter;
+    float dd[3] = {dp.x, dp.y, dp.z};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const size_t o = (size_t)d * M + p;
         const float vh = u[o];
         const float Ft = f[d] - a.gammaf * vh;
-        G[o] = Ft;
-        u[o] = vh + hdt * Ft;
+        float un = vh + hdt * Ft;
+        if (last) {
+            a.G[o] = Ft;
+        } else {
+            un = un + hdt2 * Ft;
+            dd[d] += a.dtf * un;
+        }
+        u[o] = un;
+    }
+    a.dl[~k & 1][p] = make_float4(dd[0], dd[1], dd[2], 0.f);
+    if (last) return;
+    const float4 r = a.rec[p];
+    a.pg[~k & 1][p] = make_float4(r.x + dd[0], r.y + dd[1], r.z + dd[2], r.w);
+    const float dr2 = dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2];
+    if (!(dr2 <= a.half_skin2f)) {
+        if (!isfinite(dr2)) atomicOr(a.flags, ERR_NONFINITE);
+        atomicOr(&a.loop->req, 1u << k);
     }
 }
 
@@ -493,13 +512,13 @@ __device__ __forceinline__ unsigned long long unpermute_one(const PpaArgs &a, in
     const double *x = cb ? a.x1 : a.x0;
     const size_t M = a.M;
     const int p = a.pos_of[s];
-    const float4 dp = a.u0 ? a.dl[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 dp = a.u0 ? a.dl[a.loop->par][p] : make_float4(0.f, 0.f, 0.f, 0.f);
     const float dd[3] = {dp.x, dp.y, dp.z};
     double f2 = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         xs[d * M + s] = x[d * M + p] + (double)dd[d];
-        const double f = a.u0 ? (double)(cb ? a.G1 : a.G0)[d * M + p] : (cb ? a.F1 : a.F0)[d * M + p];
+        const double f = a.u0 ? (double)a.G[d * M + p] : a.F[d * M + p];
         f2 += f * f;
     }
     const int i = s % a.N;
@@ -560,100 +579,35 @@ __global__ void k_ppa_iota(int *__restrict__ a, int n)
 
 inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 
-constexpr int PPA_BUILD_LAUNCHES = 9;        // kernels of one list build
-constexpr int PPA_LAUNCHES_PER_ITER = 2 + PPA_BUILD_LAUNCHES;   // direct launches of one step
-
-// the list build (each kernel returns at once unless a build is requested)
-void enqueue_build(const PpaArgs &a, cudaStream_t st, int *bsum)
+// ends a pass: the buffer that a build wrote becomes the one in use
+__global__ void k_ppa_end(PpaArgs a, int len, cudaGraphConditionalHandle h, int in_graph)
 {
-    const int nbs = nblk(a.ncell, 1024);
+    a.flags[3] ^= a.flags[1];
+    const bool more = loop_finish(a.loop, len, a.steps, a.flags);
+    if (in_graph) cudaGraphSetConditional(h, more ? 1u : 0u);
+}
+
+// one pass: the list build (each kernel returns at once unless a build is
+// requested), `len` steps, the end kernel (h: the loop's condition in a graph)
+void enqueue_pass(const PpaArgs &a, cudaStream_t st, int *bsum, bool mixed, int len, cudaGraphConditionalHandle h,
+                  bool in_graph)
+{
+    const int nbs = nblk(a.ncell, 1024), nbm = nblk(a.M, PPA_BLOCK);
     k_ppa_bin<<<nblk(a.M, 256), 256, 0, st>>>(a);
     k_scan1<<<nbs, 1024, 0, st>>>(a.count, a.start, bsum, a.ncell, a.flags);
     k_scan2<<<nbs, 1024, 0, st>>>(a.start, bsum, a.ncell, nbs, a.flags);
     k_ppa_scatter<<<nblk(a.M, 256), 256, 0, st>>>(a);
-    k_ppa_cellsort<<<nblk(a.ncell, 256), 256, 0, st>>>(a);
     k_ppa_permute<<<nblk(a.M, 256), 256, 0, st>>>(a);
-    k_ppa_flip<<<1, 1, 0, st>>>(a);
-    k_ppa_partners<<<nblk(a.M, 256), 256, 0, st>>>(a);
-    k_ppa_nlist<<<nblk(a.M, PPA_BLOCK), PPA_BLOCK, 0, st>>>(a);
-}
-
-void enqueue_drift(const PpaArgs &a, cudaStream_t st, bool mixed)
-{
-    const int nbm = nblk(a.M, PPA_BLOCK);
-    if (mixed) k_ppa_drift_mixed<<<nbm, PPA_BLOCK, 0, st>>>(a);
-    else k_ppa_drift_f64<<<nbm, PPA_BLOCK, 0, st>>>(a);
-}
-
-void enqueue_force(const PpaArgs &a, cudaStream_t st, bool mixed, double half)
-{
-    const int nbm = nblk(a.M, PPA_BLOCK);
-    if (mixed) k_ppa_force_mixed<<<nbm, PPA_BLOCK, 0, st>>>(a, (float)half);
-    else k_ppa_force_f64<<<nbm, PPA_BLOCK, 0, st>>>(a, half);
-}
-
-void enqueue_step(const PpaArgs &a, cudaStream_t st, int *bsum, bool mixed)
-{
-    enqueue_drift(a, st, mixed);
-    enqueue_build(a, st, bsum);
-    enqueue_force(a, st, mixed, 0.5);
-}
-
-// arms the conditional build node of a captured step with the build request
-__global__ void k_ppa_arm(const unsigned *__restrict__ flags, cudaGraphConditionalHandle h)
-{
-    cudaGraphSetConditional(h, (flags[1] && !flags[0]) ? 1u : 0u);
-}
-
-// A graph of PPA_GRAPH_ITERS steps: drift, the arm kernel, a conditional node
-// holding the list build (run only when a monomer has left its skin), force.
-bool capture_steps(const PpaArgs &a, cudaStream_t s1, cudaStream_t s2, int *bsum, bool mixed,
-                   cudaGraphExec_t *out)
-{
-    cudaGraph_t g = nullptr;
-    if (cudaGraphCreate(&g, 0) != cudaSuccess) return false;
-    bool ok = cudaStreamBeginCaptureToGraph(s1, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
-              cudaSuccess;
-    for (int i = 0; ok && i < PPA_GRAPH_ITERS; ++i) {
-        enqueue_drift(a, s1, mixed);
-        cudaGraphConditionalHandle h;
-        ok = cudaGraphConditionalHandleCreate(&h, g, 0, 0) == cudaSuccess;
-        if (!ok) break;
-        k_ppa_arm<<<1, 1, 0, s1>>>(a.flags, h);
-        cudaStreamCaptureStatus cs;
-        cudaGraph_t cg = nullptr;
-        const cudaGraphNode_t *deps = nullptr;
-        size_t nd = 0;
-        ok = cudaStreamGetCaptureInfo(s1, &cs, nullptr, &cg, &deps, nullptr, &nd) == cudaSuccess;
-        if (!ok) break;
-        cudaGraphNodeParams cp{};
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeIf;
-        cp.conditional.size = 1;
-        cudaGraphNode_t cn;
-        ok = cudaGraphAddNode(&cn, cg, deps, nullptr, nd, &cp) == cudaSuccess &&
-             cudaStreamUpdateCaptureDependencies(s1, &cn, nullptr, 1, cudaStreamSetCaptureDependencies) ==
-                 cudaSuccess;
-        if (!ok) break;
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        ok = cudaStreamBeginCaptureToGraph(s2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
-             cudaSuccess;
-        if (!ok) break;
-        enqueue_build(a, s2, bsum);
-        ok = cudaStreamEndCapture(s2, &body) == cudaSuccess;
-        if (!ok) break;
-        enqueue_force(a, s1, mixed, 0.5);
+    k_ppa_nlist<<<nbm, PPA_BLOCK, 0, st>>>(a);
+    for (int k = 0; k < len; ++k) {
+        if (mixed) {
+            k_ppa_step_mixed<<<nbm, PPA_BLOCK, 0, st>>>(a, k);
+        } else {
+            k_ppa_force_f64<<<nbm, PPA_BLOCK, 0, st>>>(a, k);
+            k_ppa_drift_f64<<<nbm, PPA_BLOCK, 0, st>>>(a, k);
+        }
     }
-    cudaGraph_t g_out = nullptr;
-    const bool ended = cudaStreamEndCapture(s1, &g_out) == cudaSuccess;
-    ok = ok && ended && cudaGetLastError() == cudaSuccess && cudaGraphInstantiate(out, g, 0) == cudaSuccess;
-    cudaGraphDestroy(g);
-    if (!ok) {
-        cudaGetLastError();
-        *out = nullptr;
-    }
-    return ok;
+    k_ppa_end<<<1, 1, 0, st>>>(a, len, h, in_graph);
 }
 
 // Eq. 22's left-hand side (2 x + exp(-2 x) - 1) / (2 x^2); a series below
@@ -709,6 +663,7 @@ kg_status kg_primitive_path(kg_ctx *c, int melt, const kg_ppa_params *pp, double
     a.kf = (float)k;
     a.invR0sqf = (float)(1.0 / a.R0sq);
     a.half_skin2f = (float)a.half_skin2;
+    a.n_iter = pp->n_iter;
 
     const size_t m3 = 3 * (size_t)M;
     const int nbs = nblk(a.ncell, 1024);
@@ -723,22 +678,24 @@ kg_status kg_primitive_path(kg_ctx *c, int melt, const kg_ppa_params *pp, double
     if (mixed) {
         a.u0 = (float *)get(sizeof(float) * m3);
         a.u1 = (float *)get(sizeof(float) * m3);
-        a.G0 = (float *)get(sizeof(float) * m3);
-        a.G1 = (float *)get(sizeof(float) * m3);
+        a.G = (float *)get(sizeof(float) * m3);
     } else {
         a.v0 = (double *)get(sizeof(double) * m3);
         a.v1 = (double *)get(sizeof(double) * m3);
-        a.F0 = (double *)get(sizeof(double) * m3);
-        a.F1 = (double *)get(sizeof(double) * m3);
+        a.F = (double *)get(sizeof(double) * m3);
         a.xb = (double *)get(sizeof(double) * m3);
     }
     a.slot0 = (int *)get(sizeof(int) * M);
     a.slot1 = (int *)get(sizeof(int) * M);
     a.rec = (float4 *)get(sizeof(float4) * M);
-    a.pg = (float4 *)get(sizeof(float4) * M);
-    a.dl = (float4 *)get(sizeof(float4) * M);
     a.off = (float4 *)get(sizeof(float4) * M);
-    if (mixed) a.bvec = (float4 *)get(sizeof(float4) * M);
+    if (mixed) {
+        a.bvec = (float4 *)get(sizeof(float4) * M);
+        for (int b = 0; b < 2; ++b) {
+            a.pg[b] = (float4 *)get(sizeof(float4) * M);
+            a.dl[b] = (float4 *)get(sizeof(float4) * M);
+        }
+    }
     a.bp = (int2 *)get(sizeof(int2) * M);
     a.pos_of = (int *)get(sizeof(int) * M);
     a.cellof = (int *)get(sizeof(int) * M);
@@ -748,17 +705,18 @@ kg_status kg_primitive_path(kg_ctx *c, int melt, const kg_ppa_params *pp, double
     a.list = (int *)get(sizeof(int) * M);
     a.nl = (unsigned *)get(sizeof(unsigned) * (size_t)PPA_MAXNB * M);
     a.nn = (int *)get(sizeof(int) * M);
-    a.flags = (unsigned *)get(sizeof(unsigned) * 4);
+    a.flags = (unsigned *)get(sizeof(unsigned) * 8);
+    a.loop = (LoopDev *)get(sizeof(LoopDev));
+    a.steps = (long long *)get(sizeof(long long));
     int *bsum = (int *)get(sizeof(int) * (size_t)nbs);
     double *d_xs = (double *)get(sizeof(double) * m3);
     double *d_lpp = (double *)get(sizeof(double) * n_ch);
     unsigned long long *d_fmax = (unsigned long long *)get(2 * sizeof(unsigned long long));   // max |F|, sum nn
-    cudaStream_t gs = nullptr, gs2 = nullptr;
+    cudaStream_t gs = nullptr;
     cudaGraphExec_t gexec = nullptr;
     auto done = [&](kg_status r) {
         if (gexec) cudaGraphExecDestroy(gexec);
         if (gs) cudaStreamDestroy(gs);
-        if (gs2) cudaStreamDestroy(gs2);
         cudaStreamSynchronize(c->stream);
         for (void *p : bufs) dev_free(c, p);
         return r;
@@ -772,26 +730,22 @@ kg_status kg_primitive_path(kg_ctx *c, int melt, const kg_ppa_params *pp, double
     static const unsigned one = 1u;
     if (cudaMemcpyAsync(a.flags + 1, &one, sizeof(unsigned), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return done(KG_ERR_CUDA);
-    // the first build (into cell order) and force, from rest (v = 0, no kick)
-    enqueue_build(a, st, bsum);
-    enqueue_force(a, st, mixed, 0.0);
-    c->launches += 2 + PPA_BUILD_LAUNCHES;
-    long long left = pp->n_iter, graph_steps = 0;
-    if (left >= 2 * PPA_GRAPH_ITERS && cudaStreamCreateWithFlags(&gs, cudaStreamNonBlocking) == cudaSuccess &&
-        cudaStreamCreateWithFlags(&gs2, cudaStreamNonBlocking) == cudaSuccess &&
-        capture_steps(a, gs, gs2, bsum, mixed, &gexec)) {
-        for (; left >= PPA_GRAPH_ITERS; left -= PPA_GRAPH_ITERS, graph_steps += PPA_GRAPH_ITERS)
-            if (cudaGraphLaunch(gexec, st) != cudaSuccess) return done(KG_ERR_CUDA);
+    // the build into cell order, then n_iter + 1 steps from rest
+    const long long steps = pp->n_iter + 1;
+    const int len = steps >= PPA_GRAPH_MIN ? PPA_PASS : PPA_DIRECT_PASS;
+    loop_begin(st, a.loop, steps, len);
+    if (len == PPA_PASS && cudaStreamCreateWithFlags(&gs, cudaStreamNonBlocking) == cudaSuccess &&
+        capture_loop(gs, &gexec, [&](cudaGraphConditionalHandle h) { enqueue_pass(a, gs, bsum, mixed, len, h, true); })) {
+        if (cudaGraphLaunch(gexec, st) != cudaSuccess) return done(KG_ERR_CUDA);
+    } else {                                           // a pass does one step at least; none is left for the last ones
+        for (long long i = 0; i < steps; ++i) enqueue_pass(a, st, bsum, mixed, len, cudaGraphConditionalHandle{}, false);
     }
-    c->launches += 3 * graph_steps + PPA_LAUNCHES_PER_ITER * left;   // + the graphs' builds, below
-    for (; left > 0; --left) enqueue_step(a, st, bsum, mixed);
     k_ppa_unpermute<<<nblk(M, 256), 256, 0, st>>>(a, d_xs, d_fmax, d_fmax + 1);
     k_ppa_lengths<<<nblk(32LL * n_ch, 256), 256, 0, st>>>(d_xs, M, N, d_lpp);
-    c->launches += 2;
     if (cudaGetLastError() != cudaSuccess) return done(KG_ERR_CUDA);
 
     std::vector<double> h_lpp((size_t)n_ch);
-    unsigned h_flags[4] = {0, 0, 0, 0};
+    unsigned h_flags[8] = {};
     unsigned long long h_fmax[2] = {0, 0};
     if (cudaMemcpyAsync(h_lpp.data(), d_lpp, sizeof(double) * n_ch, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaMemcpyAsync(h_flags, a.flags, sizeof(h_flags), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -800,7 +754,7 @@ kg_status kg_primitive_path(kg_ctx *c, int melt, const kg_ppa_params *pp, double
     if (x_out && cudaMemcpyAsync(x_out, d_xs, sizeof(double) * m3, cudaMemcpyDefault, st) != cudaSuccess)
         return done(KG_ERR_CUDA);
     if (cudaStreamSynchronize(st) != cudaSuccess) return done(KG_ERR_CUDA);
-    if (graph_steps) c->launches += PPA_BUILD_LAUNCHES * (long long)h_flags[2];   // upper bound: all builds
+    c->launches += 5 + (mixed ? 1 : 2) * steps + (long long)h_flags[6];   // the passes' other kernels: counted there
     const unsigned e = h_flags[0];
     if (e & ERR_OVERSTRETCH) return done(KG_ERR_BOND_OVERSTRETCH);
     if (e & ERR_NONFINITE) return done(KG_ERR_NONFINITE);

@@ -231,19 +231,63 @@ __device__ __forceinline__ void md_cell_xyz(const MeltDev &md, int cell, int &cx
     cz = ((b / (md.nbk * md.nbk)) << 2) | (l >> 4);
 }
 
+// Conversions between binary64, binary32 and integers in 32-bit integer
+// instructions, for the ordinary range of their arguments; the rest takes the
+// conversion instruction.  A binary64 conversion or rounding occupies the
+// binary64 pipe, two lanes a clock per SM here, like an addition: 16 clocks a
+// warp, where these take 5 to 15 instructions of the 128-lane integer and
+// logic pipes.  Same results as the instructions, bit for bit.
+__device__ __forceinline__ double f32_to_f64(float f)
+{
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (double)f;            // zero, subnormal, infinite or NaN
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+__device__ __forceinline__ float f64_to_f32(double d)                // to nearest even
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u >= 253u) return __double2float_rn(d);               // outside [2^-126, 2^127) in size
+    const unsigned long long r = (((unsigned long long)hi << 32) | lo) + 0x0fffffffu + ((lo >> 29) & 1u);
+    return __uint_as_float((__funnelshift_l((unsigned)r, (unsigned)(r >> 32), 3) - (0x180u << 23)) | (hi & 0x80000000u));
+}
+
+// floor(p) as an integer; g: the same as binary64
+__device__ __forceinline__ int floor_f64(double p, double &g)
+{
+    const unsigned hi = (unsigned)__double2hiint(p), lo = (unsigned)__double2loint(p);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
+    if ((unsigned)e >= 30u) {                                        // below 1 or from 2^30 in size, infinite, NaN
+        if (e < 0) {
+            g = (hi >> 31) && ((hi << 1) | lo) ? -1.0 : 0.0;
+            return (int)g;
+        }
+        g = floor(p);
+        return (int)g;
+    }
+    const unsigned m = __funnelshift_l(lo, hi, 11) | 0x80000000u;    // the significand's top 32 bits: [1, 2) 2^31
+    unsigned t = m >> (31 - e);
+    if (hi >> 31) t += ((m << (e + 1)) | (lo << 11)) != 0u;          // away from zero below it
+    const int z = __clz((int)t);                                     // t in [1, 2^30]
+    const unsigned n = t << z;
+    g = __hiloint2double((int)((hi & 0x80000000u) | ((unsigned)(1023 + 31 - z) << 20) | ((n << 1) >> 12)), (int)(n << 21));
+    return hi >> 31 ? -(int)t : (int)t;
+}
+
 // Cell of a binary64 coordinate on a grid of n cells of side h = L / n per
 // period: g = floor(x / h) of the unwrapped coordinate, taken modulo n, and
 // the offset x - g h from that cell's corner, rounded once to binary32.
 // n h differs from L by at most an ulp of L, so the offsets of monomers in
-// different periodic images stay consistent to ~1e-14 sigma.  Four binary64
-// operations (binary64 issues at a small fraction of the binary32 rate on
-// this GPU), each explicitly rounded so that every kernel inlining it
-// computes the same bits.
+// different periodic images stay consistent to ~1e-14 sigma.  Two binary64
+// operations, each explicitly rounded so that every kernel inlining it
+// computes the same bits; floor and conversions in integer instructions.
 __device__ __forceinline__ int cell_of(double x, double h, double invh, int n, float &off)
 {
-    const double g = floor(__dmul_rn(x, invh));
-    off = __double2float_rn(__fma_rn(-g, h, x));
-    const int c = (int)g % n;
+    double g;
+    const int k = floor_f64(__dmul_rn(x, invh), g);
+    off = f64_to_f32(__fma_rn(-g, h, x));
+    const int c = k % n;
     return c < 0 ? c + n : c;
 }
 

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(256) k_ppa_bin(PpaArgs a)
     for (int d = 0; d < 3; ++d) {
         double xd = x[(size_t)d * a.M + p];
         if (a.u0) {                                    // mixed: fold d into the binary64 position
-            xd += (double)dd[d];
+            xd += f32_to_f64(dd[d]);
             x[(size_t)d * a.M + p] = xd;
         }
         cc[d] = cell_of(xd, a.h, a.invh, a.nc, o[d]);

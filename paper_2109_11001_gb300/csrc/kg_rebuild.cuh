@@ -33,9 +33,9 @@ __device__ __forceinline__ unsigned bin_md_one(const SimDev &S, int s, double *_
     double xs[3];
     if (xb64) {                        // mixed: the build position plus the displacement since
         const float4 e = dread[s];
-        xs[0] = __dadd_rn(xb64[s], (double)e.x);
-        xs[1] = __dadd_rn(xb64[Mp + s], (double)e.y);
-        xs[2] = __dadd_rn(xb64[2 * Mp + s], (double)e.z);
+        xs[0] = __dadd_rn(xb64[s], f32_to_f64(e.x));
+        xs[1] = __dadd_rn(xb64[Mp + s], f32_to_f64(e.y));
+        xs[2] = __dadd_rn(xb64[2 * Mp + s], f32_to_f64(e.z));
     } else {
         xs[0] = x[s];
         xs[1] = x[Mp + s];

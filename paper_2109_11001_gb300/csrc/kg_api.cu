@@ -20,12 +20,26 @@ using kg::dev_free;
 
 namespace kg {
 
+// A program that passes no stream usually works on the default stream: the
+// inputs it hands over, and buffers that its allocator hands out again, can
+// still be in use by work queued there, which a non-blocking stream does not
+// wait for by itself.
+void follow_default(kg_ctx *c)
+{
+    if (!c->own_stream) return;
+    if (!c->order_ev && cudaEventCreateWithFlags(&c->order_ev, cudaEventDisableTiming) != cudaSuccess) return;
+    cudaEventRecord(c->order_ev, cudaStreamLegacy);
+    cudaStreamWaitEvent(c->stream, c->order_ev, 0);
+}
+
 void *dev_alloc(kg_ctx *c, size_t bytes)
 {
     bytes = (bytes + 255) & ~(size_t)255;
     void *p = nullptr;
-    if (c->have_alloc) p = c->alloc.alloc(bytes, c->alloc.user);
-    else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+    if (c->have_alloc) {
+        p = c->alloc.alloc(bytes, c->alloc.user);
+        follow_default(c);
+    } else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
     if (p) cudaMemsetAsync(p, 0, bytes, c->stream);
     return p;
 }
@@ -435,6 +449,7 @@ void kg_destroy(kg_ctx *c)
     dev_free(c, c->bidx);
     dev_free(c, c->brec);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
+    if (c->order_ev) cudaEventDestroy(c->order_ev);
     kg::graphs_reset(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -454,6 +469,7 @@ kg_status kg_load_config(kg_ctx *c, int melt, const double *x, const double *v, 
     if (!x) return KG_ERR_INVALID_ARG;
     const MeltDev &md = c->sim.melt[melt];
     const size_t Mm = md.M, Mp = c->Mp;
+    kg::follow_default(c);
     for (int d = 0; d < 3; ++d)
         KG_TRY(cudaMemcpyAsync(c->x + d * Mp + md.off, x + d * Mm, Mm * sizeof(double), cudaMemcpyDefault, c->stream));
     if (c->precision == KG_MIXED) {   // build position = the loaded one, no displacement since

@@ -49,6 +49,7 @@ struct kg_ctx {
     long long *d_step = nullptr;   // device step counter (index of the step being run)
     bool d_step_stale = true;      // host must write it before the next step
     cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
+    cudaEvent_t order_ev = nullptr;    // follow_default
     cudaGraphExec_t gexec[kg::LOOP_MAX / 4] = {};   // captured step loops with bodies of 4, 8, 12 and 16 steps
     bool graph_failed = false;
     kg::LoopDev *loop = nullptr;   // their state on the device
@@ -141,6 +142,8 @@ struct kg_ctx {
 namespace kg {
 
 // device memory through the context's allocator (zero-filled on the context's stream)
+// a context's own stream waits for the work queued on the default stream so far
+void follow_default(kg_ctx *c);
 void *dev_alloc(kg_ctx *c, size_t bytes);
 void dev_free(kg_ctx *c, void *p);
 

@@ -42,7 +42,7 @@ def _run(kg, m, calls, one_by_one, **options):
 
 
 # two threads per monomer and binary64 systems take the loop at every size
-@pytest.mark.parametrize("options", [dict(threads_per_monomer=2), dict(precision=1)])
+@pytest.mark.parametrize("options", [dict(threads_per_monomer=2), dict(precision=0)])
 @pytest.mark.parametrize("skin", [0.1, 0.3, 0.8])
 def test_loop_matches_one_launch_per_step(kg, options, skin):
     m = KI.random_walk_melt(30, 41, 0.85, 1.0, 17)

@@ -63,7 +63,7 @@ struct ViewMove {
     __device__ __forceinline__ int cur(int p) const { return swap_slot(b.cur(p), kind, A, B, pA, pB, N, off); }
 };
 
-__device__ __forceinline__ double d2(const DBC &C, int a, int b) { return dist2_exact(C.x, C.Mp, C.md.L, a, b); }
+__device__ __forceinline__ double d2(const DBC &C, int a, int b) { return dist2_exact(C.x, C.Mp, C.md.L, C.md.invLf, a, b); }
 
 // Swap-bond criterion d2(a, b) <= 1.3^2, decided exactly: the binary32 record
 // distance settles every pair outside the band [db_lo, db_hi), which bounds
@@ -204,8 +204,8 @@ __device__ double vcos(const DBC &C, const V &v, int chain, int i)
     double b1[3], b2[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        b1[k] = min_image_exact(C.x[k * C.Mp + b] - C.x[k * C.Mp + a], L);
-        b2[k] = min_image_exact(C.x[k * C.Mp + c] - C.x[k * C.Mp + b], L);
+        b1[k] = min_image_exact(C.x[k * C.Mp + b] - C.x[k * C.Mp + a], L, C.md.invLf);
+        b2[k] = min_image_exact(C.x[k * C.Mp + c] - C.x[k * C.Mp + b], L, C.md.invLf);
     }
     return (b1[0] * b2[0] + b1[1] * b2[1] + b1[2] * b2[2])
            / (sqrt(b1[0] * b1[0] + b1[1] * b1[1] + b1[2] * b1[2])

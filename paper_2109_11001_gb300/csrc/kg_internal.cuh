@@ -189,21 +189,6 @@ __device__ __forceinline__ int melt_of(const SimDev &S, int s)
     return m;
 }
 
-// binary64 minimum image evaluated exactly as d - L*rint(d/L), no contraction
-__device__ __forceinline__ double min_image_exact(double d, double L)
-{
-    return __dsub_rn(d, __dmul_rn(L, rint(__ddiv_rn(d, L))));
-}
-
-// squared binary64 distance between slots s and t, ((dx*dx + dy*dy) + dz*dz)
-__device__ __forceinline__ double dist2_exact(const double *__restrict__ x, int Mp, double L, int s, int t)
-{
-    const double dx = min_image_exact(__dsub_rn(x[t], x[s]), L);
-    const double dy = min_image_exact(__dsub_rn(x[Mp + t], x[Mp + s]), L);
-    const double dz = min_image_exact(__dsub_rn(x[2 * Mp + t], x[2 * Mp + s]), L);
-    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
 __device__ __forceinline__ unsigned pack_code(int cx, int cy, int cz)
 {
     return (unsigned)cx | ((unsigned)cy << CODE_BITS) | ((unsigned)cz << (2 * CODE_BITS));
@@ -289,6 +274,38 @@ __device__ __forceinline__ int cell_of(double x, double h, double invh, int n, f
     off = f64_to_f32(__fma_rn(-g, h, x));
     const int c = k % n;
     return c < 0 ? c + n : c;
+}
+
+// Number of box lengths that a minimum image takes off d, rint(d / L), in
+// binary32 where that settles it: the binary32 quotient is good to 2e-3 below
+// 1e4 box lengths, so 0.02 from a half its nearest integer is the binary64
+// one's.  `sure` false: it does not (or d is not finite).
+__device__ __forceinline__ float image_of(double d, float invL, bool &sure)
+{
+    const float y = f64_to_f32(d) * invL, k = rintf(y);
+    sure = fabsf(y - k) < 0.48f && fabsf(y) < 1e4f;
+    return k;
+}
+
+// d - L*rint(d/L) as written, no contraction.  Most vectors here join
+// monomers of the same image (k = 0 leaves d as it is) or near ones, so the
+// binary64 divide and rounding, ~12 of the thin pipe's operations, are rarely
+// taken.
+__device__ __forceinline__ double min_image_exact(double d, double L, float invL)
+{
+    bool sure;
+    const float k = image_of(d, invL, sure);
+    if (!sure) return __dsub_rn(d, __dmul_rn(L, rint(__ddiv_rn(d, L))));
+    return k == 0.f ? d : __dsub_rn(d, __dmul_rn(L, f32_to_f64(k)));
+}
+
+// squared binary64 distance between slots s and t, ((dx*dx + dy*dy) + dz*dz)
+__device__ __forceinline__ double dist2_exact(const double *__restrict__ x, int Mp, double L, float invL, int s, int t)
+{
+    const double dx = min_image_exact(__dsub_rn(x[t], x[s]), L, invL);
+    const double dy = min_image_exact(__dsub_rn(x[Mp + t], x[Mp + s]), L, invL);
+    const double dz = min_image_exact(__dsub_rn(x[2 * Mp + t], x[2 * Mp + s]), L, invL);
+    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
 // Minimum-image vector from gather record i to gather record j (binary32):

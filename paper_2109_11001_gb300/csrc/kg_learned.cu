@@ -109,8 +109,8 @@ __device__ void move_features(const DBC &C, const V &v, int c, int b, const Cand
         double e1[3], e2[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            e1[k] = min_image_exact(C.x[k * C.Mp + w] - C.x[k * C.Mp + u], md.L);
-            e2[k] = min_image_exact(C.x[k * C.Mp + Y] - C.x[k * C.Mp + X], md.L);
+            e1[k] = min_image_exact(C.x[k * C.Mp + w] - C.x[k * C.Mp + u], md.L, md.invLf);
+            e2[k] = min_image_exact(C.x[k * C.Mp + Y] - C.x[k * C.Mp + X], md.L, md.invLf);
         }
         val = (e1[0] * e2[0] + e1[1] * e2[1] + e1[2] * e2[2])
               / (sqrt(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]) *
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(256) k_bond_max(const SimDev *__restrict__ Sp,
     if (s < S.M) {
         const MeltDev &md = S.melt[melt_of(S, s)];
         const int i = (s - md.off) % md.N;
-        if (i < md.N - 1) r2 = dist2_exact(x, S.Mp, md.L, comp_of[s], comp_of[s + 1]);
+        if (i < md.N - 1) r2 = dist2_exact(x, S.Mp, md.L, md.invLf, comp_of[s], comp_of[s + 1]);
     }
     for (int o = 16; o > 0; o >>= 1) r2 = fmax(r2, __shfl_xor_sync(FULL, r2, o));
     if ((threadIdx.x & 31) == 0 && r2 > 0.0) atomicMax(bmax2, (unsigned long long)__double_as_longlong(r2));

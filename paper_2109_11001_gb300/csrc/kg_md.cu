@@ -907,7 +907,7 @@ NlArgs nl_args(const kg_ctx *c)
     a.rl2 = c->sim.rl2;
     for (int m = 0; m < c->sim.n_melts; ++m) {
         const MeltDev &md = c->sim.melt[m];
-        a.melt[m] = MeltNl{md.off, md.cell_off, md.nbk, md.nc, md.hf, md.nl_lo, md.nl_hi, md.L};
+        a.melt[m] = MeltNl{md.off, md.cell_off, md.nbk, md.nc, md.hf, md.nl_lo, md.nl_hi, md.invLf, md.L};
     }
     return a;
 }

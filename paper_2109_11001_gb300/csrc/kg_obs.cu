@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(256) k_hist(const double *__restrict__ x, int 
         for (int b = threadIdx.x; b < 2 * nbins; b += blockDim.x) sh[b] = 0;
         __syncthreads();
     }
-    const float half = (float)(0.49 * L), binsf = (float)nbins, per = (float)((double)nbins / R0);
+    const float invL = (float)(1.0 / L), half = (float)(0.49 * L), binsf = (float)nbins, per = (float)((double)nbins / R0);
     // rounding of the binary32 length (relative 3 2^-24, and the bin's) and cosine (absolute 12 2^-24), in bins, doubled
     const float ulp = 5.9604644775390625e-8f, tol = 32.0f * binsf * ulp;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < M; r += gridDim.x * blockDim.x) {
@@ -232,11 +232,11 @@ __global__ void __launch_bounds__(256) k_hist(const double *__restrict__ x, int 
         auto bond = [&](int from, int to, Bond64 &b, float3 &f) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) b.v[k] = x[(size_t)k * Mp + to] - x[(size_t)k * Mp + from];
-            f = make_float3((float)b.v[0], (float)b.v[1], (float)b.v[2]);
+            f = make_float3(f64_to_f32(b.v[0]), f64_to_f32(b.v[1]), f64_to_f32(b.v[2]));
             if (!(fmaxf(fmaxf(fabsf(f.x), fabsf(f.y)), fabsf(f.z)) < half)) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) b.v[k] = min_image_exact(b.v[k], L);
-                f = make_float3((float)b.v[0], (float)b.v[1], (float)b.v[2]);
+                for (int k = 0; k < 3; ++k) b.v[k] = min_image_exact(b.v[k], L, invL);
+                f = make_float3(f64_to_f32(b.v[0]), f64_to_f32(b.v[1]), f64_to_f32(b.v[2]));
             }
         };
         if (i + 1 >= N) continue;
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(256) k_gr_sort(const float4 *__restrict__ rec,
 // bin of a pair by the binary64 definition (-1: none)
 __device__ __noinline__ int gr_exact(const GrArgs &A, int p, int k)
 {
-    const double r = sqrt(dist2_exact(A.x, A.Mp, A.Ld, A.list[p], A.list[k]));
+    const double r = sqrt(dist2_exact(A.x, A.Mp, A.Ld, A.invL, A.list[p], A.list[k]));
     return r < A.r_max ? (int)__ddiv_rn(r, A.dr) : -1;
 }
 

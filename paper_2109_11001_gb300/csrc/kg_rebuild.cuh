@@ -141,7 +141,7 @@ __device__ __forceinline__ bool cellrank_one(int p, const int *__restrict__ cell
 // ---------------------------------------------------------------------------
 struct MeltNl {
     int off, cell_off, nbk, nc;
-    float h, lo, hi;
+    float h, lo, hi, invL;
     double L;
 };
 
@@ -261,7 +261,7 @@ __device__ __forceinline__ unsigned nlist_one(const NlArgs &A, int s)
             const unsigned e = out[(size_t)k * Mp];
             const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
             const float r2 = nl_r2(ri, nl_ld<READ_ONLY>(A.recb + t), q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1, h);
-            const bool keep = r2 < lo || dist2_exact(A.x, A.Mp, md.L, s, t) < A.rl2;
+            const bool keep = r2 < lo || dist2_exact(A.x, A.Mp, md.L, md.invL, s, t) < A.rl2;
             if (keep) out[(size_t)(w++) * Mp] = e;
         }
         cnt = w;
@@ -309,7 +309,7 @@ __device__ __forceinline__ unsigned nlist_finish(const NlArgs &A, int s, int m, 
             const int t = (int)(e & IDX_MASK), q = (int)(e >> IDX_BITS);
             const float v = nl_v(A.recb[t], rs.x - (float)(q % 3 - 1) * ms.h, rs.y - (float)((q / 3) % 3 - 1) * ms.h,
                                  rs.z - (float)(q / 9 - 1) * ms.h, ms.hi);
-            const bool keep = k < cs && (v < ms.lo - ms.hi || dist2_exact(A.x, A.Mp, ms.L, ss, t) < A.rl2);
+            const bool keep = k < cs && (v < ms.lo - ms.hi || dist2_exact(A.x, A.Mp, ms.L, ms.invL, ss, t) < A.rl2);
             const unsigned bal = __ballot_sync(FULL, keep);
             if (keep) row[(size_t)(kept + __popc(bal & ((1u << lane) - 1u))) * Mp] = e;
             kept += __popc(bal);

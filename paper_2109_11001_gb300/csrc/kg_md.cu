@@ -27,7 +27,6 @@ namespace kg {
 // U_MLJ^n(r) = c1 r^-n - c2 r^-6 + 1 for r < r_c (Eqs. 5-6, shifted by +epsilon);
 // fr = (dU/dr)/r, so the force on i from j at d = x_j - x_i is fr * d.
 // ---------------------------------------------------------------------------
-template <bool ENERGY>
 __device__ __forceinline__ float mlj_fr(const StageDev &st, float r2, float &U)
 {
     const float ir2 = __fdividef(1.0f, r2);
@@ -47,11 +46,10 @@ __device__ __forceinline__ float mlj_fr(const StageDev &st, float r2, float &U)
     } else {
         rn = exp2f(-0.5f * st.nf * log2f(r2));
     }
-    if (ENERGY) U = st.c1f * rn - st.c2f * ir6 + 1.0f;
+    U = st.c1f * rn - st.c2f * ir6 + 1.0f;
     return (st.c2x6f * ir6 - st.c1xnf * rn) * ir2;
 }
 
-template <bool ENERGY>
 __device__ __forceinline__ double mlj_fr(const StageDev &st, double r2, double &U)
 {
     const double ir2 = 1.0 / r2;
@@ -69,7 +67,7 @@ __device__ __forceinline__ double mlj_fr(const StageDev &st, double r2, double &
     } else {
         rn = exp2(-0.5 * st.n * log2(r2));
     }
-    if (ENERGY) U = st.c1 * rn - st.c2 * ir6 + 1.0;
+    U = st.c1 * rn - st.c2 * ir6 + 1.0;
     return (6.0 * st.c2 * ir6 - st.n * st.c1 * rn) * ir2;
 }
 
@@ -155,51 +153,46 @@ struct GeoF64 {
     __device__ __forceinline__ double3 rel_nl(unsigned e) const { return rel((int)(e & IDX_MASK)); }
 };
 
-template <bool ENERGY, typename T, typename T3>
+template <typename T, typename T3>
 __device__ __forceinline__ void pair_term(const StageDev &st, T rc2, T3 d, T3 &F, double *e)
 {
     const T r2 = dot3(d, d);
-    if (!ENERGY) {                       // branch-free: a warp evaluates the force for some lane anyway
+    if (r2 < rc2) {
         T U;
-        T fr = mlj_fr<false>(st, r2, U);
-        fr = r2 < rc2 ? fr : (T)0;
-        F.x += fr * d.x; F.y += fr * d.y; F.z += fr * d.z;
-    } else if (r2 < rc2) {
-        T U;
-        const T fr = mlj_fr<ENERGY>(st, r2, U);
+        const T fr = mlj_fr(st, r2, U);
         F.x += fr * d.x; F.y += fr * d.y; F.z += fr * d.z;
         e[0] += 0.5 * (double)U;
         e[3] -= 0.5 * (double)(fr * r2);
     }
 }
 
-// Pair forces on s from its Verlet-list entries k = k0, k0 + stride, ...
-// (both directions are stored), four entries in flight.
-template <bool ENERGY, class G>
+// Pair forces on s from its Verlet list (both directions are stored), four
+// entries in flight.
+template <class G>
 __device__ __forceinline__ void pair_forces(const G &g, const SimDev &S, const StageDev &st, int s,
-                                            const unsigned *__restrict__ nl, int cnt, int k0, int stride,
+                                            const unsigned *__restrict__ nl, int cnt,
                                             typename G::T3 &F, double *e)
 {
     using T = typename G::T;
     using T3 = typename G::T3;
     const T rc2 = (T)S.rc2;
-    const size_t Mp = (size_t)S.Mp, step = (size_t)stride * Mp;
-    const unsigned *__restrict__ col = nl + s + (size_t)k0 * Mp;
-    int k = k0;
-    for (; k + 3 * stride < cnt; k += 4 * stride, col += 4 * step) {
+    const size_t step = (size_t)S.Mp;
+    const unsigned *__restrict__ col = nl + s;
+    int k = 0;
+    for (; k + 3 < cnt; k += 4, col += 4 * step) {
         const unsigned e0 = __ldg(col), e1 = __ldg(col + step);
         const unsigned e2 = __ldg(col + 2 * step), e3 = __ldg(col + 3 * step);
         const T3 d0 = g.rel_nl(e0), d1 = g.rel_nl(e1), d2 = g.rel_nl(e2), d3 = g.rel_nl(e3);
-        pair_term<ENERGY>(st, rc2, d0, F, e);
-        pair_term<ENERGY>(st, rc2, d1, F, e);
-        pair_term<ENERGY>(st, rc2, d2, F, e);
-        pair_term<ENERGY>(st, rc2, d3, F, e);
+        pair_term(st, rc2, d0, F, e);
+        pair_term(st, rc2, d1, F, e);
+        pair_term(st, rc2, d2, F, e);
+        pair_term(st, rc2, d3, F, e);
     }
-    for (; k < cnt; k += stride, col += step) pair_term<ENERGY>(st, rc2, g.rel_nl(__ldg(col)), F, e);
+    for (; k < cnt; ++k, col += step) pair_term(st, rc2, g.rel_nl(__ldg(col)), F, e);
 }
 
 // Bond (Eq. 10) and bending (Eq. 4) forces on s from its chain partners.
-template <bool ENERGY, class G>
+template <class G>
 __device__ __forceinline__ void bonded_forces(const G &g, const StageDev &st, const MeltDev &md,
                                               typename G::T rc2, int4 bp, typename G::T3 &F, double *e,
                                               unsigned &err)
@@ -225,20 +218,18 @@ __device__ __forceinline__ void bonded_forces(const G &g, const StageDev &st, co
             if (qmin > (T)0 && q < qmin) {           // continuation beyond r* (kg_params.fene_qmin)
                 fr = kf * frcp(qmin);
                 if (!(r2 < (T)4 * R0sq)) err |= ERR_OVERSTRETCH;
-                if (ENERGY) Uf = st_c<T>(st, 7) + kf * (r2 - st_c<T>(st, 6)) / ((T)2 * qmin);
+                Uf = st_c<T>(st, 7) + kf * (r2 - st_c<T>(st, 6)) / ((T)2 * qmin);
             } else {
                 if (!(r2 < R0sq)) err |= ERR_OVERSTRETCH;
                 q = fmax(q, (T)1e-6);                    // finite even when flagged
                 fr = kf * frcp(q);
-                if (ENERGY) Uf = (T)-0.5 * kf * R0sq * flog(q);
+                Uf = (T)-0.5 * kf * R0sq * flog(q);
             }
             T U = 0;
-            if (r2 < rc2) fr += mlj_fr<ENERGY>(st, r2, U);
+            if (r2 < rc2) fr += mlj_fr(st, r2, U);
             F.x += fr * d.x; F.y += fr * d.y; F.z += fr * d.z;
-            if (ENERGY) {
-                e[1] += 0.5 * ((double)U + (double)Uf);
-                e[3] -= 0.5 * (double)(fr * r2);
-            }
+            e[1] += 0.5 * ((double)U + (double)Uf);
+            e[3] -= 0.5 * (double)(fr * r2);
         }
     }
     // bending kappa (1 - b1.b2 / |b1||b2|) at the vertices s-1, s, s+1
@@ -251,7 +242,7 @@ __device__ __forceinline__ void bonded_forces(const G &g, const StageDev &st, co
             F.x += kap * ((B0.x * inv - c1 * Bm1.x) - (Bm1.x * inv - c2 * B0.x));
             F.y += kap * ((B0.y * inv - c1 * Bm1.y) - (Bm1.y * inv - c2 * B0.y));
             F.z += kap * ((B0.z * inv - c1 * Bm1.z) - (Bm1.z * inv - c2 * B0.z));
-            if (ENERGY) e[2] += (double)kap * (1.0 - (double)cs);
+            e[2] += (double)kap * (1.0 - (double)cs);
         }
         if (hp2) {                           // vertex s+1, s is its first end: -kappa g1
             const T l1 = dot3(B0, B0), l2 = dot3(Bp1, Bp1), inv = frsqrt(l1 * l2), cs = dot3(B0, Bp1) * inv;
@@ -270,10 +261,10 @@ __device__ __forceinline__ void bonded_forces(const G &g, const StageDev &st, co
     }
 }
 
-// Conservative force on slot s (chain position i of N) and, with ENERGY, its
+// Conservative force on slot s (chain position i of N) and its
 // shares of the energies: e[0] pair (1/2 per pair), e[1] bond (1/2 per bond),
 // e[2] bending (the angle whose vertex is s), e[3] virial (1/2 per pair/bond).
-template <bool ENERGY, class G>
+template <class G>
 __device__ __forceinline__ typename G::T3 force_on(const G &g, const SimDev &S, const StageDev &st,
                                                    const MeltDev &md, int s, int4 bp,
                                                    const unsigned *__restrict__ nl, int cnt,
@@ -281,8 +272,8 @@ __device__ __forceinline__ typename G::T3 force_on(const G &g, const SimDev &S, 
 {
     using T = typename G::T;
     typename G::T3 F = mk<T>(0, 0, 0);
-    pair_forces<ENERGY>(g, S, st, s, nl, cnt, 0, 1, F, e);
-    bonded_forces<ENERGY>(g, st, md, (T)S.rc2, bp, F, e, err);
+    pair_forces(g, S, st, s, nl, cnt, F, e);
+    bonded_forces(g, st, md, (T)S.rc2, bp, F, e, err);
     return F;
 }
 
@@ -660,7 +651,7 @@ __global__ void __launch_bounds__(128) k_forces(const SimDev *__restrict__ Sp, c
         G gg = g;
         gg.melt(md, m);
         gg.self(s);
-        const auto F = force_on<true>(gg, S, st, md, s, bp[s], nl, __ldg(nn + s), e, err);
+        const auto F = force_on(gg, S, st, md, s, bp[s], nl, __ldg(nn + s), e, err);
         const int Mp = S.Mp;
         if (Fout) {
             Fout[s] = (double)F.x; Fout[Mp + s] = (double)F.y; Fout[2 * Mp + s] = (double)F.z;

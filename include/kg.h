@@ -112,7 +112,7 @@ typedef struct {
                                  not depend on it; in KG_MIXED a re-sort forces a Verlet
                                  build, whose timing moves positions at the binary32
                                  rounding level (~1e-7 sigma)                           */
-    int block_size;           /* threads per block of the fused step kernel: 64, 128
+    int block_size;           /* threads per block of the mixed step kernel: 64, 128
                                  or 256 (<= 0: 128); results do not depend on it        */
     int precision;            /* KG_FP64 or KG_MIXED                                    */
     int flags;                /* KG_FLAG_*                                              */

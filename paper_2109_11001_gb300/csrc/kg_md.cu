@@ -288,12 +288,19 @@ __device__ __forceinline__ typename G::T3 force_on(const G &g, const SimDev &S, 
 //    the mixed path (offset from the build-time cell corner + displacement, a
 //    shift for the stencil code), with a margin above their rounding; only the
 //    pairs that may lie within r_c, about a third to a half of the list, take
-//    the binary64 minimum image, distance and force, in list order;
+//    the binary64 minimum image, distance and force;
+//  * the near pairs of a warp's 32 monomers form one queue, worked through a pair
+//    a lane; the results go through shared memory to their owners, who add them
+//    in list order.  Popping its own pairs, a lane waited for the largest of 32
+//    numbers of near pairs (about 9 against a mean of 4 to 5);
 //  * a bond's inverse length is one reciprocal square root that serves its own
 //    1/r^2, both its angles and all their gradients.
-// Each lane pops its own candidates from a mask, so a warp runs the binary64
-// part for its largest number of near pairs (about 8) and not for its longest
-// list (15 to 21).  80,000 monomers, n = 12, skin 0.3: 157 -> 99 us.
+// Blocks of 64, whatever block_size says: the pipe is the SM's, so the SM with
+// the most blocks sets the time, and 80,000 monomers are 4.1 blocks of 128 per
+// SM (five on some) but 8.2 of 64.  80,000 monomers, n = 12, skin 0.3, 50 steps
+// with 14 list builds: 9016 -> 5726 us with the first and last point, 4984 with
+// the queue and the small blocks (of which 2% the queue; at exponents that take
+// log2 and exp2 a pair is four times the work).  200,000: 228 -> 208 us a step.
 // ---------------------------------------------------------------------------
 // r^-n for the stage from 1/r^2 and 1/r^6
 __device__ __forceinline__ double inv_rn64(const StageDev &st, double r2, double ir2, double ir6)
@@ -380,7 +387,10 @@ __device__ __forceinline__ void bonded64(const GeoF64 &g, const StageDev &st, do
     }
 }
 
-__global__ void __launch_bounds__(256) k_step_f64(const SimDev *__restrict__ Sp, const StageDev *__restrict__ stp,
+constexpr int F64_BLOCK = 64;
+constexpr int F64_PAIRS = 192;           // near pairs of a warp that one round takes (mean about 110)
+
+__global__ void __launch_bounds__(F64_BLOCK) k_step_f64(const SimDev *__restrict__ Sp, const StageDev *__restrict__ stp,
                                                  double *__restrict__ x, double *__restrict__ u,
                                                  const double4_32a *__restrict__ pcur, double4_32a *__restrict__ pnext,
                                                  const double4_32a *__restrict__ xb, const float4 *__restrict__ recb,
@@ -404,29 +414,31 @@ __global__ void __launch_bounds__(256) k_step_f64(const SimDev *__restrict__ Sp,
     const SimDev &S = *Sp;
     const StageDev &st = *stp;
     const long long step = *stepp + (loop ? 1 + kstep : 0);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double pf_s[F64_BLOCK / 32][3 * F64_PAIRS];
+    __shared__ unsigned pair_s[F64_BLOCK / 32][F64_PAIRS];
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    double *const pf = pf_s[threadIdx.x >> 5];
+    unsigned *const pair = pair_s[threadIdx.x >> 5];
     bool rebuild = false;
     unsigned err = 0;
-    if (s < S.M) {
-        const int slot = __ldg(slot_of + s);
-        const int m = melt_of(S, slot);
-        const MeltDev &md = S.melt[m];
-        const int rel = slot - md.off;
-        GeoF64 g{pcur, md.L, md.invL, {}};
-        g.self(s);
-        const int Mp = S.Mp, cnt = __ldg(nn + s);
+    const bool live = s < S.M;
+    const int cnt = live ? __ldg(nn + s) : 0;
+    const int kmax = __reduce_max_sync(0xffffffffu, cnt);
+    double3 F = make_double3(0., 0., 0.);
+    {
+        const int slot = __ldg(slot_of + (live ? s : 0));
+        const MeltDev &md = S.melt[melt_of(S, slot)];
         const unsigned *__restrict__ col = nl + s;
-        const float4 gi = __ldg(gcur + s);
+        const float4 gi = __ldg(gcur + (live ? s : 0));
         const float h = md.hf, near2 = S.rc2f * (1.0f + 2e-5f);   // >> the records' rounding (~1e-6 in r^2)
-        double3 F = make_double3(0., 0., 0.);
-        for (int k0 = 0; k0 < cnt; k0 += 32) {
+        for (int k0 = 0; k0 < kmax; k0 += 32) {
             unsigned mask = 0;
             const int kn = min(32, cnt - k0);
             for (int k = 0; k < kn; k += 4) {
                 unsigned e[4];
                 float4 p[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) e[i] = __ldg(col + (size_t)(k0 + min(k + i, kn - 1)) * Mp);
+                for (int i = 0; i < 4; ++i) e[i] = __ldg(col + (size_t)(k0 + min(k + i, kn - 1)) * S.Mp);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) p[i] = __ldg(gcur + (e[i] & IDX_MASK));
 #pragma unroll
@@ -439,14 +451,55 @@ __global__ void __launch_bounds__(256) k_step_f64(const SimDev *__restrict__ Sp,
                     mask |= (unsigned)(close && k + i < kn) << (k + i);
                 }
             }
-            while (mask) {
-                const int k = __ffs(mask) - 1;
-                mask &= mask - 1;
-                const double3 d = g.rel((int)(__ldg(col + (size_t)(k0 + k) * Mp) & IDX_MASK));
-                const double r2 = dot3(d, d);
-                if (r2 < S.rc2) add64(mlj_fr64(st, r2, 1.0 / r2), d, F);
+            // the warp's near pairs in order of lane and list: this lane's are [first, first + n)
+            const int n = __popc(mask);
+            int first = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, first, o);
+                if (lane >= o) first += t;
+            }
+            const int total = __shfl_sync(0xffffffffu, first, 31);
+            first -= n;
+            for (int b = 0; b < total; b += F64_PAIRS) {
+                unsigned left = mask;
+                for (int i = first - b; left; ++i) {
+                    const int k = __ffs(left) - 1;
+                    left &= left - 1;
+                    if (i >= 0 && i < F64_PAIRS)
+                        pair[i] = (__ldg(col + (size_t)(k0 + k) * S.Mp) & IDX_MASK) | ((unsigned)lane << IDX_BITS);
+                }
+                __syncwarp();
+                for (int i = lane; i < min(F64_PAIRS, total - b); i += 32) {
+                    const int own = s - lane + (int)(pair[i] >> IDX_BITS);
+                    const MeltDev &mo = S.melt[melt_of(S, __ldg(slot_of + own))];
+                    GeoF64 g{pcur, mo.L, mo.invL, {}};
+                    g.self(own);
+                    const double3 d = g.rel((int)(pair[i] & IDX_MASK));
+                    const double r2 = dot3(d, d);
+                    const double fr = r2 < S.rc2 ? mlj_fr64(st, r2, 1.0 / r2) : 0.0;
+                    pf[i] = fr * d.x;
+                    pf[F64_PAIRS + i] = fr * d.y;
+                    pf[2 * F64_PAIRS + i] = fr * d.z;
+                }
+                __syncwarp();
+                for (int i = max(first - b, 0); i < min(first + n - b, F64_PAIRS); ++i) {
+                    F.x += pf[i];
+                    F.y += pf[F64_PAIRS + i];
+                    F.z += pf[2 * F64_PAIRS + i];
+                }
+                __syncwarp();
             }
         }
+    }
+    if (live) {
+        const int slot = __ldg(slot_of + s);
+        const int m = melt_of(S, slot);
+        const MeltDev &md = S.melt[m];
+        const int rel = slot - md.off;
+        GeoF64 g{pcur, md.L, md.invL, {}};
+        g.self(s);
+        const int Mp = S.Mp;
         bonded64(g, st, md.kappa, S.rc2, __ldg(bp + s), F, err);
         const double3 gn = gauss3_d(draw(S.seed, m, 0, (unsigned long long)step, (uint32_t)rel));
         double3 v = make_double3(u[s], u[Mp + s], u[2 * Mp + s]);
@@ -925,8 +978,7 @@ static void launch_step_kernel(kg_ctx *c, cudaStream_t st, int cur, LoopDev *loo
         step_mixed_launch(c, st, cur, loop, k);
         return;
     }
-    const int nb = nblk(c->M, c->block);
-    k_step_f64<<<nb, c->block, 0, st>>>(c->d_sim, c->d_stage, c->x, (double *)c->u, c->pos64[cur], c->pos64[cur ^ 1],
+    k_step_f64<<<nblk(c->M, F64_BLOCK), F64_BLOCK, 0, st>>>(c->d_sim, c->d_stage, c->x, (double *)c->u, c->pos64[cur], c->pos64[cur ^ 1],
                                         c->xb, c->recb, c->pg[cur], c->pg[cur ^ 1], c->nl, c->nn, c->slot_of, c->bp, c->flags, c->d_step, loop, k);
 }
 

@@ -50,6 +50,20 @@ struct LoopDev {
     unsigned req;            // bit k: step k of the pass asked for a list rebuild (later ones of the pass are skipped)
 };
 
+// Non-zero if step k of a pass (or a step launched by itself, lp null) does not
+// run: a latched error, the end of the loop, or a build asked for by an earlier
+// step of the pass (this step's own bit may already be set by another block).
+// The three words are loaded together.
+__device__ __forceinline__ unsigned step_off(const unsigned *flags, const LoopDev *lp, int k)
+{
+    const unsigned err = *(const volatile unsigned *)flags;
+    if (!lp) return err;
+    const volatile LoopDev *v = lp;
+    const int n = v->n;
+    const unsigned req = v->req;
+    return err | (unsigned)(k >= n) | (req & ((1u << k) - 1u));
+}
+
 // Ends a pass of `len` steps: counts the steps done (those up to the first
 // that asked for a build), passes the request on (flags[1]) and returns true if
 // another pass has to run.  flags[6] counts the pass's kernels other than these

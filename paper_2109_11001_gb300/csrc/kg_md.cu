@@ -401,14 +401,7 @@ __global__ void __launch_bounds__(F64_BLOCK) k_step_f64(const SimDev *__restrict
                                                  const long long *__restrict__ stepp, LoopDev *loop, int kstep)
 {
     __shared__ unsigned stop;
-    if (threadIdx.x == 0) {                // a latched error, the end of the loop or an earlier step's rebuild request
-        unsigned f = *(volatile unsigned *)flags;
-        if (loop) {
-            const volatile LoopDev *lp = loop;
-            if (kstep >= lp->n || (lp->req & ((1u << kstep) - 1u))) f = 1u;
-        }
-        stop = f;
-    }
+    if (threadIdx.x == 0) stop = step_off(flags, loop, kstep);
     __syncthreads();
     if (stop) return;
     const SimDev &S = *Sp;

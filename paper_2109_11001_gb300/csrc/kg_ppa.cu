@@ -123,16 +123,11 @@ __device__ __forceinline__ double min_image(double d, const PpaArgs &a)
     return __dsub_rn(d, __dmul_rn(a.L, rint(__dmul_rn(d, a.invL))));
 }
 
-// the stop test of a step kernel, one thread's answer for the block: a latched
-// error, the end of the loop, or an earlier step of the pass that asked for a
-// build (this step's own bit may already be set)
-__device__ __forceinline__ bool step_off(const PpaArgs &a, int k)
+// step_off (kg_internal.cuh), one thread's answer for the block
+__device__ __forceinline__ bool block_off(const PpaArgs &a, int k)
 {
     __shared__ unsigned off;
-    if (threadIdx.x == 0) {
-        const volatile LoopDev *lp = a.loop;
-        off = *(volatile unsigned *)a.flags | (unsigned)(k >= lp->n) | (lp->req & ((1u << k) - 1u));
-    }
+    if (threadIdx.x == 0) off = step_off(a.flags, a.loop, k);
     __syncthreads();
     return off != 0u;
 }
@@ -145,7 +140,7 @@ __device__ __forceinline__ bool is_fixed(const float4 &r) { return (__float_as_u
 // v <- v + (dt/2) F; x <- x + dt v; request a rebuild past skin / 2
 __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_drift_f64(PpaArgs a, int k)
 {
-    if (step_off(a, k) || *a.steps + k == a.n_iter) return;
+    if (block_off(a, k) || *a.steps + k == a.n_iter) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.M || is_fixed(a.rec[p])) return;
     const int cb = step_buf(a);
@@ -349,7 +344,7 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_nlist(PpaArgs a)
 // bonds; F <- F_c(x) - gamma v; v <- v + half dt F (half = 0 for the first force)
 __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_force_f64(PpaArgs a, int k)
 {
-    if (step_off(a, k)) return;
+    if (block_off(a, k)) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.M || is_fixed(a.rec[p])) return;
     const int cb = step_buf(a);
@@ -416,7 +411,7 @@ __global__ void __launch_bounds__(PPA_BLOCK) k_ppa_step_mixed(PpaArgs a, int k)
         const int i = q & 31, c = i < 27 ? (q < 32 ? i % 3 : q < 64 ? (i / 3) % 3 : i / 9) - 1 : 0;
         sh[q] = (float)c * a.hf;
     }
-    if (step_off(a, k)) return;
+    if (block_off(a, k)) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.M) return;
     const float4 *__restrict__ pg = a.pg[k & 1], *__restrict__ dl = a.dl[k & 1];

@@ -3,7 +3,7 @@
 // per monomer.
 //
 // What bounds a small system is not work but the chain of dependent waits: as
-// separate launches a step is a begin kernel, a conditional graph node and a
+// separate launches a step was a begin kernel, a conditional graph node and a
 // step kernel, each a launch of several microseconds around one or two
 // microseconds of load latency.  Here a step is one grid barrier and one round
 // of gathers:
@@ -31,8 +31,8 @@
 // Measured, 50 steps and a read of the state of 80,000 monomers (skin 0.3, n =
 // 12, dt = 0.01; a build every third or fourth step), against captured graphs
 // of separate launches: 1743 -> 1117 us.
-// Larger systems keep the graphs: there the step is work and the launches are
-// not.
+// Larger systems go in whole tiles (kg_resident_tiled.cu) or, from 1280
+// monomers per SM, through the captured loop (kg_md.cu).
 //
 // Systems of at most 128 monomers per SM take kg_resident_small.cu.
 //

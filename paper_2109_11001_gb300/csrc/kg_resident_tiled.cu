@@ -86,7 +86,8 @@ __global__ void __launch_bounds__(TILE, 5) k_resident_tiled(const __grid_constan
                                     [&](bool far, unsigned err) {
                                         if (err) atomicOr(A.errw, err);
                                         gb.note((far ? REQ : 0u) | (err ? FAIL : 0u));
-                                    });
+                                    },
+                                    []() { return true; });
         told = gb.sync();
         rebuild = (told & REQ) != 0u;
         if (told & (FAIL | GAVE_UP)) break;

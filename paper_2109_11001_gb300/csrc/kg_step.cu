@@ -44,16 +44,7 @@ __global__ void __launch_bounds__(256, 8) k_step32(const __grid_constant__ StepA
     __shared__ float dk[96];
     __shared__ unsigned stop;
     step_block_setup(dk);
-    if (threadIdx.x == 0) {
-        unsigned st = *(volatile unsigned *)P.flags;               // a latched error stops the run
-        if (P.loop) {                                              // so do the end of the loop and a rebuild request of
-            const volatile LoopDev *lp = P.loop;                   //   an earlier step of the pass (this one's own bit
-            if (P.k >= lp->n || (lp->req & ((1u << P.k) - 1u))) st = 1u;   //   may already be set by another block)
-        }
-        stop = st;
-    }
-    __syncthreads();
-    if (stop) return;                                              // block-uniform
+    if (threadIdx.x == 0) stop = step_off(P.flags, P.loop, P.k);
     const long long step = *P.stepp + (P.loop ? 1 + P.k : 0);
     step_tile<N4, TPM, true>(P, blockIdx.x * blockDim.x, P.dcur, P.dnext, P.pcur, P.pnext, step, dk,
                              // the rebuild vote per warp (no block barrier: a warp with short
@@ -64,7 +55,9 @@ __global__ void __launch_bounds__(256, 8) k_step32(const __grid_constant__ StepA
                                      else atomicOr(P.flags + 1, 1u);
                                  }
                                  if (err) atomicOr(P.flags, err);
-                             });
+                             },
+                             // the block's answer arrives with the first loads of the tile
+                             [&]() { __syncthreads(); return !stop; });
 }
 
 // 4n of a stage exponent with its own kernel instantiation, 0 otherwise

@@ -198,7 +198,8 @@ constexpr int STEP_ILP = 4;      // Verlet-list entries in flight per lane
 // with the zero shift (code 13), a valid gather whose term is masked.
 // READ_ONLY: nothing it loads is written in the same launch (non-coherent
 // loads).  vote(rebuild, err), by every lane of the warp: its monomer left its
-// skin, and its error bits.
+// skin, and its error bits.  go(), by every thread once its first loads are
+// under way: false if the block does not run the step after all.
 template <bool READ_ONLY, typename T>
 __device__ __forceinline__ T step_ld(const T *p)
 {
@@ -206,10 +207,10 @@ __device__ __forceinline__ T step_ld(const T *p)
     else return *p;
 }
 
-template <int N4, int TPM, bool READ_ONLY, class VOTE>
+template <int N4, int TPM, bool READ_ONLY, class VOTE, class GO>
 __device__ __forceinline__ void step_tile(const StepArgs &P, int t0, const float4 *dcur, float4 *dnext,
                                           const float4 *pcur, float4 *pnext, long long step, const float *dk,
-                                          VOTE vote)
+                                          VOTE vote, GO go)
 {
     constexpr bool RO = READ_ONLY;
     const int lane = threadIdx.x & 31;
@@ -217,16 +218,17 @@ __device__ __forceinline__ void step_tile(const StepArgs &P, int t0, const float
     const int s = t / TPM, sub = t % TPM;
     const bool live = s < P.M;
     const int cnt = live ? step_ld<RO>(P.nn + s) : 0;
-    const int kmax = __reduce_max_sync(0xffffffffu, cnt);
     unsigned err = 0;
     float3 F = make_float3(0.f, 0.f, 0.f), gn = F;
-    int slot = 0, m = 0;
+    int slot = 0;
     float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
     if (live) {
         slot = __ldg(P.slot_of + s);
-        m = melt_index(P, slot);
         pi = step_ld<RO>(pcur + s);
     }
+    if (!go()) return;                     // the same for the whole block
+    const int kmax = __reduce_max_sync(0xffffffffu, cnt);
+    const int m = live ? melt_index(P, slot) : 0;
     const MeltStep &md = P.melt[m];
     const float h = md.h, rc2 = P.rc2;
     const unsigned self = (unsigned)(live ? s : 0) | (13u << IDX_BITS);

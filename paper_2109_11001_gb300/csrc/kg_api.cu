@@ -32,7 +32,7 @@ void follow_default(kg_ctx *c)
     cudaStreamWaitEvent(c->stream, c->order_ev, 0);
 }
 
-void *dev_alloc(kg_ctx *c, size_t bytes)
+void *dev_alloc(kg_ctx *c, size_t bytes, size_t clear)
 {
     bytes = (bytes + 255) & ~(size_t)255;
     void *p = nullptr;
@@ -40,7 +40,7 @@ void *dev_alloc(kg_ctx *c, size_t bytes)
         p = c->alloc.alloc(bytes, c->alloc.user);
         follow_default(c);
     } else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
-    if (p) cudaMemsetAsync(p, 0, bytes, c->stream);
+    if (p) cudaMemsetAsync(p, 0, std::min(bytes, clear), c->stream);
     return p;
 }
 

@@ -144,7 +144,7 @@ namespace kg {
 // device memory through the context's allocator (zero-filled on the context's stream)
 // a context's own stream waits for the work queued on the default stream so far
 void follow_default(kg_ctx *c);
-void *dev_alloc(kg_ctx *c, size_t bytes);
+void *dev_alloc(kg_ctx *c, size_t bytes, size_t clear = ~(size_t)0);   // the first `clear` bytes zero
 void dev_free(kg_ctx *c, void *p);
 
 constexpr int GRAPH_STEPS = 10;          // MD steps between re-sort tests

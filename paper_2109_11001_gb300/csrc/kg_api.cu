@@ -505,9 +505,10 @@ kg_status kg_load_config(kg_ctx *c, int melt, const double *x, const double *v, 
         unsigned f[8];
         KG_TRY(cudaMemcpyAsync(f, c->flags, sizeof(f), cudaMemcpyDeviceToHost, c->stream));
         KG_TRY(cudaStreamSynchronize(c->stream));
-        c->launches += 6LL * (long long)f[6];
+        c->launches += (long long)f[6];
     }
     KG_TRY(cudaMemsetAsync(c->flags, 0, 16 * sizeof(unsigned), c->stream));
+    c->builds_seen = 0;                      // counted in flags[5]
     // a rebuild cut short by an earlier error may have left cell counts behind
     KG_TRY(cudaMemsetAsync(c->ccount, 0, sizeof(int) * (size_t)c->ncell_md, c->stream));
     KG_TRY(kg::resident_reset(c));

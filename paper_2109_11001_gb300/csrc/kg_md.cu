@@ -14,8 +14,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cstddef>
-#include <cstdlib>
 
 #include "kg_host.h"
 #include "kg_rebuild.cuh"

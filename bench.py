@@ -66,7 +66,7 @@ def bytes_per_monomer_at_skin(precision, skin):
 
 # DRAM bytes per monomer of the mixed step kernel from ncu captures of the
 # 1.6M-monomer case, by skin, and the hash of the step kernel's source
-# (kg_step.cu) they were taken on (reported as null for another skin or once
+# (kg_step.cu, kg_step.cuh) they were taken on (reported as null for another skin or once
 # the source changes)
 NCU_TRAFFIC = {"bytes_per_monomer": {0.5: 196.8, 0.6: 213.9}, "src_sha1": "e627455da1f4382bbc2b14cf2e2c30d8d440a189"}
 
@@ -89,8 +89,11 @@ def prelude_stages(kg):
 
 
 def src_sha1():
-    with open(os.path.join(ROOT, "paper_2109_11001_gb300", "csrc", "kg_step.cu"), "rb") as f:
-        return hashlib.sha1(f.read()).hexdigest()
+    h = hashlib.sha1()
+    for name in ("kg_step.cu", "kg_step.cuh"):
+        with open(os.path.join(ROOT, "paper_2109_11001_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
 
 
 def peaks():
@@ -636,7 +639,7 @@ KAPPA_SCAN = [(0.0, 100, 200), (0.5, 200, 150), (1.0, 400, 100), (1.5, 800, 50),
 
 def batched_secondary(kg, torch, args, local):
     """Eight melts of a kappa scan (20k-200k monomers each) advanced by the
-    same launches in one context (graphs of separate launches, and persistent
+    same launches in one context (captured loop, and persistent
     cooperative launches), against the same melts run one context at a time;
     4 x (50 MD steps + one DB sweep at R_MC) after the dt-ramped prelude."""
     import kg_inputs as KI

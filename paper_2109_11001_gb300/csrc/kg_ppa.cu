@@ -38,7 +38,7 @@
 // step loop of the MD path (kg_md.cu): passes of the list build, which returns
 // at once without a request, and PPA_PASS steps, those after a request left to
 // the next pass.  A contraction rebuilds its list every few steps: 200 steps
-// of 200,000 monomers with 51 builds took 11.5 ms with drift and force apart
+// of 200,000 monomers with 51 builds take 6.8 ms, and took 11.3 with drift and force apart
 // and a conditional node per step.
 //
 // Two force kernels.  Binary64 (KG_FP64): minimum-image distances and forces
@@ -75,7 +75,7 @@ namespace {
 constexpr double PPA_RC = 1.122462048309373;   // 2^(1/6)
 constexpr int PPA_MAXNB = 128;                  // list entries per monomer (overflow: capacity error)
 constexpr int PPA_CELL_CAP = 1024;              // monomers per cell the build accepts
-constexpr int PPA_PASS = 6;                     // steps per pass of the captured loop (even)
+constexpr int PPA_PASS = 6;                     // steps per pass of the captured loop (even; a build every 4 to 7 steps)
 constexpr int PPA_DIRECT_PASS = 2;              // the same without a graph
 constexpr long long PPA_GRAPH_MIN = 16;         // steps that are worth a capture (~0.2 ms; more than one pass)
 constexpr int PPA_BLOCK = 128;

@@ -30,7 +30,7 @@
 //
 // Measured, 50 steps and a read of the state of 80,000 monomers (skin 0.3, n =
 // 12, dt = 0.01; a build every third or fourth step), against captured graphs
-// of separate launches: 1743 -> 1117 us.
+// of separate launches: 1748 -> 1090 us.
 // Larger systems go in whole tiles (kg_resident_tiled.cu) or, from 1280
 // monomers per SM, through the captured loop (kg_md.cu).
 //

@@ -110,7 +110,7 @@ __device__ double swap_part(const DBC &C, const V &v, WarpCand &wc, const Attemp
 constexpr int EVAL_WARPS_U = 4;                 // attempts (warps) per block of k_db_eval
 
 // (128, 12): at most 40 registers; the partner scans are latency-bound, and
-// more resident warps beat the spills (160,000 attempts: 168 us)
+// more resident warps beat the spills (160,000 attempts: 157 us)
 __global__ void __launch_bounds__(32 * EVAL_WARPS_U, 12) k_db_eval(const SimDev *__restrict__ Sp,
                                                               const StageDev *__restrict__ stp,
                                                               const double *__restrict__ x,

@@ -264,7 +264,7 @@ __device__ __forceinline__ DBC make_dbc(const SimDev &S, const StageDev &st, int
 // slowest one, so it is cut in two: the draw and the partner scan of the drawn
 // bond, one warp per record (most sets are empty, and done); then, for a
 // non-empty set, E::TASKS independent parts on as many warps.  160,000
-// attempts of a 1.6M-monomer melt (21 swaps): 536 us, against about 1,450 as two
+// attempts of a 1.6M-monomer melt (21 swaps): 521 us, against about 1,450 as two
 // launches a round with the host reading the finished flags now and then, an
 // attempt evaluated by one warp and the dE of a swap by one lane.
 // round[RS m + 0..5] of one of two buffers (by round parity: commits write the

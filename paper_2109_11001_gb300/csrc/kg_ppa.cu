@@ -521,7 +521,10 @@ __device__ __forceinline__ unsigned long long unpermute_one(const PpaArgs &a, in
 }
 
 // positions back to slot order; the largest net force on a mobile monomer
-// (a warp maximum, then one atomic per warp) and the sum of the list lengths
+// (a warp maximum, then one atomic per warp) and the sum of the list lengths.
+// A first build cut short (a cell over PPA_CELL_CAP: flags[2] is 0) has not
+// written the index arrays, which are not cleared beforehand, and nothing has
+// moved: buffer 0 holds the positions in slot order.
 __global__ void __launch_bounds__(256) k_ppa_unpermute(PpaArgs a, double *__restrict__ xs,
                                                       unsigned long long *__restrict__ fmax_bits,
                                                       unsigned long long *__restrict__ nn_sum)
@@ -529,9 +532,12 @@ __global__ void __launch_bounds__(256) k_ppa_unpermute(PpaArgs a, double *__rest
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long fb = 0ull;                      // bits of a non-negative double order like it
     unsigned long long nb = 0ull;
-    if (s < a.M) {
+    if (s < a.M && a.flags[2]) {
         fb = unpermute_one(a, s, xs);
         nb = (unsigned long long)a.nn[s];              // list lengths, storage order (any order sums)
+    } else if (s < a.M) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) xs[(size_t)d * a.M + s] = a.x0[(size_t)d * a.M + s];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

@@ -153,13 +153,13 @@ struct UniformEval {
     const float4 *rec;
     const int *comp_of, *slot_of;
     long long sweep;
-    unsigned *flags;
+    unsigned *errw;              // RoundArgs::errw
     WarpCand *wc;                // set by the kernel
     static constexpr int TASKS = UNIFORM_TASKS;
     __device__ DBC dbc(int m) const { return make_dbc(*S, *st, m, x, pid, cell, start, list, rec, st->T); }
     __device__ void say(unsigned err) const
     {
-        if (err && (threadIdx.x & 31) == 0) atomicOr(flags, err);
+        if (err && (threadIdx.x & 31) == 0) atomicOr(errw, err);
     }
     __device__ void scan(int m, int k, int, Attempt &a)
     {
@@ -290,6 +290,7 @@ RoundArgs round_args(kg_ctx *c)
     r.old = (int *)c->scratch;
     r.stats = c->db_stats;
     r.flags = c->flags;
+    r.errw = (unsigned *)(c->dbbar + 3);
     return r;
 }
 
@@ -308,9 +309,10 @@ cudaError_t db_sweep(kg_ctx *c, const std::vector<long long> &K, long long *host
             c->slot_of, att, c->sweep, c->flags);
     // ordered commit in rounds (kg_db.cuh)
     db_rounds_reset(c);
+    const RoundArgs ra = round_args(c);
     const UniformEval ev{c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist, c->dbrec,
-                         c->comp_of, c->slot_of, c->sweep, c->flags, nullptr};
-    const cudaError_t e = rounds_launch(c, k_db_rounds, 32 * ROUND_WARPS, 0, tot, nm, round_args(c), ev);
+                         c->comp_of, c->slot_of, c->sweep, ra.errw, nullptr};
+    const cudaError_t e = rounds_launch(c, k_db_rounds, 32 * ROUND_WARPS, 0, tot, nm, ra, ev);
     if (e != cudaSuccess) return e;
     c->launches += 1;
     db_finish(c, host_stats);

@@ -294,6 +294,7 @@ struct RoundArgs {
     int *old;                    // [2 M]: slot maps of the two chains of a commit, per melt
     long long *stats;
     unsigned *flags;
+    unsigned *errw;              // error bits of this launch (zero at launch), the evaluator's among them
     unsigned long long *bar;     // three barrier words, zero at launch
     unsigned spin;
     long long most;              // rounds (attempts + 1)
@@ -496,29 +497,34 @@ __device__ bool commit_pass(P &pol, const RoundArgs &A, int m, const int *round,
     return true;
 }
 
-// all rounds of a sweep; every block of a cooperative launch (ev, pol as above)
+// All rounds of a sweep; every block of a cooperative launch (ev, pol as above).
+// Errors of the evaluations go to a word of this launch, so the status word is
+// the same for a block however late it starts: block 0 writes it after a
+// barrier at which every block has arrived.  A round that saw an error ends the
+// sweep before its commit.
 template <int THREADS, class E, class P>
 __device__ void rounds_body(E &ev, P &pol, const RoundArgs &R)
 {
-    __shared__ unsigned acc_s[2], out_s;
-    const bool stop = *(volatile unsigned *)R.flags != 0u;     // a latched error stops the sweep; written only after
-    if (threadIdx.x < 2) acc_s[threadIdx.x] = 0u;              //   every block has arrived at the first barrier
+    __shared__ unsigned acc_s[2], out_s, stop_s;
+    if (threadIdx.x < 2) acc_s[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) stop_s = *(volatile unsigned *)R.flags;
     __syncthreads();
-    if (stop) return;
+    if (stop_s) return;                                        // a latched error stops the sweep
     GridBar gb{R.bar, acc_s, &out_s, R.spin, 0};
     unsigned told = 0;
     for (long long r = 0; r <= R.most; ++r) {
         int *round = R.round + (r & 1) * RS * MAX_MELTS, *next = R.round + ((r + 1) & 1) * RS * MAX_MELTS;
         restale_pass<THREADS>(ev, R, round, r == 0);
-        if (threadIdx.x == 0 && r > 0 && *(volatile unsigned *)R.flags) gb.note(FAIL);
+        if (threadIdx.x == 0 && *(volatile unsigned *)R.errw) gb.note(FAIL);
         if ((told = gb.sync()) & (FAIL | GAVE_UP)) break;
         bool left = false;
         for (int m = 0; m < R.sim->n_melts; ++m) left |= commit_pass(pol, R, m, round, next);
         if (threadIdx.x == 0 && left) gb.note(REQ);
         told = gb.sync();
-        if (!(told & REQ) || (told & (FAIL | GAVE_UP))) break;
+        if (!(told & REQ) || (told & GAVE_UP)) break;
     }
     if (threadIdx.x == 0 && (told & GAVE_UP)) atomicOr(R.flags, ERR_TIMEOUT);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (told & FAIL)) atomicOr(R.flags, *(volatile unsigned *)R.errw);
 }
 
 RoundArgs round_args(kg_ctx *c);                // kg_db.cu
@@ -538,7 +544,7 @@ cudaError_t rounds_launch(kg_ctx *c, KERNEL K, int threads, size_t smem, long lo
     if (per < 1) return cudaErrorCooperativeLaunchTooLarge;
     const long long want = (tot + threads - 1) / threads;      // a thread looks at one record
     const long long nb = std::min((long long)per * nsm, std::max((long long)nm, std::max(want, 1LL)));
-    e = cudaMemsetAsync(c->dbbar, 0, 3 * sizeof(unsigned long long), c->stream);
+    e = cudaMemsetAsync(c->dbbar, 0, 4 * sizeof(unsigned long long), c->stream);   // and the error word
     if (e != cudaSuccess) return e;
     r.bar = c->dbbar;
     r.spin = ROUNDS_SPIN;

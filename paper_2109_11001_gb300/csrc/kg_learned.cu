@@ -338,7 +338,7 @@ struct LearnedEval {
     const int *pid, *cell, *start, *list;
     const int *comp_of, *slot_of;
     long long sweep;
-    unsigned *flags;
+    unsigned *errw;              // RoundArgs::errw
     LearnedArgs la;
     const MlpSmem *W;            // set by the kernel
     WarpProp *wp;
@@ -346,7 +346,7 @@ struct LearnedEval {
     __device__ DBC dbc(int m) const { return make_dbc(*S, *st, m, x, pid, cell, start, list, la.rec, st->T); }
     __device__ void say(unsigned err) const
     {
-        if (err && (threadIdx.x & 31) == 0) atomicOr(flags, err);
+        if (err && (threadIdx.x & 31) == 0) atomicOr(errw, err);
     }
     __device__ void scan(int m, int k, int g, Attempt &a)
     {
@@ -372,7 +372,7 @@ struct LearnedEval {
     {
         const double q_fwd = a.p + p[0], q_rev = p[1] + p[2];
         if (!(q_rev > 0.0) || !(q_fwd > 0.0)) {
-            atomicOr(flags, ERR_DB_INTERNAL);
+            atomicOr(errw, ERR_DB_INTERNAL);
             return false;
         }
         return accept_u(S->seed, m, sweep, k) < exp(-a.dE / st->T) * q_rev / q_fwd;
@@ -543,9 +543,10 @@ cudaError_t db_sweep_learned(kg_ctx *c, const std::vector<long long> &K, double 
     // ordered commit in rounds (kg_db.cuh)
     db_rounds_reset(c);
     cudaFuncSetAttribute(k_dbl_rounds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eval_smem());
+    const RoundArgs ra = round_args(c);
     const LearnedEval ev{c->d_sim, c->d_stage, c->x, c->pid, c->dbcell, c->dbstart, c->dblist,
-                         c->comp_of, c->slot_of, c->sweep, c->flags, la, nullptr, nullptr};
-    const cudaError_t e = rounds_launch(c, k_dbl_rounds, 32 * EVAL_WARPS, eval_smem(), tot, nm, round_args(c), ev);
+                         c->comp_of, c->slot_of, c->sweep, ra.errw, la, nullptr, nullptr};
+    const cudaError_t e = rounds_launch(c, k_dbl_rounds, 32 * EVAL_WARPS, eval_smem(), tot, nm, ra, ev);
     if (e != cudaSuccess) return e;
     c->launches += 2;
     if (log && tot > 0) {

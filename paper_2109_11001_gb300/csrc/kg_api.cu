@@ -21,15 +21,28 @@ using kg::dev_free;
 namespace kg {
 
 // A program that passes no stream usually works on the default stream: the
-// inputs it hands over, and buffers that its allocator hands out again, can
-// still be in use by work queued there, which a non-blocking stream does not
-// wait for by itself.
+// inputs and output buffers it hands over, and memory that its allocator hands
+// out again, can still be in use by work queued there, which a non-blocking
+// stream does not wait for by itself.  Nothing to do if that work is done,
+// which the query tells for less than the event and the wait cost.
 void follow_default(kg_ctx *c)
 {
-    if (!c->own_stream) return;
+    if (!c->own_stream || cudaStreamQuery(cudaStreamLegacy) == cudaSuccess) return;
+    cudaGetLastError();
     if (!c->order_ev && cudaEventCreateWithFlags(&c->order_ev, cudaEventDisableTiming) != cudaSuccess) return;
     cudaEventRecord(c->order_ev, cudaStreamLegacy);
     cudaStreamWaitEvent(c->stream, c->order_ev, 0);
+}
+
+void follow_default_for(kg_ctx *c, const void *out)
+{
+    cudaPointerAttributes a;
+    if (!out || !c->own_stream) return;
+    if (cudaPointerGetAttributes(&a, out) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) follow_default(c);
 }
 
 void *dev_alloc(kg_ctx *c, size_t bytes, size_t clear)
@@ -537,6 +550,7 @@ kg_status kg_get_config(kg_ctx *c, int melt, double *x, double *v, int *pid)
     const size_t Mm = md.M;
     // one kernel for everything asked for, into the caller's memory where it
     // is this GPU's, else into scratch and copied from there
+    for (const void *out : {(const void *)x, (const void *)v, (const void *)pid}) kg::follow_default_for(c, out);
     const char *lo[3] = {(const char *)x, (const char *)v, (const char *)pid};
     const size_t bytes[3] = {3 * Mm * sizeof(double), 3 * Mm * sizeof(double), Mm * sizeof(int)};
     bool direct = true;                                    // no two outputs share memory
@@ -968,6 +982,7 @@ kg_status kg_forces(kg_ctx *c, int melt, double *F, double *e4)
     const size_t Mm = md.M, Mp = c->Mp;
     if (F) {
         kg::to_slots(c, melt, c->fout, c->scratch, 3);
+        kg::follow_default_for(c, F);
         KG_TRY(cudaMemcpyAsync(F, c->scratch, 3 * Mm * sizeof(double), cudaMemcpyDefault, c->stream));
     }
     std::vector<double> part((size_t)nb * 5);
@@ -1203,6 +1218,7 @@ kg_status kg_observables(kg_ctx *c, int melt, kg_obs *out, double *r2n, double *
     if (r2n) {
         if (md.N > KG_R2N_MAX_CHAIN_LEN) return KG_ERR_INVALID_ARG;
         if (!kg::r2n_eval(c, melt, c->scratch)) return KG_ERR_CUDA;
+        kg::follow_default_for(c, r2n);
         KG_TRY(cudaMemcpyAsync(r2n, c->scratch, sizeof(double) * md.N, cudaMemcpyDefault, c->stream));
     }
     if (bond_hist || cos_hist) {

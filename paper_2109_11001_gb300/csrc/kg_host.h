@@ -141,9 +141,10 @@ struct kg_ctx {
 
 namespace kg {
 
-// device memory through the context's allocator (zero-filled on the context's stream)
 // a context's own stream waits for the work queued on the default stream so far
 void follow_default(kg_ctx *c);
+void follow_default_for(kg_ctx *c, const void *out);   // the same before it writes a caller's device memory
+// device memory through the context's allocator (zero-filled on the context's stream)
 void *dev_alloc(kg_ctx *c, size_t bytes, size_t clear = ~(size_t)0);   // the first `clear` bytes zero
 void dev_free(kg_ctx *c, void *p);
 

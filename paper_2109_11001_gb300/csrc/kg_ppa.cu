@@ -766,6 +766,7 @@ kg_status kg_primitive_path(kg_ctx *c, int melt, const kg_ppa_params *pp, double
         cudaMemcpyAsync(h_flags, a.flags, sizeof(h_flags), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaMemcpyAsync(h_fmax, d_fmax, sizeof(h_fmax), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return done(KG_ERR_CUDA);
+    kg::follow_default_for(c, x_out);
     if (x_out && cudaMemcpyAsync(x_out, d_xs, sizeof(double) * m3, cudaMemcpyDefault, st) != cudaSuccess)
         return done(KG_ERR_CUDA);
     if (cudaStreamSynchronize(st) != cudaSuccess) return done(KG_ERR_CUDA);

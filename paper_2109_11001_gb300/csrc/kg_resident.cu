@@ -207,13 +207,22 @@ __global__ void __launch_bounds__(RES_BLOCK, RES_MIN_BLOCKS) k_resident(const __
 // while a block has one tile of 256).  Every block has to be resident at once;
 // the limits are what the kernels' __launch_bounds__ guarantee for every
 // exponent.
+//
+// Dilute systems: a list build scans every cell, here from a block per 64 to
+// 256 monomers, there from the whole GPU.  At 85 to 90 cells per monomer the
+// resident loops are still ahead (us per step against the captured loop; 1,000
+// monomers 7.8 / 9.4, 19,000 9.5 / 14.1, 90,000 17.3 / 31.2), the work per
+// block grows with the cells, and no use of so empty a box is known, so the
+// rule ends there.
 constexpr int TILED_MOST = 5 * 256;
+constexpr long long DILUTE_CELLS = 64;           // cells per monomer
 
 int resident_kind(kg_ctx *c)
 {
     if (c->precision != KG_MIXED || c->resident_failed) return RES_NONE;
     if (c->tpm != 1 && !(c->p.flags & KG_FLAG_PERSISTENT)) return RES_NONE;
     if (c->res_sms < 0) cudaDeviceGetAttribute(&c->res_sms, cudaDevAttrMultiProcessorCount, c->device);
+    if (c->ncell_md > DILUTE_CELLS * c->M + 4096) return c->p.flags & KG_FLAG_PERSISTENT ? RES_TILED : RES_NONE;
     if (c->buckets && c->M <= SMALL_OWN * SMALL_MIN_BLOCKS * c->res_sms) return RES_SMALL;
     if (c->M <= RES_BLOCK * RES_MIN_BLOCKS * c->res_sms) return RES_WIDE;
     return c->M <= TILED_MOST * c->res_sms || (c->p.flags & KG_FLAG_PERSISTENT) ? RES_TILED : RES_NONE;
@@ -268,9 +277,14 @@ cudaError_t resident_launch(kg_ctx *c, int K, int skip_block, unsigned spin)
 }
 
 // Barrier words and segment totals; for the small kernel bucket counts (two
-// sets), members and records.  Cells of the usual grids hold 2.4 to 5
-// monomers; grids whose mean is above a third of a bucket (cell_scale well
-// above 1) do not use them.
+// sets), members and records, 648 bytes a cell.  Cells of the usual grids hold
+// 2.4 to 5 monomers; grids whose mean is above a third of a bucket (cell_scale
+// well above 1) do not use them, nor do those with more than eight cells per
+// monomer: a thousand monomers in a box of side 500 have 44 million cells.  At
+// the limit the buckets of 19,000 monomers take 100 MB (one thread per monomer
+// without them: 7.4 against 6.0 us per step there).
+constexpr long long BUCKET_CELLS = 8;            // cells per monomer
+
 bool resident_alloc(kg_ctx *c)
 {
     double most = 0.0;
@@ -278,7 +292,7 @@ bool resident_alloc(kg_ctx *c)
         const MeltDev &md = c->sim.melt[m];
         most = std::max(most, (double)md.M / ((double)md.nc * md.nc * md.nc));
     }
-    c->buckets = 3.0 * most <= BUCKET;
+    c->buckets = 3.0 * most <= BUCKET && c->ncell_md <= BUCKET_CELLS * c->M + 512;
     const int kind = resident_kind(c);
     if (c->precision != KG_MIXED) return true;
     c->resbar = (unsigned long long *)dev_alloc(c, 4 * sizeof(unsigned long long) +

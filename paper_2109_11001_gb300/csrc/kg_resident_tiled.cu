@@ -104,7 +104,9 @@ __global__ void __launch_bounds__(TILE, 5) k_resident_tiled(const __grid_constan
 
 cudaError_t tiled_launch(const ResArgs &a, int n4, int sms, cudaStream_t st)
 {
-    const int nb = std::min((a.st.M + TILE - 1) / TILE, 5 * sms);      // what __launch_bounds__ guarantees
+    // a block per tile, or (dilute systems) per segment of the cells that a list
+    // build scans, up to what __launch_bounds__ guarantees
+    const int nb = std::min(std::max((a.st.M + TILE - 1) / TILE, (a.ncell + RES_SEG - 1) / RES_SEG), 5 * sms);
     return KG_RESIDENT_LAUNCH(k_resident_tiled, n4, nb, TILE, a, st);
 }
 

@@ -219,9 +219,9 @@ constexpr long long DILUTE_CELLS = 64;           // cells per monomer
 
 int resident_kind(kg_ctx *c)
 {
+    if (c->res_sms < 0) cudaDeviceGetAttribute(&c->res_sms, cudaDevAttrMultiProcessorCount, c->device);
     if (c->precision != KG_MIXED || c->resident_failed) return RES_NONE;
     if (c->tpm != 1 && !(c->p.flags & KG_FLAG_PERSISTENT)) return RES_NONE;
-    if (c->res_sms < 0) cudaDeviceGetAttribute(&c->res_sms, cudaDevAttrMultiProcessorCount, c->device);
     if (c->ncell_md > DILUTE_CELLS * c->M + 4096) return c->p.flags & KG_FLAG_PERSISTENT ? RES_TILED : RES_NONE;
     if (c->buckets && c->M <= SMALL_OWN * SMALL_MIN_BLOCKS * c->res_sms) return RES_SMALL;
     if (c->M <= RES_BLOCK * RES_MIN_BLOCKS * c->res_sms) return RES_WIDE;

@@ -308,6 +308,16 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
             md.nl_lo = (float)(rl * rl - 2.0 * er2);
             md.nl_hi = (float)(rl * rl + 2.0 * er2);
         }
+        {   // near test of the binary64 step on gather records: offset (<= h) and
+            // displacement (<= skin / 2) are rounded once each and once as their
+            // sum, for both monomers; their difference (<= h + skin), the cell
+            // side and the shifted difference (<= r_c near the cutoff) once each.
+            // The margin is twice the resulting bound at r_c, 2e-5 r_c^2 at least
+            // (the usual cells need a quarter of that).
+            const double ec = (6.0 * md.h + 3.0 * c->p.skin + RC) * std::ldexp(1.0, -24);
+            const double er2 = 2.0 * RC * std::sqrt(3.0) * ec + 3.0 * ec * ec + 4.0 * RC * RC * std::ldexp(1.0, -24);
+            md.near2 = (float)(RC * RC + std::max(2.0 * er2, 2e-5 * RC * RC));
+        }
         if (md.nc > (1 << kg::CODE_BITS)) return fail(KG_ERR_INVALID_ARG);
         md.hdb = ml.box / md.ndb; md.invhdb = 1.0 / md.hdb;
         md.hdbf = (float)md.hdb;

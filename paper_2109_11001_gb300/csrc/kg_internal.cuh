@@ -101,6 +101,7 @@ struct MeltDev {
     double h, invh;
     float hf;
     float nl_lo, nl_hi;      // binary32 prefilter: r^2 < nl_lo in, r^2 >= nl_hi out
+    float near2;             // binary64 step: pairs with r^2 >= near2 on the gather records lie beyond r_c
     // double-bridging grid (cells >= db_bond_max); binary32 records on it decide
     // the swap-bond criterion outside the band [db_lo, db_hi) around db_bond_max^2
     int ndb, dbcell_off;

@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(F64_BLOCK) k_step_f64(const SimDev *__restrict
         const MeltDev &md = S.melt[melt_of(S, slot)];
         const unsigned *__restrict__ col = nl + s;
         const float4 gi = __ldg(gcur + (live ? s : 0));
-        const float h = md.hf, near2 = S.rc2f * (1.0f + 2e-5f);   // >> the records' rounding (~1e-6 in r^2)
+        const float h = md.hf, near2 = md.near2;
         for (int k0 = 0; k0 < kmax; k0 += 32) {
             unsigned mask = 0;
             const int kn = min(32, cnt - k0);

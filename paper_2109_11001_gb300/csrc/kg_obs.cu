@@ -10,31 +10,72 @@
 
 namespace kg {
 
+// <R^2(n)> of short chains in binary64: one thread per chain and lag, one warp
+// per block with as many chains as fit (a step of a warp is seven operations of
+// the binary64 pipe, 112 clocks of an SM's; four warps a block took 2 us more for
+// few chains).  The scaling and the two reductions that the kernel below needs
+// first cost about 3 us, which short chains do not earn back.  In us, the former
+// binary64 kernel / this / the one below, with the sum over chains: 3 chains of 3
+// 8.0 / 8.3 / 10.5, 10 of 20 12.4 / 13.6 / 12.5, 10,000 of 3 692 / 101 / 164, 10,000
+// of 20 738 / 197 / 183.
+constexpr int R2N_SHORT = 20, R2N_THREADS = 128;
+
+__global__ void __launch_bounds__(32) k_r2n_short(const double *__restrict__ x, long long Mp, int off, int n_ch, int N,
+                                                 double *__restrict__ out /* [n_ch][N] */,
+                                                 const int *__restrict__ comp_of /* NULL: slot order */)
+{
+    __shared__ double pos[3][32];
+    const int per = 32 / N, c0 = blockIdx.x * per, n_here = min(per, n_ch - c0) * N;
+    const int t = threadIdx.x, n = t % N;
+    const long long base = (long long)off + (long long)c0 * N;
+    if (t < n_here) {
+        const long long j = comp_of ? (long long)comp_of[base + t] : base + t;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) pos[d][t] = x[d * Mp + j];
+    }
+    __syncwarp();
+    if (t >= n_here) return;
+    double s = 0.0;
+    if (n > 0)
+        for (int i = t - n; i + n < t - n + N; ++i) {
+            const double dx = pos[0][i + n] - pos[0][i], dy = pos[1][i + n] - pos[1][i], dz = pos[2][i + n] - pos[2][i];
+            s += dx * dx + dy * dy + dz * dz;
+        }
+    out[(size_t)c0 * N + t] = s;
+}
+
 // <R^2(n)> of one chain and a share of its lags (block (c, y) of gridDim.y):
 // sum_i |x_{i+n} - x_i|^2 for every lag n.  In binary64 the three differences
 // and three fused multiply-adds of a pair are 96 clocks of an SM's binary64
-// pipe per warp (two lanes a clock), and nothing else counts: 500 chains of
-// 800 took 2584 us, and take 518 us here (the wide integer multiplies bound it).  Here a chain's positions become 53-bit integers t = (x -
-// x_0) 2^(52-e), 2^e above the chain's extent, split as t = 2^30 hi + lo, and a
-// pair's t^2 = 2^60 dhi^2 + 2^31 dhi dlo + dlo^2 is three products a component,
+// pipe per warp (two lanes a clock), and nothing else counts.  Here a chain's
+// positions become 53-bit integers t = (x - x_0) 2^(52-e), 2^e above the chain's
+// extent, split as t = 2^30 hi + lo, and a pair's t^2 = 2^60 dhi^2 + 2^31 dhi dlo + dlo^2 is three products a component,
 // accumulated as 64-bit integers: dhi^2 exactly, dhi dlo exactly (moved to
 // binary64 every R2N_CHUNK terms, before it can overflow), dlo^2 from the upper
 // 22 of its 30 bits (2^-21 of a unit of dhi^2).  The quantum, 2^(e-52), is of
 // the order of one binary64 ulp at the chain's extent.
-// A thread takes R2N_W consecutive lags at once: monomer i + n0 + k serves lag
+// A thread takes W consecutive lags at once: monomer i + n0 + k serves lag
 // k of step i and lag k - 1 of step i + 1, so one shared-memory read of a
 // position (six words, each array padded by one word in 32 against bank
-// conflicts between lanes four monomers apart) serves R2N_W pairs.  The window
+// conflicts between lanes four monomers apart) serves W pairs.  The window
 // at the short end of the lags and its mirror image at the long end go to
 // the same thread, so threads have equal work.
+// W is 4 where that fills the GPU, where the wide integer multiplies bound it
+// (r2n_launch), else 1: four times as many threads with a quarter of the work,
+// and a step of one warp alone is a chain of latencies.  In us, binary64 / W = 4 /
+// W = 1, with the sum over chains: 20 chains of 100 33 / 45 / 21, 10 of 200 68 /
+// 83 / 31, 3 of 1600 2623 / 431 / 149, 100 of 800 712 / 238 / 150; 300 of 800 1351
+// / 312 / 350, 1000 of 1600 17802 / 2899 / 3474.  W = 2 is nowhere the best by
+// more than 2%.
 // A chain with a position that is not finite takes binary64, which says so.
 // The row stride Mp is 64-bit: a caller's rows may sit 2^30 or more doubles
 // apart, and every index into x is formed in 64-bit arithmetic.
-constexpr int R2N_W = 4, R2N_CHUNK = 256, R2N_THREADS = 128;
+constexpr int R2N_CHUNK = 256;
 
 // words of one of the six arrays of a chain of N monomers; sh: padding shift (31: none, the longest chains)
 __host__ __device__ __forceinline__ int r2n_words(int N, int sh) { return N + (N >> sh); }
 
+template <int W>
 __global__ void __launch_bounds__(R2N_THREADS) k_r2n_chain(const double *__restrict__ x, long long Mp, int off, int N,
                                                           double *__restrict__ out /* [n_ch][N] */,
                                                           const int *__restrict__ comp_of /* NULL: slot order */,
@@ -93,7 +134,7 @@ __global__ void __launch_bounds__(R2N_THREADS) k_r2n_chain(const double *__restr
     }
     __syncthreads();
     const double unit = scalbn(1.0, 2 * (e - 52) + 30);
-    const int nwin = (N - 1 + R2N_W - 1) / R2N_W;   // windows of lags 1 + R2N_W w ...
+    const int nwin = (N - 1 + W - 1) / W;   // windows of lags 1 + W w ...
     auto get = [&](int i, int *p) {
         const int w = i + (i >> sh);
 #pragma unroll
@@ -103,12 +144,12 @@ __global__ void __launch_bounds__(R2N_THREADS) k_r2n_chain(const double *__restr
         for (int half = 0; half < 2; ++half) {
             const int w = half ? nwin - 1 - u : u;
             if (half && w == u) break;
-            const int n0 = 1 + R2N_W * w;
-            long long hh[R2N_W], hl[R2N_W], ll[R2N_W];
-            double mid[R2N_W];
-            int ring[R2N_W][6];                      // monomers i + n0 ... i + n0 + 3, at (i + k) % 4
+            const int n0 = 1 + W * w;
+            long long hh[W], hl[W], ll[W];
+            double mid[W];
+            int ring[W][6];                      // monomers i + n0 ... i + n0 + 3, at (i + k) % 4
 #pragma unroll
-            for (int k = 0; k < R2N_W; ++k) {
+            for (int k = 0; k < W; ++k) {
                 hh[k] = hl[k] = ll[k] = 0;
                 mid[k] = 0.0;
                 if (k) get(min(n0 + k - 1, N - 1), ring[k - 1]);
@@ -122,37 +163,38 @@ __global__ void __launch_bounds__(R2N_THREADS) k_r2n_chain(const double *__restr
                     ll[k] += (long long)dq * dq;
                 }
             };
-            const int full = max(0, N - n0 - (R2N_W - 1));      // steps whose R2N_W lags all end in the chain
+            const int full = max(0, N - n0 - (W - 1));      // steps whose W lags all end in the chain
             int i = 0;
-            for (; i + R2N_W <= full; i += R2N_W) {
+#pragma unroll (W == 1 ? 4 : 1)
+            for (; i + W <= full; i += W) {
 #pragma unroll
-                for (int r = 0; r < R2N_W; ++r) {
+                for (int r = 0; r < W; ++r) {
                     int a[6];
                     get(i + r, a);
-                    get(i + r + n0 + R2N_W - 1, ring[(r + R2N_W - 1) % R2N_W]);
+                    get(i + r + n0 + W - 1, ring[(r + W - 1) % W]);
 #pragma unroll
-                    for (int k = 0; k < R2N_W; ++k) pair(k, a, ring[(r + k) % R2N_W]);
+                    for (int k = 0; k < W; ++k) pair(k, a, ring[(r + k) % W]);
                 }
-                if ((i & (R2N_CHUNK - 1)) == R2N_CHUNK - R2N_W) {
+                if ((i & (R2N_CHUNK - 1)) == R2N_CHUNK - W) {
 #pragma unroll
-                    for (int k = 0; k < R2N_W; ++k) {
+                    for (int k = 0; k < W; ++k) {
                         mid[k] += (double)hl[k];
                         hl[k] = 0;
                     }
                 }
             }
-            for (; i + n0 < N; ++i) {                // the ends, lag by lag (at most 2 R2N_W - 2 steps)
+            for (; i + n0 < N; ++i) {                // the ends, lag by lag (at most 2 W - 2 steps)
                 int a[6], p[6];
                 get(i, a);
 #pragma unroll
-                for (int k = 0; k < R2N_W; ++k)
+                for (int k = 0; k < W; ++k)
                     if (i + n0 + k < N) {
                         get(i + n0 + k, p);
                         pair(k, a, p);
                     }
             }
 #pragma unroll
-            for (int k = 0; k < R2N_W; ++k)
+            for (int k = 0; k < W; ++k)
                 if (n0 + k < N)
                     out[(size_t)c * N + n0 + k] =
                         ((double)hh[k] * 1073741824.0 + (2.0 * (mid[k] + (double)hl[k]) + (double)ll[k] * 6.103515625e-05)) *
@@ -278,28 +320,55 @@ __global__ void __launch_bounds__(256) k_hist(const double *__restrict__ x, int 
 // Dynamic shared memory of k_r2n_chain for chains of N monomers (six words a
 // monomer, padded where that fits); above 48 KiB the kernel's opt-in limit is
 // raised first.  False if N is too long.
+template <int W>
 static bool r2n_shared(int N, size_t &smem, int &sh)
 {
     sh = 24 * (size_t)r2n_words(N, 5) <= (size_t)R2N_SMEM_MAX ? 5 : 31;
     smem = 24 * (size_t)r2n_words(N, sh);
     if (N < 1 || smem > (size_t)R2N_SMEM_MAX) return false;
     if (smem <= 48 * 1024 - 256) return true;
-    return cudaFuncSetAttribute(k_r2n_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+    return cudaFuncSetAttribute(k_r2n_chain<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+}
+
+// blocks of a chain when each thread takes two windows of W lags
+template <int W>
+static int r2n_split(int N)
+{
+    const int pairs = ((N - 1 + W - 1) / W + 1) / 2;
+    return std::max(1, (pairs + R2N_THREADS - 1) / R2N_THREADS);
+}
+
+template <int W>
+static bool r2n_chains(const double *x, long long Mp, int off, int n_ch, int N, const int *comp_of, double *tmp,
+                       cudaStream_t st)
+{
+    size_t smem = 0;
+    int sh = 5;
+    if (!r2n_shared<W>(N, smem, sh)) return false;
+    // few chains: the lags of a chain over several blocks, to about eight per SM
+    const int split = std::max(1, std::min(r2n_split<W>(N), 152 * 8 / n_ch));
+    k_r2n_chain<W><<<dim3(n_ch, split), R2N_THREADS, smem, st>>>(x, Mp, off, N, tmp, comp_of, sh);
+    return cudaGetLastError() == cudaSuccess;
 }
 
 // <R^2(n)> of n_ch chains of N monomers from x (rows Mp apart); tmp: [n_ch][N]
 static bool r2n_launch(const double *x, long long Mp, int off, int n_ch, int N, const int *comp_of, double *tmp,
                        double *out, cudaStream_t st)
 {
-    size_t smem = 0;
-    int sh = 5;
-    if (!r2n_shared(N, smem, sh)) return false;
-    // few chains: the lags of a chain over several blocks, to about eight per SM
-    const int pairs = ((N - 1 + R2N_W - 1) / R2N_W + 1) / 2;
-    const int most = std::max(1, (pairs + R2N_THREADS - 1) / R2N_THREADS);
-    const int split = std::max(1, std::min(most, 152 * 8 / n_ch));
-    k_r2n_chain<<<dim3(n_ch, split), R2N_THREADS, smem, st>>>(x, Mp, off, N, tmp, comp_of, sh);
-    if (cudaGetLastError() != cudaSuccess) return false;
+    if (N <= R2N_SHORT) {
+        const int per = 32 / N;
+        k_r2n_short<<<(n_ch + per - 1) / per, 32, 0, st>>>(x, Mp, off, n_ch, N, tmp, comp_of);
+        if (cudaGetLastError() != cudaSuccess) return false;
+    } else {
+        // four lags a thread: blocks three quarters full, two or more per SM
+        // (300 of 800: 312 against 350 us, 100 of 800: 238 / 150; 1000 of 400,
+        // blocks 39% full: 389 / 302)
+        const int split = r2n_split<4>(N), pairs = (N + 6) / 8;
+        const bool four = 4 * pairs >= 3 * split * R2N_THREADS && (long long)n_ch * split >= 2 * 150;
+        if (!(four ? r2n_chains<4>(x, Mp, off, n_ch, N, comp_of, tmp, st)
+                   : r2n_chains<1>(x, Mp, off, n_ch, N, comp_of, tmp, st)))
+            return false;
+    }
     k_r2n_reduce<<<(N + 31) / 32, dim3(32, R2N_ROWS), 0, st>>>(tmp, n_ch, N, out);
     return cudaGetLastError() == cudaSuccess;
 }

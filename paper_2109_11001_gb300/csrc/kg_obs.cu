@@ -67,10 +67,16 @@ __global__ void __launch_bounds__(32) k_r2n_short(const double *__restrict__ x, 
 // 83 / 31, 3 of 1600 2623 / 431 / 149, 100 of 800 712 / 238 / 150; 300 of 800 1351
 // / 312 / 350, 1000 of 1600 17802 / 2899 / 3474.  W = 2 is nowhere the best by
 // more than 2%.
-// A chain with a position that is not finite takes binary64, which says so.
+// A chain with a position that is not finite takes binary64, which says so, and
+// so does one whose extent is more than R2N_EXTENT times its shortest bond: the
+// quantum goes with the extent and the differences of near monomers are exact in
+// binary64 (chains of 1600 at kappa = 3.5 reach about 400; the sums' error stays
+// below binary64's for walks, as emulated in 128 bits: 1e-16 against 1e-16 to 5e-16
+// for 2 x 20 to 30 x 800; straight rods pass it from 1,500 to 2,000 monomers).
 // The row stride Mp is 64-bit: a caller's rows may sit 2^30 or more doubles
 // apart, and every index into x is formed in 64-bit arithmetic.
 constexpr int R2N_CHUNK = 256;
+constexpr float R2N_EXTENT = 2048.0f;
 
 // words of one of the six arrays of a chain of N monomers; sh: padding shift (31: none, the longest chains)
 __host__ __device__ __forceinline__ int r2n_words(int N, int sh) { return N + (N >> sh); }
@@ -82,30 +88,48 @@ __global__ void __launch_bounds__(R2N_THREADS) k_r2n_chain(const double *__restr
                                                           int sh)
 {
     extern __shared__ __align__(16) int words[];   // hi x, y, z, lo x, y, z (first the warps' extents)
-    static_assert(2 * 24 >= 8 * (R2N_THREADS / 32), "the extents fit the shortest chain's words");
+    static_assert((R2N_SHORT + 1) * 24 >= 12 * (R2N_THREADS / 32), "the extents and bonds fit the shortest chain's words");
     double *ext_s = reinterpret_cast<double *>(words);
+    float *bond_s = reinterpret_cast<float *>(ext_s + R2N_THREADS / 32);
     const int c = blockIdx.x, P = r2n_words(N, sh);
     const long long base = (long long)off + (long long)c * N;
     const long long j0 = comp_of ? (long long)comp_of[base] : base;
     const double o[3] = {x[j0], x[Mp + j0], x[2 * Mp + j0]};
     double ext = 0.0;
+    float bond2 = 3.0e38f;                          // the shortest bond, squared
     bool bad = false;
     for (int i = threadIdx.x; i < N; i += R2N_THREADS) {
         const long long j = comp_of ? (long long)comp_of[base + i] : base + i;
+        const int i1 = min(i + 1, N - 1);
+        const long long j1 = comp_of ? (long long)comp_of[base + i1] : base + i1;
+        float b2 = 0.f;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const double t = fabs(x[d * Mp + j] - o[d]);
+            const double xd = x[d * Mp + j], t = fabs(xd - o[d]);
+            const float b = f64_to_f32(x[d * Mp + j1] - xd);
             bad |= !isfinite(t);
             ext = fmax(ext, t);
+            b2 = fmaf(b, b, b2);
         }
+        if (i1 > i) bond2 = fminf(bond2, b2);
     }
 #pragma unroll
-    for (int w = 16; w > 0; w >>= 1) ext = fmax(ext, __shfl_xor_sync(0xffffffffu, ext, w));
-    if ((threadIdx.x & 31) == 0) ext_s[threadIdx.x >> 5] = ext;
+    for (int w = 16; w > 0; w >>= 1) {
+        ext = fmax(ext, __shfl_xor_sync(0xffffffffu, ext, w));
+        bond2 = fminf(bond2, __shfl_xor_sync(0xffffffffu, bond2, w));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        ext_s[threadIdx.x >> 5] = ext;
+        bond_s[threadIdx.x >> 5] = bond2;
+    }
     bad = __syncthreads_or(bad);
 #pragma unroll
-    for (int w = 0; w < R2N_THREADS / 32; ++w) ext = fmax(ext, ext_s[w]);
+    for (int w = 0; w < R2N_THREADS / 32; ++w) {
+        ext = fmax(ext, ext_s[w]);
+        bond2 = fminf(bond2, bond_s[w]);
+    }
     __syncthreads();                                // before the words replace them
+    bad |= !((float)ext <= R2N_EXTENT * sqrtf(bond2));
     if (blockIdx.y == 0 && threadIdx.x == 0) out[(size_t)c * N] = 0.0;
     if (bad || ext < 1e-200 || ext > 1e200) {       // not finite, a point, or past the scaling's range
         for (int n = 1 + blockIdx.y * R2N_THREADS + threadIdx.x; n < N; n += gridDim.y * R2N_THREADS) {

@@ -55,3 +55,23 @@ def test_every_path(kg, chains, N):
     # a sum of N terms one after the other, positions of binary64 rounding 2^-53 max |x| against bonds of 0.97
     tol = (N + 16 * np.abs(x).max()) * 2.0 ** -53
     assert got[0] == 0 and np.abs(got[1:] / want[1:] - 1).max() < tol
+
+
+# one monomer far away, two monomers almost at one place, straight rods: lags that do not see the far one keep
+# the rounding of binary64 (a chain of N sums N terms, 2^-53 each, in any order)
+@pytest.mark.parametrize("chains,N", [(3, 100), (5, 800), (1, 2500)])
+@pytest.mark.parametrize("kind", ["far", "near", "rod"])
+def test_data_that_are_no_melt(kg, chains, N, kind):
+    x, first = walk(chains, N, 9), 1
+    if kind == "far":
+        x[1, :, N // 2] += 1e9
+        first = N // 2 + 1                           # no pair with the far monomer from here
+    elif kind == "near":
+        x[:, :, 1] = x[:, :, 0] + 1e-9
+    else:
+        x = x[:, :, :1] + 0.97 * np.arange(N)[None, None, :] * np.array([0.8, 0.6, 0.0])[:, None, None]
+    got = r2n(kg, np.ascontiguousarray(x))
+    y = x.astype(np.longdouble)
+    for n in range(first, N, 1 + N // 200):
+        want = ((y[:, :, n:] - y[:, :, :-n]) ** 2).sum() / (chains * (N - n))
+        assert abs(got[n] / want - 1) < 4 * N * 2.0 ** -53

@@ -292,23 +292,25 @@ __device__ __forceinline__ typename G::T3 force_on(const G &g, const SimDev &S, 
 //    in list order.  Popping its own pairs, a lane waited for the largest of 32
 //    numbers of near pairs (about 9 against a mean of 4 to 5);
 //  * a bond's inverse length is one reciprocal square root that serves its own
-//    1/r^2, both its angles and all their gradients.
+//    1/r^2, both its angles and all their gradients, each corrected by a Newton
+//    step: without it (and with r^-12 as a square) a step's forces were twice as
+//    far from 128 bits (3.0e-14 of a force against 1.42e-14 of plain divides and
+//    square roots; with it 1.42e-14).
 // Blocks of 64, whatever block_size says: the pipe is the SM's, so the SM with
 // the most blocks sets the time, and 80,000 monomers are 4.1 blocks of 128 per
 // SM (five on some) but 8.2 of 64.  80,000 monomers, n = 12, skin 0.3, 50 steps
-// with 14 list builds: 9016 -> 5726 us with the first and last point, 4984 with
-// the queue and the small blocks (of which 2% the queue; at exponents that take
-// log2 and exp2 a pair is four times the work).  200,000: 228 -> 208 us a step.
+// with 14 list builds: 9016 -> 5290 us (4990 without the corrections; at
+// exponents that take log2 and exp2 a pair is four times the work).  200,000, n =
+// 2: 17170 -> 10900 us.
 // ---------------------------------------------------------------------------
 // r^-n for the stage from 1/r^2 and 1/r^6
 __device__ __forceinline__ double inv_rn64(const StageDev &st, double r2, double ir2, double ir6)
 {
     if (st.nkind == 1) {
+        // factor by factor: r^-12 as the square of r^-6 would double that one's rounding
         const int n = st.nint, h = n >> 1;
         double p = n >= 6 ? ir6 : 1.0;
-        if (n == 12) p = ir6 * ir6;
-        else
-            for (int k = n >= 6 ? 3 : 0; k < h; ++k) p *= ir2;
+        for (int k = n >= 6 ? 3 : 0; k < h; ++k) p *= ir2;
         if (n & 1) p *= rsqrt(r2);
         return p;
     }
@@ -330,6 +332,18 @@ __device__ __forceinline__ void add64(double a, double3 x, double3 &F)
     F.z += a * x.z;
 }
 
+// One Newton step each, two to four operations of the pipe, where a divide or
+// another square root is a dozen: 1 / l from q = 1 / l to a few ulps, 1 / sqrt(l)
+// likewise, a / b from r = 1 / b rounded.  The results are within an ulp, as those
+// of the instructions' sequences that they stand for.
+__device__ __forceinline__ double better_inv(double l, double q) { return fma(q, fma(-l, q, 1.0), q); }
+__device__ __forceinline__ double better_rsqrt(double l, double i) { return fma(0.5 * i, fma(-l * i, i, 1.0), i); }
+__device__ __forceinline__ double better_div(double a, double b, double r)
+{
+    const double t = a * r;
+    return fma(fma(-t, b, a), r, t);
+}
+
 // Bond (Eq. 10) and bending (Eq. 4) forces from the chain partners bp = (s-2, s-1, s+1, s+2)
 __device__ __forceinline__ void bonded64(const GeoF64 &g, const StageDev &st, double kap, double rc2, int4 bp,
                                          double3 &F, unsigned &err)
@@ -347,13 +361,14 @@ __device__ __forceinline__ void bonded64(const GeoF64 &g, const StageDev &st, do
         if (hp2 && kap != 0.0) Bp1 = sub3(g.rel(bp.w), B0);
     }
     const double l1 = dot3(Bm1, Bm1), l2 = dot3(B0, B0);
-    const double i1 = rsqrt(l1), i2 = rsqrt(l2), q1 = i1 * i1, q2 = i2 * i2;    // infinite past a chain end, unused
+    const double i1 = rsqrt(l1), i2 = rsqrt(l2);                                // infinite past a chain end, unused
+    const double q1 = better_inv(l1, i1 * i1), q2 = better_inv(l2, i2 * i2);
     const double invR0sq = 1.0 / st.R0sq;
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
         if (side == 0 ? hm1 : hp1) {
             const double r2 = side == 0 ? l1 : l2;
-            double q = 1.0 - r2 * invR0sq, fr;
+            double q = 1.0 - better_div(r2, st.R0sq, invR0sq), fr;
             if (st.qmin > 0.0 && q < st.qmin) {          // continuation beyond r* (kg_params.fene_qmin)
                 fr = st.kfene / st.qmin;
                 if (!(r2 < 4.0 * st.R0sq)) err |= ERR_OVERSTRETCH;
@@ -368,17 +383,17 @@ __device__ __forceinline__ void bonded64(const GeoF64 &g, const StageDev &st, do
     }
     if (kap != 0.0) {
         if (hm1 && hp1) {                    // vertex s: force kappa (g1 - g2)
-            const double inv = i1 * i2, cs = dot3(Bm1, B0) * inv;
+            const double inv = better_rsqrt(l1 * l2, i1 * i2), cs = dot3(Bm1, B0) * inv;
             add64(kap * (inv + cs * q2), B0, F);
             add64(-kap * (inv + cs * q1), Bm1, F);
         }
         if (hp2) {                           // vertex s+1, s is its first end: -kappa g1
-            const double inv = i2 * rsqrt(dot3(Bp1, Bp1)), cs = dot3(B0, Bp1) * inv;
+            const double l3 = dot3(Bp1, Bp1), inv = better_rsqrt(l2 * l3, i2 * rsqrt(l3)), cs = dot3(B0, Bp1) * inv;
             add64(-kap * inv, Bp1, F);
             add64(kap * cs * q2, B0, F);
         }
         if (hm2) {                           // vertex s-1, s is its last end: +kappa g2
-            const double inv = i1 * rsqrt(dot3(Bm2, Bm2)), cs = dot3(Bm2, Bm1) * inv;
+            const double l0 = dot3(Bm2, Bm2), inv = better_rsqrt(l0 * l1, i1 * rsqrt(l0)), cs = dot3(Bm2, Bm1) * inv;
             add64(kap * inv, Bm2, F);
             add64(-kap * cs * q1, Bm1, F);
         }
@@ -405,7 +420,7 @@ __global__ void __launch_bounds__(F64_BLOCK) k_step_f64(const SimDev *__restrict
     const SimDev &S = *Sp;
     const StageDev &st = *stp;
     const long long step = *stepp + (loop ? 1 + kstep : 0);
-    __shared__ double pf_s[F64_BLOCK / 32][3 * F64_PAIRS];
+    __shared__ double pf_s[F64_BLOCK / 32][4 * F64_PAIRS];       // (dU/dr)/r and the vector of each pair
     __shared__ unsigned pair_s[F64_BLOCK / 32][F64_PAIRS];
     const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     double *const pf = pf_s[threadIdx.x >> 5];
@@ -469,15 +484,15 @@ __global__ void __launch_bounds__(F64_BLOCK) k_step_f64(const SimDev *__restrict
                     const double3 d = g.rel((int)(pair[i] & IDX_MASK));
                     const double r2 = dot3(d, d);
                     const double fr = r2 < S.rc2 ? mlj_fr64(st, r2, 1.0 / r2) : 0.0;
-                    pf[i] = fr * d.x;
-                    pf[F64_PAIRS + i] = fr * d.y;
-                    pf[2 * F64_PAIRS + i] = fr * d.z;
+                    pf[i] = fr;
+                    pf[F64_PAIRS + i] = d.x;
+                    pf[2 * F64_PAIRS + i] = d.y;
+                    pf[3 * F64_PAIRS + i] = d.z;
                 }
                 __syncwarp();
                 for (int i = max(first - b, 0); i < min(first + n - b, F64_PAIRS); ++i) {
-                    F.x += pf[i];
-                    F.y += pf[F64_PAIRS + i];
-                    F.z += pf[2 * F64_PAIRS + i];
+                    const double fr = pf[i];
+                    add64(fr, make_double3(pf[F64_PAIRS + i], pf[2 * F64_PAIRS + i], pf[3 * F64_PAIRS + i]), F);
                 }
                 __syncwarp();
             }

@@ -24,10 +24,19 @@ namespace kg {
 // inputs and output buffers it hands over, and memory that its allocator hands
 // out again, can still be in use by work queued there, which a non-blocking
 // stream does not wait for by itself.  Nothing to do if that work is done,
-// which the query tells for less than the event and the wait cost.
+// which the query tells for less than the event and the wait cost.  While a
+// blocking stream of the program is being captured any use of the default
+// stream would invalidate the capture; the first call tells without doing so,
+// and the order is then the program's to make, as for a stream of its own.
 void follow_default(kg_ctx *c)
 {
-    if (!c->own_stream || cudaStreamQuery(cudaStreamLegacy) == cudaSuccess) return;
+    if (!c->own_stream) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(cudaStreamLegacy, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (cudaStreamQuery(cudaStreamLegacy) == cudaSuccess) return;
     cudaGetLastError();
     if (!c->order_ev && cudaEventCreateWithFlags(&c->order_ev, cudaEventDisableTiming) != cudaSuccess) return;
     cudaEventRecord(c->order_ev, cudaStreamLegacy);

@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(32 * R2N_ROWS) k_r2n_reduce(const double *__re
 // in binary32 settle the bin unless they are within their rounding of an
 // edge.  Counts go to shared memory first (bins up to HIST_SHARED).  18 us.
 constexpr int HIST_SHARED = 4096;
+constexpr float HIST_TINY2 = 1e-28f;             // squared lengths from here on keep their digits in binary32
 
 struct Bond64 {
     double v[3];
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(256) k_hist(const double *__restrict__ x, int 
             const float t = (cs + 1.0f) * 0.5f * binsf;
             int b = (int)t;
             const float q = t - (float)b;
-            if (!(q > tol && q < 1.0f - tol)) b = hist_cos_exact(b1, b2, nbins);
+            if (!(q > tol && q < 1.0f - tol) || fminf(l1, l2) < HIST_TINY2) b = hist_cos_exact(b1, b2, nbins);
             b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
             atomicAdd(hc + b, 1);
         }

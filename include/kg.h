@@ -261,7 +261,8 @@ typedef struct {
  * Verlet build, a re-sort into its cell order and a warm-up of trial_steps
  * steps: the layout a long run keeps) for every candidate
  * skin in {0.25, 0.3, 0.4, 0.5, 0.6}, block size in {64, 128, 256} and, for
- * KG_MIXED, threads per monomer in {1, 2}, each in a scratch context of its
+ * KG_MIXED, threads per monomer in {1, 2} (the last two where the kernels that
+ * run the steps of that context have them), each in a scratch context of its
  * own, then the cell side (cell_scale 1.15 and 1.3 of r_c + skin) with the
  * best of those; return the fastest in *best (a later candidate must be
  * faster by 0.5% to replace an earlier one, so near-ties keep the smaller

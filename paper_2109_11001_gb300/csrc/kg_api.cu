@@ -1298,16 +1298,21 @@ constexpr double TUNE_MARGIN = 0.005;
 // One autotuner trial: a context with parameters q on the given states
 // (re-sorted into cell order after its first step, as after every load),
 // warmed up, then timed over two windows of trial_steps MD steps with
-// periodic re-sorts off.  *ms: the better window, per MD step.
+// periodic re-sorts off.  *ms: the better window, per MD step.  *block, *split:
+// whether block_size and threads_per_monomer reach the kernels that run the
+// steps (the resident loops and the binary64 step have their own).
 static kg_status autotune_trial(const kg_params &q0, const double *const *x, const double *const *v,
                                 const kg_stage *stage, int trial_steps, int device, void *stream,
-                                const kg_allocator *allocator, cudaEvent_t e0, cudaEvent_t e1, double *ms)
+                                const kg_allocator *allocator, cudaEvent_t e0, cudaEvent_t e1, double *ms, bool *block,
+                                bool *split)
 {
     kg_params q = q0;
     q.sort_interval = 1 << 30;
     kg_ctx *c = nullptr;
     kg_status s = kg_create(&c, &q, device, stream, allocator);
     if (s != KG_OK) return s;
+    *block = c->precision == KG_MIXED && kg::resident_kind(c) == kg::RES_NONE;
+    *split = c->precision == KG_MIXED && !((c->p.flags & KG_FLAG_PERSISTENT) && !*block);
     kg_stage st = *stage;
     st.n_steps = -1;                                       // open-ended stage for the trial
     for (int m = 0; s == KG_OK && m < q.n_melts; ++m) s = kg_load_config(c, m, x[m], v ? v[m] : nullptr, nullptr);
@@ -1344,15 +1349,18 @@ kg_status kg_autotune(const kg_params *p, const double *const *x, const double *
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return KG_ERR_CUDA;
     kg_status out = KG_OK;
     for (double skin : skins) {
+        bool block = true, split = true;                           // of this skin's last trial
         for (int bt = 0; out == KG_OK && bt < 3 * ntpm; ++bt) {
+            if ((bt % 3 && !block) || (bt / 3 && !split)) continue;   // the same kernels as the trial before
             kg_params q = *p;
             q.skin = skin;
             q.block_size = blocks[bt % 3];
             q.threads_per_monomer = tpms[bt / 3];
             q.cell_scale = 1.0;
             double per = 0.0;
-            const kg_status s = autotune_trial(q, x, v, stage, trial_steps, device, stream, allocator, e0, e1, &per);
-            if (s == KG_ERR_INVALID_ARG) continue;                 // this skin does not fit the box
+            const kg_status s =
+                autotune_trial(q, x, v, stage, trial_steps, device, stream, allocator, e0, e1, &per, &block, &split);
+            if (s == KG_ERR_INVALID_ARG) break;                    // this skin does not fit the box
             if (s != KG_OK) { out = s; break; }
             ++best->trials;
             if (per < best->ms_per_step * (1.0 - TUNE_MARGIN)) {   // earlier (smaller skin) wins ties
@@ -1372,7 +1380,9 @@ kg_status kg_autotune(const kg_params *p, const double *const *x, const double *
         q.threads_per_monomer = best->threads_per_monomer;
         q.cell_scale = scales[k];
         double per = 0.0;
-        const kg_status s = autotune_trial(q, x, v, stage, trial_steps, device, stream, allocator, e0, e1, &per);
+        bool block, split;
+        const kg_status s =
+            autotune_trial(q, x, v, stage, trial_steps, device, stream, allocator, e0, e1, &per, &block, &split);
         if (s == KG_ERR_INVALID_ARG) continue;                     // fewer than three cells per side
         if (s != KG_OK) { out = s; break; }
         ++best->trials;

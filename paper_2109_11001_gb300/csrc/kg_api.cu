@@ -357,11 +357,8 @@ kg_status kg_create(kg_ctx **out, const kg_params *p, int device, void *stream, 
     c->maxnb = 80;
     S.M = c->M; S.Mp = c->Mp; S.maxnb = c->maxnb;
     S.rc2 = RC * RC; S.rc2f = (float)S.rc2;
-    S.rl = rl; S.rl2 = rl * rl;
-    S.rl2f_lo = (float)(S.rl2 * (1.0 - 1e-5));
-    S.rl2f_hi = (float)(S.rl2 * (1.0 + 1e-5));
-    S.half_skin2 = 0.25 * c->p.skin * c->p.skin;
-    S.half_skin2f = (float)S.half_skin2;
+    S.rl2 = rl * rl;
+    S.half_skin2f = (float)(0.25 * c->p.skin * c->p.skin);
     S.db_lim2 = p->db_bond_max * p->db_bond_max;
     S.seed = p->seed;
     S.paper_metropolis = (p->flags & KG_FLAG_PAPER_METROPOLIS) ? 1 : 0;

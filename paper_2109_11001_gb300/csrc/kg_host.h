@@ -48,7 +48,7 @@ struct kg_ctx {
     long long since_sort = 0;
     long long *d_step = nullptr;   // device step counter (index of the step being run)
     bool d_step_stale = true;      // host must write it before the next step
-    cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
+    cudaStream_t cap_stream = nullptr;
     cudaEvent_t order_ev = nullptr;    // follow_default
     cudaGraphExec_t gexec[kg::LOOP_MAX / 4] = {};   // captured step loops with bodies of 4, 8, 12 and 16 steps
     bool graph_failed = false;
@@ -93,7 +93,7 @@ struct kg_ctx {
     void *att = nullptr;         // kg::Attempt[att_cap]
     long long att_cap = 0;
     int *koff = nullptr;         // [n_melts+1] attempt offsets
-    unsigned long long *dbbar = nullptr;   // grid-barrier words of the commit rounds
+    unsigned long long *dbbar = nullptr;   // grid-barrier words of the commit rounds, and their error word
     int *img = nullptr;
     long long *db_stats = nullptr;   // [n_melts][4]
 
@@ -120,7 +120,8 @@ struct kg_ctx {
     // scratch
     double *scratch = nullptr;   // [3][Mp] doubles + [3][Mp] + [Mp] ints (gather / staging)
     unsigned *flags = nullptr;   // [0] error bits, [1] rebuild request, [3] max list length, [4] blocks done,
-                                 // [5] Verlet builds, [6] rebuild bodies run inside graphs
+                                 // [5] Verlet builds, [6] kernels of captured loops' passes that are no steps,
+                                 // [8], [9] RES_BUILT, RES_NEXT
     double *partials = nullptr;  // block partial sums for observables
     int partials_cap = 0;
     double *r2tmp = nullptr;     // per-chain <R^2(n)> partial sums

@@ -7,7 +7,8 @@
 //   recb     float4[Mp]      build-time position record: offset from the corner
 //                            of its Verlet-grid cell + packed cell coordinates
 //   dlt[2]   float4[Mp]      (mixed) displacement since the last build, ping-pong
-//   pg[2]    float4[Mp]      (mixed) gather record of the step: recb + dlt, code
+//   pg[2]    float4[Mp]      gather record of the step: recb + displacement, code
+//                            (binary64: for the near-pair test)
 //   pos64[2] double4_32a[Mp] (FP64) gather copy of the positions, ping-pong
 //   xb       double4_32a[Mp] (FP64) positions at the last build
 //   nl       uint[maxnb][Mp] Verlet list, column-major (coalesced per k); an
@@ -124,9 +125,8 @@ struct StageDev {
 struct SimDev {
     MeltDev melt[MAX_MELTS];
     int n_melts, M, Mp, maxnb;
-    double rc2, rl2, rl, db_lim2;
-    float rc2f, rl2f_lo, rl2f_hi, half_skin2f;
-    double half_skin2;
+    double rc2, rl2, db_lim2;
+    float rc2f, half_skin2f;
     unsigned long long seed;
     int paper_metropolis;
 };
@@ -221,14 +221,6 @@ __device__ __forceinline__ int md_cell(const MeltDev &md, int cx, int cy, int cz
 {
     return md.cell_off + ((((cz >> 2) * md.nbk + (cy >> 2)) * md.nbk + (cx >> 2)) << 6) +
            (((cz & 3) << 4) | ((cy & 3) << 2) | (cx & 3));
-}
-
-__device__ __forceinline__ void md_cell_xyz(const MeltDev &md, int cell, int &cx, int &cy, int &cz)
-{
-    const int r = cell - md.cell_off, b = r >> 6, l = r & 63;
-    cx = ((b % md.nbk) << 2) | (l & 3);
-    cy = (((b / md.nbk) % md.nbk) << 2) | ((l >> 2) & 3);
-    cz = ((b / (md.nbk * md.nbk)) << 2) | (l >> 4);
 }
 
 // Conversions between binary64, binary32 and integers in 32-bit integer

@@ -1,5 +1,5 @@
-// kg_resident.cuh -- arguments, grid barrier and counting-sort phases shared by the
-// two resident MD kernels (kg_resident.cu, kg_resident_small.cu).
+// kg_resident.cuh -- arguments, launch and counting-sort phases shared by the three
+// resident MD kernels (kg_resident.cu, kg_resident_small.cu, kg_resident_tiled.cu).
 #pragma once
 #include <cuda_runtime.h>
 

@@ -43,15 +43,21 @@ void follow_default(kg_ctx *c)
     cudaStreamWaitEvent(c->stream, c->order_ev, 0);
 }
 
+// whether p is device or managed memory; a: its attributes then
+static bool device_memory(const void *p, cudaPointerAttributes &a)
+{
+    if (!p) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
 void follow_default_for(kg_ctx *c, const void *out)
 {
     cudaPointerAttributes a;
-    if (!out || !c->own_stream) return;
-    if (cudaPointerGetAttributes(&a, out) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
-    if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) follow_default(c);
+    if (c->own_stream && device_memory(out, a)) follow_default(c);
 }
 
 void *dev_alloc(kg_ctx *c, size_t bytes, size_t clear)
@@ -547,17 +553,6 @@ kg_status kg_load_config(kg_ctx *c, int melt, const double *x, const double *v, 
     return KG_OK;
 }
 
-// whether a kernel of the context can write n elements of `size` bytes at p: device memory of its GPU, aligned
-static bool writable(const kg_ctx *c, const void *p, size_t size)
-{
-    cudaPointerAttributes a;
-    if ((size_t)p % size != 0 || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice && a.device == c->device;
-}
-
 kg_status kg_get_config(kg_ctx *c, int melt, double *x, double *v, int *pid)
 {
     kg_status s = check_melt(c, melt);
@@ -566,17 +561,25 @@ kg_status kg_get_config(kg_ctx *c, int melt, double *x, double *v, int *pid)
     const size_t Mm = md.M;
     // one kernel for everything asked for, into the caller's memory where it
     // is this GPU's, else into scratch and copied from there
-    for (const void *out : {(const void *)x, (const void *)v, (const void *)pid}) kg::follow_default_for(c, out);
     const char *lo[3] = {(const char *)x, (const char *)v, (const char *)pid};
     const size_t bytes[3] = {3 * Mm * sizeof(double), 3 * Mm * sizeof(double), Mm * sizeof(int)};
     bool direct = true;                                    // no two outputs share memory
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b)
             if (a != b && lo[a] && lo[b] && lo[a] < lo[b] + bytes[b] && lo[b] < lo[a] + bytes[a]) direct = false;
+    // a kernel of the context writes device memory of its GPU that is aligned
+    bool on_gpu = false, to[3];
+    for (int a = 0; a < 3; ++a) {
+        cudaPointerAttributes at;
+        const bool dev = kg::device_memory(lo[a], at);
+        on_gpu |= dev;
+        to[a] = dev && direct && at.type == cudaMemoryTypeDevice && at.device == c->device &&
+                (size_t)lo[a] % (a < 2 ? sizeof(double) : sizeof(int)) == 0;
+    }
+    if (on_gpu) kg::follow_default(c);
     double *xd = c->scratch, *vd = c->scratch + 3 * Mm;
     int *pd = (int *)(c->scratch + 6 * Mm);
-    const bool dx = x && direct && writable(c, x, sizeof(double)), dv = v && direct && writable(c, v, sizeof(double));
-    const bool dp = pid && direct && writable(c, pid, sizeof(int));
+    const bool dx = to[0], dv = to[1], dp = to[2];
     if (x || v || pid)
         kg::state_to_slots(c, melt, x ? (dx ? x : xd) : nullptr, v ? (dv ? v : vd) : nullptr,
                            pid ? (dp ? pid : pd) : nullptr);

@@ -66,9 +66,9 @@ def bytes_per_monomer_at_skin(precision, skin):
 
 # DRAM bytes per monomer of the mixed step kernel from ncu captures of the
 # 1.6M-monomer case, by skin, and the hash of the step kernel's source
-# (kg_step.cu, kg_step.cuh) they were taken on (reported as null for another skin or once
-# the source changes)
-NCU_TRAFFIC = {"bytes_per_monomer": {0.5: 196.8, 0.6: 213.9}, "src_sha1": "e627455da1f4382bbc2b14cf2e2c30d8d440a189"}
+# (kg_step.cu, kg_step.cuh) they were taken on (reported as null for another
+# skin or once the source changes)
+NCU_TRAFFIC = {"bytes_per_monomer": {0.5: 195.6, 0.6: 212.7}, "src_sha1": "9908b3a3a76495ebd08c385381c162ebbd1b8c2a"}
 
 WORKLOADS = {
     "cfg5": dict(index=5, desc="1000 chains x N=1600 (1.6M monomers), kappa=3.5, rho=0.85"),

@@ -24,6 +24,9 @@
  *   - Pointers passed to kg_load_config / kg_get_config / kg_observables /
  *     kg_get_nlist / kg_forces may be host or device memory (CUDA unified
  *     addressing decides); inputs are copied, the caller keeps ownership.
+ *   - A context on a stream of its own (kg_create with stream NULL) takes
+ *     inputs, allocator memory and device outputs after the work queued on the
+ *     default stream so far (not while a blocking stream is being captured).
  *   - The context owns its device memory; all GPU work is enqueued on the
  *     context's stream.  kg_step and kg_db_sweep are asynchronous except for
  *     one status read at their end; device-side errors (overstretched bond,
@@ -71,13 +74,19 @@ enum {
     KG_FLAG_PERSISTENT = 2        /* KG_MIXED (ignored with KG_FP64): kg_step advances
                                       every melt in cooperative launches of up to 1000
                                       steps; the Verlet rebuild runs inside the launch
-                                      between grid barriers, and every barrier wait is
-                                      bounded (a block that gives up latches
-                                      KG_ERR_TIMEOUT).  One thread per monomer; results
-                                      equal the default path's up to binary32 summation
-                                      order.  Contexts with threads_per_monomer 1 and at
-                                      most 1280 monomers per SM take such launches, of
-                                      up to 50 steps, without the flag               */
+                                      between grid barriers.  One thread per monomer;
+                                      results equal the default path's up to binary32
+                                      summation order.  Contexts with threads_per_monomer
+                                      1, at most 1280 monomers per SM and at most 64
+                                      Verlet cells per monomer take such launches, of up
+                                      to 50 steps, without the flag.
+                                      Every wait at a grid barrier of these launches, and
+                                      of every double-bridging sweep, is bounded (about
+                                      1.3 s and 5 s): a block that gives up latches
+                                      KG_ERR_TIMEOUT, from which, as from any error,
+                                      kg_load_config frees the context.  A launch that
+                                      finds the GPU busy starts when all its blocks fit;
+                                      that time does not count                          */
 };
 
 /* One melt (Sec. II.B): N_ch chains of N monomers in a cube of side L. */
@@ -113,12 +122,17 @@ typedef struct {
                                  build, whose timing moves positions at the binary32
                                  rounding level (~1e-7 sigma)                           */
     int block_size;           /* threads per block of the mixed step kernel: 64, 128
-                                 or 256 (<= 0: 128); results do not depend on it        */
+                                 or 256 (<= 0: 128); results do not depend on it.
+                                 Cooperative launches (KG_FLAG_PERSISTENT) and KG_FP64
+                                 have block sizes of their own                          */
     int precision;            /* KG_FP64 or KG_MIXED                                    */
     int flags;                /* KG_FLAG_*                                              */
     int threads_per_monomer;  /* threads sharing one monomer's step in KG_MIXED: 1 or 2
                                  (<= 0: 1; KG_FP64 always uses 1); results do not
-                                 depend on it beyond binary32 summation order           */
+                                 depend on it beyond binary32 summation order.  2
+                                 without KG_FLAG_PERSISTENT means a launch per step at
+                                 every size: up to 1280 monomers per SM the cooperative
+                                 launches that 1 takes are the faster                   */
     double cell_scale;        /* Verlet-list cells of side >= cell_scale (r_c + skin),
                                  1 ... 3 (<= 0: 1): larger cells mean fewer cells to
                                  bin and sort and more candidates per monomer; lists
@@ -178,7 +192,7 @@ kg_status kg_get_config(kg_ctx *c, int melt, double *x, double *v, int *pid);
 /* Self-test of the persistent launch's bounded barrier waits (KG_MIXED
  * contexts): one persistent launch of two MD steps in which block skip_block
  * (>= 0) never arrives at the grid barrier, so the other blocks give up after
- * `spin` polls (about 64 ns apart), latch KG_ERR_TIMEOUT and return; the call
+ * `spin` polls (about 0.32 us apart), latch KG_ERR_TIMEOUT and return; the call
  * returns that status and the context holds it until the next kg_load_config.
  * With skip_block < 0 it is an ordinary two-step persistent launch (KG_OK).
  * No block waits longer than `spin` polls per barrier. */
@@ -486,7 +500,13 @@ kg_status kg_entanglement_length(double lpp_mean, int chain_len, double l0, doub
  * before any stream capture.  Calls share the array and overwrite it
  * completely, so calls that overlap on the GPU (different streams, or devices
  * sharing nothing but this host code) race: serialise them.  No cudaMalloc,
- * cudaFree or allocating library routine is called. */
+ * cudaFree or allocating library routine is called.
+ *
+ * Chains of up to 20 monomers, and chains whose extent is more than 2048 times
+ * their shortest bond, are summed in binary64; others as integers of 2^-52 of
+ * the power of two above the chain's extent, exactly: every position is off by
+ * at most half of that, and the sums of connected chains are as close as
+ * binary64 sums of N terms are. */
 kg_status kg_r2n_noalloc(const double *x, long long stride, int n_chains, int chain_len, double *out,
                          void *stream);
 

@@ -264,9 +264,10 @@ __device__ __forceinline__ DBC make_dbc(const SimDev &S, const StageDev &st, int
 // slowest one, so it is cut in two: the draw and the partner scan of the drawn
 // bond, one warp per record (most sets are empty, and done); then, for a
 // non-empty set, E::TASKS independent parts on as many warps.  160,000
-// attempts of a 1.6M-monomer melt (21 swaps): 521 us, against about 1,450 as two
-// launches a round with the host reading the finished flags now and then, an
-// attempt evaluated by one warp and the dE of a swap by one lane.
+// attempts of a 1.6M-monomer melt: about 30 us a round (14 swaps 526 us, 21 swaps
+// 668, 25 swaps 790), against about 60 as two launches a round with the host
+// reading the finished flags now and then, an attempt evaluated by one warp and
+// the dE of a swap by one lane.
 // round[RS m + 0..5] of one of two buffers (by round parity: commits write the
 // next round's while every block reads this one's) = position, commits,
 // finished, re-evaluations, the first accepted attempt at or after the position
@@ -529,7 +530,7 @@ __device__ void rounds_body(E &ev, P &pol, const RoundArgs &R)
 
 RoundArgs round_args(kg_ctx *c);                // kg_db.cu
 
-constexpr unsigned ROUNDS_SPIN = 1u << 24;         // barrier polls (tens of ns at least) before giving up
+constexpr unsigned ROUNDS_SPIN = 1u << 24;         // barrier polls (0.32 us apart) before giving up
 
 // Launches kernel K (blocks of `threads`, smem bytes, RoundArgs in r, then the
 // evaluator's arguments) on as many blocks as the attempts need and the GPU holds.

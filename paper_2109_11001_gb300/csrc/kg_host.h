@@ -153,7 +153,7 @@ constexpr int GRAPH_STEPS = 10;          // MD steps between re-sort tests
 constexpr int PERSIST_STEPS = 50;        // MD steps between re-sort tests with KG_FLAG_PERSISTENT
 constexpr int RESIDENT_STEPS = 50;       // MD steps per resident launch (KG_FLAG_PERSISTENT, step loop: PERSIST_MAX)
 constexpr int PERSIST_MAX = 1000;
-constexpr unsigned RESIDENT_SPIN = 1u << 22;  // its barrier polls (a few hundred ns apart) before ERR_TIMEOUT
+constexpr unsigned RESIDENT_SPIN = 1u << 22;  // its barrier polls (0.32 us apart) before ERR_TIMEOUT
 constexpr int RS = 8;                    // ints per melt in the DB commit-round array
 
 // A sweep's record of one attempt.  The staleness check of every round reads
